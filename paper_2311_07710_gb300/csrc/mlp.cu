@@ -424,53 +424,197 @@ __device__ __forceinline__ long long visit(long long a, long long s, long long c
   return (a * i + s) % count;
 }
 
+// The elementwise kernels below take W columns per thread (two, in 16-byte
+// accesses, where n and m are even) and ROWS_PER rows per grid y: the
+// per-feature constants are read (and converted) once, no index is divided,
+// and the rows' loads are in flight together.  What bounds them is memory or,
+// where a value is converted, GB300's float64 pipe (two lanes per clock per
+// SM, conversions included).
+constexpr int ROWS_PER = 16;
+constexpr int BATCH = 8;            // rows loaded before the first is used
+
+template <int W>
+__device__ __forceinline__ void load_cols(const double* __restrict__ p, double (&v)[W]) {
+  if constexpr (W == 2) {
+    const double2 q = __ldcs(reinterpret_cast<const double2*>(p));
+    v[0] = q.x;
+    v[1] = q.y;
+  } else {
+    v[0] = __ldcs(p);
+  }
+}
+
 // u = bf16((fl32(v) - mean) * scale) for rows [row0, row0+rows) of v = [C | B]
-__global__ void k_prep_input(const double* __restrict__ C, const double* __restrict__ B, int n, int m, long long row0,
-                             int rows, const float* __restrict__ mean, const float* __restrict__ scale,
-                             bf16* __restrict__ U, int ldu) {
-  const int F = n + m;
-  const long long total = (long long)rows * F;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    const int r = (int)(i / F), f = (int)(i % F);
-    const long long smp = row0 + r;
-    const double v = f < n ? C[smp * n + f] : B[smp * m + (f - n)];
-    U[(size_t)r * ldu + f] = __float2bfloat16_rn(__fmul_rn(__fsub_rn((float)v, mean[f]), scale[f]));
+template <int W>
+__global__ void __launch_bounds__(256)
+    k_prep_input(const double* __restrict__ C, const double* __restrict__ B, int n, int m, long long row0, int rows,
+                 const float* __restrict__ mean, const float* __restrict__ scale, bf16* __restrict__ U, int ldu) {
+  const int f = (blockIdx.x * 256 + threadIdx.x) * W;
+  if (f >= n + m) return;
+  const double* src = f < n ? C + (size_t)row0 * n + f : B + (size_t)row0 * m + (f - n);
+  const size_t ld = f < n ? n : m;
+  float mu[W], sc[W];
+#pragma unroll
+  for (int i = 0; i < W; ++i) { mu[i] = mean[f + i]; sc[i] = scale[f + i]; }
+  const int r1 = min(rows, (int)(blockIdx.y + 1) * ROWS_PER);
+  for (int r = blockIdx.y * ROWS_PER; r < r1; r += BATCH) {
+    double v[BATCH][W];
+#pragma unroll
+    for (int k = 0; k < BATCH; ++k)
+      if (r + k < r1) load_cols<W>(src + (r + k) * ld, v[k]);
+#pragma unroll
+    for (int k = 0; k < BATCH; ++k) {
+      if (r + k >= r1) break;
+      bf16 h[W];
+#pragma unroll
+      for (int i = 0; i < W; ++i) h[i] = __float2bfloat16_rn(__fmul_rn(__fsub_rn((float)v[k][i], mu[i]), sc[i]));
+      bf16* d = U + (size_t)(r + k) * ldu + f;
+      if constexpr (W == 2) *reinterpret_cast<__nv_bfloat162*>(d) = __nv_bfloat162(h[0], h[1]);
+      else *d = h[0];
+    }
   }
 }
 
 // t = (fl32(v) - omean) * oinv, float32, for rows [0, count) of [X | Y]
-__global__ void k_prep_target(const double* __restrict__ X, const double* __restrict__ Y, int n, int m,
-                              long long count, const float* __restrict__ omean, const float* __restrict__ oinv,
-                              float* __restrict__ T, int ldt) {
-  const int F = n + m;
-  const long long total = count * F;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    const long long r = i / F;
-    const int f = (int)(i % F);
-    const double v = f < n ? X[r * n + f] : Y[r * m + (f - n)];
-    T[r * ldt + f] = __fmul_rn(__fsub_rn((float)v, omean[f]), oinv[f]);
+template <int W>
+__global__ void __launch_bounds__(256)
+    k_prep_target(const double* __restrict__ X, const double* __restrict__ Y, int n, int m, long long count,
+                  const float* __restrict__ omean, const float* __restrict__ oinv, float* __restrict__ T, int ldt) {
+  const int f = (blockIdx.x * 256 + threadIdx.x) * W;
+  if (f >= n + m) return;
+  const double* src = f < n ? X + f : Y + (f - n);
+  const size_t ld = f < n ? n : m;
+  float mu[W], sc[W];
+#pragma unroll
+  for (int i = 0; i < W; ++i) { mu[i] = omean[f + i]; sc[i] = oinv[f + i]; }
+  for (long long b = blockIdx.y; b * ROWS_PER < count; b += gridDim.y) {
+    const long long r1 = min(count, (b + 1) * ROWS_PER);
+    for (long long r = b * ROWS_PER; r < r1; r += BATCH) {
+      double v[BATCH][W];
+#pragma unroll
+      for (int k = 0; k < BATCH; ++k)
+        if (r + k < r1) load_cols<W>(src + (r + k) * ld, v[k]);
+#pragma unroll
+      for (int k = 0; k < BATCH; ++k) {
+        if (r + k >= r1) break;
+        float t[W];
+#pragma unroll
+        for (int i = 0; i < W; ++i) t[i] = __fmul_rn(__fsub_rn((float)v[k][i], mu[i]), sc[i]);
+        if constexpr (W == 2) *reinterpret_cast<float2*>(T + (r + k) * ldt + f) = make_float2(t[0], t[1]);
+        else T[(r + k) * ldt + f] = t[0];
+      }
+    }
   }
 }
 
-// per-feature mean and population std over `count` rows (two passes, float64);
-// std below 1e-8 counts as 1
-__global__ void k_fit_stats(const double* __restrict__ V, long long count, int nf, float* __restrict__ mean,
-                            float* __restrict__ scale, float* __restrict__ stdv) {
-  const int f = blockIdx.x * blockDim.x + threadIdx.x;
+// The sum of (hi, lo) and x, the rounding error kept (Knuth's two-sum), plus a
+// low-order term.
+__device__ __forceinline__ void pair_add(float& hi, float& lo, float x, float xl) {
+  const float t = __fadd_rn(hi, x), b = __fsub_rn(t, hi);
+  const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, b)), __fsub_rn(x, b));
+  hi = t;
+  lo = __fadd_rn(lo, __fadd_rn(e, xl));
+}
+
+// Per-feature mean and sum of squared deviations of a range of rows, one pass:
+// deviations from the range's first row.  That row is one of the data, so its
+// squared distance from the mean is at most FIT_ROWS times the range's
+// variance, and the cancellation in M2 costs at most about that factor of a
+// rounding.  In float64 the pass takes three float64-pipe operations a value
+// (1.27 ms for 4096 x 60000 values at that pipe's rate); it takes the difference
+// there, and the sums run on float32 pairs: the difference's bits split into
+// 24 + 23 (truncated at 2^-46 of it), products and sums with their exact
+// rounding errors.  Values whose square or its error leaves float32's range
+// take the float64 sums.  Two arrays per launch (grid z) and short ranges, so
+// that the blocks fill whole waves (ranges of 256 rows, one array a launch: a
+// little over two waves, 1.48 ms; the two-pass form before, 157 blocks of one
+// column per thread: 4.8 ms).
+constexpr int FIT_ROWS = 64;
+struct FitPair {
+  const double* v[2];
+  double* mean[2];       // [ranges x nf]
+  double* m2[2];
+};
+__global__ void __launch_bounds__(256) k_fit_part(FitPair a, long long count, int nf) {
+  const int f = blockIdx.x * 256 + threadIdx.x;
   if (f >= nf) return;
-  double s = 0.0;
-  for (long long r = 0; r < count; ++r) s += V[r * nf + f];
-  const double mu = s / (double)count;
-  double q = 0.0;
-  for (long long r = 0; r < count; ++r) {
-    const double d = V[r * nf + f] - mu;
-    q += d * d;
+  const double* V = a.v[blockIdx.z];
+  for (long long b = blockIdx.y; b * FIT_ROWS < count; b += gridDim.y) {
+    const long long r0 = b * FIT_ROWS;
+    const int rows = (int)min((long long)FIT_ROWS, count - r0);
+    const double* p = V + (size_t)r0 * nf + f;
+    const double K = isfinite(p[0]) ? p[0] : 0.0;
+    float sh = 0.f, sl = 0.f, qh = 0.f, ql = 0.f;
+    double sd = 0.0, qd = 0.0;
+    for (int r = 0; r < rows; r += BATCH) {
+      double v[BATCH];                             // all in flight before the first is used
+#pragma unroll
+      for (int k = 0; k < BATCH; ++k) v[k] = r + k < rows ? __ldcs(p + (size_t)(r + k) * nf) : K;
+#pragma unroll
+      for (int k = 0; k < BATCH; ++k) {            // (a row past the end adds 0)
+        const double d = v[k] - K;
+        const unsigned hw = (unsigned)__double2hiint(d), lw = (unsigned)__double2loint(d);
+        const unsigned e = (hw >> 20) & 0x7FFu, sg = hw & 0x80000000u;
+        if (e - 973u <= 113u) {                    // 2^-50 <= |d| < 2^64
+          const float hi = __uint_as_float(sg | ((e - 896u) << 23) | (__funnelshift_l(lw, hw, 3) & 0x7FFFFFu));
+          const float lo = __fmul_rn(__fsub_rn(__uint_as_float(0x4B000000u | ((lw >> 6) & 0x7FFFFFu)), 8388608.f),
+                                     __uint_as_float(sg | ((e - 942u) << 23)));
+          pair_add(sh, sl, hi, lo);
+          const float q = __fmul_rn(hi, hi);
+          pair_add(qh, ql, q, __fmaf_rn(__fadd_rn(hi, hi), lo, __fmaf_rn(hi, hi, -q)));
+        } else if (((hw << 1) | lw) != 0u) {       // not a zero
+          sd += d;
+          qd = fma(d, d, qd);
+        }
+      }
+    }
+    const double s = (double)sh + (double)sl + sd, q = (double)qh + (double)ql + qd;
+    const double c = s * (1.0 / (double)rows), t = fma(-s, c, q);
+    a.mean[blockIdx.z][(size_t)b * nf + f] = K + c;
+    a.m2[blockIdx.z][(size_t)b * nf + f] = t < 0.0 ? 0.0 : t;    // (a NaN stays one)
   }
+}
+
+// the ranges merged in order (Chan, Golub & LeVeque 1983): per-feature mean and
+// population std over all rows; std below 1e-8 counts as 1.  The merge weights
+// are the same for every feature: the block's threads form 128 at a time.
+struct FitOut {
+  float* mean[2];
+  float* scale[2];
+  float* stdv[2];        // null: not kept
+};
+__global__ void __launch_bounds__(128) k_fit_merge(FitPair a, long long count, int nf, FitOut o) {
+  __shared__ double sw[128], sv[128];
+  const int f = blockIdx.x * 128 + threadIdx.x;
+  const double *pm = a.mean[blockIdx.z], *p2 = a.m2[blockIdx.z];
+  const long long nb = (count + FIT_ROWS - 1) / FIT_ROWS;
+  double mu = 0.0, q = 0.0;
+  if (f < nf) { mu = pm[f]; q = p2[f]; }
+  for (long long b0 = 1; b0 < nb; b0 += 128) {
+    const long long b = b0 + threadIdx.x;
+    __syncthreads();
+    if (b < nb) {
+      const double na = (double)(b * FIT_ROWS), c = (double)min((long long)FIT_ROWS, count - b * FIT_ROWS);
+      sw[threadIdx.x] = c / (na + c);
+      sv[threadIdx.x] = na * c / (na + c);
+    }
+    __syncthreads();
+    if (f >= nf) continue;
+    const int n = (int)min(128LL, nb - b0);
+#pragma unroll 4
+    for (int i = 0; i < n; ++i) {
+      const double mb = pm[(size_t)(b0 + i) * nf + f], d = mb - mu;
+      mu = isfinite(d) ? fma(d, sw[i], mu) : mu + mb;    // an infinite mean stays one
+      q = fma(d * d, sv[i], q + p2[(size_t)(b0 + i) * nf + f]);
+    }
+  }
+  if (f >= nf) return;
   double sd = sqrt(q / (double)count);
   if (sd < 1e-8) sd = 1.0;
-  mean[f] = (float)mu;
-  scale[f] = (float)(1.0 / sd);
-  if (stdv) stdv[f] = (float)sd;
+  const int z = blockIdx.z;
+  o.mean[z][f] = (float)mu;
+  o.scale[z][f] = (float)(1.0 / sd);
+  if (o.stdv[z]) o.stdv[z][f] = (float)sd;
 }
 
 __global__ void k_gather_rows(const bf16* __restrict__ src, int ld, long long a, long long s, long long count,
@@ -498,19 +642,34 @@ __global__ void __launch_bounds__(256) k_grad_tiles(const float* __restrict__ in
                                                     float* __restrict__ colpart, int ldc, double* __restrict__ lossp) {
   __shared__ float tile[32][33];
   __shared__ double red[8];
+  __shared__ long long smp_of[32];
   const int f0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int f = f0 + tx;
-  double ls = 0.0;
+  // the squared error in float32 pairs (product and sum with their exact
+  // rounding errors, about 2^-48 relative): a thread's four terms would take
+  // eight float64-pipe operations (conversions included), one conversion pair
+  // here; terms whose square or its error leaves float32's range go to ld
+  float lh = 0.f, ll = 0.f;
+  double ld = 0.0;
+  if (MODE == 0) {   // the rows' samples, one 64-bit remainder each
+    if (ty == 0 && r0 + tx < rows) smp_of[tx] = visit(a, sft, count, row0 + r0 + tx);
+    __syncthreads();
+  }
+#pragma unroll
   for (int i = ty; i < 32; i += 8) {
     const int r = r0 + i;
     float g = 0.f;
     if (r < rows && f < F) {
       const float o = in[(size_t)r * ldi + f];
       if (MODE == 0) {
-        const long long smp = visit(a, sft, count, row0 + r);
-        const float d = __fsub_rn(o, T[(size_t)smp * ldt + f]);
-        ls += (double)d * (double)d;
+        const float d = __fsub_rn(o, T[(size_t)smp_of[i] * ldt + f]);
+        if (fabsf(d) > 1e-10f && fabsf(d) < 1e15f) {
+          const float ph = __fmul_rn(d, d);
+          pair_add(lh, ll, ph, __fmaf_rn(d, d, -ph));
+        } else {
+          ld += (double)d * (double)d;
+        }
         g = __fmul_rn(d, scale);
       } else {
         g = o;
@@ -530,8 +689,13 @@ __global__ void __launch_bounds__(256) k_grad_tiles(const float* __restrict__ in
     if (ff < F && rr < rows) gt[(size_t)ff * ldgt + rr] = __float2bfloat16_rn(tile[tx][i]);
   }
   if (MODE == 0) {
-    for (int o = 16; o > 0; o >>= 1) ls += __shfl_down_sync(0xffffffffu, ls, o);
-    if (tx == 0) red[ty] = ls;
+    for (int o = 16; o > 0; o >>= 1) {
+      const float xh = __shfl_down_sync(0xffffffffu, lh, o), xl = __shfl_down_sync(0xffffffffu, ll, o);
+      pair_add(lh, ll, xh, xl);
+    }
+    if (__any_sync(0xffffffffu, ld != 0.0))       // warp-uniform (a NaN too)
+      for (int o = 16; o > 0; o >>= 1) ld += __shfl_down_sync(0xffffffffu, ld, o);
+    if (tx == 0) red[ty] = (double)lh + (double)ll + ld;
     __syncthreads();
     if (tx == 0 && ty == 0) {
       double t = 0.0;
@@ -549,18 +713,21 @@ __global__ void k_colsum(const float* __restrict__ part, int ntiles, int F, int 
   out[f] = s;
 }
 
-// acc += inv * sum(parts) (one block of 256 threads, fixed order)
-__global__ void k_loss_acc(const double* __restrict__ parts, int n, double inv, double* __restrict__ acc) {
-  __shared__ double red[256];
+// acc += inv * sum(parts) (one block of 1024 threads, fixed order)
+__global__ void __launch_bounds__(1024) k_loss_acc(const double* __restrict__ parts, int n, double inv,
+                                                   double* __restrict__ acc) {
+  __shared__ double red[32];
   double s = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) s += parts[i];
-  red[threadIdx.x] = s;
+#pragma unroll 4
+  for (int i = threadIdx.x; i < n; i += 1024) s += parts[i];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
+  if (threadIdx.x < 32) {
+    s = red[threadIdx.x];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (threadIdx.x == 0) *acc += inv * s;
   }
-  if (threadIdx.x == 0) *acc += inv * red[0];
 }
 
 __global__ void k_transpose_bf16(const bf16* __restrict__ in, int ldi, int rows, int cols, bf16* __restrict__ out,
@@ -589,35 +756,56 @@ __device__ __forceinline__ float adam_one(float w, float g, float& m, float& v, 
   return w - a.lr * (m * a.c1) / (sqrtf(v * a.c2) + a.eps);
 }
 
-// Adam on a rows x cols weight (all float32 arrays row-major, ld = cols), then
-// the bf16 copy [rows x ldb] and the transposed bf16 copy [cols x ldt].
+// Adam on a rows x cols weight (all float32 arrays row-major, ld = cols, a
+// multiple of 4), then the bf16 copy [rows x ldb] and the transposed bf16 copy
+// [cols x ldt].  Bound by memory (28 bytes read and written per weight and 4
+// for the copies): 64 x 64 tiles, four columns per thread in 16-byte accesses,
+// the transposed copy in 128-byte runs.
+constexpr int ADAM_T = 64;
 __global__ void __launch_bounds__(256) k_adam_mat(float* __restrict__ W, float* __restrict__ mW,
                                                   float* __restrict__ vW, const float* __restrict__ g, int rows,
                                                   int cols, AdamArgs a, bf16* __restrict__ Wb, int ldb,
                                                   bf16* __restrict__ Wt, int ldt) {
-  __shared__ bf16 t[32][34];
-  const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-    const int r = r0 + i, c = c0 + threadIdx.x;
+  __shared__ bf16 t[ADAM_T][ADAM_T + 2];          // [column][row]
+  const int c0 = blockIdx.x * ADAM_T, r0 = blockIdx.y * ADAM_T;
+  const int cl = (threadIdx.x & 15) * 4, c = c0 + cl;
+#pragma unroll
+  for (int k = 0; k < ADAM_T / 16; ++k) {
+    const int rl = (threadIdx.x >> 4) + 16 * k, r = r0 + rl;
     if (r < rows && c < cols) {
-      const size_t k = (size_t)r * cols + c;
-      float w = W[k];
+      const size_t o = (size_t)r * cols + c;
+      float4 w = *reinterpret_cast<const float4*>(W + o);
       if (a.update) {
-        float m = mW[k], v = vW[k];
-        w = adam_one(w, g[k], m, v, a);
-        W[k] = w;
-        mW[k] = m;
-        vW[k] = v;
+        float4 m = *reinterpret_cast<const float4*>(mW + o), v = *reinterpret_cast<const float4*>(vW + o);
+        const float4 gg = *reinterpret_cast<const float4*>(g + o);
+        w.x = adam_one(w.x, gg.x, m.x, v.x, a);
+        w.y = adam_one(w.y, gg.y, m.y, v.y, a);
+        w.z = adam_one(w.z, gg.z, m.z, v.z, a);
+        w.w = adam_one(w.w, gg.w, m.w, v.w, a);
+        *reinterpret_cast<float4*>(W + o) = w;
+        *reinterpret_cast<float4*>(mW + o) = m;
+        *reinterpret_cast<float4*>(vW + o) = v;
       }
-      const bf16 h = __float2bfloat16_rn(w);
-      Wb[(size_t)r * ldb + c] = h;
-      t[i][threadIdx.x] = h;
+      const __nv_bfloat162 h0 = __floats2bfloat162_rn(w.x, w.y), h1 = __floats2bfloat162_rn(w.z, w.w);
+      uint2 q;
+      q.x = *reinterpret_cast<const uint32_t*>(&h0);
+      q.y = *reinterpret_cast<const uint32_t*>(&h1);
+      *reinterpret_cast<uint2*>(Wb + (size_t)r * ldb + c) = q;
+      t[cl][rl] = h0.x;
+      t[cl + 1][rl] = h0.y;
+      t[cl + 2][rl] = h1.x;
+      t[cl + 3][rl] = h1.y;
     }
   }
   __syncthreads();
-  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-    const int c = c0 + i, r = r0 + threadIdx.x;
-    if (r < rows && c < cols) Wt[(size_t)c * ldt + r] = t[threadIdx.x][i];
+  const int rp = (threadIdx.x & 31) * 2;          // ldt is even and r0 + rp too: 4-byte stores
+#pragma unroll
+  for (int k = 0; k < ADAM_T / 8; ++k) {
+    const int cc = (threadIdx.x >> 5) + 8 * k;
+    if (c0 + cc >= cols || r0 + rp >= rows) continue;
+    bf16* d = Wt + (size_t)(c0 + cc) * ldt + r0 + rp;
+    if (r0 + rp + 1 < rows) *reinterpret_cast<uint32_t*>(d) = *reinterpret_cast<const uint32_t*>(&t[cc][rp]);
+    else *d = t[cc][rp];
   }
 }
 
@@ -639,20 +827,54 @@ __global__ void k_f32_to_bf16_2d(const float* __restrict__ in, int rows, int col
   }
 }
 
-// [x0 | y0] = omean + ostd * o in float64, rows [row0, row0+rows)
-__global__ void k_write_pred(const float* __restrict__ O, int ldo, int rows, int n, int m,
-                             const float* __restrict__ omean, const float* __restrict__ ostd, long long row0,
-                             double* __restrict__ X0, double* __restrict__ Y0) {
-  const int F = n + m;
-  const long long total = (long long)rows * F;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    const int r = (int)(i / F), f = (int)(i % F);
-    const double v = __dadd_rn((double)omean[f], __dmul_rn((double)ostd[f], (double)O[(size_t)r * ldo + f]));
-    const long long smp = row0 + r;
-    if (f < n) {
-      if (X0) X0[smp * n + f] = v;
-    } else if (Y0) {
-      Y0[smp * m + (f - n)] = v;
+// float -> double by integer instructions (the conversion instruction issues on
+// the float64 pipe): the same value for every float (NaN payloads aside)
+__device__ __forceinline__ double widen(float x) {
+  const unsigned u = __float_as_uint(x), e = (u >> 23) & 0xFFu;
+  if (e - 1u >= 254u) return (double)x;           // zero, subnormal, infinite, NaN
+  return __hiloint2double((int)((u & 0x80000000u) | (((u >> 3) & 0x0FFFFFFFu) + 0x38000000u)), (int)(u << 29));
+}
+
+// [x0 | y0] = omean + ostd * o in float64, rows [row0, row0+rows).  The product
+// of two floats is exact in float64, so one fused multiply-add rounds like the
+// separate addition: one float64-pipe operation per value instead of five.
+template <int W>
+__global__ void __launch_bounds__(256)
+    k_write_pred(const float* __restrict__ O, int ldo, int rows, int n, int m, const float* __restrict__ omean,
+                 const float* __restrict__ ostd, long long row0, double* __restrict__ X0, double* __restrict__ Y0) {
+  const int f = (blockIdx.x * 256 + threadIdx.x) * W;
+  if (f >= n + m) return;
+  double* dst = f < n ? X0 : Y0;
+  if (!dst) return;
+  const size_t ld = f < n ? n : m;
+  dst += (size_t)row0 * ld + (f < n ? f : f - n);
+  double mu[W], sd[W];
+#pragma unroll
+  for (int i = 0; i < W; ++i) { mu[i] = (double)omean[f + i]; sd[i] = (double)ostd[f + i]; }
+  const int r1 = min(rows, (int)(blockIdx.y + 1) * ROWS_PER);
+  for (int r = blockIdx.y * ROWS_PER; r < r1; r += BATCH) {
+    float o[BATCH][W];
+#pragma unroll
+    for (int k = 0; k < BATCH; ++k) {
+      if (r + k >= r1) break;
+      const float* p = O + (size_t)(r + k) * ldo + f;
+      if constexpr (W == 2) {
+        const float2 q = __ldcs(reinterpret_cast<const float2*>(p));
+        o[k][0] = q.x;
+        o[k][1] = q.y;
+      } else {
+        o[k][0] = __ldcs(p);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < BATCH; ++k) {
+      if (r + k >= r1) break;
+      double* d = dst + (r + k) * ld;
+      if constexpr (W == 2)
+        *reinterpret_cast<double2*>(d) =
+            make_double2(__fma_rn(sd[0], widen(o[k][0]), mu[0]), __fma_rn(sd[1], widen(o[k][1]), mu[1]));
+      else
+        *d = __fma_rn(sd[0], widen(o[k][0]), mu[0]);
     }
   }
 }
@@ -758,6 +980,11 @@ cudaError_t gemm_tn(const bf16* A, int lda, const bf16* B, int ldb, int M, int N
 
 inline int grid_for(long long total, int threads = 256) {
   return (int)std::max<long long>(1, std::min<long long>((total + threads - 1) / threads, 16LL * num_sms()));
+}
+// two columns per thread: pairs do not straddle [n | m] and every row of both
+// arrays starts on 16 bytes
+inline bool two_columns(int n, int m, const void* p, const void* q) {
+  return n % 2 == 0 && m % 2 == 0 && ((uintptr_t)p & 15) == 0 && ((uintptr_t)q & 15) == 0;
 }
 inline int r8(long long v) { return (int)((v + 7) / 8 * 8); }
 
@@ -926,7 +1153,7 @@ void backward(pdqp_ws_s* w, int rows, const float* T, long long a, long long sft
     const float scale = (float)(2.0 / ((double)rows * F));
     k_grad_tiles<0><<<grid, blk, 0, s>>>(w->O, Fp, T, Fp, a, sft, count, row0, rows, F, scale, w->dOb, Fp, w->dOt,
                                          mb, w->colpart, w->ldc, w->lossp);
-    k_loss_acc<<<1, 256, 0, s>>>(w->lossp, (int)(grid.x * grid.y), 1.0 / ((double)rows * F), w->lossacc);
+    k_loss_acc<<<1, 1024, 0, s>>>(w->lossp, (int)(grid.x * grid.y), 1.0 / ((double)rows * F), w->lossacc);
   }
   WsLayer& o = w->L[w->depth];
   k_colsum<<<(F + 255) / 256, 256, 0, s>>>(w->colpart, rt, F, w->ldc, o.gb);
@@ -969,8 +1196,8 @@ void adam(pdqp_ws_s* w, float lr, float b1, float b2, float eps, cudaStream_t s)
   a.c2 = (float)(1.0 / (1.0 - std::pow((double)b2, (double)w->step)));
   a.update = 1;
   for (WsLayer& l : w->L) {
-    dim3 grid((l.in + 31) / 32, (l.out + 31) / 32), blk(32, 8);
-    k_adam_mat<<<grid, blk, 0, s>>>(l.W, l.mW, l.vW, l.gW, l.out, l.in, a, l.Wb, l.in, l.Wt, l.ldt);
+    dim3 grid((l.in + ADAM_T - 1) / ADAM_T, (l.out + ADAM_T - 1) / ADAM_T);
+    k_adam_mat<<<grid, 256, 0, s>>>(l.W, l.mW, l.vW, l.gW, l.out, l.in, a, l.Wb, l.in, l.Wt, l.ldt);
     k_adam_vec<<<(l.out + 255) / 256, 256, 0, s>>>(l.b, l.mb, l.vb, l.gb, l.out, a);
   }
 }
@@ -978,13 +1205,20 @@ void adam(pdqp_ws_s* w, float lr, float b1, float b2, float eps, cudaStream_t s)
 void refresh_copies(WsLayer& l, cudaStream_t s) {
   AdamArgs a{};
   a.update = 0;
-  dim3 grid((l.in + 31) / 32, (l.out + 31) / 32), blk(32, 8);
-  k_adam_mat<<<grid, blk, 0, s>>>(l.W, l.mW, l.vW, l.gW, l.out, l.in, a, l.Wb, l.in, l.Wt, l.ldt);
+  dim3 grid((l.in + ADAM_T - 1) / ADAM_T, (l.out + ADAM_T - 1) / ADAM_T);
+  k_adam_mat<<<grid, 256, 0, s>>>(l.W, l.mW, l.vW, l.gW, l.out, l.in, a, l.Wb, l.in, l.Wt, l.ldt);
+}
+
+// the elementwise kernels' grid over `rows` rows of arrays p, q
+dim3 row_grid(const pdqp_ws_s* w, const void* p, const void* q, long long rows) {
+  const int per = two_columns(w->n, w->m, p, q) ? 512 : 256;
+  return dim3((w->F + per - 1) / per, (unsigned)std::min<long long>((rows + ROWS_PER - 1) / ROWS_PER, 32768));
 }
 
 // normalised inputs of rows [row0, row0+rows) -> U -> H0 = U P'
 void project(pdqp_ws_s* w, const double* C, const double* B, long long row0, int rows, bf16* H0, cudaStream_t s) {
-  k_prep_input<<<grid_for((long long)rows * w->F), 256, 0, s>>>(C, B, w->n, w->m, row0, rows, w->in_mean,
+  auto prep = two_columns(w->n, w->m, C, B) ? k_prep_input<2> : k_prep_input<1>;
+  prep<<<row_grid(w, C, B, rows), 256, 0, s>>>(C, B, w->n, w->m, row0, rows, w->in_mean,
                                                                 w->in_scale, w->U, w->Fp);
   gemm(w, w->U, w->Fp, w->P, w->Fp, rows, w->d, w->F, epi_of(nullptr, H0, w->d, nullptr, 0), s);
 }
@@ -1243,20 +1477,38 @@ pdqp_status pdqp_ws_fit(pdqp_ws_handle w, const double* C, const double* B, cons
     if (count < 1) throw WsFail{PDQP_ERR_INVALID, "count >= 1"};
     need_data(w, C, B, X, Y, mem, true);
     const int n = w->n, m = w->m;
+    // partials of two arrays at a time: mean and M2 per range of FIT_ROWS rows
+    const long long nb = (count + FIT_ROWS - 1) / FIT_ROWS;
+    const size_t need = 4 * (size_t)nb * (size_t)std::max(n, m) * (sizeof(double) / sizeof(float));
+    if (need > w->work_floats) {
+      WCK(cudaStreamSynchronize(s));
+      wfree(w, w->work);
+      w->work = nullptr;
+      w->work_floats = 0;
+      w->work = walloc<float>(w, need);
+      w->work_floats = need;
+    }
+    // the statistics of the inputs `in` and of the targets `out`, nf columns each, from feature f0
+    auto stats = [&](const double* in, const double* out, int nf, int f0) {
+      double* part = reinterpret_cast<double*>(w->work);
+      const size_t len = (size_t)nb * nf;
+      const FitPair p{{in, out}, {part, part + 2 * len}, {part + len, part + 3 * len}};
+      const FitOut o{{w->in_mean + f0, w->out_mean + f0}, {w->in_scale + f0, w->out_inv + f0}, {nullptr, w->out_std + f0}};
+      k_fit_part<<<dim3((nf + 255) / 256, (unsigned)std::min<long long>(nb, 32768), 2), 256, 0, s>>>(p, count, nf);
+      k_fit_merge<<<dim3((nf + 127) / 128, 1, 2), 128, 0, s>>>(p, count, nf, o);
+      WCK(cudaGetLastError());
+    };
     {
       DevView<double> c(C, (size_t)count * n, mem, s), x(X, (size_t)count * n, mem, s);
-      k_fit_stats<<<(n + 127) / 128, 128, 0, s>>>(c.p, count, n, w->in_mean, w->in_scale, nullptr);
-      k_fit_stats<<<(n + 127) / 128, 128, 0, s>>>(x.p, count, n, w->out_mean, w->out_inv, w->out_std);
-      WCK(cudaGetLastError());
-      WCK(cudaStreamSynchronize(s));
+      stats(c.p, x.p, n, 0);
+      if (mem != PDQP_MEM_DEVICE) WCK(cudaStreamSynchronize(s));
     }
     if (m > 0) {
       DevView<double> b(B, (size_t)count * m, mem, s), y(Y, (size_t)count * m, mem, s);
-      k_fit_stats<<<(m + 127) / 128, 128, 0, s>>>(b.p, count, m, w->in_mean + n, w->in_scale + n, nullptr);
-      k_fit_stats<<<(m + 127) / 128, 128, 0, s>>>(y.p, count, m, w->out_mean + n, w->out_inv + n, w->out_std + n);
-      WCK(cudaGetLastError());
-      WCK(cudaStreamSynchronize(s));
+      stats(b.p, y.p, m, n);
+      if (mem != PDQP_MEM_DEVICE) WCK(cudaStreamSynchronize(s));
     }
+    WCK(cudaStreamSynchronize(s));
     w->have_norm = true;
   });
 }
@@ -1274,7 +1526,8 @@ pdqp_status pdqp_ws_grad(pdqp_ws_handle w, const double* C, const double* B, con
         x(X, (size_t)count * n, mem, s), y(Y, (size_t)count * m, mem, s);
     float* T = walloc<float>(w, (size_t)count * w->Fp);
     try {
-      k_prep_target<<<grid_for(count * w->F), 256, 0, s>>>(x.p, y.p, n, m, count, w->out_mean, w->out_inv, T, w->Fp);
+      (two_columns(n, m, x.p, y.p) ? k_prep_target<2> : k_prep_target<1>)<<<row_grid(w, x.p, y.p, count), 256, 0, s>>>(
+          x.p, y.p, n, m, count, w->out_mean, w->out_inv, T, w->Fp);
       project(w, c.p, b.p, 0, (int)count, w->H[0], s);
       forward(w, (int)count, s);
       WCK(cudaMemsetAsync(w->lossacc, 0, sizeof(double), s));
@@ -1328,7 +1581,8 @@ pdqp_status pdqp_ws_train(pdqp_ws_handle w, const pdqp_ws_train_options* opt, co
     }
     {
       DevView<double> x(X, (size_t)count * n, mem, s), y(Y, (size_t)count * m, mem, s);
-      k_prep_target<<<grid_for(count * F), 256, 0, s>>>(x.p, y.p, n, m, count, w->out_mean, w->out_inv, w->Tall, Fp);
+      (two_columns(n, m, x.p, y.p) ? k_prep_target<2> : k_prep_target<1>)<<<row_grid(w, x.p, y.p, count), 256, 0, s>>>(
+          x.p, y.p, n, m, count, w->out_mean, w->out_inv, w->Tall, Fp);
       finish(w, s);
     }
     const long long steps = count / batch;
@@ -1376,7 +1630,7 @@ pdqp_status pdqp_ws_infer(pdqp_ws_handle w, const double* C, const double* B, in
         const int rows = (int)std::min<long long>(w->maxb, count - r0);
         project(w, c.p, b.p, r0, rows, w->H[0], s);
         forward(w, rows, s);
-        k_write_pred<<<grid_for((long long)rows * w->F), 256, 0, s>>>(w->O, w->Fp, rows, n, m, w->out_mean,
+        (two_columns(n, m, x0, y0) ? k_write_pred<2> : k_write_pred<1>)<<<row_grid(w, x0, y0, rows), 256, 0, s>>>(w->O, w->Fp, rows, n, m, w->out_mean,
                                                                       w->out_std, r0, x0, y0);
       }
       finish(w, s);
