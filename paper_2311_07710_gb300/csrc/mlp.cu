@@ -18,7 +18,7 @@
 // A and B into a 4-stage shared-memory ring with TMA (128-byte swizzle),
 // thread 0 of warp 1 issues tcgen05.mma (M=128, N=256, K=16, kind::f16 with
 // bf16 A and B) on each stage into one of two float32 accumulators in tensor
-// memory and releases the stage with tcgen05.commit, and warps 2..5 drain the
+// memory and releases the stage with tcgen05.commit, and warps 2..9 drain the
 // other accumulator with tcgen05.ld into the fused epilogue (warp w reads TMEM
 // lanes 32 (w mod 4) .. +32), so a tile's epilogue overlaps the next tile's
 // main loop.  Split-K: a unit takes a range of k slices and writes raw float32
@@ -51,7 +51,8 @@ constexpr int A_BYTES = BM * BK * 2;                    // 16 KiB
 template <int BN> struct Tile {
   static constexpr int B_BYTES = BN * BK * 2;           // 16 or 32 KiB
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /* alignment */ + 256 /* barriers */;
+  static constexpr int EPI_BYTES = 8 * 32 * 20 * 4;     // the epilogue warps' stages (EPI_LD floats a row)
+  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /* alignment */ + 256 /* barriers */ + EPI_BYTES;
 };
 constexpr uint64_t WAIT_NS = 200000000ULL;            // a wait gives up after 0.2 s without progress
 
@@ -62,6 +63,7 @@ struct Epi {
   const bf16* mask;              // [M x ldm]: keep where mask > 0, else 0 (ReLU derivative), or null
   int ldo, ldm;
   int relu;
+  int vec;                       // the outputs and the mask start on 16 (8) bytes: 4 columns per access
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -144,82 +146,126 @@ __device__ __forceinline__ float epi_value(float r, int row, int col, const Epi&
   return r;
 }
 
-// Epilogue of 32 accumulator columns of one row: the raw float32 split-K
-// partial of split z (ld = N), or the fused epilogue into the outputs.
-__device__ __forceinline__ void store_chunk(const uint32_t (&v)[32], int row, int cb, int z, int M, int N,
+// Epilogue of a warp's 32 x 16 accumulator values (rows row0.., columns cb..
+// below nend), staged in `stg` (32 rows of EPI_LD floats): the raw float32 split-K
+// partial of split z (ld = N), or the fused epilogue into the outputs.  A lane
+// holds one accumulator row, so storing from its registers touches 32 rows at a
+// time in 16-byte pieces; through shared memory four lanes store a row's 64
+// contiguous bytes, eight rows an instruction.  The short-K products of the
+// network are bound by this path and its dependent instructions (512 x 30000 x
+// 64: 31 us with four epilogue warps, float32 or bf16 alike), so the common
+// case reads all its values first and takes its branches outside the loops,
+// and eight warps drain an accumulator, two per 32 TMEM lanes.
+constexpr int EPI_LD = 20;
+constexpr int EPI_WARPS = 8;
+constexpr int GEMM_NT = 64 + 32 * EPI_WARPS;   // TMA, MMA and epilogue warps
+__device__ __forceinline__ void store_chunk(const float* stg, int row0, int cb, int z, int M, int N, int nend,
                                             const Epi& epi, float* __restrict__ partial) {
-  if (partial) {   // raw float32 partial of this k range, ld = N
-    float* dst = partial + ((size_t)z * M + row) * N + cb;
-    if (cb + 32 <= N && (N & 3) == 0) {
+  const int lane = threadIdx.x & 31;
+  const bool vec = cb + 16 <= nend && row0 + 32 <= M && epi.vec &&
+                   (partial ? (N & 3) == 0 : (epi.ldo & 3) == 0 && (!epi.mask || (epi.ldm & 3) == 0));
+  if (vec) {
+    const int col = cb + (lane & 3) * 4, row = row0 + (lane >> 2);
+    float4 v[4];
 #pragma unroll
-      for (int i = 0; i < 32; i += 4)
-        *(float4*)(dst + i) = make_float4(__uint_as_float(v[i]), __uint_as_float(v[i + 1]),
-                                          __uint_as_float(v[i + 2]), __uint_as_float(v[i + 3]));
-    } else {
+    for (int i = 0; i < 4; ++i)
+      v[i] = *reinterpret_cast<const float4*>(stg + (8 * i + (lane >> 2)) * EPI_LD + (lane & 3) * 4);
+    if (partial) {
+      float* d = partial + ((size_t)z * M + row) * N + col;
 #pragma unroll
-      for (int i = 0; i < 32; ++i)
-        if (cb + i < N) dst[i] = __uint_as_float(v[i]);
+      for (int i = 0; i < 4; ++i) *reinterpret_cast<float4*>(d + (size_t)(8 * i) * N) = v[i];
+      return;
+    }
+    if (epi.bias) {
+      const float4 b = make_float4(__ldg(epi.bias + col), __ldg(epi.bias + col + 1), __ldg(epi.bias + col + 2),
+                                   __ldg(epi.bias + col + 3));
+#pragma unroll
+      for (int i = 0; i < 4; ++i) { v[i].x += b.x; v[i].y += b.y; v[i].z += b.z; v[i].w += b.w; }
+    }
+    if (epi.relu) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        v[i].x = fmaxf(v[i].x, 0.f); v[i].y = fmaxf(v[i].y, 0.f);
+        v[i].z = fmaxf(v[i].z, 0.f); v[i].w = fmaxf(v[i].w, 0.f);
+      }
+    }
+    if (epi.mask) {
+      const bf16* mk = epi.mask + (size_t)row * epi.ldm + col;
+      uint2 q[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) q[i] = *reinterpret_cast<const uint2*>(mk + (size_t)(8 * i) * epi.ldm);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const __nv_bfloat162 a = *reinterpret_cast<const __nv_bfloat162*>(&q[i].x);
+        const __nv_bfloat162 b = *reinterpret_cast<const __nv_bfloat162*>(&q[i].y);
+        if (!(__low2float(a) > 0.f)) v[i].x = 0.f;
+        if (!(__high2float(a) > 0.f)) v[i].y = 0.f;
+        if (!(__low2float(b) > 0.f)) v[i].z = 0.f;
+        if (!(__high2float(b) > 0.f)) v[i].w = 0.f;
+      }
+    }
+    const size_t o = (size_t)row * epi.ldo + col;
+    if (epi.out_f) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) *reinterpret_cast<float4*>(epi.out_f + o + (size_t)(8 * i) * epi.ldo) = v[i];
+    }
+    if (epi.out_b) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const __nv_bfloat162 h0 = __floats2bfloat162_rn(v[i].x, v[i].y), h1 = __floats2bfloat162_rn(v[i].z, v[i].w);
+        uint2 q;
+        q.x = *reinterpret_cast<const uint32_t*>(&h0);
+        q.y = *reinterpret_cast<const uint32_t*>(&h1);
+        *reinterpret_cast<uint2*>(epi.out_b + o + (size_t)(8 * i) * epi.ldo) = q;
+      }
     }
     return;
   }
-  float r[32];
-#pragma unroll
-  for (int i = 0; i < 32; ++i) r[i] = __uint_as_float(v[i]);
-  if (cb + 32 <= N) {
-#pragma unroll
-    for (int i = 0; i < 32; ++i) r[i] = epi_value(r[i], row, cb + i, epi);
-    const size_t o = (size_t)row * epi.ldo + cb;
-    if (epi.out_f) {
-      if ((epi.ldo & 3) == 0) {
-#pragma unroll
-        for (int i = 0; i < 32; i += 4) *(float4*)(epi.out_f + o + i) = make_float4(r[i], r[i + 1], r[i + 2], r[i + 3]);
-      } else {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) epi.out_f[o + i] = r[i];
-      }
+  // ragged rows or columns, unaligned rows: one column per lane, two rows at a time
+  const int col = cb + (lane & 15);
+  if (col >= nend) return;
+  for (int i = lane >> 4; i < 32; i += 2) {
+    const int row = row0 + i;
+    if (row >= M) return;
+    const float v = stg[i * EPI_LD + (lane & 15)];
+    if (partial) {
+      partial[((size_t)z * M + row) * N + col] = v;
+      continue;
     }
-    if (epi.out_b) {
-      if ((epi.ldo & 7) == 0) {
-#pragma unroll
-        for (int i = 0; i < 32; i += 8) {
-          uint4 q;
-          __nv_bfloat162 h0 = __floats2bfloat162_rn(r[i], r[i + 1]), h1 = __floats2bfloat162_rn(r[i + 2], r[i + 3]),
-                         h2 = __floats2bfloat162_rn(r[i + 4], r[i + 5]), h3 = __floats2bfloat162_rn(r[i + 6], r[i + 7]);
-          q.x = *(uint32_t*)&h0;
-          q.y = *(uint32_t*)&h1;
-          q.z = *(uint32_t*)&h2;
-          q.w = *(uint32_t*)&h3;
-          *(uint4*)(epi.out_b + o + i) = q;
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) epi.out_b[o + i] = __float2bfloat16_rn(r[i]);
-      }
-    }
-  } else {   // the ragged last columns: a test per column keeps the indexing static
-#pragma unroll
-    for (int i = 0; i < 32; ++i) {
-      if (cb + i < N) {
-        const float x = epi_value(r[i], row, cb + i, epi);
-        const size_t o = (size_t)row * epi.ldo + cb + i;
-        if (epi.out_f) epi.out_f[o] = x;
-        if (epi.out_b) epi.out_b[o] = __float2bfloat16_rn(x);
-      }
-    }
+    const float x = epi_value(v, row, col, epi);
+    const size_t o = (size_t)row * epi.ldo + col;
+    if (epi.out_f) epi.out_f[o] = x;
+    if (epi.out_b) epi.out_b[o] = __float2bfloat16_rn(x);
   }
 }
 
-// 32 float32 accumulator columns of this warp's TMEM lanes, from column address taddr
-__device__ __forceinline__ void tmem_ld32(uint32_t (&v)[32], uint32_t taddr) {
+// 16 float32 accumulator columns of this warp's TMEM lanes, from column address taddr
+__device__ __forceinline__ void tmem_ld16(uint32_t (&v)[16], uint32_t taddr) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
       : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
-        "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
-        "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
       : "r"(taddr));
   asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+}
+
+// One warp's share of an accumulator (TMEM base address of its lanes, columns
+// 16 half, 16 half + 32, ... of width) through its stage into the outputs.
+__device__ __forceinline__ void drain(float* stg, uint32_t tmem, int half, int width, int row0, int n0, int z, int M,
+                                      int N, const Epi& epi, float* __restrict__ partial) {
+  const int lane = threadIdx.x & 31, nend = min(n0 + width, N);
+  for (int c0 = 16 * half; c0 < width && n0 + c0 < N; c0 += 32) {
+    uint32_t v[16];
+    tmem_ld16(v, tmem + (uint32_t)c0);
+    __syncwarp();                             // the previous chunk has left the stage
+#pragma unroll
+    for (int i = 0; i < 16; i += 4)
+      *reinterpret_cast<float4*>(stg + lane * EPI_LD + i) =
+          make_float4(__uint_as_float(v[i]), __uint_as_float(v[i + 1]), __uint_as_float(v[i + 2]),
+                      __uint_as_float(v[i + 3]));
+    __syncwarp();
+    store_chunk(stg, row0, n0 + c0, z, M, N, nend, epi, partial);
+  }
 }
 
 // D = A B' (bf16 A, B K-major, float32 accumulation in tensor memory), persistent:
@@ -227,14 +273,14 @@ __device__ __forceinline__ void tmem_ld32(uint32_t (&v)[32], uint32_t taddr) {
 // blockIdx.x + gridDim.x, ... (a unit is one BM x BN tile of one k split;
 // the tiles in bands of tile rows, see `unit`).
 // Warp roles: warp 0 lane 0 issues the TMA loads of every unit through the
-// STAGES ring, warp 1 lane 0 the MMAs, warps 2..5 drain the accumulators
+// STAGES ring, warp 1 lane 0 the MMAs, warps 2..9 drain the accumulators
 // (warp w reads TMEM lanes 32 (w mod 4) .. +32).  Two accumulators of BN
 // columns: the epilogue of one unit overlaps the main loop of the next.
 // Every wait is bounded (WAIT_NS without progress, or the error flag), after
 // which the roles leave their loops, the copies in flight land, and the TMEM
 // is freed.
 template <int BN>
-__global__ void __launch_bounds__(192, 1)
+__global__ void __launch_bounds__(GEMM_NT, 1)
     k_gemm_tn_p(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int M, int N,
                 int K, int ktps, int splits, Epi epi, float* __restrict__ partial, int* err) {
   constexpr int STAGE_BYTES = Tile<BN>::STAGE_BYTES;
@@ -245,6 +291,7 @@ __global__ void __launch_bounds__(192, 1)
   uint64_t* acc_full = empty + STAGES;       // [2]: the MMAs of a unit are done
   uint64_t* acc_empty = acc_full + 2;        // [2]: the epilogue has read the accumulator
   uint32_t* tmem_slot = (uint32_t*)(acc_empty + 2);
+  float* epi_stage = (float*)(sm + STAGES * STAGE_BYTES + 256);
   __shared__ volatile int s_fail;
   __shared__ int s_issued;                   // stage loads issued, for the cleanup
   __shared__ volatile int s_progress;        // stages consumed by the MMA issuer
@@ -263,7 +310,7 @@ __global__ void __launch_bounds__(192, 1)
     }
     for (int q = 0; q < 2; ++q) {
       mbar_init(&acc_full[q], 1);
-      mbar_init(&acc_empty[q], 4);           // one arrival per epilogue warp
+      mbar_init(&acc_empty[q], EPI_WARPS);   // one arrival per epilogue warp
     }
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
@@ -363,12 +410,8 @@ __global__ void __launch_bounds__(192, 1)
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;\n");
-      const int row = m0 + sp * 32 + lane;
-      for (int c0 = 0; c0 < BN; c0 += 32) {
-        uint32_t v[32];
-        tmem_ld32(v, tmem + ((uint32_t)(sp * 32) << 16) + (uint32_t)(buf * BN + c0));
-        if (row < M) store_chunk(v, row, n0 + c0, z, M, N, epi, splits > 1 ? partial : nullptr);
-      }
+      drain(epi_stage + (warp - 2) * 32 * EPI_LD, tmem + ((uint32_t)(sp * 32) << 16) + (uint32_t)(buf * BN),
+            (warp - 2) >> 2, BN, m0 + sp * 32, n0, z, M, N, epi, splits > 1 ? partial : nullptr);
       asm volatile("tcgen05.fence::before_thread_sync;\n");
       __syncwarp();
       if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(&acc_empty[buf])) : "memory");
@@ -389,6 +432,207 @@ __global__ void __launch_bounds__(192, 1)
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(2 * BN));
 }
 
+// --------------------------------------------------------------------------
+// The same product on CTA pairs (cta_group::2): a cluster of two CTAs works on
+// one 256 x bn tile.  Each CTA loads its 128 rows of A and its half of the bn rows of
+// B, the even CTA's thread issues M = 256 MMAs that read both CTAs' shared memory,
+// and each CTA drains the 128 rows that its tensor memory holds.  Per MMA step a
+// CTA then moves 16 KB through shared memory (TMA write and tensor-core read of
+// 4 KB of A and 4 KB of B) instead of 24 KB: with one CTA per tile the 192 bytes
+// a clock exceed the 128 of the shared memory, which bound k_gemm_tn_p.
+// bn (a multiple of 16, <= 256) is chosen so that the tiles fill the waves
+// (plan_pairs).  Barriers: `full` lives in the even CTA and counts both CTAs'
+// bytes; `empty` and `acc_full` are signalled in both CTAs by a multicast commit;
+// `acc_empty` in the even CTA takes an arrival of each CTA's epilogue warps.
+// Every wait is bounded as in k_gemm_tn_p; both CTAs meet at a cluster barrier
+// before they leave, so no signal reaches shared memory that is gone.
+constexpr int P_STAGES = 6;
+constexpr int P_B_BYTES = 128 * BK * 2;                 // at most 128 rows of B per CTA
+constexpr int P_STAGE_BYTES = A_BYTES + P_B_BYTES;      // 32 KiB
+constexpr int P_SMEM_BYTES = P_STAGES * P_STAGE_BYTES + 1024 + 256 + EPI_WARPS * 32 * EPI_LD * 4;
+
+__device__ __forceinline__ uint32_t mapa_u32(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+// a load into this CTA whose bytes count on the barrier at cluster address bar
+__device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* map, uint32_t bar, int x, int y) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], "
+      "[%2];\n" ::"r"(smem_u32(dst)),
+      "l"((uint64_t)map), "r"(bar), "r"(x), "r"(y)
+      : "memory");
+}
+__device__ __forceinline__ void commit_pair(uint64_t* bar) {   // arrives on this barrier in both CTAs
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n" ::"r"(
+          smem_u32(bar)),
+      "h"((uint16_t)3));
+}
+
+__global__ void __launch_bounds__(GEMM_NT, 1) __cluster_dims__(2, 1, 1)
+    k_gemm_tn_pair(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int M, int N,
+                   int K, int bn, int ktps, int splits, Epi epi, float* __restrict__ partial, int* err) {
+  extern __shared__ __align__(1024) unsigned char smraw[];
+  unsigned char* sm = (unsigned char*)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
+  uint64_t* full = (uint64_t*)(sm + P_STAGES * P_STAGE_BYTES);
+  uint64_t* empty = full + P_STAGES;
+  uint64_t* acc_full = empty + P_STAGES;     // [2]
+  uint64_t* acc_empty = acc_full + 2;        // [2]
+  uint32_t* tmem_slot = (uint32_t*)(acc_empty + 2);
+  float* epi_stage = (float*)(sm + P_STAGES * P_STAGE_BYTES + 256);
+  __shared__ volatile int s_fail;
+  __shared__ int s_issued;
+  __shared__ volatile int s_progress;        // stages consumed (even CTA), stages granted (odd CTA)
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = blockIdx.x & 1;
+  const bool leader = rank == 0;
+  const int tn = (N + bn - 1) / bn, tm = (M + 2 * BM - 1) / (2 * BM);
+  const int KT = (K + BK - 1) / BK;
+  const int units = tm * tn * splits;
+  const int u0 = blockIdx.x >> 1, du = gridDim.x >> 1;
+  const uint32_t half_bytes = (uint32_t)(bn / 2) * BK * 2;
+
+  if (threadIdx.x == 0) {
+    s_fail = 0;
+    s_issued = 0;
+    s_progress = 0;
+    for (int q = 0; q < P_STAGES; ++q) {
+      mbar_init(&full[q], 1);
+      mbar_init(&empty[q], 1);
+    }
+    for (int q = 0; q < 2; ++q) {
+      mbar_init(&acc_full[q], 1);
+      mbar_init(&acc_empty[q], 2 * EPI_WARPS);   // the epilogue warps of both CTAs
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  if (warp == 0) {   // both CTAs: two accumulators of 256 float32 columns
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_slot)),
+                 "r"(512));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;\n");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;\n");
+  __syncthreads();
+  cluster_sync();                            // the peer's barriers are initialised
+  asm volatile("tcgen05.fence::after_thread_sync;\n");
+  const uint32_t tmem = *tmem_slot;
+
+  // tiles in bands of tile rows, as k_gemm_tn_p (4 x 256 rows)
+  constexpr int GROUP = 4;
+  auto unit = [&](int u, int& m0, int& n0, int& kt0, int& nk, int& z) {
+    z = u / (tm * tn);
+    const int t = u - z * (tm * tn);
+    const int band = t / (GROUP * tn), first = band * GROUP;
+    const int rows = min(tm - first, GROUP);
+    const int q = t - band * GROUP * tn;
+    m0 = (first + q % rows) * 2 * BM;
+    n0 = (q / rows) * bn;
+    kt0 = z * ktps;
+    nk = min(KT, kt0 + ktps) - kt0;
+  };
+
+  if (warp == 0 && lane == 0) {   // TMA producer of this CTA's halves
+    int i = 0;
+    for (int u = u0; u < units && !s_fail; u += du) {
+      int m0, n0, kt0, nk, z;
+      unit(u, m0, n0, kt0, nk, z);
+      for (int k = 0; k < nk; ++k, ++i) {
+        const int q = i % P_STAGES;
+        if (i >= P_STAGES && !mbar_wait(&empty[q], ((i / P_STAGES) - 1) & 1, err, &s_progress)) {
+          s_fail = 1;
+          break;
+        }
+        if (!leader) s_progress = i + 1;
+        unsigned char* a = sm + q * P_STAGE_BYTES;
+        if (leader) mbar_expect_tx(&full[q], 2 * (A_BYTES + half_bytes));
+        const uint32_t bar = mapa_u32(smem_u32(&full[q]), 0);
+        tma_load_2d_pair(a, &mapA, bar, (kt0 + k) * BK, m0 + (int)rank * BM);
+        tma_load_2d_pair(a + A_BYTES, &mapB, bar, (kt0 + k) * BK, n0 + (int)rank * (bn / 2));
+        s_issued = i + 1;
+      }
+    }
+  } else if (warp == 1 && lane == 0 && leader) {   // MMA issuer
+    const uint32_t idesc = instr_desc(2 * BM, bn);
+    int i = 0, lt = 0;
+    for (int u = u0; u < units && !s_fail; u += du, ++lt) {
+      int m0, n0, kt0, nk, z;
+      unit(u, m0, n0, kt0, nk, z);
+      const int buf = lt & 1;
+      if (!mbar_wait(&acc_empty[buf], ((lt >> 1) & 1) ^ 1, err)) {
+        s_fail = 1;
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;\n");
+      const uint32_t acc_tm = tmem + (uint32_t)(buf * 256);
+      for (int k = 0; k < nk; ++k, ++i) {
+        const int q = i % P_STAGES;
+        if (!mbar_wait(&full[q], (i / P_STAGES) & 1, err)) {
+          s_fail = 1;
+          break;
+        }
+        s_progress = i + 1;
+        asm volatile("tcgen05.fence::after_thread_sync;\n");
+        const unsigned char* a = sm + q * P_STAGE_BYTES;
+        const uint64_t da = smem_desc(a), db = smem_desc(a + A_BYTES);
+#pragma unroll
+        for (int kk = 0; kk < BK / 16; ++kk) {
+          const uint64_t step = (uint64_t)((kk * 16 * 2) >> 4);
+          const uint32_t acc = (k > 0 || kk > 0) ? 1u : 0u;
+          asm volatile(
+              "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
+              " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(acc_tm),
+              "l"(da + step), "l"(db + step), "r"(idesc), "r"(acc));
+        }
+        commit_pair(&empty[q]);
+      }
+      if (s_fail) break;
+      commit_pair(&acc_full[buf]);
+    }
+  } else if (warp >= 2) {   // epilogue of this CTA's 128 rows
+    const int sp = warp & 3;
+    const uint32_t ae0 = mapa_u32(smem_u32(&acc_empty[0]), 0), ae1 = mapa_u32(smem_u32(&acc_empty[1]), 0);
+    int lt = 0;
+    for (int u = u0; u < units; u += du, ++lt) {
+      int m0, n0, kt0, nk, z;
+      unit(u, m0, n0, kt0, nk, z);
+      const int buf = lt & 1;
+      if (s_fail || !mbar_wait(&acc_full[buf], (lt >> 1) & 1, err, &s_progress)) {
+        s_fail = 1;
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;\n");
+      drain(epi_stage + (warp - 2) * 32 * EPI_LD, tmem + ((uint32_t)(sp * 32) << 16) + (uint32_t)(buf * 256),
+            (warp - 2) >> 2, bn, m0 + (int)rank * BM + sp * 32, n0, z, M, N, epi, splits > 1 ? partial : nullptr);
+      asm volatile("tcgen05.fence::before_thread_sync;\n");
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];\n" ::"r"(buf ? ae1 : ae0)
+                     : "memory");
+    }
+  }
+  __syncwarp();
+  asm volatile("tcgen05.fence::before_thread_sync;\n");
+  __syncthreads();
+  cluster_sync();
+  if (s_fail && threadIdx.x == 0) {   // record the failure; let the copies in flight land (both CTAs' count on the leader)
+    atomicExch(err, 1);
+    const int issued = s_issued;
+    if (leader)
+      for (int i = max(0, issued - P_STAGES); i < issued; ++i) {
+        int never = 0;
+        mbar_wait(&full[i % P_STAGES], (i / P_STAGES) & 1, &never);
+      }
+  }
+  __syncthreads();
+  cluster_sync();
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(512));
+}
+
 // The bounded wait of the tensor-core kernels on an mbarrier that nothing
 // completes: it gives up after WAIT_NS and raises the error flag, as a GEMM
 // whose copies or MMAs never landed would (the host then reads
@@ -403,17 +647,33 @@ __global__ void k_wait_probe(int* err) {
   if (threadIdx.x == 0 && !mbar_wait(&bar, 0, err)) atomicExch(err, 1);
 }
 
-// Sum of the split-K partials in a fixed order, then the epilogue.
-__global__ void k_splitk_epi(const float* __restrict__ part, int splits, int M, int N, Epi epi) {
-  const long long MN = (long long)M * N;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < MN; i += (long long)gridDim.x * blockDim.x) {
-    float r = 0.f;
-    for (int z = 0; z < splits; ++z) r += part[z * MN + i];
-    const int row = (int)(i / N), col = (int)(i % N);
-    r = epi_value(r, row, col, epi);
+// Sum of the split-K partials in a fixed order, then the epilogue: W columns
+// per thread (4 where N and the leading dimensions allow), a row per grid y.
+template <int W>
+__global__ void __launch_bounds__(128) k_splitk_epi(const float* __restrict__ part, int splits, int M, int N, Epi epi) {
+  const size_t MN = (size_t)M * N;
+  const int col = (blockIdx.x * 128 + threadIdx.x) * W;
+  if (col >= N) return;
+  for (int row = blockIdx.y; row < M; row += gridDim.y) {
+    const float* p = part + (size_t)row * N + col;
+    float r[W];
+#pragma unroll
+    for (int i = 0; i < W; ++i) r[i] = 0.f;
+    for (int z = 0; z < splits; ++z) {
+      if constexpr (W == 4) {
+        const float4 q = *reinterpret_cast<const float4*>(p + z * MN);
+        r[0] += q.x; r[1] += q.y; r[2] += q.z; r[3] += q.w;
+      } else {
+        r[0] += p[z * MN];
+      }
+    }
     const size_t o = (size_t)row * epi.ldo + col;
-    if (epi.out_f) epi.out_f[o] = r;
-    if (epi.out_b) epi.out_b[o] = __float2bfloat16_rn(r);
+#pragma unroll
+    for (int i = 0; i < W; ++i) {
+      const float v = epi_value(r[i], row, col + i, epi);
+      if (epi.out_f) epi.out_f[o + i] = v;
+      if (epi.out_b) epi.out_b[o + i] = __float2bfloat16_rn(v);
+    }
   }
 }
 
@@ -927,20 +1187,51 @@ static int num_sms() {   // of the current device, read once (a thread-safe stat
 // the B tile width: 256 when N fills it, else 128
 inline int tile_n(int N) { return N >= 256 ? 256 : 128; }
 
-// number of K splits: enough blocks to cover the SMs, at least 4 k-tiles each
-int plan_splits(int M, int N, int K, int requested) {
-  const int BN = tile_n(N);
+// How a product runs: on CTA pairs (256 x bn tiles) or single CTAs (128 x bn),
+// and in how many splits of K.
+struct GemmPlan {
+  int pair, bn, splits;
+};
+
+// Splits: with fewer 128 x 256 (128) tiles than SMs, enough to cover the SMs,
+// at least 4 k-tiles each.  Pairs where M and N fill their tiles (a pair on
+// M <= 128 would idle one CTA).  A product on pairs takes the tile width whose
+// waves cost least: per k-tile a tile lasts as long as it is wide (plus about 32
+// columns' worth of the A side), its epilogue about ten k-tiles; the epilogue
+// of all but the last tile hides behind the next tile's main loop or the other
+// way round.  So 256 for long products with many tiles, less where that
+// leaves the last wave nearly empty or the epilogue of a single wave shows.
+GemmPlan plan_gemm(int M, int N, int K, int requested) {
+  GemmPlan p;
+  p.bn = tile_n(N);
   const int KT = (K + BK - 1) / BK;
   int splits = requested;
   if (splits <= 0) {
-    const long long tiles = (long long)((M + BM - 1) / BM) * ((N + BN - 1) / BN);
+    const long long t = (long long)((M + BM - 1) / BM) * ((N + p.bn - 1) / p.bn);
     splits = 1;
-    if (tiles < num_sms()) splits = (int)std::min<long long>(KT / 4, (num_sms() + tiles - 1) / tiles);
+    if (t < num_sms()) splits = (int)std::min<long long>(KT / 4, (num_sms() + t - 1) / t);
   }
   splits = std::max(1, std::min(splits, KT));
   const int ktps = (KT + splits - 1) / splits;
-  return (KT + ktps - 1) / ktps;
+  p.splits = (KT + ktps - 1) / ktps;
+  p.pair = M > 128 && N >= 256;
+  if (p.pair) {
+    const long long tm = (M + 2 * BM - 1) / (2 * BM), pairs = std::max(1, num_sms() / 2);
+    const long long kt = (KT + p.splits - 1) / p.splits;
+    long long best = 0;
+    for (int bn = 256; bn >= 128; bn -= 16) {
+      const long long waves = (tm * ((N + bn - 1) / bn) * p.splits + pairs - 1) / pairs;
+      const long long main = kt * (bn + 32), epi = 10LL * bn;
+      const long long cost = waves * std::max(main, epi) + std::min(main, epi);
+      if (best == 0 || cost < best) {
+        best = cost;
+        p.bn = bn;
+      }
+    }
+  }
+  return p;
 }
+int plan_splits(int M, int N, int K, int requested) { return plan_gemm(M, N, K, requested).splits; }
 
 size_t splitk_floats(int M, int N, int K, int splits) {
   const int s = plan_splits(M, N, K, splits);
@@ -952,28 +1243,41 @@ size_t splitk_floats(int M, int N, int K, int splits) {
 cudaError_t gemm_tn(const bf16* A, int lda, const bf16* B, int ldb, int M, int N, int K, const Epi& epi, int splits,
                     float* work, size_t work_floats, int* err, cudaStream_t s) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaErrorInvalidValue;
-  const int BN = tile_n(N);
+  const GemmPlan plan = plan_gemm(M, N, K, splits);
+  const int BN = plan.bn;
   CUtensorMap ma, mb;
-  if (!make_map(&ma, A, M, K, lda, BM) || !make_map(&mb, B, N, K, ldb, BN)) return cudaErrorInvalidValue;
+  if (!make_map(&ma, A, M, K, lda, BM) || !make_map(&mb, B, N, K, ldb, plan.pair ? BN / 2 : BN))
+    return cudaErrorInvalidValue;
   static std::once_flag attr;
   std::call_once(attr, [] {
     cudaFuncSetAttribute(k_gemm_tn_p<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, Tile<128>::SMEM_BYTES);
     cudaFuncSetAttribute(k_gemm_tn_p<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, Tile<256>::SMEM_BYTES);
+    cudaFuncSetAttribute(k_gemm_tn_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, P_SMEM_BYTES);
   });
+  Epi ep = epi;
+  ep.vec = ((uintptr_t)epi.out_f & 15) == 0 && ((uintptr_t)epi.out_b & 7) == 0 && ((uintptr_t)epi.mask & 7) == 0 &&
+           ((uintptr_t)work & 15) == 0;
   const int KT = (K + BK - 1) / BK;
-  int sp = plan_splits(M, N, K, splits);
+  int sp = plan.splits;
   if (sp > 1 && (!work || work_floats < (size_t)sp * M * N)) sp = 1;
   const int ktps = (KT + sp - 1) / sp;
-  const long long units = (long long)((N + BN - 1) / BN) * ((M + BM - 1) / BM) * sp;
-  const int grid = (int)std::min<long long>(units, num_sms());
-  if (BN == 256)
-    k_gemm_tn_p<256><<<grid, 192, Tile<256>::SMEM_BYTES, s>>>(ma, mb, M, N, K, ktps, sp, epi, work, err);
+  const int bm = plan.pair ? 2 * BM : BM;
+  const long long units = (long long)((N + BN - 1) / BN) * ((M + bm - 1) / bm) * sp;
+  if (plan.pair)
+    k_gemm_tn_pair<<<2 * (int)std::min<long long>(units, num_sms() / 2), GEMM_NT, P_SMEM_BYTES, s>>>(
+        ma, mb, M, N, K, BN, ktps, sp, ep, work, err);
+  else if (BN == 256)
+    k_gemm_tn_p<256><<<(int)std::min<long long>(units, num_sms()), GEMM_NT, Tile<256>::SMEM_BYTES, s>>>(
+        ma, mb, M, N, K, ktps, sp, ep, work, err);
   else
-    k_gemm_tn_p<128><<<grid, 192, Tile<128>::SMEM_BYTES, s>>>(ma, mb, M, N, K, ktps, sp, epi, work, err);
+    k_gemm_tn_p<128><<<(int)std::min<long long>(units, num_sms()), GEMM_NT, Tile<128>::SMEM_BYTES, s>>>(
+        ma, mb, M, N, K, ktps, sp, ep, work, err);
   if (sp > 1) {
-    const long long MN = (long long)M * N;
-    const int blocks = (int)std::min<long long>((MN + 255) / 256, 8LL * num_sms());
-    k_splitk_epi<<<blocks, 256, 0, s>>>(work, sp, M, N, epi);
+    const int rows = std::min(M, 32768);
+    if ((N & 3) == 0 && ((uintptr_t)work & 15) == 0)
+      k_splitk_epi<4><<<dim3((N / 4 + 127) / 128, rows), 128, 0, s>>>(work, sp, M, N, epi);
+    else
+      k_splitk_epi<1><<<dim3((N + 127) / 128, rows), 128, 0, s>>>(work, sp, M, N, epi);
   }
   return cudaGetLastError();
 }
