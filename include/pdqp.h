@@ -373,8 +373,8 @@ pdqp_status pdqp_kkt(pdqp_handle h, const double *x, const double *y, double *pa
  * library's device image that every GPU loading the library holds until the
  * process exits.  The first call on each device looks up that array's device
  * address (cudaGetSymbolAddress) with the device current; make the first call
- * on a device before any stream capture.  Every call zeroes and reuses the
- * same array, so calls whose device work overlaps (on different streams or
+ * on a device before any stream capture.  Every call resets the array's block
+ * counter and reuses the same array, so calls whose device work overlaps (on different streams or
  * from different threads) race on it: order them on one stream. */
 pdqp_status pdqp_kkt_noalloc(int64_t n, int64_t m, int64_t m_eq,
                              const int32_t *Q_rowptr, const int32_t *Q_col, const double *Q_val,

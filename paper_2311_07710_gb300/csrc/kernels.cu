@@ -31,162 +31,6 @@ static int pick_lanes(long long nnz, long long rows) {
   return L;
 }
 
-#define DISPATCH_L(L, ...)                                  \
-  switch (L) {                                              \
-    case 2: { constexpr int LL = 2; __VA_ARGS__; } break;   \
-    case 4: { constexpr int LL = 4; __VA_ARGS__; } break;   \
-    case 8: { constexpr int LL = 8; __VA_ARGS__; } break;   \
-    case 16: { constexpr int LL = 16; __VA_ARGS__; } break; \
-    default: { constexpr int LL = 32; __VA_ARGS__; } break; \
-  }
-
-// --------------------------------------------------------------------------
-// Per-row relative KKT kernels on separate Q, A, A' CSR arrays (used by
-// pdqp_kkt_noalloc, which takes caller-owned arrays).
-// Relative KKT error (Section 5 "Progress metric", equality/bound form) in
-// float64, for NIT iterates at once, measured on the original problem:
-// (Ax)_i = (A~ x~)_i / D1_i, (Qx)_j = (Q~ x~)_j / D2_j, (A'y)_j = (A~' y~)_j / D2_j.
-// Partial sums go to part[block][field]; k_kkt_finish_noalloc finishes them.
-// --------------------------------------------------------------------------
-struct KktArgs {
-  Csr<double> A, Q, At;                 // scaled (or original with D = null)
-  const double* x[2];                   // float64 iterates (scaled space)
-  const double* y[2];
-  const float* dx[2];                   // mixed mode: iterate = base + delta
-  const float* dy[2];
-  const double* xhi;
-  const double* yhi;
-  const double* ax;                     // anchors (scaled); null: delta from base (mixed)
-  const double* ay;
-  const double* D1;                     // null = 1
-  const double* D2;
-  const double *b, *c, *l, *u;          // original data
-  double* prodAx[2];                    // optional: store A~x~ etc. (mixed-mode correction)
-  double* prodQx[2];
-  double* prodATy[2];
-  double* part;
-  int n, m, m_eq;
-};
-
-template <bool MIXED>
-__device__ __forceinline__ double it_x(const KktArgs& a, int it, int k) {
-  if (MIXED) return a.xhi[k] + (double)a.dx[it][k];
-  return a.x[it][k];
-}
-template <bool MIXED>
-__device__ __forceinline__ double it_y(const KktArgs& a, int it, int k) {
-  if (MIXED) return a.yhi[k] + (double)a.dy[it][k];
-  return a.y[it][k];
-}
-
-template <int L, int NIT, bool MIXED>
-__global__ void __launch_bounds__(256) k_kkt_m(KktArgs a) {
-  // fields: it*4 + {0 max|viol|, 1 max|Ax|, 2 b'y, 3 |dy|^2}, 8: max|b|
-  double f[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-  const int rpb = 256 / L, lane = threadIdx.x % L;
-  for (int base = blockIdx.x * rpb; base < a.m; base += gridDim.x * rpb) {
-    const int row = base + threadIdx.x / L;
-    const bool valid = row < a.m;
-    double s[NIT];
-#pragma unroll
-    for (int it = 0; it < NIT; ++it) s[it] = 0.0;
-    if (valid) {
-      for (int k = a.A.rp[row] + lane; k < a.A.rp[row + 1]; k += L) {
-        const double v = a.A.val[k];
-        const int cidx = a.A.col[k];
-#pragma unroll
-        for (int it = 0; it < NIT; ++it) s[it] = fma(v, it_x<MIXED>(a, it, cidx), s[it]);
-      }
-    }
-#pragma unroll
-    for (int it = 0; it < NIT; ++it) s[it] = group_sum<L>(s[it]);
-    if (valid && lane == 0) {
-      const double d1 = a.D1 ? a.D1[row] : 1.0;
-      const double bi = a.b[row];
-#pragma unroll
-      for (int it = 0; it < NIT; ++it) {
-        if (a.prodAx[it]) a.prodAx[it][row] = s[it];
-        const double Ax = s[it] / d1;
-        const double viol = row < a.m_eq ? fabs(Ax - bi) : fmax(bi - Ax, 0.0);
-        f[it * 4 + 0] = nmax(f[it * 4 + 0], viol);
-        f[it * 4 + 1] = nmax(f[it * 4 + 1], fabs(Ax));
-        const double yt = it_y<MIXED>(a, it, row);
-        f[it * 4 + 2] += bi * (d1 * yt);
-        const double dy = MIXED ? (double)a.dy[it][row] : (a.ay ? yt - a.ay[row] : 0.0);
-        f[it * 4 + 3] += dy * dy;
-      }
-      f[8] = nmax(f[8], fabs(bi));
-    }
-  }
-  const bool is_max[9] = {true, true, false, false, true, true, false, false, true};
-  block_reduce<9>(f, is_max);
-  if (threadIdx.x == 0)
-    for (int k = 0; k < 9; ++k) a.part[blockIdx.x * 32 + k] = f[k];
-}
-
-template <int L, int NIT, bool MIXED>
-__global__ void __launch_bounds__(256) k_kkt_n(KktArgs a) {
-  // fields (offset 9): it*7 + {0 max|res|, 1 max|Qx|, 2 max|A'y|, 3 x'Qx, 4 c'x,
-  // 5 sum(l lam+ - u lam-), 6 |dx|^2}, 14: max|c|
-  double f[15];
-#pragma unroll
-  for (int k = 0; k < 15; ++k) f[k] = 0.0;
-  const int rpb = 256 / L, lane = threadIdx.x % L;
-  for (int base = blockIdx.x * rpb; base < a.n; base += gridDim.x * rpb) {
-    const int row = base + threadIdx.x / L;
-    const bool valid = row < a.n;
-    double sq[NIT], sa[NIT];
-#pragma unroll
-    for (int it = 0; it < NIT; ++it) { sq[it] = 0.0; sa[it] = 0.0; }
-    if (valid) {
-      for (int k = a.Q.rp[row] + lane; k < a.Q.rp[row + 1]; k += L) {
-        const double v = a.Q.val[k];
-        const int cidx = a.Q.col[k];
-#pragma unroll
-        for (int it = 0; it < NIT; ++it) sq[it] = fma(v, it_x<MIXED>(a, it, cidx), sq[it]);
-      }
-      if (a.m > 0)
-        for (int k = a.At.rp[row] + lane; k < a.At.rp[row + 1]; k += L) {
-          const double v = a.At.val[k];
-          const int cidx = a.At.col[k];
-#pragma unroll
-          for (int it = 0; it < NIT; ++it) sa[it] = fma(v, it_y<MIXED>(a, it, cidx), sa[it]);
-        }
-    }
-#pragma unroll
-    for (int it = 0; it < NIT; ++it) { sq[it] = group_sum<L>(sq[it]); sa[it] = group_sum<L>(sa[it]); }
-    if (valid && lane == 0) {
-      const double d2 = a.D2 ? a.D2[row] : 1.0;
-      const double cj = a.c[row], lj = a.l[row], uj = a.u[row];
-      const bool lf = isfinite(lj), uf = isfinite(uj);
-#pragma unroll
-      for (int it = 0; it < NIT; ++it) {
-        if (a.prodQx[it]) { a.prodQx[it][row] = sq[it]; a.prodATy[it][row] = sa[it]; }
-        const double Qx = sq[it] / d2, ATy = sa[it] / d2;
-        const double xt = it_x<MIXED>(a, it, row);
-        const double xj = d2 * xt;
-        const double g = Qx + cj - ATy;
-        const double lam = (lf && uf) ? g : (lf ? fmax(g, 0.0) : (uf ? fmin(g, 0.0) : 0.0));
-        double* fi = f + it * 7;
-        fi[0] = nmax(fi[0], fabs(g - lam));
-        fi[1] = nmax(fi[1], fabs(Qx));
-        fi[2] = nmax(fi[2], fabs(ATy));
-        fi[3] += xj * Qx;
-        fi[4] += cj * xj;
-        fi[5] += (lam > 0.0 ? lj * lam : 0.0) - (lam < 0.0 ? uj * (-lam) : 0.0);
-        const double dx = MIXED ? (double)a.dx[it][row] : (a.ax ? xt - a.ax[row] : 0.0);
-        fi[6] += dx * dx;
-      }
-      f[14] = nmax(f[14], fabs(cj));
-    }
-  }
-  const bool is_max[15] = {true, true, true, false, false, false, false,
-                           true, true, true, false, false, false, false, true};
-  block_reduce<15>(f, is_max);
-  if (threadIdx.x == 0)
-    for (int k = 0; k < 15; ++k) a.part[blockIdx.x * 32 + 9 + k] = f[k];
-}
-
 // relKKT parts from the reduced fields of iterate `it`
 __device__ void kkt_from_fields(const double* F, int it, double* out) {
   const double maxviol = F[it * 4 + 0], maxAx = F[it * 4 + 1], by = F[it * 4 + 2];
@@ -202,22 +46,6 @@ __device__ void kkt_from_fields(const double* F, int it, double* out) {
   double rel = nmax(nmax(rp, rd), rg);
   if (pobj != pobj || dobj != dobj) rel = pobj - dobj;   // NaN
   out[0] = rp; out[1] = rd; out[2] = rg; out[3] = rel; out[4] = pobj; out[5] = dobj;
-}
-
-// reduce the partials of k_kkt_m / k_kkt_n (fields 0..23) in thread 0
-__device__ void reduce_kkt_partials(const double* __restrict__ part, int nblk, double* F) {
-  double f[24];
-#pragma unroll
-  for (int k = 0; k < 24; ++k) f[k] = 0.0;
-  const bool is_max[24] = {true, true, false, false, true, true, false, false, true,
-                           true, true, true, false, false, false, false,
-                           true, true, true, false, false, false, false, true};
-  for (int b = threadIdx.x; b < nblk; b += blockDim.x)
-#pragma unroll
-    for (int k = 0; k < 24; ++k) f[k] = is_max[k] ? nmax(f[k], part[b * 32 + k]) : f[k] + part[b * 32 + k];
-  block_reduce<24>(f, is_max);
-  if (threadIdx.x == 0)
-    for (int k = 0; k < 24; ++k) F[k] = f[k];
 }
 
 // ==========================================================================
@@ -2577,16 +2405,120 @@ static_assert(PDQP_NOALLOC_MAX_BLOCKS * (256 / 32) >= PDQP_NOALLOC_MAX_ROWS, "no
 
 // 8192 blocks x 32 partial sums x 8 bytes = 2 MiB per device.
 static __device__ __align__(256) double g_noalloc_scratch[PDQP_NOALLOC_MAX_BLOCKS * 32];
+// blocks of the call in flight that have written their partial sums
+static __device__ unsigned g_noalloc_ticket;
 
 static std::mutex g_noalloc_mu;
-static double* g_noalloc_addr[PDQP_NOALLOC_MAX_DEVICES] = {};
+struct NoallocAddr {
+  double* scratch;
+  unsigned* ticket;
+};
+static NoallocAddr g_noalloc_addr[PDQP_NOALLOC_MAX_DEVICES] = {};
 
-// The variant of the finishing step that writes the six parts to caller memory.
-__global__ void k_kkt_finish_noalloc(const double* __restrict__ part, int nblk, double* __restrict__ out) {
-  __shared__ double F[24];
-  pdqp::reduce_kkt_partials(part, nblk, F);
-  if (threadIdx.x == 0) pdqp::kkt_from_fields(F, 0, out);
+namespace pdqp {
+
+// sum over an aligned group of L lanes (L a power of two <= 32)
+__device__ __forceinline__ double lanes_sum(double s, int L) {
+  for (int o = L >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
 }
+
+struct NoallocArgs {
+  Csr<double> A, Q, At;
+  const double *x, *y, *b, *c, *l, *u;
+  int n, m, m_eq, LA, LN, gm, gn;
+  double* part;         // [max(gm, gn)][32]
+  unsigned* ticket;     // 0 at launch
+  double* out;
+};
+
+// Relative KKT error (Section 5 "Progress metric", equality/bound form) in
+// float64 of one point on the original problem, on separate Q, A, A' arrays.
+// Blocks [0, gm) take rows of A, blocks [gm, gm + gn) rows of Q and A', L lanes
+// per row; the last block to finish folds the partial sums.  A control-loop
+// problem (n = 172) is all latency: one launch behind the ticket's reset took
+// the place of a 2 KB reset and three launches.
+__global__ void __launch_bounds__(256) k_kkt_noalloc(NoallocArgs a) {
+  if ((int)blockIdx.x < a.gm) {
+    // fields: 0 max|viol|, 1 max|Ax|, 2 b'y, 8 max|b| (3..7 stay 0)
+    double f[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+    const int L = a.LA, row = blockIdx.x * (256 / L) + threadIdx.x / L, lane = threadIdx.x & (L - 1);
+    const bool valid = row < a.m;
+    double s = 0.0;
+    if (valid)
+      for (int k = a.A.rp[row] + lane; k < a.A.rp[row + 1]; k += L) s = fma(a.A.val[k], a.x[a.A.col[k]], s);
+    s = lanes_sum(s, L);
+    if (valid && lane == 0) {
+      const double bi = a.b[row];
+      f[0] = row < a.m_eq ? fabs(s - bi) : fmax(bi - s, 0.0);
+      f[1] = fabs(s);
+      f[2] = bi * a.y[row];
+      f[8] = fabs(bi);
+    }
+    const bool is_max[9] = {true, true, false, false, true, true, false, false, true};
+    block_reduce<9>(f, is_max);
+    if (threadIdx.x == 0)
+      for (int k = 0; k < 9; ++k) a.part[(size_t)blockIdx.x * 32 + k] = f[k];
+  } else {
+    // fields: 0 max|res|, 1 max|Qx|, 2 max|A'y|, 3 x'Qx, 4 c'x, 5 sum(l lam+ - u lam-), 14 max|c|
+    double f[15];
+#pragma unroll
+    for (int k = 0; k < 15; ++k) f[k] = 0.0;
+    const int blk = (int)blockIdx.x - a.gm;
+    const int L = a.LN, row = blk * (256 / L) + threadIdx.x / L, lane = threadIdx.x & (L - 1);
+    const bool valid = row < a.n;
+    double sq = 0.0, sa = 0.0;
+    if (valid) {
+      for (int k = a.Q.rp[row] + lane; k < a.Q.rp[row + 1]; k += L) sq = fma(a.Q.val[k], a.x[a.Q.col[k]], sq);
+      if (a.m > 0)
+        for (int k = a.At.rp[row] + lane; k < a.At.rp[row + 1]; k += L) sa = fma(a.At.val[k], a.y[a.At.col[k]], sa);
+    }
+    sq = lanes_sum(sq, L);
+    sa = lanes_sum(sa, L);
+    if (valid && lane == 0) {
+      const double cj = a.c[row], lj = a.l[row], uj = a.u[row], xj = a.x[row];
+      const bool lf = isfinite(lj), uf = isfinite(uj);
+      const double g = sq + cj - sa;
+      const double lam = (lf && uf) ? g : (lf ? fmax(g, 0.0) : (uf ? fmin(g, 0.0) : 0.0));
+      f[0] = fabs(g - lam);
+      f[1] = fabs(sq);
+      f[2] = fabs(sa);
+      f[3] = xj * sq;
+      f[4] = cj * xj;
+      f[5] = (lam > 0.0 ? lj * lam : 0.0) - (lam < 0.0 ? uj * (-lam) : 0.0);
+      f[14] = fabs(cj);
+    }
+    const bool is_max[15] = {true, true, true, false, false, false, false,
+                             true, true, true, false, false, false, false, true};
+    block_reduce<15>(f, is_max);
+    if (threadIdx.x == 0)
+      for (int k = 0; k < 15; ++k) a.part[(size_t)blk * 32 + 9 + k] = f[k];
+  }
+  __shared__ bool last;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
+    __threadfence();
+  }
+  __syncthreads();
+  if (!last) return;
+  double f[24];
+#pragma unroll
+  for (int k = 0; k < 24; ++k) f[k] = 0.0;
+  const bool is_max[24] = {true, true, false, false, true, true, false, false, true,
+                           true, true, true, false, false, false, false,
+                           true, true, true, false, false, false, false, true};
+  for (int b = threadIdx.x; b < max(a.gm, a.gn); b += 256)
+#pragma unroll
+    for (int k = 0; k < 24; ++k) {
+      const double v = b < (k < 9 ? a.gm : a.gn) ? __ldcg(a.part + (size_t)b * 32 + k) : 0.0;
+      f[k] = is_max[k] ? nmax(f[k], v) : f[k] + v;
+    }
+  block_reduce<24>(f, is_max);
+  if (threadIdx.x == 0) kkt_from_fields(f, 0, a.out);
+}
+
+}  // namespace pdqp
 
 extern "C" pdqp_status pdqp_kkt_noalloc(int64_t n, int64_t m, int64_t m_eq, const int32_t* Q_rowptr,
                                         const int32_t* Q_col, const double* Q_val, int64_t nnz_Q,
@@ -2623,19 +2555,20 @@ extern "C" pdqp_status pdqp_kkt_noalloc(int64_t n, int64_t m, int64_t m_eq, cons
   cudaStream_t s = (cudaStream_t)stream;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= PDQP_NOALLOC_MAX_DEVICES) return PDQP_ERR_CUDA;
-  double* scratch = nullptr;
+  NoallocAddr mem{};
   {
-    // once per device, with that device current: the device address of the array
+    // once per device, with that device current: the device addresses of the arrays
     std::lock_guard<std::mutex> lock(g_noalloc_mu);
-    if (!g_noalloc_addr[dev]) {
-      void* p = nullptr;
-      if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p) {
+    if (!g_noalloc_addr[dev].scratch) {
+      void *p = nullptr, *q = nullptr;
+      if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p ||
+          cudaGetSymbolAddress(&q, g_noalloc_ticket) != cudaSuccess || !q) {
         cudaGetLastError();
         return PDQP_ERR_CUDA;
       }
-      g_noalloc_addr[dev] = (double*)p;
+      g_noalloc_addr[dev] = NoallocAddr{(double*)p, (unsigned*)q};
     }
-    scratch = g_noalloc_addr[dev];
+    mem = g_noalloc_addr[dev];
   }
   const int LA = pdqp::pick_lanes(nnz_A, m);
   const int LN = pdqp::pick_lanes(nnz_Q + nnz_A, n);
@@ -2643,18 +2576,15 @@ extern "C" pdqp_status pdqp_kkt_noalloc(int64_t n, int64_t m, int64_t m_eq, cons
   const int gn = pdqp::cdiv(n, 256 / LN);
   const int nblk = gm > gn ? gm : gn;
   if (nblk > PDQP_NOALLOC_MAX_BLOCKS) return PDQP_ERR_INVALID;   // unreachable by the sizes above
-  // blocks that one of the two kernels does not launch contribute zeros
-  if (cudaMemsetAsync(scratch, 0, (size_t)nblk * 32 * sizeof(double), s) != cudaSuccess) return PDQP_ERR_CUDA;
-  pdqp::KktArgs a{};
+  if (cudaMemsetAsync(mem.ticket, 0, sizeof(unsigned), s) != cudaSuccess) return PDQP_ERR_CUDA;
+  pdqp::NoallocArgs a{};
   a.A = Csr<double>{A_rowptr, A_col, A_val};
   a.Q = Csr<double>{Q_rowptr, Q_col, Q_val};
   a.At = Csr<double>{At_rowptr, At_col, At_val};
-  a.x[0] = x; a.x[1] = x; a.y[0] = y; a.y[1] = y;
-  a.b = b; a.c = c; a.l = l; a.u = u;
-  a.part = scratch;
+  a.x = x; a.y = y; a.b = b; a.c = c; a.l = l; a.u = u;
   a.n = (int)n; a.m = (int)m; a.m_eq = (int)m_eq;
-  if (gm > 0) { DISPATCH_L(LA, pdqp::launch(pdqp::k_kkt_m<LL, 1, false>, gm, 256, 0, s, a)); }
-  DISPATCH_L(LN, pdqp::launch(pdqp::k_kkt_n<LL, 1, false>, gn, 256, 0, s, a));
-  pdqp::launch(k_kkt_finish_noalloc, 1, 256, 0, s, (const double*)scratch, nblk, parts);
+  a.LA = LA; a.LN = LN; a.gm = gm; a.gn = gn;
+  a.part = mem.scratch; a.ticket = mem.ticket; a.out = parts;
+  pdqp::launch(pdqp::k_kkt_noalloc, gm + gn, 256, 0, s, a);
   return cudaGetLastError() == cudaSuccess ? PDQP_OK : PDQP_ERR_CUDA;
 }
