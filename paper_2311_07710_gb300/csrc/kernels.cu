@@ -1129,29 +1129,30 @@ __device__ double refine_max_eig_warp(const double* __restrict__ al, const doubl
   return 0.5 * (lo + hi);
 }
 
-// A bracket [lo, hi) of lambda_max of the k x k tridiagonal, about 1e-6 of its
-// Gershgorin scale wide, that float64 Sturm counts at both ends confirm: four
-// float32 multisection rounds (alf, be2f: the tridiagonal divided by the
-// scale, written here), a margin of 2^-16 of the scale on both sides, then one
-// float64 round whose outer lanes sit on the ends.  Falls back to the
-// Gershgorin bracket when the check fails.  One warp.
-__device__ void bracket_max_eig_warp(const double* __restrict__ al, const double* __restrict__ be,
-                                     const double* __restrict__ be2, float* __restrict__ alf,
-                                     float* __restrict__ be2f, int k, double& lo, double& hi) {
+// The float32 bracket [flo, fhi) of lambda_max / G of the k x k tridiagonal, G
+// its Gershgorin scale, by four multisection rounds (alf, be2f: the
+// tridiagonal divided by G, written here).  A float32 Sturm count is the exact
+// count of a tridiagonal whose entries differ by a few float32 roundings of
+// the scale (Wilkinson 1965, chapter 5; with the conversions at most 2^-21 of G
+// in norm), so the bracket widened by LZ_F32_MARGIN holds the eigenvalue.
+// False where float32 cannot resolve it.  One warp.
+constexpr double LZ_F32_MARGIN = 0x1p-19;
+__device__ bool bracket_max_eig_f32_warp(const double* __restrict__ al, const double* __restrict__ be,
+                                         const double* __restrict__ be2, float* __restrict__ alf,
+                                         float* __restrict__ be2f, int k, double& glo, double& ghi, double& G,
+                                         float& flo, float& fhi) {
   const int lane = threadIdx.x & 31;
-  double glo, ghi;
   gershgorin_warp(al, be, k, glo, ghi);
-  lo = glo;
-  hi = ghi;
-  const double G = fmax(fabs(glo), fabs(ghi));
-  if (!(G > 1e-280 && G < 1e280) || ghi - glo <= 1e-5 * G) return;
+  G = fmax(fabs(glo), fabs(ghi));
+  if (!(G > 1e-280 && G < 1e280) || ghi - glo <= 1e-5 * G) return false;
   const double iG = 1.0 / G;
   for (int i = lane; i < k; i += 32) {
     alf[i] = (float)(al[i] * iG);
     if (i < k - 1) be2f[i] = (float)(be2[i] * iG * iG);
   }
   __syncwarp();
-  float flo = (float)(glo * iG), fhi = (float)(ghi * iG);
+  flo = (float)(glo * iG);
+  fhi = (float)(ghi * iG);
   for (int round = 0; round < 4; ++round) {
     const float step = (fhi - flo) * (1.f / 33.f);
     const float x = flo + step * (float)(lane + 1);
@@ -1165,11 +1166,20 @@ __device__ void bracket_max_eig_warp(const double* __restrict__ al, const double
       flo = nlo;
     }
   }
-  const double clo = fmax(glo, ((double)flo - 0x1p-16) * G);
-  const double chi = fmin(ghi, ((double)fhi + 0x1p-16) * G);
-  const double step = (chi - clo) * (1.0 / 31.0);
+  return true;
+}
+
+// One float64 round over [lo, hi) whose outer lanes sit on its ends: confirms
+// it and narrows it to about 1e-6 of the scale, or falls back to the
+// Gershgorin bracket.  One warp.
+__device__ void confirm_bracket_warp(const double* __restrict__ al, const double* __restrict__ be2, int k, double glo,
+                                     double ghi, double& lo, double& hi) {
+  const int lane = threadIdx.x & 31;
+  const double clo = lo, chi = hi, step = (chi - clo) * (1.0 / 31.0);
   const double x = lane == 31 ? chi : clo + step * (double)lane;
   const unsigned ge = __ballot_sync(0xffffffffu, sturm_count(al, be2, k, x) < k);
+  lo = glo;
+  hi = ghi;
   if ((ge & 1u) && !(ge >> 31)) {              // lambda_max in [clo, chi)
     const int t = 31 - __clz(ge);
     lo = clo + step * (double)t;
@@ -1232,11 +1242,29 @@ __global__ void __launch_bounds__(NT) k_lz_beta(LzArgs a, double tol, int max_st
   const int o = (threadIdx.x >> 6) & 1, second = (threadIdx.x >> 5) & 1, lane = threadIdx.x & 31;
   const double plo = st.pi_lam_prev[o], phi = st.pi_hi_prev[o];   // bracket of theta_{k-1}
   if (ritz && !done_in[o] && !second) {           // warp-uniform
-    double lo, hi;
-    bracket_max_eig_warp(s_al(o), s_be(o), s_be2(o), s_alf(o), s_be2f(o), k, lo, hi);
-    const double mag = fmax(fabs(lo), fabs(hi));
-    const double gap = fmax(fmax(lo - phi, plo - hi), 0.0);   // least |theta_k - theta_{k-1}|
-    const bool go_on = k < max_steps && beta[o] > 1e-12 * mag && gap > tol * mag;
+    // far from the stop the float32 bracket shows that the step goes on, and
+    // the float64 round (three float64-pipe operations a row and lane) is not needed
+    double glo, ghi, G;
+    float flo, fhi;
+    const bool f32 = bracket_max_eig_f32_warp(s_al(o), s_be(o), s_be2(o), s_alf(o), s_be2f(o), k, glo, ghi, G, flo,
+                                              fhi);
+    double lo = glo, hi = ghi;
+    if (f32) {
+      lo = fmax(glo, ((double)flo - LZ_F32_MARGIN) * G);
+      hi = fmin(ghi, ((double)fhi + LZ_F32_MARGIN) * G);
+    }
+    auto goes_on = [&]() {
+      const double mag = fmax(fabs(lo), fabs(hi));
+      const double gap = fmax(fmax(lo - phi, plo - hi), 0.0);   // least |theta_k - theta_{k-1}|
+      return k < max_steps && beta[o] > 1e-12 * mag && gap > tol * mag;
+    };
+    bool go_on = goes_on();
+    if (!go_on && f32) {                          // warp-uniform
+      lo = fmax(glo, ((double)flo - 0x1p-16) * G);
+      hi = fmin(ghi, ((double)fhi + 0x1p-16) * G);
+      confirm_bracket_warp(s_al(o), s_be2(o), k, glo, ghi, lo, hi);
+      go_on = goes_on();
+    }
     if (lane == 0) {
       s_lo[o] = lo;
       s_hi[o] = hi;
