@@ -112,25 +112,31 @@ typedef struct {
   int32_t spmv_threads;      /* iteration-kernel variant: 256 or 512 threads per row
                                 block, 1 = pipelined persistent (cp.async prefetch of
                                 the next row block), 2 = a whole chunk of iterations
-                                in one launch of a 16-CTA thread-block cluster (8 where
-                                16 cannot be resident) with a
-                                cluster barrier after each half-step (problems of at
-                                most 64 row blocks of A and of P, no row longer than a
-                                row block, no low-rank term; else PDQP_ERR_INVALID),
+                                in one launch, a CTA or a thread-block cluster of up
+                                to 16 (8 where 16 cannot be resident) per instance
+                                with a barrier after each half-step (asked for:
+                                problems of at most 64 row blocks of A and of P, no
+                                row longer than a row block, no low-rank term; else
+                                PDQP_ERR_INVALID),
                                 3 = family handles (pdqp_create_family; no row longer
                                 than a row block, no low-rank term; else
                                 PDQP_ERR_INVALID): the iteration vectors interleaved
                                 by member, v[j * members + i], one warp per row for 32
                                 members, so one matrix entry meets 128 members in one
                                 coalesced load,
-                                0 = autotuned: 3 for an eligible family handle, else
-                                the first full chunk of a handle's first solve in each
-                                precision times two rounds of 3 iterations of each
-                                eligible variant and keeps the fastest for that
-                                precision; the choice is also kept for the process per
-                                problem shape, so later handles of the same sizes,
-                                nonzeros and row blocks start with it (all variants
-                                give bitwise identical iterates) */
+                                0 = chosen: 3 for an eligible family handle; 2 where
+                                every instance's vectors fit a CTA's shared memory and
+                                the instances are many or small; for a low-rank term
+                                over short rows of P, kernels that read the factor once
+                                per iteration (pdqp_info reports them as 4, which
+                                cannot be asked for); else the first full chunk of a
+                                handle's first solve in each precision times two
+                                rounds of 4 iterations of each of 256, 512 and 1 and
+                                keeps the fastest for that precision; the choice is
+                                also kept for the process per problem shape, so later
+                                handles of the same sizes, nonzeros and row blocks
+                                start with it (all variants give bitwise identical
+                                iterates) */
   int32_t no_graphs;         /* 0: replay each full chunk of check_period iterations
                                 and its check as one captured CUDA graph; 1: launch
                                 every kernel directly */
@@ -181,8 +187,8 @@ typedef struct {
 /* Per-kernel device time of the solver's hot loop, measured with CUDA events
  * recorded on the solve's stream around every launch while profiling is on.
  * kind 0 = dual half-step, 1 = primal half-step, 2 = relKKT check + restart,
- * 3 = the one-launch cluster chunk (spmv_threads 2: both half-steps of a
- * chunk's iterations per launch).  Scaling, norms, start point and output are
+ * 3 = the one-launch chunk (spmv_threads 2: both half-steps of a chunk's
+ * iterations per launch).  Scaling, norms, start point and output are
  * not timed. */
 typedef struct {
   int64_t launches[4];

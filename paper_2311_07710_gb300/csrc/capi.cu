@@ -42,7 +42,7 @@ struct pdqp_problem {
   std::vector<pdqp_info> infos;                       // per instance, from the last solve
   std::vector<void*> allocs;
   int tuned_nt[2] = {0, 0};                           // autotuned variant per precision (0: not yet)
-  cudaEvent_t tune_ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
+  cudaEvent_t tune_ev[4] = {nullptr, nullptr, nullptr, nullptr};
   // Where the last solve stopped (what pdqp_get_state exports): its parameters,
   // the step-table position (iterations run since the table was last filled;
   // 0 at a check) and the iterations of the solve loop.
@@ -623,6 +623,18 @@ void tuned_store(const Work& w, bool mixed, int nt) {
   g_tuned[tune_key(w, mixed)] = nt;
 }
 
+void alloc_chunk(pdqp_problem* h, bool mixed, cudaStream_t s);   // with the device scans, below
+
+// options.spmv_threads = 2: at most 64 row blocks of A and of P, no row longer
+// than a row block, no low-rank term, and 3n + 2m values (with a row block's
+// staging) within 200 KB.
+bool chunk_asked_ok(const Work& w, bool mixed) {
+  const size_t sv = mixed ? sizeof(float) : sizeof(double);
+  const size_t head = (BNNZ * sv + (BROWS + 1) * sizeof(int) + 15) / 16 * 16;
+  return w.r == 0 && w.A.nlseg == 0 && w.P.nlseg == 0 && w.A.nblk <= 64 && w.P.nblk <= 64 && w.P.nblk > 0 &&
+         head + (3 * (size_t)w.n + 2 * (size_t)w.m) * sv <= 200 * 1024;
+}
+
 pdqp_status solve_impl(pdqp_problem* h, const pdqp_options& o, const double* x0, const double* y0,
                        double* x_out, double* y_out, pdqp_info* info, int mem, cudaStream_t s) {
   const double t0 = now_s();
@@ -635,11 +647,10 @@ pdqp_status solve_impl(pdqp_problem* h, const pdqp_options& o, const double* x0,
   check_space(x_out, mem, "x_out");
   check_space(y_out, mem, "y_out");
   const bool mixed = o.precision == PDQP_PREC_MIXED;
-  const bool cluster_ok = pdqp::chunk_cluster_ok(w, mixed);
-  if (o.spmv_threads == 2 && !cluster_ok)
+  const bool chunk_ok = pdqp::chunk_ok(w, mixed);
+  if (o.spmv_threads == 2 && !(chunk_ok && chunk_asked_ok(w, mixed)))
     throw Fail{PDQP_ERR_INVALID, "options.spmv_threads = 2 needs at most 64 row blocks of A and of P, no row "
                                  "longer than a row block, no low-rank term and 3n + 2m values within 200 KB"};
-  if (cluster_ok) pdqp::prepare_chunk_cluster();
   // family handles run on member-interleaved vectors unless a row-block
   // variant is asked for (no low-rank term, no long rows)
   const bool il_ok = w.fam_il && w.r == 0;
@@ -665,6 +676,17 @@ pdqp_status solve_impl(pdqp_problem* h, const pdqp_options& o, const double* x0,
   if (w.detect) alloc_infeas(h, s);
   SolveParams p = make_params(o);
   if (use_il) p.spmv_threads = 3;
+  // the one-launch chunk: asked for, or chosen where every instance fits it
+  const bool use_chunk = !use_il && !mp && chunk_ok && (o.spmv_threads == 2 || (o.spmv_threads == 0 && pdqp::chunk_pays(w, mixed)));
+  if (use_chunk) {
+    alloc_chunk(h, mixed, s);
+    p.spmv_threads = 2;
+  }
+  // the iteration-kernel variant, where nothing above fixes it: the one this
+  // shape was tuned to, or timed on the first chunk (below)
+  const bool autotune = o.spmv_threads == 0 && !use_il && !mp && !use_chunk;
+  int& tuned = h->tuned_nt[mixed ? 1 : 0];
+  if (autotune && !tuned) tuned = tuned_lookup(w, mixed);
   w.mp = mp ? 1 : 0;
   w.mp_accelerate = p.accelerate;
   if (mp) {
@@ -734,6 +756,7 @@ pdqp_status solve_impl(pdqp_problem* h, const pdqp_options& o, const double* x0,
     pdqp::scale_apply(sw, mixed, s);
   }
   pdqp::scale_apply(w, mixed, s, rep_vals ? &sw : nullptr);
+  if (use_chunk) pdqp::chunk_fill_values(w, mixed, s);
 
   // spectral norms of the scaled matrices (a resumed solve keeps its own)
   const bool run_lanczos = !resuming && !(o.norm_A > 0.0 && o.norm_Q > 0.0);
@@ -793,17 +816,13 @@ pdqp_status solve_impl(pdqp_problem* h, const pdqp_options& o, const double* x0,
   // two rounds of TUNE iterations with each candidate (interleaved, so that no
   // candidate always runs first on a cold cache), keeps the fastest by its
   // better round and runs the rest of the chunk with it; the iterates do not
-  // depend on the variant.  Problems of a few row blocks also try the
-  // one-launch cluster chunk.  Each candidate's iterations are captured into a
+  // depend on the variant.  Each candidate's iterations are captured into a
   // graph and replayed, as the solve loop runs them (direct launches would
   // charge the per-iteration variants launch gaps that graphs do not have);
   // with the event profiler on, they are launched directly.
-  static const int kCand[4] = {256, 512, 1, 2};
-  const int ncand = cluster_ok ? 4 : 3;
+  static const int kCand[3] = {256, 512, 1};
+  constexpr int ncand = 3;
   constexpr int TUNE = 4, ROUNDS = 2;
-  const bool autotune = o.spmv_threads == 0 && !use_il && !mp;
-  int& tuned = h->tuned_nt[mixed ? 1 : 0];
-  if (autotune && !tuned) tuned = tuned_lookup(w, mixed);   // a handle of the same shape tuned before
   if (autotune && tuned) p.spmv_threads = tuned;
   while (w.bst_host->running > 0) {
     const long long len = std::min<long long>(o.check_period, o.max_iter - k_total);
@@ -813,13 +832,13 @@ pdqp_status solve_impl(pdqp_problem* h, const pdqp_options& o, const double* x0,
     if (tune_now) {
       for (auto& e : h->tune_ev)
         if (!e) CK(cudaEventCreate(&e));
-      float best_ms[4] = {0.f, 0.f, 0.f, 0.f};
+      float best_ms[ncand] = {0.f, 0.f, 0.f};
       int j = 0;
       const bool replay = !w.prof.on && !o.no_graphs;
       if (replay) pdqp::iterate(w, 0, mixed, 1, s, 0);   // one-time setup of the pipelined variant
       for (int r = 0; r < ROUNDS; ++r) {
-        cudaGraphExec_t ex[4] = {nullptr, nullptr, nullptr, nullptr};
-        long long kern[4] = {0, 0, 0, 0};
+        cudaGraphExec_t ex[ncand] = {nullptr, nullptr, nullptr};
+        long long kern[ncand] = {0, 0, 0};
         if (replay)
           for (int c = 0; c < ncand; ++c) ex[c] = capture_iterations(h, TUNE, mixed, kCand[c], j + c * TUNE, &kern[c]);
         CK(cudaEventRecord(h->tune_ev[0], s));
@@ -1764,6 +1783,47 @@ void device_scan(const int* in, int len, int* out, std::vector<void*>& tmp, cuda
   CK(cudaGetLastError());
 }
 
+// The one-launch chunk's slice layout (chunk.cu), built on the first solve that
+// runs it: structure once per handle, the scaled values by every solve.
+void alloc_chunk(pdqp_problem* h, bool mixed, cudaStream_t s) {
+  Work& w = h->w;
+  ChunkPlan& ck = w.chunk;
+  if (!ck.built) {
+    pdqp::chunk_plan_instances(w);
+    ck.inst = dalloc<ChunkInst>(h, w.count);
+    to_device(ck.inst, ck.order.data(), ck.order.size(), s);
+    ck.sp = dalloc<int>(h, (size_t)ck.slices + 1);
+    TmpFree tmp;
+    tmp.s = s;
+    int* wid = (int*)pool_alloc((size_t)std::max(ck.slices, 1) * sizeof(int), s);
+    tmp.v.push_back(wid);
+    pdqp::chunk_widths(w, wid, s);
+    device_scan(wid, ck.slices, ck.sp, tmp.v, s);
+    int2* dg = (int2*)pool_alloc((size_t)w.count * sizeof(int2), s);
+    tmp.v.push_back(dg);
+    pdqp::chunk_groups(w, dg, s);
+    std::vector<int2> groups((size_t)w.count);
+    CK(cudaMemcpyAsync(groups.data(), dg, groups.size() * sizeof(int2), cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    long long total = 0;
+    for (const int2& g : groups) total += (long long)g.x + g.y;
+    ck.ngroups = total;
+    pdqp::chunk_plan_order(w, groups);
+    to_device(ck.inst, ck.order.data(), ck.order.size(), s);
+    ck.idx = dalloc<unsigned>(h, (size_t)total * 32);
+    pdqp::chunk_fill_index(w, s);
+    for (auto& t : ck.side)
+      if (!t) CK(cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking));
+    for (cudaEvent_t* e : {&ck.fork, &ck.join[0], &ck.join[1]})
+      if (!*e) CK(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+    CK(cudaGetLastError());
+    ck.built = true;
+  }
+  if (mixed && !ck.valf) ck.valf = dalloc<float2>(h, (size_t)ck.ngroups * 32);
+  if (!mixed && !ck.vald) ck.vald = dalloc<double2>(h, (size_t)ck.ngroups * 32);
+  if (ck.cls[mixed ? 1 : 0].empty()) pdqp::chunk_plan_classes(w, mixed);
+}
+
 // A batch handed over as one block-diagonal problem: instance i owns the
 // variables [xoff_i, xoff_i + n_i) and the rows [yoff_i, yoff_i + m_i), in
 // order; Q (N rows) and A (M rows) are CSR over the whole stack with global
@@ -2495,6 +2555,10 @@ void pdqp_destroy(pdqp_handle h) {
   for (auto& c : h->cgraphs)
     if (c.exec) cudaGraphExecDestroy(c.exec);
   if (h->cap) cudaStreamDestroy(h->cap);
+  for (auto& t : h->w.chunk.side)
+    if (t) cudaStreamDestroy(t);
+  for (cudaEvent_t e : {h->w.chunk.fork, h->w.chunk.join[0], h->w.chunk.join[1]})
+    if (e) cudaEventDestroy(e);
   if (h->tmpl) pdqp_destroy(h->tmpl);
   delete h;
 }

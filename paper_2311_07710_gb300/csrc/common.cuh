@@ -232,3 +232,11 @@ __device__ __forceinline__ double r_mul(double a, double b) { return __dmul_rn(a
 __device__ __forceinline__ float r_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double r_fma(double a, double b, double c) { return __fma_rn(a, b, c); }
 
+// s + v x, one term of a row sum of the half-steps: in float32 the product is
+// rounded, then the sum (products pass through shared memory in the row-block
+// kernels); in float64 one fused multiply-add, since GB300 retires two float64
+// lanes per clock per SM and the two operations a nonzero bound the small
+// instances' half-steps.  Every variant forms its row sums with it.
+__device__ __forceinline__ float r_dot(float v, float x, float s) { return __fadd_rn(s, __fmul_rn(v, x)); }
+__device__ __forceinline__ double r_dot(double v, double x, double s) { return __fma_rn(v, x, s); }
+

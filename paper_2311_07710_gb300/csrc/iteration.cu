@@ -5,16 +5,13 @@
 //   k_primal : rows of P = [Q | -A'] gathering [x_md ; y+] -- g = Q x_md + c - A'y+,
 //              x+ = proj_[l,u](x - tau g), x_bar+ = (1 - 1/beta) x_bar + x+/beta,
 //              and the next iteration's x_md and x_tilde
-// with their pipelined persistent variants, the segment sums of long rows,
-// and the host loop that launches a chunk of iterations.
-#include <cooperative_groups.h>
-
+// with their pipelined persistent variants, the member-interleaved family
+// kernels, the segment sums of long rows, and the host loop that launches a
+// chunk of iterations (a whole chunk in one launch: chunk.cu).
 #include <algorithm>
-#include <mutex>
 
 #include "rowblock.cuh"
-
-namespace cg = cooperative_groups;
+#include "rowupdate.cuh"
 
 namespace pdqp {
 
@@ -40,33 +37,6 @@ struct DualB {
   const int* __restrict__ act;          // row block of each CUDA block (null: the block index)
 };
 
-template <typename V> __device__ __forceinline__ V step_sigma(const StepEntry& e);
-template <> __device__ __forceinline__ double step_sigma<double>(const StepEntry& e) { return e.sigma_d; }
-template <> __device__ __forceinline__ float step_sigma<float>(const StepEntry& e) { return e.sigma_d_f; }
-template <typename V> __device__ __forceinline__ V step_tau(const StepEntry& e);
-template <> __device__ __forceinline__ double step_tau<double>(const StepEntry& e) { return e.tau_p; }
-template <> __device__ __forceinline__ float step_tau<float>(const StepEntry& e) { return e.tau_p_f; }
-template <typename V> __device__ __forceinline__ V step_ib(const StepEntry& e);
-template <> __device__ __forceinline__ double step_ib<double>(const StepEntry& e) { return e.inv_beta; }
-template <> __device__ __forceinline__ float step_ib<float>(const StepEntry& e) { return e.inv_beta_f; }
-template <typename V> __device__ __forceinline__ V step_ibn(const StepEntry& e);
-template <> __device__ __forceinline__ double step_ibn<double>(const StepEntry& e) { return e.inv_beta_next; }
-template <> __device__ __forceinline__ float step_ibn<float>(const StepEntry& e) { return e.inv_beta_next_f; }
-template <typename V> __device__ __forceinline__ V step_thn(const StepEntry& e);
-template <> __device__ __forceinline__ double step_thn<double>(const StepEntry& e) { return e.theta_next; }
-template <> __device__ __forceinline__ float step_thn<float>(const StepEntry& e) { return e.theta_next_f; }
-
-// The dual update of one row from its sum s = (A x_tilde)_r: y+ and y_bar+
-// (shared by the row-block and the member-interleaved kernels).
-template <typename V>
-__device__ __forceinline__ void dual_update(const StepEntry& e, V s, V yo, V bi, V yb, V lo, bool ineq, V& yn,
-                                            V& ybn) {
-  const V sigma = step_sigma<V>(e), ib = step_ib<V>(e);
-  yn = r_fma(-sigma, r_sub(s, bi), yo);                       // y - sigma (A x_tilde - b)
-  if (ineq) yn = fmax(yn, lo);
-  ybn = r_fma(ib, yn, r_mul(r_sub(V(1), ib), yb));            // (1 - 1/beta) y_bar + y+/beta
-}
-
 template <typename V>
 __device__ __forceinline__ void dual_row(const DualB<V>& a, const StepEntry& e, int r, V s, V yo, V bi, V yb,
                                          V lo) {
@@ -76,10 +46,21 @@ __device__ __forceinline__ void dual_row(const DualB<V>& a, const StepEntry& e, 
   a.ynew[r] = yn;
 }
 
-// The dual half-step of row block bk (one CUDA block): prod and srp are the
-// block's staging buffers; GM is how x_tilde is gathered (see stage_products).
-template <typename V, int NT, int GM>
-__device__ __forceinline__ void dual_block(const DualB<V>& a, int bk, int j, V* prod, int* srp) {
+__device__ __forceinline__ float staged_sum(const float* prod, const float*, int e, int end) {
+  float s = 0.f;
+  for (; e < end; ++e) s += prod[e];
+  return s;
+}
+__device__ __forceinline__ double staged_sum(const double* sval, const double* sx, int e, int end) {
+  double s = 0.0;
+  for (; e < end; ++e) s = r_dot(sval[e], sx[e], s);
+  return s;
+}
+
+// The dual half-step of row block bk (one CUDA block): prod, sx and srp are the
+// block's staging buffers.
+template <typename V, int NT>
+__device__ __forceinline__ void dual_block(const DualB<V>& a, int bk, int j, V* prod, V* sx, int* srp) {
   const int tid = threadIdx.x;
   const int inst = a.blk_inst[bk];
   if (a.st[inst].status != ST_RUNNING) return;    // uniform over the block
@@ -87,20 +68,23 @@ __device__ __forceinline__ void dual_block(const DualB<V>& a, int bk, int j, V* 
   const int nr = r1 - r0;
   const int e0 = a.A.rp[r0];
   const int ne = a.A.rp[r1] - e0;
-  // operands of this thread's first row, fetched before the SpMV
+  // operands of this thread's first row, fetched before the gathers
   V yo = V(0), bi = V(0), yb = V(0), lo = V(0);
-  if (tid < nr) {
-    const int r = r0 + tid;
-    yo = a.yold[r]; bi = a.b[r]; yb = a.ybar[r];
-    if (a.ylo) lo = a.ylo[r];
-  }
-  const StepEntry& es = a.tab[inst * a.C + j];
+  auto mid = [&]() {
+    if (tid < nr) {
+      const int r = r0 + tid;
+      yo = a.yold[r]; bi = a.b[r]; yb = a.ybar[r];
+      if (a.ylo) lo = a.ylo[r];
+    }
+    return true;
+  };
+  if (ne > BNNZ && !mid()) return;
   if (ne <= BNNZ) {
-    stage_products<NT, GM>(a.A, a.xt, e0, ne, r0, nr, prod, srp);
+    if (!stage_rows<NT>(a.A, a.xt, e0, ne, r0, nr, prod, sx, srp, mid)) return;
     __syncthreads();
+    const StepEntry& es = a.tab[inst * a.C + j];
     for (int t = tid; t < nr; t += NT) {
-      V s = V(0);
-      for (int e = srp[t]; e < srp[t + 1]; ++e) s += prod[e];
+      const V s = staged_sum(prod, sx, srp[t], srp[t + 1]);
       const int r = r0 + t;
       if (t >= BNT) {
         yo = a.yold[r]; bi = a.b[r]; yb = a.ybar[r];
@@ -113,24 +97,25 @@ __device__ __forceinline__ void dual_block(const DualB<V>& a, int bk, int j, V* 
       const int2 sg = a.blk_seg[bk];
       V s = V(0);
       for (int q = 0; q < sg.y; ++q) s += a.lpart[sg.x + q];
-      dual_row(a, es, r0, s, yo, bi, yb, lo);
+      dual_row(a, a.tab[inst * a.C + j], r0, s, yo, bi, yb, lo);
     }
   } else {   // a single row longer than a block
     V s = V(0);
     for (int e = e0 + tid; e < e0 + ne; e += NT)
-      s += a.A.val[e] * gather_load<GM>(a.xt + a.A.col[e]);
+      s += a.A.val[e] * __ldg(a.xt + a.A.col[e]);
     s = block_sum(s);
-    if (tid == 0) dual_row(a, es, r0, s, yo, bi, yb, lo);
+    if (tid == 0) dual_row(a, a.tab[inst * a.C + j], r0, s, yo, bi, yb, lo);
   }
 }
 
 template <typename V, int NT>
 __global__ void __launch_bounds__(NT, MinBlocks<V, NT>::value) k_dual(DualB<V> a, int j) {
   __shared__ V prod[BNNZ];
+  __shared__ V sx[sizeof(V) == 8 ? BNNZ : 1];
   __shared__ int srp[BROWS + 1];
   const int bk = a.act ? a.act[blockIdx.x] : (int)blockIdx.x;   // compacted batches: running blocks only
   if (bk < 0) return;                                             // padding of a compacted grid
-  dual_block<V, NT, GATHER_LDG>(a, bk, j, prod, srp);
+  dual_block<V, NT>(a, bk, j, prod, sx, srp);
 }
 
 // --------------------------------------------------------------------------
@@ -159,19 +144,6 @@ struct PrimalB {
   const int* __restrict__ act;          // row block of each CUDA block (null: the block index)
 };
 
-// The primal update of one row from g = (Q x_md - A'y+)_r + c_r (+ the
-// low-rank term): x+, x_bar+ and the next iteration's x_md and x_tilde
-// (shared by the row-block and the member-interleaved kernels).
-template <typename V>
-__device__ __forceinline__ void primal_update(const StepEntry& e, V g, V xo, V xb0, V lr, V ur, V& xn, V& xb, V& zo,
-                                              V& xtn) {
-  const V tau = step_tau<V>(e), ib = step_ib<V>(e), ibn = step_ibn<V>(e), thn = step_thn<V>(e);
-  xn = fmin(fmax(r_fma(-tau, g, xo), lr), ur);               // proj_X(x - tau g)
-  xb = r_fma(ib, xn, r_mul(r_sub(V(1), ib), xb0));            // (1 - 1/beta) x_bar + x+/beta
-  zo = r_fma(ibn, xn, r_mul(r_sub(V(1), ibn), xb));           // next x_md
-  xtn = r_fma(thn, r_sub(xn, xo), xn);                        // next x_tilde
-}
-
 template <typename V, bool LR = false>
 __device__ __forceinline__ void primal_row(const PrimalB<V>& a, const StepEntry& e, int r, V s, V xo, V xb0,
                                            V cr, V lr, V ur) {
@@ -186,8 +158,8 @@ __device__ __forceinline__ void primal_row(const PrimalB<V>& a, const StepEntry&
 }
 
 // The primal half-step of row block bk (one CUDA block), as dual_block.
-template <typename V, int NT, bool LR, int GM>
-__device__ __forceinline__ void primal_block(const PrimalB<V>& a, int bk, int j, V* prod, int* srp) {
+template <typename V, int NT, bool LR>
+__device__ __forceinline__ void primal_block(const PrimalB<V>& a, int bk, int j, V* prod, V* sx, int* srp) {
   const int tid = threadIdx.x;
   const int inst = a.blk_inst[bk];
   if (a.st[inst].status != ST_RUNNING) return;    // uniform over the block
@@ -196,17 +168,20 @@ __device__ __forceinline__ void primal_block(const PrimalB<V>& a, int bk, int j,
   const int e0 = a.P.rp[r0];
   const int ne = a.P.rp[r1] - e0;
   V xo = V(0), xb = V(0), cr = V(0), lr = V(0), ur = V(0);
-  if (tid < nr) {
-    const int r = r0 + tid;
-    xo = a.x[r]; xb = a.xbar[r]; cr = a.c[r]; lr = a.l[r]; ur = a.u[r];
-  }
-  const StepEntry& es = a.tab[inst * a.C + j];
+  auto mid = [&]() {
+    if (tid < nr) {
+      const int r = r0 + tid;
+      xo = a.x[r]; xb = a.xbar[r]; cr = a.c[r]; lr = a.l[r]; ur = a.u[r];
+    }
+    return true;
+  };
+  if (ne > BNNZ && !mid()) return;
   if (ne <= BNNZ) {
-    stage_products<NT, GM>(a.P, a.zin, e0, ne, r0, nr, prod, srp);
+    if (!stage_rows<NT>(a.P, a.zin, e0, ne, r0, nr, prod, sx, srp, mid)) return;
     __syncthreads();
+    const StepEntry& es = a.tab[inst * a.C + j];
     for (int t = tid; t < nr; t += NT) {
-      V s = V(0);
-      for (int e = srp[t]; e < srp[t + 1]; ++e) s += prod[e];
+      const V s = staged_sum(prod, sx, srp[t], srp[t + 1]);
       const int r = r0 + t;
       if (t >= BNT) { xo = a.x[r]; xb = a.xbar[r]; cr = a.c[r]; lr = a.l[r]; ur = a.u[r]; }
       primal_row<V, LR>(a, es, r, s, xo, xb, cr, lr, ur);
@@ -216,14 +191,14 @@ __device__ __forceinline__ void primal_block(const PrimalB<V>& a, int bk, int j,
       const int2 sg = a.blk_seg[bk];
       V s = V(0);
       for (int q = 0; q < sg.y; ++q) s += a.lpart[sg.x + q];
-      primal_row<V, LR>(a, es, r0, s, xo, xb, cr, lr, ur);
+      primal_row<V, LR>(a, a.tab[inst * a.C + j], r0, s, xo, xb, cr, lr, ur);
     }
   } else {
     V s = V(0);
     for (int e = e0 + tid; e < e0 + ne; e += NT)
-      s += a.P.val[e] * gather_load<GM>(a.zin + a.P.col[e]);
+      s += a.P.val[e] * __ldg(a.zin + a.P.col[e]);
     s = block_sum(s);
-    if (tid == 0) primal_row<V, LR>(a, es, r0, s, xo, xb, cr, lr, ur);
+    if (tid == 0) primal_row<V, LR>(a, a.tab[inst * a.C + j], r0, s, xo, xb, cr, lr, ur);
   }
 }
 
@@ -232,242 +207,14 @@ __device__ __forceinline__ void primal_block(const PrimalB<V>& a, int bk, int j,
 template <typename V, int NT, bool LR = false>
 __global__ void __launch_bounds__(NT, MinBlocks<V, NT, LR>::value) k_primal(PrimalB<V> a, int j) {
   __shared__ V prod[BNNZ];
+  __shared__ V sx[sizeof(V) == 8 ? BNNZ : 1];
   __shared__ int srp[BROWS + 1];
   const int bk = a.act ? a.act[blockIdx.x] : (int)blockIdx.x;
   if (bk < 0) return;
   // (the dual half-step measured no gain from it: 202.6 -> 203.9 ms of a control-QP
   // batch solve, against 225.4 -> 219.9 here)
   prefetch_ahead(a.P, a.act, (int)blockIdx.x, (int)gridDim.x);
-  primal_block<V, NT, LR, GATHER_LDG>(a, bk, j, prod, srp);
-}
-
-// --------------------------------------------------------------------------
-// A whole chunk of iterations in one launch, for small problems (whose
-// per-iteration kernels are bound by launch and gather latency): one cluster
-// of C = 16 CTAs (8 where 16 cannot be co-scheduled).  Every CTA keeps its own copy of x_tilde and of both
-// [x_md ; y] buffers in shared memory and gathers from it; after each
-// half-step it writes the rows it updated into every CTA's copy (distributed
-// shared memory) and the cluster meets at a barrier (release / acquire).  CTA
-// c takes row blocks c, c + C, ... of A and of P.  The row arithmetic
-// is that of k_dual / k_primal, so the iterates are bitwise theirs, and every
-// result still goes to global memory for the checks.  Every thread of every
-// CTA takes the same 2 * len + 1 barriers: no path leaves the loop early
-// (blocks of an instance that stopped are skipped).  No low-rank term, no
-// long rows, and the copies must fit in shared memory (the host checks).
-// --------------------------------------------------------------------------
-constexpr int CHUNK_NT = 512;
-constexpr int CHUNK_MAX_BLOCKS = 64;               // row blocks of A and of P, each
-constexpr int CHUNK_SMEM_MAX = 200 * 1024;
-
-// every thread of the cluster arrives (release) and waits (acquire); the
-// unaligned form does not need the warp converged at the barrier
-__device__ __forceinline__ void cluster_barrier() {
-  asm volatile("barrier.cluster.arrive.release;\n" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire;\n" ::: "memory");
-}
-
-template <typename V>
-constexpr size_t chunk_head_bytes() {     // staging buffers, rounded to 16 bytes
-  return ((size_t)BNNZ * sizeof(V) + (BROWS + 1) * sizeof(int) + 15) / 16 * 16;
-}
-template <typename V>
-static size_t chunk_smem_bytes(int n, int m) {
-  return chunk_head_bytes<V>() + (size_t)(3 * (size_t)n + 2 * (size_t)m) * sizeof(V);
-}
-
-// write v into slot p of every CTA's copy (p: this CTA's shared address)
-template <typename V>
-__device__ __forceinline__ void broadcast(cg::cluster_group& cl, int ctas, V* p, V v) {
-  for (int q = 0; q < ctas; ++q) *cl.map_shared_rank(p, q) = v;
-}
-
-// Resident row blocks: where every CTA takes at most one row block of A and
-// one of P, each CTA keeps its blocks in shared memory for the launch: the
-// row offsets, column indices and values, and the rows' own operands (of A:
-// b, y_bar, the inequality flag and the mixed-precision lower bound; of P: x,
-// x_bar, c, l, u), which only this CTA updates.  A half-step's dependent chain
-// then runs from the gathers out of the shared-memory vector copies to the
-// writes into every CTA's copies, straight from registers, with no global
-// round trip on it (the results still go to global memory for the checks).
-// The products val[e] * v[col[e]], the row sums in order and the row updates
-// are dual_block / primal_block's, so the iterates stay theirs.
-constexpr int RES_ROWS = 5;   // operand rows per resident block
-template <typename V>
-struct ResBlock {
-  int r0, nr, ne;
-  V* val;            // [BNNZ]
-  V* row[RES_ROWS];  // [BROWS] each
-  int* col;          // [BNNZ]
-  int* srp;          // [BROWS + 1]
-};
-template <typename V>
-__host__ __device__ inline size_t chunk_res_offset(int n, int m) {   // behind the vector copies, 16-byte aligned
-  return (chunk_head_bytes<V>() + (size_t)(3 * (size_t)n + 2 * (size_t)m) * sizeof(V) + 15) / 16 * 16;
-}
-template <typename V>
-constexpr size_t chunk_res_block_bytes() {   // one resident block, a multiple of 16 bytes
-  return ((size_t)(BNNZ + RES_ROWS * BROWS) * sizeof(V) + (size_t)BNNZ * sizeof(int) + (BROWS + 1) * sizeof(int) +
-          15) / 16 * 16;
-}
-template <typename V>
-constexpr size_t chunk_res_bytes() { return 2 * chunk_res_block_bytes<V>(); }
-template <typename V>
-__device__ __forceinline__ ResBlock<V> res_view(unsigned char* base) {
-  ResBlock<V> rb;
-  rb.val = reinterpret_cast<V*>(base);
-  for (int k = 0; k < RES_ROWS; ++k) rb.row[k] = rb.val + BNNZ + k * BROWS;
-  rb.col = reinterpret_cast<int*>(rb.val + BNNZ + RES_ROWS * BROWS);
-  rb.srp = rb.col + BNNZ;
-  rb.r0 = rb.nr = rb.ne = 0;
-  return rb;
-}
-template <typename V>
-__device__ __forceinline__ void res_load(const BCsr<V>& M, int b, ResBlock<V>& rb, const V* o0, const V* o1,
-                                         const V* o2, const V* o3, const V* o4) {
-  const int r0 = M.blk[b], r1 = M.blk[b + 1];
-  const int e0 = M.rp[r0];
-  rb.r0 = r0;
-  rb.nr = r1 - r0;
-  rb.ne = M.rp[r1] - e0;   // <= BNNZ: no long rows in the cluster chunk
-  for (int t = threadIdx.x; t <= rb.nr; t += CHUNK_NT) rb.srp[t] = M.rp[r0 + t] - e0;
-  for (int e = threadIdx.x; e < rb.ne; e += CHUNK_NT) {
-    rb.col[e] = M.col[e0 + e];
-    rb.val[e] = M.val[e0 + e];
-  }
-  const V* src[RES_ROWS] = {o0, o1, o2, o3, o4};
-  for (int t = threadIdx.x; t < rb.nr; t += CHUNK_NT)
-#pragma unroll
-    for (int k = 0; k < RES_ROWS; ++k) rb.row[k][t] = src[k] ? src[k][r0 + t] : V(0);
-}
-
-static_assert(BROWS <= CHUNK_NT, "a resident block's rows take one thread each");
-
-// dual_block on a resident block: rows[0] b, [1] y_bar, [2] 1 for an
-// inequality row, [3] the lower bound; y^k from the shared-memory copy yk, y+
-// into every CTA's copy at ycopy
-template <typename V>
-__device__ __forceinline__ void dual_block_res(const DualB<V>& a, int bk, int j, V* prod, ResBlock<V>& rb,
-                                               cg::cluster_group& cl, int ctas, const V* yk, V* ycopy) {
-  const int tid = threadIdx.x;
-  const int inst = a.blk_inst[bk];
-  if (a.st[inst].status != ST_RUNNING) return;    // uniform over the block
-  const StepEntry& es = a.tab[inst * a.C + j];
-  for (int e = tid; e < rb.ne; e += CHUNK_NT) prod[e] = rb.val[e] * a.xt[rb.col[e]];
-  __syncthreads();
-  if (tid < rb.nr) {
-    V s = V(0);
-    for (int e = rb.srp[tid]; e < rb.srp[tid + 1]; ++e) s += prod[e];
-    const int r = rb.r0 + tid;
-    V yn, ybn;
-    dual_update<V>(es, s, yk[r], rb.row[0][tid], rb.row[1][tid], rb.row[3][tid], rb.row[2][tid] != V(0), yn, ybn);
-    rb.row[1][tid] = ybn;
-    a.ybar[r] = ybn;
-    a.ynew[r] = yn;
-    broadcast(cl, ctas, ycopy + r, yn);
-  }
-}
-
-// primal_block on a resident block: rows[0] x, [1] x_bar, [2] c, [3] l, [4] u;
-// the next x_md into every CTA's copy at zcopy, the next x_tilde at xcopy
-template <typename V>
-__device__ __forceinline__ void primal_block_res(const PrimalB<V>& a, int bk, int j, V* prod, ResBlock<V>& rb,
-                                                 cg::cluster_group& cl, int ctas, V* zcopy, V* xcopy) {
-  const int tid = threadIdx.x;
-  const int inst = a.blk_inst[bk];
-  if (a.st[inst].status != ST_RUNNING) return;
-  const StepEntry& es = a.tab[inst * a.C + j];
-  for (int e = tid; e < rb.ne; e += CHUNK_NT) prod[e] = rb.val[e] * a.zin[rb.col[e]];
-  __syncthreads();
-  if (tid < rb.nr) {
-    V s = V(0);
-    for (int e = rb.srp[tid]; e < rb.srp[tid + 1]; ++e) s += prod[e];
-    const int r = rb.r0 + tid;
-    const V g = r_add(s, rb.row[2][tid]);
-    V xn, xb, zo, xtn;
-    primal_update<V>(es, g, rb.row[0][tid], rb.row[1][tid], rb.row[3][tid], rb.row[4][tid], xn, xb, zo, xtn);
-    rb.row[0][tid] = xn;
-    rb.row[1][tid] = xb;
-    a.xbar[r] = xb;
-    a.zout[r] = zo;
-    a.xt[r] = xtn;
-    a.x[r] = xn;
-    broadcast(cl, ctas, zcopy + r, zo);
-    broadcast(cl, ctas, xcopy + r, xtn);
-  }
-}
-
-template <typename V>
-__global__ void __launch_bounds__(CHUNK_NT)
-    k_chunk_cluster(DualB<V> da, PrimalB<V> pa, int nblkA, int nblkP, V* z0, V* z1, int n, int m, int j0,
-                    int len, int resident) {
-  extern __shared__ __align__(16) unsigned char chunk_sm[];
-  V* prod = reinterpret_cast<V*>(chunk_sm);
-  int* srp = reinterpret_cast<int*>(prod + BNNZ);
-  V* xs = reinterpret_cast<V*>(chunk_sm + chunk_head_bytes<V>());   // x_tilde
-  V* zs[2] = {xs + n, xs + n + (n + m)};                            // [x_md ; y], both buffers
-  cg::cluster_group cl = cg::this_cluster();
-  const int cta = (int)cl.block_rank(), ctas = (int)cl.num_blocks();   // the grid is one cluster
-  const int tid = threadIdx.x;
-  for (int i = tid; i < n; i += CHUNK_NT) xs[i] = __ldcg(pa.xt + i);
-  for (int i = tid; i < n + m; i += CHUNK_NT) {
-    zs[0][i] = __ldcg(z0 + i);
-    zs[1][i] = __ldcg(z1 + i);
-  }
-  // resident blocks (the host passes resident = 1 only where nblkA, nblkP <=
-  // ctas and their copies fit behind the vectors)
-  unsigned char* rbase = chunk_sm + chunk_res_offset<V>(n, m);
-  ResBlock<V> rA = res_view<V>(rbase), rP = res_view<V>(rbase + chunk_res_bytes<V>() / 2);
-  if (resident) {
-    // the inequality flags as values of V (1 or 0) in a scratch slot first
-    if (cta < nblkA) {
-      res_load(da.A, cta, rA, da.b, da.ybar, (const V*)nullptr, da.ylo, (const V*)nullptr);
-      for (int t = tid; t < rA.nr; t += CHUNK_NT) rA.row[2][t] = da.ineq[rA.r0 + t] ? V(1) : V(0);
-    }
-    if (cta < nblkP) res_load(pa.P, cta, rP, pa.x, pa.xbar, pa.c, pa.l, pa.u);
-  }
-  cluster_barrier();                              // every copy is whole before anyone writes into it
-  DualB<V> dl = da;
-  dl.xt = xs;
-  PrimalB<V> pl = pa;
-  for (int j = j0; j < j0 + len; ++j) {
-    V* zj = (j & 1) ? z1 : z0;
-    V* zn = (j & 1) ? z0 : z1;
-    V* zsj = zs[j & 1];
-    V* zsn = zs[(j + 1) & 1];
-    dl.yold = zn + n;
-    dl.ynew = zj + n;
-    for (int bk = cta; bk < nblkA; bk += ctas) {
-      __syncthreads();                            // the previous block's rows are done with prod
-      if (resident) {
-        dual_block_res<V>(dl, bk, j, prod, rA, cl, ctas, zsn + n, zsj + n);
-        continue;
-      }
-      dual_block<V, CHUNK_NT, GATHER_PLAIN>(dl, bk, j, prod, srp);
-      if (da.st[da.blk_inst[bk]].status == ST_RUNNING) {
-        const int r0 = da.A.blk[bk], nr = da.A.blk[bk + 1] - r0;
-        for (int t = tid; t < nr; t += CHUNK_NT) broadcast(cl, ctas, zsj + n + r0 + t, dl.ynew[r0 + t]);
-      }
-    }
-    cluster_barrier();
-    pl.zin = zsj;
-    pl.zout = zn;
-    for (int bk = cta; bk < nblkP; bk += ctas) {
-      __syncthreads();
-      if (resident) {
-        primal_block_res<V>(pl, bk, j, prod, rP, cl, ctas, zsn, xs);
-        continue;
-      }
-      primal_block<V, CHUNK_NT, false, GATHER_PLAIN>(pl, bk, j, prod, srp);
-      if (pa.st[pa.blk_inst[bk]].status == ST_RUNNING) {
-        const int r0 = pa.P.blk[bk], nr = pa.P.blk[bk + 1] - r0;
-        for (int t = tid; t < nr; t += CHUNK_NT) {
-          broadcast(cl, ctas, zsn + r0 + t, zn[r0 + t]);
-          broadcast(cl, ctas, xs + r0 + t, pl.xt[r0 + t]);
-        }
-      }
-    }
-    cluster_barrier();
-  }
+  primal_block<V, NT, LR>(a, bk, j, prod, sx, srp);
 }
 
 // Segment sums of the long rows: one CUDA block per segment of LSEG nonzeros
@@ -479,10 +226,7 @@ __global__ void __launch_bounds__(256) k_long_partials(BCsr<V> M, const V* __res
                                                        const DevState* __restrict__ st, V* __restrict__ out) {
   const int4 g = lseg[blockIdx.x];
   if (st[blk_inst[g.w]].status != ST_RUNNING) return;
-  V s = V(0);
-  for (int e = g.y + threadIdx.x; e < g.z; e += 256) s += M.val[e] * __ldg(vec + M.col[e]);
-  s = block_sum(s);
-  if (threadIdx.x == 0) out[blockIdx.x] = s;
+  long_segment_sum(M, vec, g, out + blockIdx.x);
 }
 
 
@@ -526,6 +270,13 @@ __device__ __forceinline__ void pipe_issue(PipeSmem<V>& sm, int s, const int4 m,
   cp_async_commit();
 }
 
+// what prod holds, and one term of a row sum from it (float32: the product;
+// float64: the gathered entry, fused with its value)
+__device__ __forceinline__ float pipe_entry(float v, float x) { return v * x; }
+__device__ __forceinline__ double pipe_entry(double, double x) { return x; }
+__device__ __forceinline__ float pipe_add(float s, float, float p) { return s + p; }
+__device__ __forceinline__ double pipe_add(double s, double v, double x) { return r_dot(v, x, s); }
+
 template <typename V, int NT>
 __global__ void __launch_bounds__(NT) k_dual_pipe(DualB<V> a, const int4* __restrict__ meta, int nblk, int j) {
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -558,13 +309,13 @@ __global__ void __launch_bounds__(NT) k_dual_pipe(DualB<V> a, const int4* __rest
 #pragma unroll
       for (int k = 0; k < BNNZ / NT; ++k) {
         const int e = tid + k * NT;
-        if (e < ne) sm.prod[e] = sm.val[s][e + off] * __ldg(a.xt + sm.col[s][e + off]);
+        if (e < ne) sm.prod[e] = pipe_entry(sm.val[s][e + off], __ldg(a.xt + sm.col[s][e + off]));
       }
       __syncthreads();
       for (int t = tid; t < nr; t += NT) {
         V acc = V(0);
         const int eb = sm.rp[s][t + roff] - e0, ee = sm.rp[s][t + 1 + roff] - e0;
-        for (int e = eb; e < ee; ++e) acc += sm.prod[e];
+        for (int e = eb; e < ee; ++e) acc = pipe_add(acc, sm.val[s][e + off], sm.prod[e]);
         const int r = r0 + t;
         if (t >= NT) {
           yo = a.yold[r]; bi = a.b[r]; yb = a.ybar[r];
@@ -621,13 +372,13 @@ __global__ void __launch_bounds__(NT) k_primal_pipe(PrimalB<V> a, const int4* __
 #pragma unroll
       for (int k = 0; k < BNNZ / NT; ++k) {
         const int e = tid + k * NT;
-        if (e < ne) sm.prod[e] = sm.val[s][e + off] * __ldg(a.zin + sm.col[s][e + off]);
+        if (e < ne) sm.prod[e] = pipe_entry(sm.val[s][e + off], __ldg(a.zin + sm.col[s][e + off]));
       }
       __syncthreads();
       for (int t = tid; t < nr; t += NT) {
         V acc = V(0);
         const int eb = sm.rp[s][t + roff] - e0, ee = sm.rp[s][t + 1 + roff] - e0;
-        for (int e = eb; e < ee; ++e) acc += sm.prod[e];
+        for (int e = eb; e < ee; ++e) acc = pipe_add(acc, sm.val[s][e + off], sm.prod[e]);
         const int r = r0 + t;
         if (t >= NT) { xo = a.x[r]; xb = a.xbar[r]; cr = a.c[r]; lr = a.l[r]; ur = a.u[r]; }
         if (a.F) primal_row<V, true>(a, es, r, acc, xo, xb, cr, lr, ur);
@@ -679,7 +430,7 @@ static int pipe_grid_p(void (*kern)(PrimalB<V>, const int4*, int, int)) {
 // instances running at the last check: the matrix streams (index + value),
 // the row pointers, each vector read or written once (the gathered vector
 // counted once); sv = bytes per value.
-static double launch_bytes(const Work& w, int kind, double sv) {
+double launch_bytes(const Work& w, int kind, double sv) {
   const BatchState& b = *w.bst_host;
   if (kind == 0) return b.run_nnzA * (sv + 4.0) + 4.0 * (b.run_m + 1.0) + sv * (b.run_n + 5.0 * b.run_m);
   return b.run_nnzP * (sv + 4.0) + 4.0 * (b.run_n + 1.0) + sv * (10.0 * b.run_n + b.run_m);
@@ -775,8 +526,8 @@ static void run_chunk(Work& w, int j0, int len, BCsr<V> A, BCsr<V> P, V* xt, V* 
 // one row for 32 members: each matrix entry is read once for them and meets
 // their 32 values of the gathered vector in one coalesced load, where the
 // member-major layout gathers 32 scattered sectors.  The row sum runs over
-// the row's entries in CSR order with separately rounded products and sums,
-// as the row-block kernels sum their staged products, and the row update is
+// the row's entries in CSR order by r_dot, as the row-block kernels sum their
+// staged entries, and the row update is
 // the same function: a member's iterates are bitwise those of its standalone
 // solve.  The vectors are transposed into this layout at the start of a
 // chunk and back at its end, so the checks, restarts and rebases run on the
@@ -834,8 +585,7 @@ __device__ __forceinline__ void il_store(V* p, const V (&v)[IlVec<V>::W]) {
 }
 
 // The row sums of this lane's W members: for each, sequential over the row's
-// entries, each product and sum rounded on its own (no fused multiply-add),
-// as prod[e] is staged and summed by the row-block kernels.  The warp reads
+// entries by r_dot, as the row-block kernels sum their staged entries.  The warp reads
 // the row's indices and values 32 at a time in one coalesced load and hands
 // each entry to all lanes by shuffle, so that the L1 data pipe (the bound of
 // this kernel) moves only the gathered members' values.  Every lane of the
@@ -863,7 +613,7 @@ __device__ __forceinline__ void il_row_sum(const FamIL<V>& a, int r, int m0, V (
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int q = 0; q < W; ++q) s[q] = r_add(s[q], r_mul(v[i], z[i][q]));
+        for (int q = 0; q < W; ++q) s[q] = r_dot(v[i], z[i][q], s[q]);
     }
     for (; k < cnt; ++k) {
       const int c = __shfl_sync(0xffffffffu, cl, k);
@@ -871,7 +621,7 @@ __device__ __forceinline__ void il_row_sum(const FamIL<V>& a, int r, int m0, V (
       V z[W];
       il_load(a.zin + (size_t)c * a.ld + m0, z);
 #pragma unroll
-      for (int q = 0; q < W; ++q) s[q] = r_add(s[q], r_mul(v, z[q]));
+      for (int q = 0; q < W; ++q) s[q] = r_dot(v, z[q], s[q]);
     }
   }
 }
@@ -1023,77 +773,6 @@ static void run_chunk_il(Work& w, int j0, int len, const V* Aval, const V* Pval,
   back(I[IL_YBAR], m, ybar, m);
 }
 
-bool chunk_cluster_ok(const Work& w, bool mixed) {
-  const size_t smem = mixed ? chunk_smem_bytes<float>(w.n, w.m) : chunk_smem_bytes<double>(w.n, w.m);
-  return w.r == 0 && w.A.nlseg == 0 && w.P.nlseg == 0 && w.A.nblk <= CHUNK_MAX_BLOCKS &&
-         w.P.nblk <= CHUNK_MAX_BLOCKS && w.P.nblk > 0 && smem <= (size_t)CHUNK_SMEM_MAX;
-}
-
-// cluster size: 16 CTAs if a 16-CTA cluster of the largest footprint fits, else 8
-static int g_chunk_ctas = 8;
-
-template <typename V>
-static int chunk_cluster_size() {
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = 16;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3(16);
-  cfg.blockDim = dim3(CHUNK_NT);
-  cfg.dynamicSmemBytes = CHUNK_SMEM_MAX;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  int clusters = 0;
-  if (cudaOccupancyMaxActiveClusters(&clusters, k_chunk_cluster<V>, &cfg) != cudaSuccess) {
-    cudaGetLastError();
-    return 8;
-  }
-  return clusters >= 1 ? 16 : 8;
-}
-
-void prepare_chunk_cluster() {
-  static std::once_flag once;
-  std::call_once(once, [] {
-    cudaFuncSetAttribute(k_chunk_cluster<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, CHUNK_SMEM_MAX);
-    cudaFuncSetAttribute(k_chunk_cluster<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, CHUNK_SMEM_MAX);
-    cudaFuncSetAttribute(k_chunk_cluster<float>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    cudaFuncSetAttribute(k_chunk_cluster<double>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    g_chunk_ctas = std::min(chunk_cluster_size<float>(), chunk_cluster_size<double>());
-  });
-}
-
-template <typename V>
-static void run_chunk_cluster(Work& w, int j0, int len, BCsr<V> A, BCsr<V> P, V* xt, V* const* Z, V* ybar,
-                              const V* b, const V* ylo, V* x, V* xbar, const V* c, const V* l, const V* u,
-                              cudaStream_t s) {
-  Profiler& Pr = w.prof;
-  DualB<V> da{A, xt, nullptr, nullptr, ybar, b, ylo, w.tab, w.blk_inst_A, w.st, w.row_ineq, w.tab_stride};
-  PrimalB<V> pa{P, nullptr, nullptr, x, xbar, xt, c, l, u, w.tab, w.blk_inst_P, w.st, w.tab_stride,
-                nullptr, nullptr, 0};
-  // kind 3: one launch holds both half-steps of `len` iterations
-  if (Pr.on) Pr.begin(3, s, len * (launch_bytes(w, 0, sizeof(V)) + launch_bytes(w, 1, sizeof(V))));
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = g_chunk_ctas;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3(g_chunk_ctas);               // one cluster
-  cfg.blockDim = dim3(CHUNK_NT);
-  const int nblkA = w.m > 0 ? w.A.nblk : 0;
-  const size_t res_end = chunk_res_offset<V>(w.n, w.m) + chunk_res_bytes<V>();
-  const int resident = nblkA <= g_chunk_ctas && w.P.nblk <= g_chunk_ctas && res_end <= (size_t)CHUNK_SMEM_MAX;
-  cfg.dynamicSmemBytes = resident ? res_end : chunk_smem_bytes<V>(w.n, w.m);
-  cfg.stream = s;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, k_chunk_cluster<V>, da, pa, nblkA, w.P.nblk, Z[0], Z[1], w.n, w.m, j0, len, resident);
-  count_launch();
-  if (Pr.on) Pr.end(s);
-}
-
 void iterate_chunk(Work& w, int len, bool mixed, int nt, cudaStream_t s, int j0, bool compact) {
   if (nt == 3) {   // a family handle on member-interleaved vectors
     if (len <= 0) return;
@@ -1108,16 +787,8 @@ void iterate_chunk(Work& w, int len, bool mixed, int nt, cudaStream_t s, int j0,
     }
     return;
   }
-  if (nt == 2) {   // the whole chunk in one cluster launch (small problems)
-    if (mixed) {
-      run_chunk_cluster<float>(w, j0, len, w.A.bscaled_f(), w.P.bscaled_f(), w.fxt, w.fZ, w.fybar, w.fb, w.fylo,
-                               w.fx, w.fxbar, w.fc, w.fl, w.fu, s);
-      w.fy = w.fZ[(j0 + len - 1) & 1] + w.n;
-    } else {
-      run_chunk_cluster<double>(w, j0, len, w.A.bscaled(), w.P.bscaled(), w.xt, w.Z, w.ybar, w.bs, nullptr, w.x,
-                                w.xbar, w.cs, w.ls, w.us, s);
-      w.y = w.Z[(j0 + len - 1) & 1] + w.n;
-    }
+  if (nt == 2) {   // the whole chunk in one launch (small instances)
+    chunk_run(w, len, mixed, s, j0);
     return;
   }
   if (nt == 1) {   // pipelined persistent kernels, 256 threads

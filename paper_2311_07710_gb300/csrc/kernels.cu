@@ -822,7 +822,7 @@ __global__ void __launch_bounds__(NT, MinBlocks<V, NT>::value) k_lz_m(BCsr<V> A,
   const int e0 = A.rp[r0];
   const int ne = A.rp[r1] - e0;
   if (ne <= BNNZ) {
-    stage_products<NT, GATHER_LDG, V, V, true>(A, vA, e0, ne, r0, nr, prod, srp, 0, gA, la.n);
+    stage_products<NT, V, V, true>(A, vA, e0, ne, r0, nr, prod, srp, 0, gA, la.n);
     __syncthreads();
     for (int t = tid; t < nr; t += NT) {
       V s = V(0);
@@ -870,7 +870,7 @@ __global__ void __launch_bounds__(NT, MinBlocks<V, NT, LR>::value) k_lz_n(BCsr<V
   if (ne <= BNNZ) {
     // once the instance's ||Q|| has converged only the A' part is gathered;
     // the v_Q entries (columns < n) are normalised as they are gathered
-    stage_products<NT, GATHER_LDG, V, V, true>(P, zin, e0, ne, r0, nr, prod, srp, doQ ? 0 : la.n, gQ, la.n);
+    stage_products<NT, V, V, true>(P, zin, e0, ne, r0, nr, prod, srp, doQ ? 0 : la.n, gQ, la.n);
     for (int t = tid; t < nr; t += NT) ssp[t] = P.split[r0 + t] - e0;
     __syncthreads();
     for (int t = tid; t < nr; t += NT) {

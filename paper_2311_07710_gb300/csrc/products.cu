@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(MP_NT, MinBlocks<double, MP_NT>::value) k_dual
     }
     return;
   }
-  stage_products<MP_NT, GATHER_LDG>(a.A, a.xg, e0, ne, r0, nr, prod, srp);
+  stage_products<MP_NT>(a.A, a.xg, e0, ne, r0, nr, prod, srp);
   __syncthreads();
   for (int t = tid; t < nr; t += MP_NT) {
     double s = 0.0;
@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(MP_NT, MinBlocks<double, MP_NT>::value) k_prim
     if (!ps.first) { qbp = a.qxb[r]; tbp = a.atyb[r]; }
   };
   if (tid < nr) operands(r0 + tid);
-  stage_products<MP_NT, GATHER_LDG>(a.P, a.zin, e0, ne, r0, nr, prod, srp, fresh ? a.n : 0);
+  stage_products<MP_NT>(a.P, a.zin, e0, ne, r0, nr, prod, srp, fresh ? a.n : 0);
   for (int t = tid; t < nr; t += MP_NT) ssp[t] = a.P.split[r0 + t] - e0;
   __syncthreads();
   const double* fr = (S.restart && S.cand_avg) ? a.sQ[1] : a.sQ[0];
@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(MP_NT, 4) k_mp_check_m(MpCheck a) {
   if (a.st[inst].status != ST_RUNNING) return;
   const int r0 = a.A.blk[bk], r1 = a.A.blk[bk + 1], nr = r1 - r0;
   const int e0 = a.A.rp[r0], ne = a.A.rp[r1] - e0;
-  stage_products<MP_NT, GATHER_LDG>(a.A, a.x, e0, ne, r0, nr, prod, srp);
+  stage_products<MP_NT>(a.A, a.x, e0, ne, r0, nr, prod, srp);
   __syncthreads();
   const double ib = a.mode ? a.tab[inst * a.C + a.last].inv_beta : 1.0;
   for (int t = threadIdx.x; t < nr; t += MP_NT) {

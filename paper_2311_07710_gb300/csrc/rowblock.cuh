@@ -4,6 +4,8 @@
 // low-rank row term.
 #pragma once
 
+#include <algorithm>
+
 #include "solver.h"
 
 namespace pdqp {
@@ -45,18 +47,6 @@ __device__ __forceinline__ T block_sum(T v) {
 // Row-block staging: the products val[e] * vec[col[e]] of one block's
 // nonzeros go to shared memory prod[0..ne); srp[t] = rp[r0+t] - e0.
 // ==========================================================================
-// How the staging gathers the vector: through the read-only path (GATHER_LDG),
-// through L2 (GATHER_CG: vectors that other CTAs of the same launch write), or
-// with plain loads of a generic pointer (GATHER_PLAIN: a copy in shared memory).
-enum { GATHER_LDG = 0, GATHER_CG = 1, GATHER_PLAIN = 2 };
-
-template <int GM, typename X>
-__device__ __forceinline__ X gather_load(const X* p) {
-  if constexpr (GM == GATHER_LDG) return __ldg(p);
-  else if constexpr (GM == GATHER_CG) return __ldcg(p);
-  else return *p;
-}
-
 // Four consecutive entries of an index or value array by one 16-byte load
 // (p 16-byte aligned).
 __device__ __forceinline__ void load4(const int* __restrict__ p, int (&v)[4]) {
@@ -83,7 +73,7 @@ __device__ __forceinline__ void load4(const double* __restrict__ p, double (&v)[
 // (a caller that needs only the sums over the columns >= cmin).
 // SC: the gathered entries of the columns below csplit are multiplied by sc
 // first (a vector kept unnormalised, normalised where it is read).
-template <int NT, int GM = GATHER_LDG, typename V, typename X, bool SC = false>
+template <int NT, typename V, typename X, bool SC = false>
 __device__ __forceinline__ void stage_products(const BCsr<V>& M, const X* __restrict__ vec, int e0, int ne,
                                                int r0, int nr, V* prod, int* srp, int cmin = 0, V sc = V(1),
                                                int csplit = 0) {
@@ -131,18 +121,74 @@ __device__ __forceinline__ void stage_products(const BCsr<V>& M, const X* __rest
               const int c = ci[k][i];
               V p = V(0);
               if (c >= cmin) {
-                const V x = (V)gather_load<GM>(vec + c);
+                const V x = (V)__ldg(vec + c);
                 p = vv[k][i] * (c < csplit ? r_mul(x, sc) : x);
               }
               prod[e] = p;
             }
           } else {
-            if (e >= 0 && e < ne) prod[e] = ci[k][i] >= cmin ? vv[k][i] * (V)gather_load<GM>(vec + ci[k][i]) : V(0);
+            if (e >= 0 && e < ne) prod[e] = ci[k][i] >= cmin ? vv[k][i] * (V)__ldg(vec + ci[k][i]) : V(0);
           }
         }
       }
     }
   }
+}
+
+// The staging of the half-steps: float32 blocks stage the products in prod;
+// float64 row sums are fused multiply-adds (r_dot), so their blocks stage the
+// values in prod and the gathered entries in sx.  `mid` runs between the first
+// quads' loads (of the matrix, which no kernel of the loop writes) and the first
+// gather: it fetches the rows' operands;
+// false ends the staging.
+template <int NT, typename V, typename Mid>
+__device__ __forceinline__ bool stage_rows(const BCsr<V>& M, const V* __restrict__ vec, int e0, int ne, int r0, int nr,
+                                           V* prod, V* sx, int* srp, Mid mid) {
+  constexpr int QPT = BNNZ / NT / 4 + 1;           // quads per thread, one more for the misalignment
+  constexpr int QPP = sizeof(V) == 4 ? 1 : 2;   // quads per phase (both phases' quads of one float64 pass in flight)
+  const int tid = threadIdx.x;
+  const int a0 = e0 & ~3, o = e0 - a0;
+  const int nq = (o + ne + 3) >> 2;
+  if (M.pf && tid == 0 && nq > 0) {                // as in stage_products
+    const unsigned long long gc = (unsigned long long)__cvta_generic_to_global(M.col + a0);
+    const unsigned long long gv = (unsigned long long)__cvta_generic_to_global(M.val + a0);
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(gc), "r"(nq * 16) : "memory");
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(gv), "r"(nq * 4 * (int)sizeof(V)) : "memory");
+  }
+  for (int t = tid; t <= nr; t += NT) srp[t] = M.rp[r0 + t] - e0;
+#pragma unroll
+  for (int h = 0; h < QPT; h += QPP) {
+    int ci[QPP][4];
+    V vv[QPP][4];
+#pragma unroll
+    for (int k = 0; k < QPP; ++k) {
+      const int q = tid + (h + k) * NT;
+      if (h + k < QPT && q < nq) {
+        load4(M.col + a0 + 4 * q, ci[k]);
+        load4(M.val + a0 + 4 * q, vv[k]);
+      }
+    }
+    if (h == 0 && !mid()) return false;
+#pragma unroll
+    for (int k = 0; k < QPP; ++k) {
+      const int q = tid + (h + k) * NT;
+      if (h + k < QPT && q < nq) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int e = 4 * q + i - o;
+          if (e >= 0 && e < ne) {
+            if constexpr (sizeof(V) == 4) {
+              prod[e] = vv[k][i] * __ldg(vec + ci[k][i]);
+            } else {
+              prod[e] = vv[k][i];
+              sx[e] = __ldg(vec + ci[k][i]);
+            }
+          }
+        }
+      }
+    }
+  }
+  return true;
 }
 
 // The index and value quads of row block b towards L2 (a bulk prefetch, a
@@ -177,11 +223,12 @@ __device__ __forceinline__ void prefetch_ahead(const BCsr<V>& M, const int* act,
 // two-phase staging above, 256 threads of float data fit 32 registers without
 // spills (8 blocks, the whole SM: k_primal 97 -> 76 us, k_dual 67 -> 51 us at
 // n=1e6 against 4 blocks at 64 registers); the float64 kernels are bound by
-// the float64 pipes and gain nothing from 5 or 6 blocks, so they keep 64
-// registers (4); NT = 512 runs 4 blocks at 32 registers.
+// the float64 pipes, and 5 blocks of one quad a phase are no faster than 4 of
+// two (an iteration at n=600000: 160.6 against 145.3 us; at n=300007 86.4 against
+// 85.3), so they keep 64 registers (4); NT = 512 runs 4 blocks at 32 registers.
 template <typename V, int NT, bool LR = false> struct MinBlocks { static constexpr int value = 4; };
 template <> struct MinBlocks<float, 256, false> { static constexpr int value = 8; };
-
+template <bool LR> struct MinBlocks<double, 512, LR> { static constexpr int value = 2; };
 
 // the row term F~_j . w (16-byte loads of the row when r allows)
 template <typename FV, typename V, typename W>
@@ -203,6 +250,37 @@ __device__ __forceinline__ V lr_row(const FV* __restrict__ F, const W* __restric
     for (int kk = 0; kk < r; ++kk) s += (V)f[kk] * (V)w[kk];
   }
   return s;
+}
+
+// Column blk of F' v from the block partials of k_lr_ft (vec, k = blk / r, blk %
+// r): a fixed-order tree over 256 threads; a float32 copy for the float32
+// iteration.
+__device__ __forceinline__ void lr_reduce_column(const double* __restrict__ part, int nparts, int r, int nv, int blk,
+                                                 double* __restrict__ w, float* __restrict__ wf) {
+  const int q = blk / r, kk = blk % r;
+  __shared__ double sh[256];
+  double s = 0.0;
+  for (int b = threadIdx.x; b < nparts; b += 256) s += part[((size_t)b * nv + q) * r + kk];
+  sh[threadIdx.x] = s;
+  __syncthreads();
+  for (int o = 128; o > 0; o >>= 1) {
+    if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    w[q * r + kk] = sh[0];
+    if (wf) wf[q * r + kk] = (float)sh[0];
+  }
+}
+
+// the sum of one segment g = {row, first nonzero, end, row block} of a long row
+template <typename V>
+__device__ __forceinline__ void long_segment_sum(const BCsr<V>& M, const V* __restrict__ vec, int4 g,
+                                                 V* __restrict__ out) {
+  V s = V(0);
+  for (int e = g.y + threadIdx.x; e < g.z; e += 256) s += M.val[e] * __ldg(vec + M.col[e]);
+  s = block_sum(s);
+  if (threadIdx.x == 0) *out = s;
 }
 
 // member-major [count][L] (member stride `stride`) <-> interleaved [L][ld],
@@ -262,5 +340,11 @@ template <> inline const float* lr_weights<float>(Work& w) { return w.wlr_f; }
 // F~' v into w.wlr / w.wlr_f for one vector (kernels.cu)
 void lowrank_ft1(Work& w, const float* F, const float* v, cudaStream_t s);
 void lowrank_ft1(Work& w, const double* F, const double* v, cudaStream_t s);
+// only the block partials of F~' v (lr_ft_grid blocks of consecutive rows each)
+void lowrank_ft_part(Work& w, const float* F, const float* v, cudaStream_t s);
+void lowrank_ft_part(Work& w, const double* F, const double* v, cudaStream_t s);
+static inline int lr_ft_grid(const Work& w) { return std::min(cdiv(w.n, LR_ROWS), 4 * w.num_sms); }
+// the row terms F~ w.wlr of nit vectors into w.lr_rows (lowrank.cu)
+void lowrank_rows(Work& w, const double* F, int nit, cudaStream_t s);
 
 }  // namespace pdqp

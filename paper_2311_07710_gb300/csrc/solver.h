@@ -103,6 +103,35 @@ struct InfState {
 constexpr int KKT_GROUP = 4;
 static_assert(KKT_CHUNK % KKT_GROUP == 0, "a relKKT chunk holds whole groups");
 
+// The one-launch chunk (chunk.cu): an instance with its slices of 32 rows, in
+// launch order; its row in sp (A's slices of all instances come first, then P's).
+struct ChunkInst {
+  int n, m, xoff, yoff;
+  int sA, nsA, sP, nsP;
+  int id;                       // instance
+};
+// Instances [first, first + count) of the launch order in one launch.
+struct ChunkClass {
+  int first, count, threads;
+  size_t smem;
+};
+struct ChunkPlan {
+  bool built = false;
+  int ctas[2] = {1, 1};                   // CTAs per instance (a cluster when > 1): float64, mixed
+  int slices = 0;
+  long long ngroups = 0;
+  std::vector<ChunkInst> order;           // launch order, largest first
+  ChunkInst* inst = nullptr;              // [count] on the device
+  int* sp = nullptr;                      // [slices + 1] starts, in groups of 32 pairs of entries
+  unsigned* idx = nullptr;                // [groups][32] two 16-bit columns
+  float2* valf = nullptr;                 // [groups][32] scaled values
+  double2* vald = nullptr;
+  std::vector<int2> groups;               // {of A, of P} per instance, in launch order
+  std::vector<ChunkClass> cls[2];         // launches: float64, mixed
+  cudaStream_t side[2] = {nullptr, nullptr};   // the second and later launches' streams
+  cudaEvent_t fork = nullptr, join[2] = {nullptr, nullptr};
+};
+
 struct Work {
   int n = 0, m = 0, m_eq = 0;   // totals over the batch (m_eq: single-instance value)
   int count = 1;                // instances stacked block-diagonally
@@ -205,6 +234,7 @@ struct Work {
   int mp_accelerate = 0;                     // its options.accelerate
   double *mp_ax = nullptr, *mp_axb = nullptr, *mp_qxb = nullptr, *mp_aty = nullptr, *mp_atyb = nullptr;
   double *mp_sA[2] = {nullptr, nullptr}, *mp_sQ[2] = {nullptr, nullptr};
+  ChunkPlan chunk;
   Profiler prof;
 };
 
@@ -246,7 +276,7 @@ void init_iterates(Work& w, const double* x0, const double* y0, const SolveParam
 // compact: launch only the row blocks of the running instances (batches; the
 // counts of the last check must be in bst_host).
 // nt: 256 or 512 threads per row block, 1 the pipelined persistent kernels, 2
-// the whole chunk in one cluster launch (only where chunk_cluster_ok), 3 the
+// the whole chunk in one launch (only where chunk_ok, plan and values built), 3 the
 // member-interleaved family kernels (only where w.fam_il, buffers allocated).
 void iterate_chunk(Work& w, int len, bool mixed, int nt, cudaStream_t s, int j0 = 0, bool compact = false);
 // iterate_chunk, or with w.mp the maintained-products kernels (float64, 256
@@ -257,9 +287,22 @@ void iterate(Work& w, int len, bool mixed, int nt, cudaStream_t s, int j0 = 0, b
 // after chunk_len iterations (mode 1), or of the start point (mode 0, which
 // also forms the A~' products of y)
 void mp_check_products(Work& w, int mode, long long chunk_len, cudaStream_t s);
-// few row blocks, no long rows, no low-rank term, the vector copies fit in shared memory
-bool chunk_cluster_ok(const Work& w, bool mixed);
-void prepare_chunk_cluster();           // once, outside any stream capture
+// Algorithmic bytes of one dual (kind 0) or primal (kind 1) launch over the
+// instances running at the last check (sv = bytes per value).
+double launch_bytes(const Work& w, int kind, double sv);
+
+// The one-launch chunk (chunk.cu): whether every instance's vectors fit a CTA
+// (no long rows, no low-rank term); the plan's parts, in the order they are built.
+bool chunk_ok(const Work& w, bool mixed);
+bool chunk_pays(const Work& w, bool mixed);               // chosen over the per-iteration kernels
+void chunk_plan_instances(Work& w);                       // w.chunk.order, slices (instance order)
+void chunk_widths(Work& w, int* wid, cudaStream_t s);     // pairs per slice
+void chunk_groups(Work& w, int2* out, cudaStream_t s);    // groups of A and of P per instance
+void chunk_plan_order(Work& w, const std::vector<int2>& groups);   // largest instances first
+void chunk_plan_classes(Work& w, bool mixed);             // w.chunk.ctas, cls of one precision
+void chunk_fill_index(Work& w, cudaStream_t s);
+void chunk_fill_values(Work& w, bool mixed, cudaStream_t s);
+void chunk_run(Work& w, int len, bool mixed, cudaStream_t s, int j0);
 void check(Work& w, const SolveParams& p, int mode, long long chunk_len, bool mixed, cudaStream_t s);
 
 // infeasibility certificates: fill the recession-cone bounds once the
