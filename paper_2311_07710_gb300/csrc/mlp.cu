@@ -18,7 +18,7 @@
 // A and B into a 4-stage shared-memory ring with TMA (128-byte swizzle),
 // thread 0 of warp 1 issues tcgen05.mma (M=128, N=256, K=16, kind::f16 with
 // bf16 A and B) on each stage into one of two float32 accumulators in tensor
-// memory and releases the stage with tcgen05.commit, and warps 2..5 drain the
+// memory and releases the stage with tcgen05.commit, and warps 2..9 drain the
 // other accumulator with tcgen05.ld into the fused epilogue (warp w reads TMEM
 // lanes 32 (w mod 4) .. +32), so a tile's epilogue overlaps the next tile's
 // main loop.  Split-K: a unit takes a range of k slices and writes raw float32
@@ -51,7 +51,8 @@ constexpr int A_BYTES = BM * BK * 2;                    // 16 KiB
 template <int BN> struct Tile {
   static constexpr int B_BYTES = BN * BK * 2;           // 16 or 32 KiB
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /* alignment */ + 256 /* barriers */;
+  static constexpr int EPI_BYTES = 8 * 32 * 20 * 4;     // the epilogue warps' stages (EPI_LD floats a row)
+  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /* alignment */ + 256 /* barriers */ + EPI_BYTES;
 };
 constexpr uint64_t WAIT_NS = 200000000ULL;            // a wait gives up after 0.2 s without progress
 
@@ -62,6 +63,7 @@ struct Epi {
   const bf16* mask;              // [M x ldm]: keep where mask > 0, else 0 (ReLU derivative), or null
   int ldo, ldm;
   int relu;
+  int vec;                       // the outputs and the mask start on 16 (8) bytes: 4 columns per access
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -144,82 +146,126 @@ __device__ __forceinline__ float epi_value(float r, int row, int col, const Epi&
   return r;
 }
 
-// Epilogue of 32 accumulator columns of one row: the raw float32 split-K
-// partial of split z (ld = N), or the fused epilogue into the outputs.
-__device__ __forceinline__ void store_chunk(const uint32_t (&v)[32], int row, int cb, int z, int M, int N,
+// Epilogue of a warp's 32 x 16 accumulator values (rows row0.., columns cb..
+// below nend), staged in `stg` (32 rows of EPI_LD floats): the raw float32 split-K
+// partial of split z (ld = N), or the fused epilogue into the outputs.  A lane
+// holds one accumulator row, so storing from its registers touches 32 rows at a
+// time in 16-byte pieces; through shared memory four lanes store a row's 64
+// contiguous bytes, eight rows an instruction.  The short-K products of the
+// network are bound by this path and its dependent instructions (512 x 30000 x
+// 64: 31 us with four epilogue warps, float32 or bf16 alike), so the common
+// case reads all its values first and takes its branches outside the loops,
+// and eight warps drain an accumulator, two per 32 TMEM lanes.
+constexpr int EPI_LD = 20;
+constexpr int EPI_WARPS = 8;
+constexpr int GEMM_NT = 64 + 32 * EPI_WARPS;   // TMA, MMA and epilogue warps
+__device__ __forceinline__ void store_chunk(const float* stg, int row0, int cb, int z, int M, int N, int nend,
                                             const Epi& epi, float* __restrict__ partial) {
-  if (partial) {   // raw float32 partial of this k range, ld = N
-    float* dst = partial + ((size_t)z * M + row) * N + cb;
-    if (cb + 32 <= N && (N & 3) == 0) {
+  const int lane = threadIdx.x & 31;
+  const bool vec = cb + 16 <= nend && row0 + 32 <= M && epi.vec &&
+                   (partial ? (N & 3) == 0 : (epi.ldo & 3) == 0 && (!epi.mask || (epi.ldm & 3) == 0));
+  if (vec) {
+    const int col = cb + (lane & 3) * 4, row = row0 + (lane >> 2);
+    float4 v[4];
 #pragma unroll
-      for (int i = 0; i < 32; i += 4)
-        *(float4*)(dst + i) = make_float4(__uint_as_float(v[i]), __uint_as_float(v[i + 1]),
-                                          __uint_as_float(v[i + 2]), __uint_as_float(v[i + 3]));
-    } else {
+    for (int i = 0; i < 4; ++i)
+      v[i] = *reinterpret_cast<const float4*>(stg + (8 * i + (lane >> 2)) * EPI_LD + (lane & 3) * 4);
+    if (partial) {
+      float* d = partial + ((size_t)z * M + row) * N + col;
 #pragma unroll
-      for (int i = 0; i < 32; ++i)
-        if (cb + i < N) dst[i] = __uint_as_float(v[i]);
+      for (int i = 0; i < 4; ++i) *reinterpret_cast<float4*>(d + (size_t)(8 * i) * N) = v[i];
+      return;
+    }
+    if (epi.bias) {
+      const float4 b = make_float4(__ldg(epi.bias + col), __ldg(epi.bias + col + 1), __ldg(epi.bias + col + 2),
+                                   __ldg(epi.bias + col + 3));
+#pragma unroll
+      for (int i = 0; i < 4; ++i) { v[i].x += b.x; v[i].y += b.y; v[i].z += b.z; v[i].w += b.w; }
+    }
+    if (epi.relu) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        v[i].x = fmaxf(v[i].x, 0.f); v[i].y = fmaxf(v[i].y, 0.f);
+        v[i].z = fmaxf(v[i].z, 0.f); v[i].w = fmaxf(v[i].w, 0.f);
+      }
+    }
+    if (epi.mask) {
+      const bf16* mk = epi.mask + (size_t)row * epi.ldm + col;
+      uint2 q[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) q[i] = *reinterpret_cast<const uint2*>(mk + (size_t)(8 * i) * epi.ldm);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const __nv_bfloat162 a = *reinterpret_cast<const __nv_bfloat162*>(&q[i].x);
+        const __nv_bfloat162 b = *reinterpret_cast<const __nv_bfloat162*>(&q[i].y);
+        if (!(__low2float(a) > 0.f)) v[i].x = 0.f;
+        if (!(__high2float(a) > 0.f)) v[i].y = 0.f;
+        if (!(__low2float(b) > 0.f)) v[i].z = 0.f;
+        if (!(__high2float(b) > 0.f)) v[i].w = 0.f;
+      }
+    }
+    const size_t o = (size_t)row * epi.ldo + col;
+    if (epi.out_f) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) *reinterpret_cast<float4*>(epi.out_f + o + (size_t)(8 * i) * epi.ldo) = v[i];
+    }
+    if (epi.out_b) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const __nv_bfloat162 h0 = __floats2bfloat162_rn(v[i].x, v[i].y), h1 = __floats2bfloat162_rn(v[i].z, v[i].w);
+        uint2 q;
+        q.x = *reinterpret_cast<const uint32_t*>(&h0);
+        q.y = *reinterpret_cast<const uint32_t*>(&h1);
+        *reinterpret_cast<uint2*>(epi.out_b + o + (size_t)(8 * i) * epi.ldo) = q;
+      }
     }
     return;
   }
-  float r[32];
-#pragma unroll
-  for (int i = 0; i < 32; ++i) r[i] = __uint_as_float(v[i]);
-  if (cb + 32 <= N) {
-#pragma unroll
-    for (int i = 0; i < 32; ++i) r[i] = epi_value(r[i], row, cb + i, epi);
-    const size_t o = (size_t)row * epi.ldo + cb;
-    if (epi.out_f) {
-      if ((epi.ldo & 3) == 0) {
-#pragma unroll
-        for (int i = 0; i < 32; i += 4) *(float4*)(epi.out_f + o + i) = make_float4(r[i], r[i + 1], r[i + 2], r[i + 3]);
-      } else {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) epi.out_f[o + i] = r[i];
-      }
+  // ragged rows or columns, unaligned rows: one column per lane, two rows at a time
+  const int col = cb + (lane & 15);
+  if (col >= nend) return;
+  for (int i = lane >> 4; i < 32; i += 2) {
+    const int row = row0 + i;
+    if (row >= M) return;
+    const float v = stg[i * EPI_LD + (lane & 15)];
+    if (partial) {
+      partial[((size_t)z * M + row) * N + col] = v;
+      continue;
     }
-    if (epi.out_b) {
-      if ((epi.ldo & 7) == 0) {
-#pragma unroll
-        for (int i = 0; i < 32; i += 8) {
-          uint4 q;
-          __nv_bfloat162 h0 = __floats2bfloat162_rn(r[i], r[i + 1]), h1 = __floats2bfloat162_rn(r[i + 2], r[i + 3]),
-                         h2 = __floats2bfloat162_rn(r[i + 4], r[i + 5]), h3 = __floats2bfloat162_rn(r[i + 6], r[i + 7]);
-          q.x = *(uint32_t*)&h0;
-          q.y = *(uint32_t*)&h1;
-          q.z = *(uint32_t*)&h2;
-          q.w = *(uint32_t*)&h3;
-          *(uint4*)(epi.out_b + o + i) = q;
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) epi.out_b[o + i] = __float2bfloat16_rn(r[i]);
-      }
-    }
-  } else {   // the ragged last columns: a test per column keeps the indexing static
-#pragma unroll
-    for (int i = 0; i < 32; ++i) {
-      if (cb + i < N) {
-        const float x = epi_value(r[i], row, cb + i, epi);
-        const size_t o = (size_t)row * epi.ldo + cb + i;
-        if (epi.out_f) epi.out_f[o] = x;
-        if (epi.out_b) epi.out_b[o] = __float2bfloat16_rn(x);
-      }
-    }
+    const float x = epi_value(v, row, col, epi);
+    const size_t o = (size_t)row * epi.ldo + col;
+    if (epi.out_f) epi.out_f[o] = x;
+    if (epi.out_b) epi.out_b[o] = __float2bfloat16_rn(x);
   }
 }
 
-// 32 float32 accumulator columns of this warp's TMEM lanes, from column address taddr
-__device__ __forceinline__ void tmem_ld32(uint32_t (&v)[32], uint32_t taddr) {
+// 16 float32 accumulator columns of this warp's TMEM lanes, from column address taddr
+__device__ __forceinline__ void tmem_ld16(uint32_t (&v)[16], uint32_t taddr) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
       : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
-        "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
-        "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
       : "r"(taddr));
   asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+}
+
+// One warp's share of an accumulator (TMEM base address of its lanes, columns
+// 16 half, 16 half + 32, ... of width) through its stage into the outputs.
+__device__ __forceinline__ void drain(float* stg, uint32_t tmem, int half, int width, int row0, int n0, int z, int M,
+                                      int N, const Epi& epi, float* __restrict__ partial) {
+  const int lane = threadIdx.x & 31, nend = min(n0 + width, N);
+  for (int c0 = 16 * half; c0 < width && n0 + c0 < N; c0 += 32) {
+    uint32_t v[16];
+    tmem_ld16(v, tmem + (uint32_t)c0);
+    __syncwarp();                             // the previous chunk has left the stage
+#pragma unroll
+    for (int i = 0; i < 16; i += 4)
+      *reinterpret_cast<float4*>(stg + lane * EPI_LD + i) =
+          make_float4(__uint_as_float(v[i]), __uint_as_float(v[i + 1]), __uint_as_float(v[i + 2]),
+                      __uint_as_float(v[i + 3]));
+    __syncwarp();
+    store_chunk(stg, row0, n0 + c0, z, M, N, nend, epi, partial);
+  }
 }
 
 // D = A B' (bf16 A, B K-major, float32 accumulation in tensor memory), persistent:
@@ -227,14 +273,14 @@ __device__ __forceinline__ void tmem_ld32(uint32_t (&v)[32], uint32_t taddr) {
 // blockIdx.x + gridDim.x, ... (a unit is one BM x BN tile of one k split;
 // the tiles in bands of tile rows, see `unit`).
 // Warp roles: warp 0 lane 0 issues the TMA loads of every unit through the
-// STAGES ring, warp 1 lane 0 the MMAs, warps 2..5 drain the accumulators
+// STAGES ring, warp 1 lane 0 the MMAs, warps 2..9 drain the accumulators
 // (warp w reads TMEM lanes 32 (w mod 4) .. +32).  Two accumulators of BN
 // columns: the epilogue of one unit overlaps the main loop of the next.
 // Every wait is bounded (WAIT_NS without progress, or the error flag), after
 // which the roles leave their loops, the copies in flight land, and the TMEM
 // is freed.
 template <int BN>
-__global__ void __launch_bounds__(192, 1)
+__global__ void __launch_bounds__(GEMM_NT, 1)
     k_gemm_tn_p(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int M, int N,
                 int K, int ktps, int splits, Epi epi, float* __restrict__ partial, int* err) {
   constexpr int STAGE_BYTES = Tile<BN>::STAGE_BYTES;
@@ -245,6 +291,7 @@ __global__ void __launch_bounds__(192, 1)
   uint64_t* acc_full = empty + STAGES;       // [2]: the MMAs of a unit are done
   uint64_t* acc_empty = acc_full + 2;        // [2]: the epilogue has read the accumulator
   uint32_t* tmem_slot = (uint32_t*)(acc_empty + 2);
+  float* epi_stage = (float*)(sm + STAGES * STAGE_BYTES + 256);
   __shared__ volatile int s_fail;
   __shared__ int s_issued;                   // stage loads issued, for the cleanup
   __shared__ volatile int s_progress;        // stages consumed by the MMA issuer
@@ -263,7 +310,7 @@ __global__ void __launch_bounds__(192, 1)
     }
     for (int q = 0; q < 2; ++q) {
       mbar_init(&acc_full[q], 1);
-      mbar_init(&acc_empty[q], 4);           // one arrival per epilogue warp
+      mbar_init(&acc_empty[q], EPI_WARPS);   // one arrival per epilogue warp
     }
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
@@ -363,12 +410,8 @@ __global__ void __launch_bounds__(192, 1)
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;\n");
-      const int row = m0 + sp * 32 + lane;
-      for (int c0 = 0; c0 < BN; c0 += 32) {
-        uint32_t v[32];
-        tmem_ld32(v, tmem + ((uint32_t)(sp * 32) << 16) + (uint32_t)(buf * BN + c0));
-        if (row < M) store_chunk(v, row, n0 + c0, z, M, N, epi, splits > 1 ? partial : nullptr);
-      }
+      drain(epi_stage + (warp - 2) * 32 * EPI_LD, tmem + ((uint32_t)(sp * 32) << 16) + (uint32_t)(buf * BN),
+            (warp - 2) >> 2, BN, m0 + sp * 32, n0, z, M, N, epi, splits > 1 ? partial : nullptr);
       asm volatile("tcgen05.fence::before_thread_sync;\n");
       __syncwarp();
       if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(&acc_empty[buf])) : "memory");
@@ -389,6 +432,207 @@ __global__ void __launch_bounds__(192, 1)
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(2 * BN));
 }
 
+// --------------------------------------------------------------------------
+// The same product on CTA pairs (cta_group::2): a cluster of two CTAs works on
+// one 256 x bn tile.  Each CTA loads its 128 rows of A and its half of the bn rows of
+// B, the even CTA's thread issues M = 256 MMAs that read both CTAs' shared memory,
+// and each CTA drains the 128 rows that its tensor memory holds.  Per MMA step a
+// CTA then moves 16 KB through shared memory (TMA write and tensor-core read of
+// 4 KB of A and 4 KB of B) instead of 24 KB: with one CTA per tile the 192 bytes
+// a clock exceed the 128 of the shared memory, which bound k_gemm_tn_p.
+// bn (a multiple of 16, <= 256) is chosen so that the tiles fill the waves
+// (plan_pairs).  Barriers: `full` lives in the even CTA and counts both CTAs'
+// bytes; `empty` and `acc_full` are signalled in both CTAs by a multicast commit;
+// `acc_empty` in the even CTA takes an arrival of each CTA's epilogue warps.
+// Every wait is bounded as in k_gemm_tn_p; both CTAs meet at a cluster barrier
+// before they leave, so no signal reaches shared memory that is gone.
+constexpr int P_STAGES = 6;
+constexpr int P_B_BYTES = 128 * BK * 2;                 // at most 128 rows of B per CTA
+constexpr int P_STAGE_BYTES = A_BYTES + P_B_BYTES;      // 32 KiB
+constexpr int P_SMEM_BYTES = P_STAGES * P_STAGE_BYTES + 1024 + 256 + EPI_WARPS * 32 * EPI_LD * 4;
+
+__device__ __forceinline__ uint32_t mapa_u32(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+// a load into this CTA whose bytes count on the barrier at cluster address bar
+__device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* map, uint32_t bar, int x, int y) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], "
+      "[%2];\n" ::"r"(smem_u32(dst)),
+      "l"((uint64_t)map), "r"(bar), "r"(x), "r"(y)
+      : "memory");
+}
+__device__ __forceinline__ void commit_pair(uint64_t* bar) {   // arrives on this barrier in both CTAs
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n" ::"r"(
+          smem_u32(bar)),
+      "h"((uint16_t)3));
+}
+
+__global__ void __launch_bounds__(GEMM_NT, 1) __cluster_dims__(2, 1, 1)
+    k_gemm_tn_pair(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int M, int N,
+                   int K, int bn, int ktps, int splits, Epi epi, float* __restrict__ partial, int* err) {
+  extern __shared__ __align__(1024) unsigned char smraw[];
+  unsigned char* sm = (unsigned char*)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
+  uint64_t* full = (uint64_t*)(sm + P_STAGES * P_STAGE_BYTES);
+  uint64_t* empty = full + P_STAGES;
+  uint64_t* acc_full = empty + P_STAGES;     // [2]
+  uint64_t* acc_empty = acc_full + 2;        // [2]
+  uint32_t* tmem_slot = (uint32_t*)(acc_empty + 2);
+  float* epi_stage = (float*)(sm + P_STAGES * P_STAGE_BYTES + 256);
+  __shared__ volatile int s_fail;
+  __shared__ int s_issued;
+  __shared__ volatile int s_progress;        // stages consumed (even CTA), stages granted (odd CTA)
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = blockIdx.x & 1;
+  const bool leader = rank == 0;
+  const int tn = (N + bn - 1) / bn, tm = (M + 2 * BM - 1) / (2 * BM);
+  const int KT = (K + BK - 1) / BK;
+  const int units = tm * tn * splits;
+  const int u0 = blockIdx.x >> 1, du = gridDim.x >> 1;
+  const uint32_t half_bytes = (uint32_t)(bn / 2) * BK * 2;
+
+  if (threadIdx.x == 0) {
+    s_fail = 0;
+    s_issued = 0;
+    s_progress = 0;
+    for (int q = 0; q < P_STAGES; ++q) {
+      mbar_init(&full[q], 1);
+      mbar_init(&empty[q], 1);
+    }
+    for (int q = 0; q < 2; ++q) {
+      mbar_init(&acc_full[q], 1);
+      mbar_init(&acc_empty[q], 2 * EPI_WARPS);   // the epilogue warps of both CTAs
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  if (warp == 0) {   // both CTAs: two accumulators of 256 float32 columns
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_slot)),
+                 "r"(512));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;\n");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;\n");
+  __syncthreads();
+  cluster_sync();                            // the peer's barriers are initialised
+  asm volatile("tcgen05.fence::after_thread_sync;\n");
+  const uint32_t tmem = *tmem_slot;
+
+  // tiles in bands of tile rows, as k_gemm_tn_p (4 x 256 rows)
+  constexpr int GROUP = 4;
+  auto unit = [&](int u, int& m0, int& n0, int& kt0, int& nk, int& z) {
+    z = u / (tm * tn);
+    const int t = u - z * (tm * tn);
+    const int band = t / (GROUP * tn), first = band * GROUP;
+    const int rows = min(tm - first, GROUP);
+    const int q = t - band * GROUP * tn;
+    m0 = (first + q % rows) * 2 * BM;
+    n0 = (q / rows) * bn;
+    kt0 = z * ktps;
+    nk = min(KT, kt0 + ktps) - kt0;
+  };
+
+  if (warp == 0 && lane == 0) {   // TMA producer of this CTA's halves
+    int i = 0;
+    for (int u = u0; u < units && !s_fail; u += du) {
+      int m0, n0, kt0, nk, z;
+      unit(u, m0, n0, kt0, nk, z);
+      for (int k = 0; k < nk; ++k, ++i) {
+        const int q = i % P_STAGES;
+        if (i >= P_STAGES && !mbar_wait(&empty[q], ((i / P_STAGES) - 1) & 1, err, &s_progress)) {
+          s_fail = 1;
+          break;
+        }
+        if (!leader) s_progress = i + 1;
+        unsigned char* a = sm + q * P_STAGE_BYTES;
+        if (leader) mbar_expect_tx(&full[q], 2 * (A_BYTES + half_bytes));
+        const uint32_t bar = mapa_u32(smem_u32(&full[q]), 0);
+        tma_load_2d_pair(a, &mapA, bar, (kt0 + k) * BK, m0 + (int)rank * BM);
+        tma_load_2d_pair(a + A_BYTES, &mapB, bar, (kt0 + k) * BK, n0 + (int)rank * (bn / 2));
+        s_issued = i + 1;
+      }
+    }
+  } else if (warp == 1 && lane == 0 && leader) {   // MMA issuer
+    const uint32_t idesc = instr_desc(2 * BM, bn);
+    int i = 0, lt = 0;
+    for (int u = u0; u < units && !s_fail; u += du, ++lt) {
+      int m0, n0, kt0, nk, z;
+      unit(u, m0, n0, kt0, nk, z);
+      const int buf = lt & 1;
+      if (!mbar_wait(&acc_empty[buf], ((lt >> 1) & 1) ^ 1, err)) {
+        s_fail = 1;
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;\n");
+      const uint32_t acc_tm = tmem + (uint32_t)(buf * 256);
+      for (int k = 0; k < nk; ++k, ++i) {
+        const int q = i % P_STAGES;
+        if (!mbar_wait(&full[q], (i / P_STAGES) & 1, err)) {
+          s_fail = 1;
+          break;
+        }
+        s_progress = i + 1;
+        asm volatile("tcgen05.fence::after_thread_sync;\n");
+        const unsigned char* a = sm + q * P_STAGE_BYTES;
+        const uint64_t da = smem_desc(a), db = smem_desc(a + A_BYTES);
+#pragma unroll
+        for (int kk = 0; kk < BK / 16; ++kk) {
+          const uint64_t step = (uint64_t)((kk * 16 * 2) >> 4);
+          const uint32_t acc = (k > 0 || kk > 0) ? 1u : 0u;
+          asm volatile(
+              "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
+              " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(acc_tm),
+              "l"(da + step), "l"(db + step), "r"(idesc), "r"(acc));
+        }
+        commit_pair(&empty[q]);
+      }
+      if (s_fail) break;
+      commit_pair(&acc_full[buf]);
+    }
+  } else if (warp >= 2) {   // epilogue of this CTA's 128 rows
+    const int sp = warp & 3;
+    const uint32_t ae0 = mapa_u32(smem_u32(&acc_empty[0]), 0), ae1 = mapa_u32(smem_u32(&acc_empty[1]), 0);
+    int lt = 0;
+    for (int u = u0; u < units; u += du, ++lt) {
+      int m0, n0, kt0, nk, z;
+      unit(u, m0, n0, kt0, nk, z);
+      const int buf = lt & 1;
+      if (s_fail || !mbar_wait(&acc_full[buf], (lt >> 1) & 1, err, &s_progress)) {
+        s_fail = 1;
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;\n");
+      drain(epi_stage + (warp - 2) * 32 * EPI_LD, tmem + ((uint32_t)(sp * 32) << 16) + (uint32_t)(buf * 256),
+            (warp - 2) >> 2, bn, m0 + (int)rank * BM + sp * 32, n0, z, M, N, epi, splits > 1 ? partial : nullptr);
+      asm volatile("tcgen05.fence::before_thread_sync;\n");
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];\n" ::"r"(buf ? ae1 : ae0)
+                     : "memory");
+    }
+  }
+  __syncwarp();
+  asm volatile("tcgen05.fence::before_thread_sync;\n");
+  __syncthreads();
+  cluster_sync();
+  if (s_fail && threadIdx.x == 0) {   // record the failure; let the copies in flight land (both CTAs' count on the leader)
+    atomicExch(err, 1);
+    const int issued = s_issued;
+    if (leader)
+      for (int i = max(0, issued - P_STAGES); i < issued; ++i) {
+        int never = 0;
+        mbar_wait(&full[i % P_STAGES], (i / P_STAGES) & 1, &never);
+      }
+  }
+  __syncthreads();
+  cluster_sync();
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(512));
+}
+
 // The bounded wait of the tensor-core kernels on an mbarrier that nothing
 // completes: it gives up after WAIT_NS and raises the error flag, as a GEMM
 // whose copies or MMAs never landed would (the host then reads
@@ -403,17 +647,33 @@ __global__ void k_wait_probe(int* err) {
   if (threadIdx.x == 0 && !mbar_wait(&bar, 0, err)) atomicExch(err, 1);
 }
 
-// Sum of the split-K partials in a fixed order, then the epilogue.
-__global__ void k_splitk_epi(const float* __restrict__ part, int splits, int M, int N, Epi epi) {
-  const long long MN = (long long)M * N;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < MN; i += (long long)gridDim.x * blockDim.x) {
-    float r = 0.f;
-    for (int z = 0; z < splits; ++z) r += part[z * MN + i];
-    const int row = (int)(i / N), col = (int)(i % N);
-    r = epi_value(r, row, col, epi);
+// Sum of the split-K partials in a fixed order, then the epilogue: W columns
+// per thread (4 where N and the leading dimensions allow), a row per grid y.
+template <int W>
+__global__ void __launch_bounds__(128) k_splitk_epi(const float* __restrict__ part, int splits, int M, int N, Epi epi) {
+  const size_t MN = (size_t)M * N;
+  const int col = (blockIdx.x * 128 + threadIdx.x) * W;
+  if (col >= N) return;
+  for (int row = blockIdx.y; row < M; row += gridDim.y) {
+    const float* p = part + (size_t)row * N + col;
+    float r[W];
+#pragma unroll
+    for (int i = 0; i < W; ++i) r[i] = 0.f;
+    for (int z = 0; z < splits; ++z) {
+      if constexpr (W == 4) {
+        const float4 q = *reinterpret_cast<const float4*>(p + z * MN);
+        r[0] += q.x; r[1] += q.y; r[2] += q.z; r[3] += q.w;
+      } else {
+        r[0] += p[z * MN];
+      }
+    }
     const size_t o = (size_t)row * epi.ldo + col;
-    if (epi.out_f) epi.out_f[o] = r;
-    if (epi.out_b) epi.out_b[o] = __float2bfloat16_rn(r);
+#pragma unroll
+    for (int i = 0; i < W; ++i) {
+      const float v = epi_value(r[i], row, col + i, epi);
+      if (epi.out_f) epi.out_f[o + i] = v;
+      if (epi.out_b) epi.out_b[o + i] = __float2bfloat16_rn(v);
+    }
   }
 }
 
@@ -424,53 +684,197 @@ __device__ __forceinline__ long long visit(long long a, long long s, long long c
   return (a * i + s) % count;
 }
 
+// The elementwise kernels below take W columns per thread (two, in 16-byte
+// accesses, where n and m are even) and ROWS_PER rows per grid y: the
+// per-feature constants are read (and converted) once, no index is divided,
+// and the rows' loads are in flight together.  What bounds them is memory or,
+// where a value is converted, GB300's float64 pipe (two lanes per clock per
+// SM, conversions included).
+constexpr int ROWS_PER = 16;
+constexpr int BATCH = 8;            // rows loaded before the first is used
+
+template <int W>
+__device__ __forceinline__ void load_cols(const double* __restrict__ p, double (&v)[W]) {
+  if constexpr (W == 2) {
+    const double2 q = __ldcs(reinterpret_cast<const double2*>(p));
+    v[0] = q.x;
+    v[1] = q.y;
+  } else {
+    v[0] = __ldcs(p);
+  }
+}
+
 // u = bf16((fl32(v) - mean) * scale) for rows [row0, row0+rows) of v = [C | B]
-__global__ void k_prep_input(const double* __restrict__ C, const double* __restrict__ B, int n, int m, long long row0,
-                             int rows, const float* __restrict__ mean, const float* __restrict__ scale,
-                             bf16* __restrict__ U, int ldu) {
-  const int F = n + m;
-  const long long total = (long long)rows * F;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    const int r = (int)(i / F), f = (int)(i % F);
-    const long long smp = row0 + r;
-    const double v = f < n ? C[smp * n + f] : B[smp * m + (f - n)];
-    U[(size_t)r * ldu + f] = __float2bfloat16_rn(__fmul_rn(__fsub_rn((float)v, mean[f]), scale[f]));
+template <int W>
+__global__ void __launch_bounds__(256)
+    k_prep_input(const double* __restrict__ C, const double* __restrict__ B, int n, int m, long long row0, int rows,
+                 const float* __restrict__ mean, const float* __restrict__ scale, bf16* __restrict__ U, int ldu) {
+  const int f = (blockIdx.x * 256 + threadIdx.x) * W;
+  if (f >= n + m) return;
+  const double* src = f < n ? C + (size_t)row0 * n + f : B + (size_t)row0 * m + (f - n);
+  const size_t ld = f < n ? n : m;
+  float mu[W], sc[W];
+#pragma unroll
+  for (int i = 0; i < W; ++i) { mu[i] = mean[f + i]; sc[i] = scale[f + i]; }
+  const int r1 = min(rows, (int)(blockIdx.y + 1) * ROWS_PER);
+  for (int r = blockIdx.y * ROWS_PER; r < r1; r += BATCH) {
+    double v[BATCH][W];
+#pragma unroll
+    for (int k = 0; k < BATCH; ++k)
+      if (r + k < r1) load_cols<W>(src + (r + k) * ld, v[k]);
+#pragma unroll
+    for (int k = 0; k < BATCH; ++k) {
+      if (r + k >= r1) break;
+      bf16 h[W];
+#pragma unroll
+      for (int i = 0; i < W; ++i) h[i] = __float2bfloat16_rn(__fmul_rn(__fsub_rn((float)v[k][i], mu[i]), sc[i]));
+      bf16* d = U + (size_t)(r + k) * ldu + f;
+      if constexpr (W == 2) *reinterpret_cast<__nv_bfloat162*>(d) = __nv_bfloat162(h[0], h[1]);
+      else *d = h[0];
+    }
   }
 }
 
 // t = (fl32(v) - omean) * oinv, float32, for rows [0, count) of [X | Y]
-__global__ void k_prep_target(const double* __restrict__ X, const double* __restrict__ Y, int n, int m,
-                              long long count, const float* __restrict__ omean, const float* __restrict__ oinv,
-                              float* __restrict__ T, int ldt) {
-  const int F = n + m;
-  const long long total = count * F;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    const long long r = i / F;
-    const int f = (int)(i % F);
-    const double v = f < n ? X[r * n + f] : Y[r * m + (f - n)];
-    T[r * ldt + f] = __fmul_rn(__fsub_rn((float)v, omean[f]), oinv[f]);
+template <int W>
+__global__ void __launch_bounds__(256)
+    k_prep_target(const double* __restrict__ X, const double* __restrict__ Y, int n, int m, long long count,
+                  const float* __restrict__ omean, const float* __restrict__ oinv, float* __restrict__ T, int ldt) {
+  const int f = (blockIdx.x * 256 + threadIdx.x) * W;
+  if (f >= n + m) return;
+  const double* src = f < n ? X + f : Y + (f - n);
+  const size_t ld = f < n ? n : m;
+  float mu[W], sc[W];
+#pragma unroll
+  for (int i = 0; i < W; ++i) { mu[i] = omean[f + i]; sc[i] = oinv[f + i]; }
+  for (long long b = blockIdx.y; b * ROWS_PER < count; b += gridDim.y) {
+    const long long r1 = min(count, (b + 1) * ROWS_PER);
+    for (long long r = b * ROWS_PER; r < r1; r += BATCH) {
+      double v[BATCH][W];
+#pragma unroll
+      for (int k = 0; k < BATCH; ++k)
+        if (r + k < r1) load_cols<W>(src + (r + k) * ld, v[k]);
+#pragma unroll
+      for (int k = 0; k < BATCH; ++k) {
+        if (r + k >= r1) break;
+        float t[W];
+#pragma unroll
+        for (int i = 0; i < W; ++i) t[i] = __fmul_rn(__fsub_rn((float)v[k][i], mu[i]), sc[i]);
+        if constexpr (W == 2) *reinterpret_cast<float2*>(T + (r + k) * ldt + f) = make_float2(t[0], t[1]);
+        else T[(r + k) * ldt + f] = t[0];
+      }
+    }
   }
 }
 
-// per-feature mean and population std over `count` rows (two passes, float64);
-// std below 1e-8 counts as 1
-__global__ void k_fit_stats(const double* __restrict__ V, long long count, int nf, float* __restrict__ mean,
-                            float* __restrict__ scale, float* __restrict__ stdv) {
-  const int f = blockIdx.x * blockDim.x + threadIdx.x;
+// The sum of (hi, lo) and x, the rounding error kept (Knuth's two-sum), plus a
+// low-order term.
+__device__ __forceinline__ void pair_add(float& hi, float& lo, float x, float xl) {
+  const float t = __fadd_rn(hi, x), b = __fsub_rn(t, hi);
+  const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, b)), __fsub_rn(x, b));
+  hi = t;
+  lo = __fadd_rn(lo, __fadd_rn(e, xl));
+}
+
+// Per-feature mean and sum of squared deviations of a range of rows, one pass:
+// deviations from the range's first row.  That row is one of the data, so its
+// squared distance from the mean is at most FIT_ROWS times the range's
+// variance, and the cancellation in M2 costs at most about that factor of a
+// rounding.  In float64 the pass takes three float64-pipe operations a value
+// (1.27 ms for 4096 x 60000 values at that pipe's rate); it takes the difference
+// there, and the sums run on float32 pairs: the difference's bits split into
+// 24 + 23 (truncated at 2^-46 of it), products and sums with their exact
+// rounding errors.  Values whose square or its error leaves float32's range
+// take the float64 sums.  Two arrays per launch (grid z) and short ranges, so
+// that the blocks fill whole waves (ranges of 256 rows, one array a launch: a
+// little over two waves, 1.48 ms; the two-pass form before, 157 blocks of one
+// column per thread: 4.8 ms).
+constexpr int FIT_ROWS = 64;
+struct FitPair {
+  const double* v[2];
+  double* mean[2];       // [ranges x nf]
+  double* m2[2];
+};
+__global__ void __launch_bounds__(256) k_fit_part(FitPair a, long long count, int nf) {
+  const int f = blockIdx.x * 256 + threadIdx.x;
   if (f >= nf) return;
-  double s = 0.0;
-  for (long long r = 0; r < count; ++r) s += V[r * nf + f];
-  const double mu = s / (double)count;
-  double q = 0.0;
-  for (long long r = 0; r < count; ++r) {
-    const double d = V[r * nf + f] - mu;
-    q += d * d;
+  const double* V = a.v[blockIdx.z];
+  for (long long b = blockIdx.y; b * FIT_ROWS < count; b += gridDim.y) {
+    const long long r0 = b * FIT_ROWS;
+    const int rows = (int)min((long long)FIT_ROWS, count - r0);
+    const double* p = V + (size_t)r0 * nf + f;
+    const double K = isfinite(p[0]) ? p[0] : 0.0;
+    float sh = 0.f, sl = 0.f, qh = 0.f, ql = 0.f;
+    double sd = 0.0, qd = 0.0;
+    for (int r = 0; r < rows; r += BATCH) {
+      double v[BATCH];                             // all in flight before the first is used
+#pragma unroll
+      for (int k = 0; k < BATCH; ++k) v[k] = r + k < rows ? __ldcs(p + (size_t)(r + k) * nf) : K;
+#pragma unroll
+      for (int k = 0; k < BATCH; ++k) {            // (a row past the end adds 0)
+        const double d = v[k] - K;
+        const unsigned hw = (unsigned)__double2hiint(d), lw = (unsigned)__double2loint(d);
+        const unsigned e = (hw >> 20) & 0x7FFu, sg = hw & 0x80000000u;
+        if (e - 973u <= 113u) {                    // 2^-50 <= |d| < 2^64
+          const float hi = __uint_as_float(sg | ((e - 896u) << 23) | (__funnelshift_l(lw, hw, 3) & 0x7FFFFFu));
+          const float lo = __fmul_rn(__fsub_rn(__uint_as_float(0x4B000000u | ((lw >> 6) & 0x7FFFFFu)), 8388608.f),
+                                     __uint_as_float(sg | ((e - 942u) << 23)));
+          pair_add(sh, sl, hi, lo);
+          const float q = __fmul_rn(hi, hi);
+          pair_add(qh, ql, q, __fmaf_rn(__fadd_rn(hi, hi), lo, __fmaf_rn(hi, hi, -q)));
+        } else if (((hw << 1) | lw) != 0u) {       // not a zero
+          sd += d;
+          qd = fma(d, d, qd);
+        }
+      }
+    }
+    const double s = (double)sh + (double)sl + sd, q = (double)qh + (double)ql + qd;
+    const double c = s * (1.0 / (double)rows), t = fma(-s, c, q);
+    a.mean[blockIdx.z][(size_t)b * nf + f] = K + c;
+    a.m2[blockIdx.z][(size_t)b * nf + f] = t < 0.0 ? 0.0 : t;    // (a NaN stays one)
   }
+}
+
+// the ranges merged in order (Chan, Golub & LeVeque 1983): per-feature mean and
+// population std over all rows; std below 1e-8 counts as 1.  The merge weights
+// are the same for every feature: the block's threads form 128 at a time.
+struct FitOut {
+  float* mean[2];
+  float* scale[2];
+  float* stdv[2];        // null: not kept
+};
+__global__ void __launch_bounds__(128) k_fit_merge(FitPair a, long long count, int nf, FitOut o) {
+  __shared__ double sw[128], sv[128];
+  const int f = blockIdx.x * 128 + threadIdx.x;
+  const double *pm = a.mean[blockIdx.z], *p2 = a.m2[blockIdx.z];
+  const long long nb = (count + FIT_ROWS - 1) / FIT_ROWS;
+  double mu = 0.0, q = 0.0;
+  if (f < nf) { mu = pm[f]; q = p2[f]; }
+  for (long long b0 = 1; b0 < nb; b0 += 128) {
+    const long long b = b0 + threadIdx.x;
+    __syncthreads();
+    if (b < nb) {
+      const double na = (double)(b * FIT_ROWS), c = (double)min((long long)FIT_ROWS, count - b * FIT_ROWS);
+      sw[threadIdx.x] = c / (na + c);
+      sv[threadIdx.x] = na * c / (na + c);
+    }
+    __syncthreads();
+    if (f >= nf) continue;
+    const int n = (int)min(128LL, nb - b0);
+#pragma unroll 4
+    for (int i = 0; i < n; ++i) {
+      const double mb = pm[(size_t)(b0 + i) * nf + f], d = mb - mu;
+      mu = isfinite(d) ? fma(d, sw[i], mu) : mu + mb;    // an infinite mean stays one
+      q = fma(d * d, sv[i], q + p2[(size_t)(b0 + i) * nf + f]);
+    }
+  }
+  if (f >= nf) return;
   double sd = sqrt(q / (double)count);
   if (sd < 1e-8) sd = 1.0;
-  mean[f] = (float)mu;
-  scale[f] = (float)(1.0 / sd);
-  if (stdv) stdv[f] = (float)sd;
+  const int z = blockIdx.z;
+  o.mean[z][f] = (float)mu;
+  o.scale[z][f] = (float)(1.0 / sd);
+  if (o.stdv[z]) o.stdv[z][f] = (float)sd;
 }
 
 __global__ void k_gather_rows(const bf16* __restrict__ src, int ld, long long a, long long s, long long count,
@@ -498,19 +902,34 @@ __global__ void __launch_bounds__(256) k_grad_tiles(const float* __restrict__ in
                                                     float* __restrict__ colpart, int ldc, double* __restrict__ lossp) {
   __shared__ float tile[32][33];
   __shared__ double red[8];
+  __shared__ long long smp_of[32];
   const int f0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int f = f0 + tx;
-  double ls = 0.0;
+  // the squared error in float32 pairs (product and sum with their exact
+  // rounding errors, about 2^-48 relative): a thread's four terms would take
+  // eight float64-pipe operations (conversions included), one conversion pair
+  // here; terms whose square or its error leaves float32's range go to ld
+  float lh = 0.f, ll = 0.f;
+  double ld = 0.0;
+  if (MODE == 0) {   // the rows' samples, one 64-bit remainder each
+    if (ty == 0 && r0 + tx < rows) smp_of[tx] = visit(a, sft, count, row0 + r0 + tx);
+    __syncthreads();
+  }
+#pragma unroll
   for (int i = ty; i < 32; i += 8) {
     const int r = r0 + i;
     float g = 0.f;
     if (r < rows && f < F) {
       const float o = in[(size_t)r * ldi + f];
       if (MODE == 0) {
-        const long long smp = visit(a, sft, count, row0 + r);
-        const float d = __fsub_rn(o, T[(size_t)smp * ldt + f]);
-        ls += (double)d * (double)d;
+        const float d = __fsub_rn(o, T[(size_t)smp_of[i] * ldt + f]);
+        if (fabsf(d) > 1e-10f && fabsf(d) < 1e15f) {
+          const float ph = __fmul_rn(d, d);
+          pair_add(lh, ll, ph, __fmaf_rn(d, d, -ph));
+        } else {
+          ld += (double)d * (double)d;
+        }
         g = __fmul_rn(d, scale);
       } else {
         g = o;
@@ -530,8 +949,13 @@ __global__ void __launch_bounds__(256) k_grad_tiles(const float* __restrict__ in
     if (ff < F && rr < rows) gt[(size_t)ff * ldgt + rr] = __float2bfloat16_rn(tile[tx][i]);
   }
   if (MODE == 0) {
-    for (int o = 16; o > 0; o >>= 1) ls += __shfl_down_sync(0xffffffffu, ls, o);
-    if (tx == 0) red[ty] = ls;
+    for (int o = 16; o > 0; o >>= 1) {
+      const float xh = __shfl_down_sync(0xffffffffu, lh, o), xl = __shfl_down_sync(0xffffffffu, ll, o);
+      pair_add(lh, ll, xh, xl);
+    }
+    if (__any_sync(0xffffffffu, ld != 0.0))       // warp-uniform (a NaN too)
+      for (int o = 16; o > 0; o >>= 1) ld += __shfl_down_sync(0xffffffffu, ld, o);
+    if (tx == 0) red[ty] = (double)lh + (double)ll + ld;
     __syncthreads();
     if (tx == 0 && ty == 0) {
       double t = 0.0;
@@ -549,18 +973,21 @@ __global__ void k_colsum(const float* __restrict__ part, int ntiles, int F, int 
   out[f] = s;
 }
 
-// acc += inv * sum(parts) (one block of 256 threads, fixed order)
-__global__ void k_loss_acc(const double* __restrict__ parts, int n, double inv, double* __restrict__ acc) {
-  __shared__ double red[256];
+// acc += inv * sum(parts) (one block of 1024 threads, fixed order)
+__global__ void __launch_bounds__(1024) k_loss_acc(const double* __restrict__ parts, int n, double inv,
+                                                   double* __restrict__ acc) {
+  __shared__ double red[32];
   double s = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) s += parts[i];
-  red[threadIdx.x] = s;
+#pragma unroll 4
+  for (int i = threadIdx.x; i < n; i += 1024) s += parts[i];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
+  if (threadIdx.x < 32) {
+    s = red[threadIdx.x];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (threadIdx.x == 0) *acc += inv * s;
   }
-  if (threadIdx.x == 0) *acc += inv * red[0];
 }
 
 __global__ void k_transpose_bf16(const bf16* __restrict__ in, int ldi, int rows, int cols, bf16* __restrict__ out,
@@ -589,35 +1016,56 @@ __device__ __forceinline__ float adam_one(float w, float g, float& m, float& v, 
   return w - a.lr * (m * a.c1) / (sqrtf(v * a.c2) + a.eps);
 }
 
-// Adam on a rows x cols weight (all float32 arrays row-major, ld = cols), then
-// the bf16 copy [rows x ldb] and the transposed bf16 copy [cols x ldt].
+// Adam on a rows x cols weight (all float32 arrays row-major, ld = cols, a
+// multiple of 4), then the bf16 copy [rows x ldb] and the transposed bf16 copy
+// [cols x ldt].  Bound by memory (28 bytes read and written per weight and 4
+// for the copies): 64 x 64 tiles, four columns per thread in 16-byte accesses,
+// the transposed copy in 128-byte runs.
+constexpr int ADAM_T = 64;
 __global__ void __launch_bounds__(256) k_adam_mat(float* __restrict__ W, float* __restrict__ mW,
                                                   float* __restrict__ vW, const float* __restrict__ g, int rows,
                                                   int cols, AdamArgs a, bf16* __restrict__ Wb, int ldb,
                                                   bf16* __restrict__ Wt, int ldt) {
-  __shared__ bf16 t[32][34];
-  const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-    const int r = r0 + i, c = c0 + threadIdx.x;
+  __shared__ bf16 t[ADAM_T][ADAM_T + 2];          // [column][row]
+  const int c0 = blockIdx.x * ADAM_T, r0 = blockIdx.y * ADAM_T;
+  const int cl = (threadIdx.x & 15) * 4, c = c0 + cl;
+#pragma unroll
+  for (int k = 0; k < ADAM_T / 16; ++k) {
+    const int rl = (threadIdx.x >> 4) + 16 * k, r = r0 + rl;
     if (r < rows && c < cols) {
-      const size_t k = (size_t)r * cols + c;
-      float w = W[k];
+      const size_t o = (size_t)r * cols + c;
+      float4 w = *reinterpret_cast<const float4*>(W + o);
       if (a.update) {
-        float m = mW[k], v = vW[k];
-        w = adam_one(w, g[k], m, v, a);
-        W[k] = w;
-        mW[k] = m;
-        vW[k] = v;
+        float4 m = *reinterpret_cast<const float4*>(mW + o), v = *reinterpret_cast<const float4*>(vW + o);
+        const float4 gg = *reinterpret_cast<const float4*>(g + o);
+        w.x = adam_one(w.x, gg.x, m.x, v.x, a);
+        w.y = adam_one(w.y, gg.y, m.y, v.y, a);
+        w.z = adam_one(w.z, gg.z, m.z, v.z, a);
+        w.w = adam_one(w.w, gg.w, m.w, v.w, a);
+        *reinterpret_cast<float4*>(W + o) = w;
+        *reinterpret_cast<float4*>(mW + o) = m;
+        *reinterpret_cast<float4*>(vW + o) = v;
       }
-      const bf16 h = __float2bfloat16_rn(w);
-      Wb[(size_t)r * ldb + c] = h;
-      t[i][threadIdx.x] = h;
+      const __nv_bfloat162 h0 = __floats2bfloat162_rn(w.x, w.y), h1 = __floats2bfloat162_rn(w.z, w.w);
+      uint2 q;
+      q.x = *reinterpret_cast<const uint32_t*>(&h0);
+      q.y = *reinterpret_cast<const uint32_t*>(&h1);
+      *reinterpret_cast<uint2*>(Wb + (size_t)r * ldb + c) = q;
+      t[cl][rl] = h0.x;
+      t[cl + 1][rl] = h0.y;
+      t[cl + 2][rl] = h1.x;
+      t[cl + 3][rl] = h1.y;
     }
   }
   __syncthreads();
-  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-    const int c = c0 + i, r = r0 + threadIdx.x;
-    if (r < rows && c < cols) Wt[(size_t)c * ldt + r] = t[threadIdx.x][i];
+  const int rp = (threadIdx.x & 31) * 2;          // ldt is even and r0 + rp too: 4-byte stores
+#pragma unroll
+  for (int k = 0; k < ADAM_T / 8; ++k) {
+    const int cc = (threadIdx.x >> 5) + 8 * k;
+    if (c0 + cc >= cols || r0 + rp >= rows) continue;
+    bf16* d = Wt + (size_t)(c0 + cc) * ldt + r0 + rp;
+    if (r0 + rp + 1 < rows) *reinterpret_cast<uint32_t*>(d) = *reinterpret_cast<const uint32_t*>(&t[cc][rp]);
+    else *d = t[cc][rp];
   }
 }
 
@@ -639,20 +1087,54 @@ __global__ void k_f32_to_bf16_2d(const float* __restrict__ in, int rows, int col
   }
 }
 
-// [x0 | y0] = omean + ostd * o in float64, rows [row0, row0+rows)
-__global__ void k_write_pred(const float* __restrict__ O, int ldo, int rows, int n, int m,
-                             const float* __restrict__ omean, const float* __restrict__ ostd, long long row0,
-                             double* __restrict__ X0, double* __restrict__ Y0) {
-  const int F = n + m;
-  const long long total = (long long)rows * F;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    const int r = (int)(i / F), f = (int)(i % F);
-    const double v = __dadd_rn((double)omean[f], __dmul_rn((double)ostd[f], (double)O[(size_t)r * ldo + f]));
-    const long long smp = row0 + r;
-    if (f < n) {
-      if (X0) X0[smp * n + f] = v;
-    } else if (Y0) {
-      Y0[smp * m + (f - n)] = v;
+// float -> double by integer instructions (the conversion instruction issues on
+// the float64 pipe): the same value for every float (NaN payloads aside)
+__device__ __forceinline__ double widen(float x) {
+  const unsigned u = __float_as_uint(x), e = (u >> 23) & 0xFFu;
+  if (e - 1u >= 254u) return (double)x;           // zero, subnormal, infinite, NaN
+  return __hiloint2double((int)((u & 0x80000000u) | (((u >> 3) & 0x0FFFFFFFu) + 0x38000000u)), (int)(u << 29));
+}
+
+// [x0 | y0] = omean + ostd * o in float64, rows [row0, row0+rows).  The product
+// of two floats is exact in float64, so one fused multiply-add rounds like the
+// separate addition: one float64-pipe operation per value instead of five.
+template <int W>
+__global__ void __launch_bounds__(256)
+    k_write_pred(const float* __restrict__ O, int ldo, int rows, int n, int m, const float* __restrict__ omean,
+                 const float* __restrict__ ostd, long long row0, double* __restrict__ X0, double* __restrict__ Y0) {
+  const int f = (blockIdx.x * 256 + threadIdx.x) * W;
+  if (f >= n + m) return;
+  double* dst = f < n ? X0 : Y0;
+  if (!dst) return;
+  const size_t ld = f < n ? n : m;
+  dst += (size_t)row0 * ld + (f < n ? f : f - n);
+  double mu[W], sd[W];
+#pragma unroll
+  for (int i = 0; i < W; ++i) { mu[i] = (double)omean[f + i]; sd[i] = (double)ostd[f + i]; }
+  const int r1 = min(rows, (int)(blockIdx.y + 1) * ROWS_PER);
+  for (int r = blockIdx.y * ROWS_PER; r < r1; r += BATCH) {
+    float o[BATCH][W];
+#pragma unroll
+    for (int k = 0; k < BATCH; ++k) {
+      if (r + k >= r1) break;
+      const float* p = O + (size_t)(r + k) * ldo + f;
+      if constexpr (W == 2) {
+        const float2 q = __ldcs(reinterpret_cast<const float2*>(p));
+        o[k][0] = q.x;
+        o[k][1] = q.y;
+      } else {
+        o[k][0] = __ldcs(p);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < BATCH; ++k) {
+      if (r + k >= r1) break;
+      double* d = dst + (r + k) * ld;
+      if constexpr (W == 2)
+        *reinterpret_cast<double2*>(d) =
+            make_double2(__fma_rn(sd[0], widen(o[k][0]), mu[0]), __fma_rn(sd[1], widen(o[k][1]), mu[1]));
+      else
+        *d = __fma_rn(sd[0], widen(o[k][0]), mu[0]);
     }
   }
 }
@@ -705,20 +1187,51 @@ static int num_sms() {   // of the current device, read once (a thread-safe stat
 // the B tile width: 256 when N fills it, else 128
 inline int tile_n(int N) { return N >= 256 ? 256 : 128; }
 
-// number of K splits: enough blocks to cover the SMs, at least 4 k-tiles each
-int plan_splits(int M, int N, int K, int requested) {
-  const int BN = tile_n(N);
+// How a product runs: on CTA pairs (256 x bn tiles) or single CTAs (128 x bn),
+// and in how many splits of K.
+struct GemmPlan {
+  int pair, bn, splits;
+};
+
+// Splits: with fewer 128 x 256 (128) tiles than SMs, enough to cover the SMs,
+// at least 4 k-tiles each.  Pairs where M and N fill their tiles (a pair on
+// M <= 128 would idle one CTA).  A product on pairs takes the tile width whose
+// waves cost least: per k-tile a tile lasts as long as it is wide (plus about 32
+// columns' worth of the A side), its epilogue about ten k-tiles; the epilogue
+// of all but the last tile hides behind the next tile's main loop or the other
+// way round.  So 256 for long products with many tiles, less where that
+// leaves the last wave nearly empty or the epilogue of a single wave shows.
+GemmPlan plan_gemm(int M, int N, int K, int requested) {
+  GemmPlan p;
+  p.bn = tile_n(N);
   const int KT = (K + BK - 1) / BK;
   int splits = requested;
   if (splits <= 0) {
-    const long long tiles = (long long)((M + BM - 1) / BM) * ((N + BN - 1) / BN);
+    const long long t = (long long)((M + BM - 1) / BM) * ((N + p.bn - 1) / p.bn);
     splits = 1;
-    if (tiles < num_sms()) splits = (int)std::min<long long>(KT / 4, (num_sms() + tiles - 1) / tiles);
+    if (t < num_sms()) splits = (int)std::min<long long>(KT / 4, (num_sms() + t - 1) / t);
   }
   splits = std::max(1, std::min(splits, KT));
   const int ktps = (KT + splits - 1) / splits;
-  return (KT + ktps - 1) / ktps;
+  p.splits = (KT + ktps - 1) / ktps;
+  p.pair = M > 128 && N >= 256;
+  if (p.pair) {
+    const long long tm = (M + 2 * BM - 1) / (2 * BM), pairs = std::max(1, num_sms() / 2);
+    const long long kt = (KT + p.splits - 1) / p.splits;
+    long long best = 0;
+    for (int bn = 256; bn >= 128; bn -= 16) {
+      const long long waves = (tm * ((N + bn - 1) / bn) * p.splits + pairs - 1) / pairs;
+      const long long main = kt * (bn + 32), epi = 10LL * bn;
+      const long long cost = waves * std::max(main, epi) + std::min(main, epi);
+      if (best == 0 || cost < best) {
+        best = cost;
+        p.bn = bn;
+      }
+    }
+  }
+  return p;
 }
+int plan_splits(int M, int N, int K, int requested) { return plan_gemm(M, N, K, requested).splits; }
 
 size_t splitk_floats(int M, int N, int K, int splits) {
   const int s = plan_splits(M, N, K, splits);
@@ -730,34 +1243,52 @@ size_t splitk_floats(int M, int N, int K, int splits) {
 cudaError_t gemm_tn(const bf16* A, int lda, const bf16* B, int ldb, int M, int N, int K, const Epi& epi, int splits,
                     float* work, size_t work_floats, int* err, cudaStream_t s) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaErrorInvalidValue;
-  const int BN = tile_n(N);
+  const GemmPlan plan = plan_gemm(M, N, K, splits);
+  const int BN = plan.bn;
   CUtensorMap ma, mb;
-  if (!make_map(&ma, A, M, K, lda, BM) || !make_map(&mb, B, N, K, ldb, BN)) return cudaErrorInvalidValue;
+  if (!make_map(&ma, A, M, K, lda, BM) || !make_map(&mb, B, N, K, ldb, plan.pair ? BN / 2 : BN))
+    return cudaErrorInvalidValue;
   static std::once_flag attr;
   std::call_once(attr, [] {
     cudaFuncSetAttribute(k_gemm_tn_p<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, Tile<128>::SMEM_BYTES);
     cudaFuncSetAttribute(k_gemm_tn_p<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, Tile<256>::SMEM_BYTES);
+    cudaFuncSetAttribute(k_gemm_tn_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, P_SMEM_BYTES);
   });
+  Epi ep = epi;
+  ep.vec = ((uintptr_t)epi.out_f & 15) == 0 && ((uintptr_t)epi.out_b & 7) == 0 && ((uintptr_t)epi.mask & 7) == 0 &&
+           ((uintptr_t)work & 15) == 0;
   const int KT = (K + BK - 1) / BK;
-  int sp = plan_splits(M, N, K, splits);
+  int sp = plan.splits;
   if (sp > 1 && (!work || work_floats < (size_t)sp * M * N)) sp = 1;
   const int ktps = (KT + sp - 1) / sp;
-  const long long units = (long long)((N + BN - 1) / BN) * ((M + BM - 1) / BM) * sp;
-  const int grid = (int)std::min<long long>(units, num_sms());
-  if (BN == 256)
-    k_gemm_tn_p<256><<<grid, 192, Tile<256>::SMEM_BYTES, s>>>(ma, mb, M, N, K, ktps, sp, epi, work, err);
+  const int bm = plan.pair ? 2 * BM : BM;
+  const long long units = (long long)((N + BN - 1) / BN) * ((M + bm - 1) / bm) * sp;
+  if (plan.pair)
+    k_gemm_tn_pair<<<2 * (int)std::min<long long>(units, num_sms() / 2), GEMM_NT, P_SMEM_BYTES, s>>>(
+        ma, mb, M, N, K, BN, ktps, sp, ep, work, err);
+  else if (BN == 256)
+    k_gemm_tn_p<256><<<(int)std::min<long long>(units, num_sms()), GEMM_NT, Tile<256>::SMEM_BYTES, s>>>(
+        ma, mb, M, N, K, ktps, sp, ep, work, err);
   else
-    k_gemm_tn_p<128><<<grid, 192, Tile<128>::SMEM_BYTES, s>>>(ma, mb, M, N, K, ktps, sp, epi, work, err);
+    k_gemm_tn_p<128><<<(int)std::min<long long>(units, num_sms()), GEMM_NT, Tile<128>::SMEM_BYTES, s>>>(
+        ma, mb, M, N, K, ktps, sp, ep, work, err);
   if (sp > 1) {
-    const long long MN = (long long)M * N;
-    const int blocks = (int)std::min<long long>((MN + 255) / 256, 8LL * num_sms());
-    k_splitk_epi<<<blocks, 256, 0, s>>>(work, sp, M, N, epi);
+    const int rows = std::min(M, 32768);
+    if ((N & 3) == 0 && ((uintptr_t)work & 15) == 0)
+      k_splitk_epi<4><<<dim3((N / 4 + 127) / 128, rows), 128, 0, s>>>(work, sp, M, N, epi);
+    else
+      k_splitk_epi<1><<<dim3((N + 127) / 128, rows), 128, 0, s>>>(work, sp, M, N, epi);
   }
   return cudaGetLastError();
 }
 
 inline int grid_for(long long total, int threads = 256) {
   return (int)std::max<long long>(1, std::min<long long>((total + threads - 1) / threads, 16LL * num_sms()));
+}
+// two columns per thread: pairs do not straddle [n | m] and every row of both
+// arrays starts on 16 bytes
+inline bool two_columns(int n, int m, const void* p, const void* q) {
+  return n % 2 == 0 && m % 2 == 0 && ((uintptr_t)p & 15) == 0 && ((uintptr_t)q & 15) == 0;
 }
 inline int r8(long long v) { return (int)((v + 7) / 8 * 8); }
 
@@ -926,7 +1457,7 @@ void backward(pdqp_ws_s* w, int rows, const float* T, long long a, long long sft
     const float scale = (float)(2.0 / ((double)rows * F));
     k_grad_tiles<0><<<grid, blk, 0, s>>>(w->O, Fp, T, Fp, a, sft, count, row0, rows, F, scale, w->dOb, Fp, w->dOt,
                                          mb, w->colpart, w->ldc, w->lossp);
-    k_loss_acc<<<1, 256, 0, s>>>(w->lossp, (int)(grid.x * grid.y), 1.0 / ((double)rows * F), w->lossacc);
+    k_loss_acc<<<1, 1024, 0, s>>>(w->lossp, (int)(grid.x * grid.y), 1.0 / ((double)rows * F), w->lossacc);
   }
   WsLayer& o = w->L[w->depth];
   k_colsum<<<(F + 255) / 256, 256, 0, s>>>(w->colpart, rt, F, w->ldc, o.gb);
@@ -969,8 +1500,8 @@ void adam(pdqp_ws_s* w, float lr, float b1, float b2, float eps, cudaStream_t s)
   a.c2 = (float)(1.0 / (1.0 - std::pow((double)b2, (double)w->step)));
   a.update = 1;
   for (WsLayer& l : w->L) {
-    dim3 grid((l.in + 31) / 32, (l.out + 31) / 32), blk(32, 8);
-    k_adam_mat<<<grid, blk, 0, s>>>(l.W, l.mW, l.vW, l.gW, l.out, l.in, a, l.Wb, l.in, l.Wt, l.ldt);
+    dim3 grid((l.in + ADAM_T - 1) / ADAM_T, (l.out + ADAM_T - 1) / ADAM_T);
+    k_adam_mat<<<grid, 256, 0, s>>>(l.W, l.mW, l.vW, l.gW, l.out, l.in, a, l.Wb, l.in, l.Wt, l.ldt);
     k_adam_vec<<<(l.out + 255) / 256, 256, 0, s>>>(l.b, l.mb, l.vb, l.gb, l.out, a);
   }
 }
@@ -978,13 +1509,20 @@ void adam(pdqp_ws_s* w, float lr, float b1, float b2, float eps, cudaStream_t s)
 void refresh_copies(WsLayer& l, cudaStream_t s) {
   AdamArgs a{};
   a.update = 0;
-  dim3 grid((l.in + 31) / 32, (l.out + 31) / 32), blk(32, 8);
-  k_adam_mat<<<grid, blk, 0, s>>>(l.W, l.mW, l.vW, l.gW, l.out, l.in, a, l.Wb, l.in, l.Wt, l.ldt);
+  dim3 grid((l.in + ADAM_T - 1) / ADAM_T, (l.out + ADAM_T - 1) / ADAM_T);
+  k_adam_mat<<<grid, 256, 0, s>>>(l.W, l.mW, l.vW, l.gW, l.out, l.in, a, l.Wb, l.in, l.Wt, l.ldt);
+}
+
+// the elementwise kernels' grid over `rows` rows of arrays p, q
+dim3 row_grid(const pdqp_ws_s* w, const void* p, const void* q, long long rows) {
+  const int per = two_columns(w->n, w->m, p, q) ? 512 : 256;
+  return dim3((w->F + per - 1) / per, (unsigned)std::min<long long>((rows + ROWS_PER - 1) / ROWS_PER, 32768));
 }
 
 // normalised inputs of rows [row0, row0+rows) -> U -> H0 = U P'
 void project(pdqp_ws_s* w, const double* C, const double* B, long long row0, int rows, bf16* H0, cudaStream_t s) {
-  k_prep_input<<<grid_for((long long)rows * w->F), 256, 0, s>>>(C, B, w->n, w->m, row0, rows, w->in_mean,
+  auto prep = two_columns(w->n, w->m, C, B) ? k_prep_input<2> : k_prep_input<1>;
+  prep<<<row_grid(w, C, B, rows), 256, 0, s>>>(C, B, w->n, w->m, row0, rows, w->in_mean,
                                                                 w->in_scale, w->U, w->Fp);
   gemm(w, w->U, w->Fp, w->P, w->Fp, rows, w->d, w->F, epi_of(nullptr, H0, w->d, nullptr, 0), s);
 }
@@ -1243,20 +1781,38 @@ pdqp_status pdqp_ws_fit(pdqp_ws_handle w, const double* C, const double* B, cons
     if (count < 1) throw WsFail{PDQP_ERR_INVALID, "count >= 1"};
     need_data(w, C, B, X, Y, mem, true);
     const int n = w->n, m = w->m;
+    // partials of two arrays at a time: mean and M2 per range of FIT_ROWS rows
+    const long long nb = (count + FIT_ROWS - 1) / FIT_ROWS;
+    const size_t need = 4 * (size_t)nb * (size_t)std::max(n, m) * (sizeof(double) / sizeof(float));
+    if (need > w->work_floats) {
+      WCK(cudaStreamSynchronize(s));
+      wfree(w, w->work);
+      w->work = nullptr;
+      w->work_floats = 0;
+      w->work = walloc<float>(w, need);
+      w->work_floats = need;
+    }
+    // the statistics of the inputs `in` and of the targets `out`, nf columns each, from feature f0
+    auto stats = [&](const double* in, const double* out, int nf, int f0) {
+      double* part = reinterpret_cast<double*>(w->work);
+      const size_t len = (size_t)nb * nf;
+      const FitPair p{{in, out}, {part, part + 2 * len}, {part + len, part + 3 * len}};
+      const FitOut o{{w->in_mean + f0, w->out_mean + f0}, {w->in_scale + f0, w->out_inv + f0}, {nullptr, w->out_std + f0}};
+      k_fit_part<<<dim3((nf + 255) / 256, (unsigned)std::min<long long>(nb, 32768), 2), 256, 0, s>>>(p, count, nf);
+      k_fit_merge<<<dim3((nf + 127) / 128, 1, 2), 128, 0, s>>>(p, count, nf, o);
+      WCK(cudaGetLastError());
+    };
     {
       DevView<double> c(C, (size_t)count * n, mem, s), x(X, (size_t)count * n, mem, s);
-      k_fit_stats<<<(n + 127) / 128, 128, 0, s>>>(c.p, count, n, w->in_mean, w->in_scale, nullptr);
-      k_fit_stats<<<(n + 127) / 128, 128, 0, s>>>(x.p, count, n, w->out_mean, w->out_inv, w->out_std);
-      WCK(cudaGetLastError());
-      WCK(cudaStreamSynchronize(s));
+      stats(c.p, x.p, n, 0);
+      if (mem != PDQP_MEM_DEVICE) WCK(cudaStreamSynchronize(s));
     }
     if (m > 0) {
       DevView<double> b(B, (size_t)count * m, mem, s), y(Y, (size_t)count * m, mem, s);
-      k_fit_stats<<<(m + 127) / 128, 128, 0, s>>>(b.p, count, m, w->in_mean + n, w->in_scale + n, nullptr);
-      k_fit_stats<<<(m + 127) / 128, 128, 0, s>>>(y.p, count, m, w->out_mean + n, w->out_inv + n, w->out_std + n);
-      WCK(cudaGetLastError());
-      WCK(cudaStreamSynchronize(s));
+      stats(b.p, y.p, m, n);
+      if (mem != PDQP_MEM_DEVICE) WCK(cudaStreamSynchronize(s));
     }
+    WCK(cudaStreamSynchronize(s));
     w->have_norm = true;
   });
 }
@@ -1274,7 +1830,8 @@ pdqp_status pdqp_ws_grad(pdqp_ws_handle w, const double* C, const double* B, con
         x(X, (size_t)count * n, mem, s), y(Y, (size_t)count * m, mem, s);
     float* T = walloc<float>(w, (size_t)count * w->Fp);
     try {
-      k_prep_target<<<grid_for(count * w->F), 256, 0, s>>>(x.p, y.p, n, m, count, w->out_mean, w->out_inv, T, w->Fp);
+      (two_columns(n, m, x.p, y.p) ? k_prep_target<2> : k_prep_target<1>)<<<row_grid(w, x.p, y.p, count), 256, 0, s>>>(
+          x.p, y.p, n, m, count, w->out_mean, w->out_inv, T, w->Fp);
       project(w, c.p, b.p, 0, (int)count, w->H[0], s);
       forward(w, (int)count, s);
       WCK(cudaMemsetAsync(w->lossacc, 0, sizeof(double), s));
@@ -1328,7 +1885,8 @@ pdqp_status pdqp_ws_train(pdqp_ws_handle w, const pdqp_ws_train_options* opt, co
     }
     {
       DevView<double> x(X, (size_t)count * n, mem, s), y(Y, (size_t)count * m, mem, s);
-      k_prep_target<<<grid_for(count * F), 256, 0, s>>>(x.p, y.p, n, m, count, w->out_mean, w->out_inv, w->Tall, Fp);
+      (two_columns(n, m, x.p, y.p) ? k_prep_target<2> : k_prep_target<1>)<<<row_grid(w, x.p, y.p, count), 256, 0, s>>>(
+          x.p, y.p, n, m, count, w->out_mean, w->out_inv, w->Tall, Fp);
       finish(w, s);
     }
     const long long steps = count / batch;
@@ -1376,7 +1934,7 @@ pdqp_status pdqp_ws_infer(pdqp_ws_handle w, const double* C, const double* B, in
         const int rows = (int)std::min<long long>(w->maxb, count - r0);
         project(w, c.p, b.p, r0, rows, w->H[0], s);
         forward(w, rows, s);
-        k_write_pred<<<grid_for((long long)rows * w->F), 256, 0, s>>>(w->O, w->Fp, rows, n, m, w->out_mean,
+        (two_columns(n, m, x0, y0) ? k_write_pred<2> : k_write_pred<1>)<<<row_grid(w, x0, y0, rows), 256, 0, s>>>(w->O, w->Fp, rows, n, m, w->out_mean,
                                                                       w->out_std, r0, x0, y0);
       }
       finish(w, s);
