@@ -8,7 +8,7 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libpdqp.so")
-SOURCES = ["kernels.cu", "iteration.cu", "chunk.cu", "products.cu", "capi.cu", "mlp.cu"]
+SOURCES = ["kernels.cu", "iteration.cu", "chunk.cu", "lowrank.cu", "products.cu", "capi.cu", "mlp.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O2", "--expt-relaxed-constexpr",
          "-I" + os.path.join(ROOT, "include"), "-I" + CSRC]

@@ -255,6 +255,7 @@ void build_long_segments(pdqp_problem* h, DCsr& M, const std::vector<int32_t>& r
   to_device(M.blk_seg, bseg.data(), bseg.size(), s);
   M.lpart_d = dalloc<double>(h, seg.size());
   M.lpart_f = dalloc<float>(h, seg.size());
+  M.kpart = dalloc<double>(h, 4 * seg.size());
   CK(cudaStreamSynchronize(s));   // the host vectors die here
 }
 
@@ -468,7 +469,8 @@ void fill_info(pdqp_info* info, const DevState& S, pdqp_status status, bool lanc
 // launch only those blocks (direct launches sized by the last check's counts)
 // instead of replaying the full-grid chunk graph.
 bool compact_now(const Work& w, const SolveParams& p) {
-  if (w.count <= 1 || p.spmv_threads == 1 || p.spmv_threads == 2 || p.spmv_threads == 3) return false;
+  if (w.count <= 1 || p.spmv_threads == 1 || p.spmv_threads == 2 || p.spmv_threads == 3 || p.spmv_threads == 4)
+    return false;
   return 2LL * w.bst_host->act_P < (long long)w.P.nblk;
 }
 
@@ -684,7 +686,9 @@ pdqp_status solve_impl(pdqp_problem* h, const pdqp_options& o, const double* x0,
   }
   // the iteration-kernel variant, where nothing above fixes it: the one this
   // shape was tuned to, or timed on the first chunk (below)
-  const bool autotune = o.spmv_threads == 0 && !use_il && !mp && !use_chunk;
+  const bool use_lr = o.spmv_threads == 0 && !use_il && !mp && pdqp::lowrank_fused_ok(w, mixed);
+  if (use_lr) p.spmv_threads = 4;
+  const bool autotune = o.spmv_threads == 0 && !use_il && !mp && !use_chunk && !use_lr;
   int& tuned = h->tuned_nt[mixed ? 1 : 0];
   if (autotune && !tuned) tuned = tuned_lookup(w, mixed);
   w.mp = mp ? 1 : 0;
@@ -1482,6 +1486,7 @@ pdqp_problem* build_family(const InstanceIn& base, int count, const double* C, c
       to_device(Mr.blk_seg, bseg.data(), bseg.size(), s);
       Mr.lpart_d = dalloc<double>(h, seg.size());
       Mr.lpart_f = dalloc<float>(h, seg.size());
+      Mr.kpart = dalloc<double>(h, 4 * seg.size());
       CK(cudaStreamSynchronize(s));
     }
     w.inst = dalloc<Inst>(h, count);
@@ -2310,6 +2315,7 @@ pdqp_status pdqp_set_lowrank_Q(pdqp_handle h, int32_t r, const float* F, int32_t
     w.wlr = dalloc<double>(h, 2 * (size_t)r);
     w.wlr_f = dalloc<float>(h, 2 * (size_t)r);
     w.lr_part = dalloc<double>(h, (size_t)((w.n + LR_ROWS - 1) / LR_ROWS) * 2 * r);
+    w.lr_rows = dalloc<double>(h, 2 * (size_t)w.n);
     to_device(w.F, hf.data(), N, s);
     to_device(w.Fo, hd.data(), N, s);
     CK(cudaStreamSynchronize(s));

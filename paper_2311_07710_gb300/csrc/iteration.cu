@@ -474,6 +474,21 @@ static void run_chunk_pipe(Work& w, int j0, int len, BCsr<V> A, BCsr<V> P, V* xt
   }
 }
 
+// The dual half-step of iteration j alone (its long rows' segments summed by
+// the kernel before it).
+template <typename V>
+void run_dual(Work& w, int j, BCsr<V> A, V* xt, V* const* Z, V* ybar, const V* b, const V* ylo, cudaStream_t s) {
+  DualB<V> da{A, xt, nullptr, nullptr, ybar, b, ylo, w.tab, w.blk_inst_A, w.st, w.row_ineq, w.tab_stride};
+  da.yold = Z[(j + 1) & 1] + w.n;
+  da.ynew = Z[j & 1] + w.n;
+  if (w.A.nlseg) { da.blk_seg = w.A.blk_seg; da.lpart = sizeof(V) == 4 ? (V*)w.A.lpart_f : (V*)w.A.lpart_d; }
+  launch(k_dual<V, 256>, w.A.nblk, 256, 0, s, da, j);
+}
+template void run_dual<float>(Work&, int, BCsr<float>, float*, float* const*, float*, const float*, const float*,
+                              cudaStream_t);
+template void run_dual<double>(Work&, int, BCsr<double>, double*, double* const*, double*, const double*,
+                               const double*, cudaStream_t);
+
 template <typename V, int NT>
 static void run_chunk(Work& w, int j0, int len, BCsr<V> A, BCsr<V> P, V* xt, V* const* Z, V* ybar, const V* b,
                       const V* ylo, V* x, V* xbar, const V* c, const V* l, const V* u, cudaStream_t s,
@@ -789,6 +804,10 @@ void iterate_chunk(Work& w, int len, bool mixed, int nt, cudaStream_t s, int j0,
   }
   if (nt == 2) {   // the whole chunk in one launch (small instances)
     chunk_run(w, len, mixed, s, j0);
+    return;
+  }
+  if (nt == 4) {   // a low-rank term over short rows
+    lowrank_run(w, len, mixed, s, j0);
     return;
   }
   if (nt == 1) {   // pipelined persistent kernels, 256 threads

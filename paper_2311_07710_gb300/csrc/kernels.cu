@@ -113,24 +113,10 @@ __global__ void k_lr_ft(const FV* __restrict__ F, int n, int r, const X* __restr
   }
 }
 
-// w[vec][k] = sum of the block partials: one CUDA block (256 threads) per
-// (vec, k), a fixed-order tree; a float32 copy for the float32 iteration
+// w[vec][k] = sum of the block partials: one CUDA block per (vec, k)
 __global__ void __launch_bounds__(256) k_lr_reduce(const double* __restrict__ part, int nparts, int r, int nv,
                                                    double* __restrict__ w, float* __restrict__ wf) {
-  const int q = blockIdx.x / r, kk = blockIdx.x % r;
-  __shared__ double sh[256];
-  double s = 0.0;
-  for (int b = threadIdx.x; b < nparts; b += 256) s += part[((size_t)b * nv + q) * r + kk];
-  sh[threadIdx.x] = s;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    w[q * r + kk] = sh[0];
-    if (wf) wf[q * r + kk] = (float)sh[0];
-  }
+  lr_reduce_column(part, nparts, r, nv, blockIdx.x, w, wf);
 }
 
 // --------------------------------------------------------------------------
@@ -161,9 +147,9 @@ struct KktB {
   const int *grp_inst_A, *grp_first_A;  // relKKT groups (KKT_GROUP row blocks of one instance)
   const int *grp_inst_P, *grp_first_P;
   const DevState* st;                   // null: no status test
-  const double* F;                      // low-rank factor F~ (null: none)
-  const double* wlr;                    // [2][r]: F~' x per iterate
-  int r;
+  const double* lr;                     // low-rank row terms (F~ F~' x)_j per iterate [2][n] (null: none)
+  const int2 *segA, *segP;              // long rows: {first segment, segments} per row block (null: none)
+  const double *longA, *longP;          // their segment sums [2] and [2][Q, A'] per segment (k_kkt_long)
 };
 
 // The row blocks [b0, b1) of relKKT group g and its instance: groups are
@@ -272,7 +258,7 @@ template <int IT, bool LR>
 __device__ __forceinline__ void kkt_n_row(const KktB& a, double (&f)[15], int r, double sq, double sa) {
   const double cj = a.c[r], lj = a.l[r], uj = a.u[r];
   double sqt = sq;
-  if constexpr (LR) sqt = r_add(sqt, lr_row<double, double, double>(a.F, a.wlr + IT * a.r, a.r, r));
+  if constexpr (LR) sqt = r_add(sqt, a.lr[(size_t)IT * a.n + r]);
   if (a.prodQx[IT]) { a.prodQx[IT][r] = sqt; a.prodATy[IT][r] = -sa; }
   const double Qx = a.iD2 ? r_mul(sqt, a.iD2[r]) : sqt, ATy = a.iD2 ? r_mul(-sa, a.iD2[r]) : -sa;
   const double xt = a.x[IT][r];
@@ -329,17 +315,16 @@ __global__ void __launch_bounds__(BNT) k_kkt_m(KktB a) {
         else kkt_m_row<NIT - 1>(a, f, r0 + t, s);
       }
     } else {
+      // a long row: its segments' sums (k_kkt_long), in order
       double s[NIT];
 #pragma unroll
       for (int it = 0; it < NIT; ++it) s[it] = 0.0;
-      for (int e = e0 + tid; e < e0 + ne; e += BNT) {
-        const double v = a.A.val[e];
-        const int c = a.A.col[e];
+      if (tid == 0) {
+        const int2 sg = a.segA[bk];
+        for (int q = 0; q < sg.y; ++q)
 #pragma unroll
-        for (int it = 0; it < NIT; ++it) s[it] = fma(v, __ldg(a.x[it] + c), s[it]);
+          for (int it = 0; it < NIT; ++it) s[it] += a.longA[2 * (size_t)(sg.x + q) + it];
       }
-#pragma unroll
-      for (int it = 0; it < NIT; ++it) s[it] = block_sum(s[it]);
       if (tid == 0) {
         kkt_m_row<0>(a, f, r0, s[0]);
         if (NIT > 1) kkt_m_row<NIT - 1>(a, f, r0, s[NIT - 1]);
@@ -351,10 +336,11 @@ __global__ void __launch_bounds__(BNT) k_kkt_m(KktB a) {
     for (int k = 0; k < 9; ++k) a.part_m[(size_t)k * a.ngrp_m + blockIdx.x] = f[k];
 }
 
-// 80 registers (3 blocks per SM): capped at 64 for 4 blocks it spills and is
-// slower (n=1e6 checks 4.67 -> 5.15 ms per solve)
+// 3 blocks per SM (80 registers): capped at 64 for 4 blocks it spills and is
+// slower (n=1e6 checks 4.67 -> 5.15 ms per solve), left alone it takes 100 and
+// runs 2 (a batch's checks 23.5 -> 29.4 ms)
 template <int NIT, bool LR>
-__global__ void __launch_bounds__(BNT) k_kkt_n(KktB a) {
+__global__ void __launch_bounds__(BNT, 3) k_kkt_n(KktB a) {
   extern __shared__ __align__(16) double kkt_sm[];
   double* sval = kkt_sm;
   double* sx = kkt_sm + BNNZ;
@@ -393,21 +379,18 @@ __global__ void __launch_bounds__(BNT) k_kkt_n(KktB a) {
         else kkt_n_row<NIT - 1, LR>(a, f, r0 + t, sq, sa);
       }
     } else {
-      const int sp = a.P.split[r0];
       double sq[NIT], sa[NIT];
 #pragma unroll
       for (int it = 0; it < NIT; ++it) { sq[it] = 0.0; sa[it] = 0.0; }
-      for (int e = e0 + tid; e < e0 + ne; e += BNT) {
-        const double v = a.P.val[e];
-        const int c = a.P.col[e];
+      if (tid == 0) {
+        const int2 sg = a.segP[bk];
+        for (int q = 0; q < sg.y; ++q)
 #pragma unroll
-        for (int it = 0; it < NIT; ++it) {
-          if (e < sp) sq[it] = fma(v, __ldg(a.x[it] + c), sq[it]);
-          else sa[it] = fma(v, __ldg(a.y[it] + (c - n)), sa[it]);
-        }
+          for (int it = 0; it < NIT; ++it) {
+            sq[it] += a.longP[4 * (size_t)(sg.x + q) + 2 * it];
+            sa[it] += a.longP[4 * (size_t)(sg.x + q) + 2 * it + 1];
+          }
       }
-#pragma unroll
-      for (int it = 0; it < NIT; ++it) { sq[it] = block_sum(sq[it]); sa[it] = block_sum(sa[it]); }
       if (tid == 0) {
         kkt_n_row<0, LR>(a, f, r0, sq[0], sa[0]);
         if (NIT > 1) kkt_n_row<NIT - 1, LR>(a, f, r0, sq[NIT - 1], sa[NIT - 1]);
@@ -419,9 +402,59 @@ __global__ void __launch_bounds__(BNT) k_kkt_n(KktB a) {
     for (int k = 0; k < 15; ++k) a.part_n[(size_t)k * a.ngrp_n + blockIdx.x] = f[k];
 }
 
+// Segment sums of the long rows for the relKKT kernels: one CUDA block per
+// segment of LSEG nonzeros of A (then of P, its Q and A' parts apart).  One
+// CUDA block walking a whole row bound the check of a problem with dense rows
+// (two rows of 1e5 nonzeros in one group: k_kkt_m 343 us).
+template <int NIT>
+__global__ void __launch_bounds__(256) k_kkt_long(KktB a, const int4* __restrict__ sA, int nA,
+                                                  const int* __restrict__ instA, const int4* __restrict__ sP,
+                                                  const int* __restrict__ instP, double* __restrict__ outA,
+                                                  double* __restrict__ outP) {
+  const bool isA = (int)blockIdx.x < nA;
+  const int q = isA ? blockIdx.x : blockIdx.x - nA;
+  const int4 g = isA ? sA[q] : sP[q];
+  if (a.st && a.st[isA ? instA[g.w] : instP[g.w]].status != ST_RUNNING) return;
+  const BCsr<double>& M = isA ? a.A : a.P;
+  const int sp = isA ? g.z : a.P.split[g.x];
+  double s[NIT], t[NIT];
+#pragma unroll
+  for (int it = 0; it < NIT; ++it) { s[it] = 0.0; t[it] = 0.0; }
+  for (int e = g.y + threadIdx.x; e < g.z; e += 256) {
+    const double v = M.val[e];
+    const int c = M.col[e];
+#pragma unroll
+    for (int it = 0; it < NIT; ++it) {
+      if (e < sp) s[it] = fma(v, __ldg(a.x[it] + c), s[it]);
+      else t[it] = fma(v, __ldg(a.y[it] + (c - a.n)), t[it]);
+    }
+  }
+#pragma unroll
+  for (int it = 0; it < NIT; ++it) {
+    s[it] = block_sum(s[it]);
+    if (!isA) t[it] = block_sum(t[it]);
+  }
+  if (threadIdx.x == 0)
+#pragma unroll
+    for (int it = 0; it < NIT; ++it) {
+      if (isA) {
+        outA[2 * (size_t)q + it] = s[it];
+      } else {
+        outP[4 * (size_t)q + 2 * it] = s[it];
+        outP[4 * (size_t)q + 2 * it + 1] = t[it];
+      }
+    }
+}
+
 // launch both relKKT kernels with their dynamic shared memory
 template <int NIT>
-static void launch_kkt(const Work& w, const KktB& a, cudaStream_t s) {
+static void launch_kkt(const Work& w, const KktB& a0, cudaStream_t s) {
+  KktB a = a0;
+  a.segA = w.A.blk_seg; a.segP = w.P.blk_seg;
+  a.longA = w.A.kpart; a.longP = w.P.kpart;
+  if (w.A.nlseg + w.P.nlseg > 0)
+    launch(k_kkt_long<NIT>, w.A.nlseg + w.P.nlseg, 256, 0, s, a, (const int4*)w.A.lseg, w.A.nlseg,
+           (const int*)w.blk_inst_A, (const int4*)w.P.lseg, (const int*)w.blk_inst_P, w.A.kpart, w.P.kpart);
   static std::once_flag attr;
   std::call_once(attr, [] {
     cudaFuncSetAttribute(k_kkt_m<NIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kkt_smem_bytes<NIT>());
@@ -429,7 +462,7 @@ static void launch_kkt(const Work& w, const KktB& a, cudaStream_t s) {
     cudaFuncSetAttribute(k_kkt_n<NIT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kkt_smem_bytes<NIT>());
   });
   if (w.m > 0) launch(k_kkt_m<NIT>, w.ngrp_A, BNT, kkt_smem_bytes<NIT>(), s, a);
-  if (a.F) launch(k_kkt_n<NIT, true>, w.ngrp_P, BNT, kkt_smem_bytes<NIT>(), s, a);
+  if (a.lr) launch(k_kkt_n<NIT, true>, w.ngrp_P, BNT, kkt_smem_bytes<NIT>(), s, a);
   else launch(k_kkt_n<NIT, false>, w.ngrp_P, BNT, kkt_smem_bytes<NIT>(), s, a);
 }
 
@@ -1890,13 +1923,25 @@ void scale_apply(Work& w, bool mixed, cudaStream_t s, const Work* tmpl) {
          (float*)nullptr);
 }
 
+// the tiles' partials of F' v (nv = 1) or F' [v0, v1] (nv = 2)
+template <typename FV, typename X>
+static void lowrank_parts(Work& w, const FV* F, const X* v0, const X* v1, cudaStream_t s) {
+  const int grid = lr_ft_grid(w);
+  if (v1) launch(k_lr_ft<FV, X, 2>, grid, 256, 0, s, F, w.n, w.r, v0, v1, w.lr_part);
+  else launch(k_lr_ft<FV, X, 1>, grid, 256, 0, s, F, w.n, w.r, v0, v1, w.lr_part);
+}
+void lowrank_ft_part(Work& w, const float* F, const float* v, cudaStream_t s) {
+  lowrank_parts<float, float>(w, F, v, nullptr, s);
+}
+void lowrank_ft_part(Work& w, const double* F, const double* v, cudaStream_t s) {
+  lowrank_parts<double, double>(w, F, v, nullptr, s);
+}
+
 // w = F' v (nv = 1) or F' [v0, v1] (nv = 2) into w.wlr
 template <typename FV, typename X>
 static void lowrank_ft(Work& w, const FV* F, const X* v0, const X* v1, cudaStream_t s) {
-  const int grid = std::min(cdiv(w.n, LR_ROWS), 4 * w.num_sms);
-  if (v1) launch(k_lr_ft<FV, X, 2>, grid, 256, 0, s, F, w.n, w.r, v0, v1, w.lr_part);
-  else launch(k_lr_ft<FV, X, 1>, grid, 256, 0, s, F, w.n, w.r, v0, v1, w.lr_part);
-  launch(k_lr_reduce, w.r * (v1 ? 2 : 1), 256, 0, s, (const double*)w.lr_part, grid, w.r, v1 ? 2 : 1, w.wlr,
+  lowrank_parts<FV, X>(w, F, v0, v1, s);
+  launch(k_lr_reduce, w.r * (v1 ? 2 : 1), 256, 0, s, (const double*)w.lr_part, lr_ft_grid(w), w.r, v1 ? 2 : 1, w.wlr,
          w.wlr_f);
 }
 
@@ -2221,7 +2266,8 @@ static void infeas_check(Work& w, const KktB& main, cudaStream_t s) {
       a.b = w.inf_zm; a.l = w.inf_lrec; a.u = w.inf_urec;
       if (w.r > 0) {
         lowrank_ft<double, double>(w, w.Fd, a.x[0], a.x[1], s);
-        a.F = w.Fd; a.wlr = w.wlr; a.r = w.r;
+        lowrank_rows(w, w.Fd, 2, s);
+    a.lr = w.lr_rows;
       }
     } else {           // dual rays: x = 0, c = 0
       a.x[0] = w.inf_zn; a.x[1] = w.inf_zn;
@@ -2283,7 +2329,8 @@ void check(Work& w, const SolveParams& p, int mode, long long chunk_len, bool mi
   }
   if (w.r > 0) {
     lowrank_ft<double, double>(w, w.Fd, a.x[0], a.x[1], s);
-    a.F = w.Fd; a.wlr = w.wlr; a.r = w.r;
+    lowrank_rows(w, w.Fd, 2, s);
+    a.lr = w.lr_rows;
   }
   if (w.il_active) {
     launch_kkt_il(w, a, s);   // a family handle on interleaved vectors (no low-rank term)
@@ -2360,7 +2407,8 @@ void eval_kkt_user(Work& w, const double* x, const double* y, cudaStream_t s) {
   a.st = nullptr;
   if (w.r > 0) {
     lowrank_ft<double, double>(w, w.Fo, x, (const double*)nullptr, s);
-    a.F = w.Fo; a.wlr = w.wlr; a.r = w.r;
+    lowrank_rows(w, w.Fo, 1, s);
+    a.lr = w.lr_rows;
   }
   launch_kkt<1>(w, a, s);
   launch(k_kkt_finish_user, 1, 1024, 0, s, (const double*)w.part_m, w.m > 0 ? w.ngrp_A : 0,

@@ -54,6 +54,7 @@ struct DCsr {
   int2* blk_seg = nullptr;    // [nblk] {first segment, segments} of a long-row block
   double* lpart_d = nullptr;  // [nlseg] segment sums, float64
   float* lpart_f = nullptr;   // [nlseg] segment sums, float32
+  double* kpart = nullptr;    // [nlseg][4] the relKKT check's segment sums (A uses 2)
   // 1 when every instance's gathered vector is small (a few L1s): the row
   // blocks' gathers hit nearby and their index and value streams set the pace,
   // so the staging prefetches those to L2 (a batch of control QPs: 8111 -> 8374
@@ -175,6 +176,7 @@ struct Work {
   double* wlr = nullptr;     // [2][r] F~' v of the current products
   float* wlr_f = nullptr;    // [2][r] the same in float32 (float32 iteration)
   double* lr_part = nullptr; // [tiles][2][r] partial sums
+  double* lr_rows = nullptr; // [2][n] the check's row terms F~ (F~' v)
   // Lanczos vectors: pu[p] (n) for A~'A~, pz[p] = [v_Q ; A~v_A] (n+m) the P input
   double *pu[2] = {nullptr, nullptr}, *pz[2] = {nullptr, nullptr};
   float *fpu[2] = {nullptr, nullptr}, *fpz[2] = {nullptr, nullptr};
@@ -276,7 +278,8 @@ void init_iterates(Work& w, const double* x0, const double* y0, const SolveParam
 // compact: launch only the row blocks of the running instances (batches; the
 // counts of the last check must be in bst_host).
 // nt: 256 or 512 threads per row block, 1 the pipelined persistent kernels, 2
-// the whole chunk in one launch (only where chunk_ok, plan and values built), 3 the
+// the whole chunk in one launch (only where chunk_ok, plan and values built), 4
+// the low-rank kernels (only where lowrank_fused_ok), 3 the
 // member-interleaved family kernels (only where w.fam_il, buffers allocated).
 void iterate_chunk(Work& w, int len, bool mixed, int nt, cudaStream_t s, int j0 = 0, bool compact = false);
 // iterate_chunk, or with w.mp the maintained-products kernels (float64, 256
@@ -303,6 +306,11 @@ void chunk_plan_classes(Work& w, bool mixed);             // w.chunk.ctas, cls o
 void chunk_fill_index(Work& w, cudaStream_t s);
 void chunk_fill_values(Work& w, bool mixed, cudaStream_t s);
 void chunk_run(Work& w, int len, bool mixed, cudaStream_t s, int j0);
+// a low-rank term over short rows of P: the fused half-step (lowrank.cu)
+bool lowrank_fused_ok(const Work& w, bool mixed);
+void lowrank_run(Work& w, int len, bool mixed, cudaStream_t s, int j0);
+template <typename V>
+void run_dual(Work& w, int j, BCsr<V> A, V* xt, V* const* Z, V* ybar, const V* b, const V* ylo, cudaStream_t s);
 void check(Work& w, const SolveParams& p, int mode, long long chunk_len, bool mixed, cudaStream_t s);
 
 // infeasibility certificates: fill the recession-cone bounds once the
