@@ -348,15 +348,25 @@ void alloc_mixed(pdqp_problem* h) {
   h->mixed_ready = true;
 }
 
+void drop_graphs(pdqp_problem* h);
+
 // The member-interleaved vectors of a family handle for one precision (on
 // the first solve that uses them).
-void alloc_il(pdqp_problem* h, bool mixed) {
+void alloc_il(pdqp_problem* h, bool mixed, int period) {
   Work& w = h->w;
   const size_t ld = (size_t)w.fam_ld, n = (size_t)w.fam_n, m = (size_t)w.fam_m;
   const size_t len[IL_SLOTS] = {n + m, n + m, n, n, n, m, n, n, n, m, m};
   for (int k = 0; k < IL_SLOTS; ++k) {
     if (mixed && !w.ilf[k]) w.ilf[k] = dalloc<float>(h, len[k] * ld);
     if (!mixed && !w.ild[k]) w.ild[k] = dalloc<double>(h, len[k] * ld);
+  }
+  if (!w.il_run) w.il_run = dalloc<int>(h, ld);
+  int& have = w.il_steps_len[mixed ? 1 : 0];
+  if (have < period) {   // a longer check period replaces the buffer the graphs point into
+    if (mixed) w.il_steps_f = dalloc<float>(h, 5 * (size_t)period * ld);
+    else w.il_steps_d = dalloc<double>(h, 5 * (size_t)period * ld);
+    if (have) drop_graphs(h);
+    have = period;
   }
   const size_t klen[ILK_SLOTS] = {n, n, m, m, m, m, n, n, n, n};
   for (int k = 0; k < ILK_SLOTS; ++k)
@@ -667,7 +677,7 @@ pdqp_status solve_impl(pdqp_problem* h, const pdqp_options& o, const double* x0,
     throw Fail{PDQP_ERR_INVALID, "options.maintained_products: a solve resumed from pdqp_set_state is not supported"};
   const bool use_il = il_ok && !mp && (o.spmv_threads == 0 || o.spmv_threads == 3);
   if (mixed) alloc_mixed(h);
-  if (use_il) alloc_il(h, mixed);
+  if (use_il) alloc_il(h, mixed, o.check_period);
   w.il_active = use_il;
   if (!use_il && !w.kkt_xx) {   // the row-block checks gather both iterates of a column at once
     w.kkt_xx = dalloc<double2>(h, std::max(w.n, 1));

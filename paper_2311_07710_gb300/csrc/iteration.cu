@@ -557,9 +557,9 @@ struct FamIL {
   const int* __restrict__ rp;          // one member's CSR (A, or P with local columns)
   const int* __restrict__ col;
   const V* __restrict__ val;           // scaled values (the same for every member)
-  int rows, ld, count, C;
-  const StepEntry* __restrict__ tab;   // [member][C]
-  const DevState* __restrict__ st;     // [member]
+  int rows, ld;
+  const V* __restrict__ steps;         // [j - j0][IL_STEPS][ld] step scalars of the chunk (k_il_steps)
+  const int* __restrict__ run;         // [ld] the member iterates
   const V* __restrict__ zin;           // gathered vector (x_tilde, or [x_md ; y+])
   // dual: yold, ynew, ybar, b, ylo (may be null), ineq;  primal: x, xbar, zout, xt, c, l, u
   const V* __restrict__ v0;
@@ -641,34 +641,58 @@ __device__ __forceinline__ void il_row_sum(const FamIL<V>& a, int r, int m0, V (
   }
 }
 
-// Per-member step entries and running flags of the block's 32 W members;
-// false when none of them runs (uniform over the block).
+// The step scalars of a chunk's iterations in member order, so that a lane
+// loads those of its members in one 16-byte access, and the members' running
+// flags.  (Each CUDA block staging its members' 64-byte table entries and
+// statuses cost 12 KB of scattered loads and a barrier before its eight rows'
+// 65 KB (A) could start.)
+enum { IL_SIGMA = 0, IL_TAU, IL_IB, IL_IBN, IL_THN, IL_STEPS };
 template <typename V>
-__device__ __forceinline__ bool il_members(const FamIL<V>& a, int j, StepEntry* es, int* run) {
-  constexpr int GM = 32 * IlVec<V>::W;
-  int any = 0;
-  for (int k = threadIdx.x; k < GM; k += blockDim.x) {
-    const int mem = blockIdx.y * GM + k;
-    const bool ok = mem < a.count && a.st[mem].status == ST_RUNNING;
-    run[k] = ok;
-    if (ok) es[k] = a.tab[(size_t)mem * a.C + j];
-    any |= ok;
+__global__ void __launch_bounds__(128) k_il_steps(const StepEntry* __restrict__ tab, int C, const DevState* __restrict__ st,
+                                                  int count, int ld, int j0, V* __restrict__ steps,
+                                                  int* __restrict__ run) {
+  const int mem = blockIdx.x * 128 + threadIdx.x, k = blockIdx.y;
+  if (mem >= ld) return;
+  const bool ok = mem < count && st[mem].status == ST_RUNNING;
+  if (k == 0) run[mem] = ok;
+  V v[IL_STEPS] = {V(0), V(0), V(0), V(0), V(0)};
+  if (ok) {
+    const StepEntry e = tab[(size_t)mem * C + j0 + k];
+    v[IL_SIGMA] = step_sigma<V>(e); v[IL_TAU] = step_tau<V>(e); v[IL_IB] = step_ib<V>(e);
+    v[IL_IBN] = step_ibn<V>(e); v[IL_THN] = step_thn<V>(e);
   }
-  return __syncthreads_or(any) != 0;
+#pragma unroll
+  for (int q = 0; q < IL_STEPS; ++q) steps[((size_t)k * IL_STEPS + q) * ld + mem] = v[q];
 }
 
 template <typename V>
-__global__ void __launch_bounds__(IL_NT, 4) k_dual_il(FamIL<V> a, int j) {
-  constexpr int W = IlVec<V>::W, GM = 32 * W;
-  __shared__ StepEntry es[GM];
-  __shared__ int run[GM];
-  if (!il_members(a, j, es, run)) return;
+__device__ __forceinline__ void il_steps(const FamIL<V>& a, int k, int q, int m0, V (&v)[IlVec<V>::W]) {
+  il_load(a.steps + ((size_t)k * IL_STEPS + q) * a.ld + m0, v);
+}
+// the running flags of this lane's members; false when no member of the warp iterates
+template <typename V>
+__device__ __forceinline__ bool il_running(const FamIL<V>& a, int m0, int (&run)[IlVec<V>::W]) {
+  int any = 0;
+#pragma unroll
+  for (int q = 0; q < IlVec<V>::W; ++q) {
+    run[q] = __ldg(a.run + m0 + q);
+    any |= run[q];
+  }
+  return __any_sync(0xffffffffu, any != 0);
+}
+
+// k: the iteration within the chunk
+template <typename V>
+__global__ void __launch_bounds__(IL_NT, 4) k_dual_il(FamIL<V> a, int k) {
+  constexpr int W = IlVec<V>::W;
   const int lane = threadIdx.x & 31;
   const int r = blockIdx.x * IL_RPB + (threadIdx.x >> 5);
   if (r >= a.rows) return;
-  const int k0 = lane * W, m0 = blockIdx.y * GM + k0;
+  const int m0 = blockIdx.y * 32 * W + lane * W;
+  int run[W];
+  if (!il_running(a, m0, run)) return;
   const size_t idx = (size_t)r * a.ld + m0;
-  V yo[W], bi[W], yb[W], lo[W], s[W], yn[W], ybn[W];
+  V yo[W], bi[W], yb[W], lo[W], s[W], sg[W], ib[W], yn[W], ybn[W];
   il_load_rw(a.v0 + idx, yo);
   il_load(a.r0 + idx, bi);
   il_load_rw(a.w1 + idx, yb);
@@ -678,9 +702,11 @@ __global__ void __launch_bounds__(IL_NT, 4) k_dual_il(FamIL<V> a, int j) {
     for (int q = 0; q < W; ++q) lo[q] = V(0);
   il_row_sum(a, r, m0, s);
   const bool ineq = a.ineq[r] != 0;
+  il_steps(a, k, IL_SIGMA, m0, sg);
+  il_steps(a, k, IL_IB, m0, ib);
 #pragma unroll
   for (int q = 0; q < W; ++q) {
-    if (run[k0 + q]) dual_update<V>(es[k0 + q], s[q], yo[q], bi[q], yb[q], lo[q], ineq, yn[q], ybn[q]);
+    if (run[q]) dual_update<V>(sg[q], ib[q], s[q], yo[q], bi[q], yb[q], lo[q], ineq, yn[q], ybn[q]);
     else { ybn[q] = yb[q]; yn[q] = a.w0[idx + q]; }    // a member that stopped keeps its values
   }
   il_store(a.w1 + idx, ybn);   // y_bar
@@ -688,28 +714,31 @@ __global__ void __launch_bounds__(IL_NT, 4) k_dual_il(FamIL<V> a, int j) {
 }
 
 template <typename V>
-__global__ void __launch_bounds__(IL_NT, 4) k_primal_il(FamIL<V> a, int j) {
-  constexpr int W = IlVec<V>::W, GM = 32 * W;
-  __shared__ StepEntry es[GM];
-  __shared__ int run[GM];
-  if (!il_members(a, j, es, run)) return;
+__global__ void __launch_bounds__(IL_NT, 4) k_primal_il(FamIL<V> a, int k) {
+  constexpr int W = IlVec<V>::W;
   const int lane = threadIdx.x & 31;
   const int r = blockIdx.x * IL_RPB + (threadIdx.x >> 5);
   if (r >= a.rows) return;
-  const int k0 = lane * W, m0 = blockIdx.y * GM + k0;
+  const int m0 = blockIdx.y * 32 * W + lane * W;
+  int run[W];
+  if (!il_running(a, m0, run)) return;
   const size_t idx = (size_t)r * a.ld + m0;
-  V xo[W], xb0[W], cr[W], lr[W], ur[W], s[W], xn[W], xb[W], zo[W], xtn[W];
+  V s[W], xo[W], xb0[W], cr[W], lr[W], ur[W], tau[W], ib[W], ibn[W], thn[W], xn[W], xb[W], zo[W], xtn[W];
   il_load_rw(a.w0 + idx, xo);
   il_load_rw(a.w1 + idx, xb0);
   il_load(a.r0 + idx, cr);
   il_load(a.r1 + idx, lr);
   il_load(a.r2 + idx, ur);
   il_row_sum(a, r, m0, s);
+  il_steps(a, k, IL_TAU, m0, tau);
+  il_steps(a, k, IL_IB, m0, ib);
+  il_steps(a, k, IL_IBN, m0, ibn);
+  il_steps(a, k, IL_THN, m0, thn);
 #pragma unroll
   for (int q = 0; q < W; ++q) {
-    if (run[k0 + q]) {
+    if (run[q]) {
       const V g = r_add(s[q], cr[q]);
-      primal_update<V>(es[k0 + q], g, xo[q], xb0[q], lr[q], ur[q], xn[q], xb[q], zo[q], xtn[q]);
+      primal_update<V>(tau[q], ib[q], ibn[q], thn[q], g, xo[q], xb0[q], lr[q], ur[q], xn[q], xb[q], zo[q], xtn[q]);
     } else {   // a member that stopped keeps its values
       xn[q] = xo[q]; xb[q] = xb0[q]; zo[q] = a.w2[idx + q]; xtn[q] = a.w3[idx + q];
     }
@@ -753,27 +782,30 @@ static void run_chunk_il(Work& w, int j0, int len, const V* Aval, const V* Pval,
   tin(b, m, m, I[IL_B]);
   tin(ylo, m, m, I[IL_YLO]);
   const int groups = ld / (32 * IlVec<V>::W);
+  V* steps = sizeof(V) == 4 ? (V*)w.il_steps_f : (V*)w.il_steps_d;
+  launch(k_il_steps<V>, dim3(cdiv(ld, 128), len), 128, 0, s, (const StepEntry*)w.tab, w.tab_stride,
+         (const DevState*)w.st, cnt, ld, j0, steps, w.il_run);
   FamIL<V> da{};
   da.rp = w.A.rp; da.col = w.A.col; da.val = Aval;
-  da.rows = m; da.ld = ld; da.count = cnt; da.C = w.tab_stride; da.tab = w.tab; da.st = w.st;
+  da.rows = m; da.ld = ld; da.steps = steps; da.run = w.il_run;
   da.zin = I[IL_XT];
   da.w1 = I[IL_YBAR]; da.r0 = I[IL_B]; da.r1 = ylo ? I[IL_YLO] : nullptr; da.ineq = w.row_ineq;
   FamIL<V> pa{};
   pa.rp = w.P.rp; pa.col = w.famP_col; pa.val = Pval;
-  pa.rows = n; pa.ld = ld; pa.count = cnt; pa.C = w.tab_stride; pa.tab = w.tab; pa.st = w.st;
+  pa.rows = n; pa.ld = ld; pa.steps = steps; pa.run = w.il_run;
   pa.w0 = I[IL_X]; pa.w1 = I[IL_XBAR]; pa.w3 = I[IL_XT]; pa.r0 = I[IL_C]; pa.r1 = I[IL_L]; pa.r2 = I[IL_U];
   for (int j = j0; j < j0 + len; ++j) {
     if (m > 0) {
       da.v0 = I[IL_Z0 + ((j + 1) & 1)] + (size_t)n * ld;   // y^k
       da.w0 = I[IL_Z0 + (j & 1)] + (size_t)n * ld;         // y^{k+1}
       if (Pr.on) Pr.begin(0, s, il_launch_bytes(w, 0, sizeof(V)));
-      launch(k_dual_il<V>, dim3(cdiv(m, IL_RPB), groups), IL_NT, 0, s, da, j);
+      launch(k_dual_il<V>, dim3(cdiv(m, IL_RPB), groups), IL_NT, 0, s, da, j - j0);
       if (Pr.on) Pr.end(s);
     }
     pa.zin = I[IL_Z0 + (j & 1)];
     pa.w2 = I[IL_Z0 + ((j + 1) & 1)];
     if (Pr.on) Pr.begin(1, s, il_launch_bytes(w, 1, sizeof(V)));
-    launch(k_primal_il<V>, dim3(cdiv(n, IL_RPB), groups), IL_NT, 0, s, pa, j);
+    launch(k_primal_il<V>, dim3(cdiv(n, IL_RPB), groups), IL_NT, 0, s, pa, j - j0);
     if (Pr.on) Pr.end(s);
   }
   // interleaved -> member-major: everything the iterations wrote

@@ -219,6 +219,10 @@ struct Work {
   bool fam_il = false;                       // eligible: no long rows, no low-rank term
   double* ild[11] = {};                      // float64 (allocated on first use)
   float* ilf[11] = {};                       // float32
+  float* il_steps_f = nullptr;               // [check period][5][fam_ld] step scalars of a chunk, member order
+  double* il_steps_d = nullptr;
+  int il_steps_len[2] = {0, 0};              // iterations they hold (float64, mixed)
+  int* il_run = nullptr;                     // [fam_ld] the member iterates
   double* ilk[10] = {};                      // the check's interleaved iterates and row sums (ILK_*)
   double* kks[6] = {};                       // the check's row sums, member-major: A x (2) [m], Q x (2), A'y (2) [n]
   bool il_active = false;                    // this solve runs the interleaved kernels
