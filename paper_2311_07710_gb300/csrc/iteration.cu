@@ -35,6 +35,7 @@ struct DualB {
   const int2* __restrict__ blk_seg;     // long rows: {first segment, segments} per block (null: none)
   const V* __restrict__ lpart;          // segment sums of the long rows
   const int* __restrict__ act;          // row block of each CUDA block (null: the block index)
+  int early;                            // launched by launch_early: no state read before grid_wait()
 };
 
 template <typename V>
@@ -63,7 +64,7 @@ template <typename V, int NT>
 __device__ __forceinline__ void dual_block(const DualB<V>& a, int bk, int j, V* prod, V* sx, int* srp) {
   const int tid = threadIdx.x;
   const int inst = a.blk_inst[bk];
-  if (a.st[inst].status != ST_RUNNING) return;    // uniform over the block
+  if (!a.early && a.st[inst].status != ST_RUNNING) return;    // uniform over the block
   const int r0 = a.A.blk[bk], r1 = a.A.blk[bk + 1];
   const int nr = r1 - r0;
   const int e0 = a.A.rp[r0];
@@ -71,6 +72,8 @@ __device__ __forceinline__ void dual_block(const DualB<V>& a, int bk, int j, V* 
   // operands of this thread's first row, fetched before the gathers
   V yo = V(0), bi = V(0), yb = V(0), lo = V(0);
   auto mid = [&]() {
+    grid_wait();
+    if (a.early && a.st[inst].status != ST_RUNNING) return false;
     if (tid < nr) {
       const int r = r0 + tid;
       yo = a.yold[r]; bi = a.b[r]; yb = a.ybar[r];
@@ -113,6 +116,7 @@ __global__ void __launch_bounds__(NT, MinBlocks<V, NT>::value) k_dual(DualB<V> a
   __shared__ V prod[BNNZ];
   __shared__ V sx[sizeof(V) == 8 ? BNNZ : 1];
   __shared__ int srp[BROWS + 1];
+  grid_trigger();
   const int bk = a.act ? a.act[blockIdx.x] : (int)blockIdx.x;   // compacted batches: running blocks only
   if (bk < 0) return;                                             // padding of a compacted grid
   dual_block<V, NT>(a, bk, j, prod, sx, srp);
@@ -142,6 +146,7 @@ struct PrimalB {
   const int2* __restrict__ blk_seg;     // long rows: {first segment, segments} per block (null: none)
   const V* __restrict__ lpart;          // segment sums of the long rows
   const int* __restrict__ act;          // row block of each CUDA block (null: the block index)
+  int early;                            // launched by launch_early: no state read before grid_wait()
 };
 
 template <typename V, bool LR = false>
@@ -162,13 +167,15 @@ template <typename V, int NT, bool LR>
 __device__ __forceinline__ void primal_block(const PrimalB<V>& a, int bk, int j, V* prod, V* sx, int* srp) {
   const int tid = threadIdx.x;
   const int inst = a.blk_inst[bk];
-  if (a.st[inst].status != ST_RUNNING) return;    // uniform over the block
+  if (!a.early && a.st[inst].status != ST_RUNNING) return;    // uniform over the block
   const int r0 = a.P.blk[bk], r1 = a.P.blk[bk + 1];
   const int nr = r1 - r0;
   const int e0 = a.P.rp[r0];
   const int ne = a.P.rp[r1] - e0;
   V xo = V(0), xb = V(0), cr = V(0), lr = V(0), ur = V(0);
   auto mid = [&]() {
+    grid_wait();
+    if (a.early && a.st[inst].status != ST_RUNNING) return false;
     if (tid < nr) {
       const int r = r0 + tid;
       xo = a.x[r]; xb = a.xbar[r]; cr = a.c[r]; lr = a.l[r]; ur = a.u[r];
@@ -209,6 +216,7 @@ __global__ void __launch_bounds__(NT, MinBlocks<V, NT, LR>::value) k_primal(Prim
   __shared__ V prod[BNNZ];
   __shared__ V sx[sizeof(V) == 8 ? BNNZ : 1];
   __shared__ int srp[BROWS + 1];
+  grid_trigger();
   const int bk = a.act ? a.act[blockIdx.x] : (int)blockIdx.x;
   if (bk < 0) return;
   // (the dual half-step measured no gain from it: 202.6 -> 203.9 ms of a control-QP
@@ -475,14 +483,15 @@ static void run_chunk_pipe(Work& w, int j0, int len, BCsr<V> A, BCsr<V> P, V* xt
 }
 
 // The dual half-step of iteration j alone (its long rows' segments summed by
-// the kernel before it).
+// the kernel before it, which may still be running: launch_early).
 template <typename V>
 void run_dual(Work& w, int j, BCsr<V> A, V* xt, V* const* Z, V* ybar, const V* b, const V* ylo, cudaStream_t s) {
   DualB<V> da{A, xt, nullptr, nullptr, ybar, b, ylo, w.tab, w.blk_inst_A, w.st, w.row_ineq, w.tab_stride};
   da.yold = Z[(j + 1) & 1] + w.n;
   da.ynew = Z[j & 1] + w.n;
   if (w.A.nlseg) { da.blk_seg = w.A.blk_seg; da.lpart = sizeof(V) == 4 ? (V*)w.A.lpart_f : (V*)w.A.lpart_d; }
-  launch(k_dual<V, 256>, w.A.nblk, 256, 0, s, da, j);
+  da.early = 1;
+  launch_early(k_dual<V, 256>, w.A.nblk, 256, 0, s, da, j);
 }
 template void run_dual<float>(Work&, int, BCsr<float>, float*, float* const*, float*, const float*, const float*,
                               cudaStream_t);
@@ -511,6 +520,10 @@ static void run_chunk(Work& w, int j0, int len, BCsr<V> A, BCsr<V> P, V* xt, V* 
     gA = w.act_grid_A > 0 ? w.act_grid_A : w.bst_host->act_A;
     gP = w.act_grid_P > 0 ? w.act_grid_P : w.bst_host->act_P;
   }
+  // One instance: its half-steps follow each other without a gap (a batch's
+  // blocks look at their instance's status before they load anything).
+  const bool early = w.count == 1 && w.r == 0 && w.A.nlseg == 0 && w.P.nlseg == 0;
+  da.early = pa.early = early;
   for (int j = j0; j < j0 + len; ++j) {
     if (w.r > 0) lowrank_ft1(w, pa.F, (const V*)Z[j & 1], s);
     if (w.m > 0) {
@@ -520,7 +533,8 @@ static void run_chunk(Work& w, int j0, int len, BCsr<V> A, BCsr<V> P, V* xt, V* 
       if (w.A.nlseg)
         launch(k_long_partials<V>, w.A.nlseg, 256, 0, s, A, (const V*)xt, (const int4*)w.A.lseg,
                (const int*)w.blk_inst_A, (const DevState*)w.st, lpA);
-      launch(k_dual<V, NT>, gA, NT, 0, s, da, j);
+      if (early) launch_early(k_dual<V, NT>, gA, NT, 0, s, da, j);
+      else launch(k_dual<V, NT>, gA, NT, 0, s, da, j);
       if (Pr.on) Pr.end(s);
     }
     pa.zin = Z[j & 1];
@@ -530,6 +544,7 @@ static void run_chunk(Work& w, int j0, int len, BCsr<V> A, BCsr<V> P, V* xt, V* 
       launch(k_long_partials<V>, w.P.nlseg, 256, 0, s, P, (const V*)pa.zin, (const int4*)w.P.lseg,
              (const int*)w.blk_inst_P, (const DevState*)w.st, lpP);
     if (w.r > 0) launch(k_primal<V, NT, true>, gP, NT, 0, s, pa, j);
+    else if (early) launch_early(k_primal<V, NT, false>, gP, NT, 0, s, pa, j);
     else launch(k_primal<V, NT, false>, gP, NT, 0, s, pa, j);
     if (Pr.on) Pr.end(s);
   }

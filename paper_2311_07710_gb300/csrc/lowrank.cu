@@ -77,11 +77,13 @@ __device__ __forceinline__ void lrf_stage(V* fs, const V* __restrict__ F, int ro
 template <typename V>
 __global__ void __launch_bounds__(LRF_NT) k_primal_lr(LrPrimal<V> a, int j) {
   extern __shared__ __align__(16) unsigned char lrf_sm[];
+  grid_trigger();
   const int j0 = blockIdx.x * a.per, rows = min(a.per, a.n - j0), r = a.r, ld = lrf_ld<V>(r), tid = threadIdx.x;
   V* fs = reinterpret_cast<V*>(lrf_sm);
   V* zs = fs + (size_t)a.per * ld;
   V* ws = zs + ((a.per + 3) & ~3);
   lrf_stage<V>(fs, a.F + (size_t)j0 * r, rows, r);
+  grid_wait();                                     // (F is the solve's own: on its way before the wait)
   if (a.st->status != ST_RUNNING) {
     asm volatile("cp.async.wait_all;\n" ::);
     return;
@@ -136,6 +138,8 @@ __global__ void __launch_bounds__(256)
     k_lr_reduce_long(const double* __restrict__ part, int nparts, int r, double* __restrict__ w, float* __restrict__ wf,
                      BCsr<V> A, const V* __restrict__ vec, const int4* __restrict__ lseg,
                      const DevState* __restrict__ st, V* __restrict__ lpart) {
+  grid_trigger();
+  grid_wait();
   if (st->status != ST_RUNNING) return;
   if ((int)blockIdx.x < r) lr_reduce_column(part, nparts, r, 1, blockIdx.x, w, wf);
   else long_segment_sum(A, vec, lseg[blockIdx.x - r], lpart + (blockIdx.x - r));
@@ -191,14 +195,14 @@ static void run_chunk_lr(Work& w, int j0, int len, BCsr<V> A, BCsr<V> P, V* xt, 
   for (int j = j0; j < j0 + len; ++j) {
     if (Pr.on) Pr.begin(0, s, launch_bytes(w, 0, sizeof(V)));
     if (j == j0) lowrank_ft_part(w, pa.F, (const V*)Z[j & 1], s);   // later ones come from k_primal_lr
-    launch(k_lr_reduce_long<V>, w.r + w.A.nlseg, 256, 0, s, (const double*)w.lr_part, grid, w.r, w.wlr, w.wlr_f, A,
+    launch_early(k_lr_reduce_long<V>, w.r + w.A.nlseg, 256, 0, s, (const double*)w.lr_part, grid, w.r, w.wlr, w.wlr_f, A,
            (const V*)xt, (const int4*)w.A.lseg, (const DevState*)w.st, lpA);
     if (w.m > 0) run_dual(w, j, A, xt, Z, ybar, b, ylo, s);
     if (Pr.on) Pr.end(s);
     pa.zin = Z[j & 1];
     pa.zout = Z[(j + 1) & 1];
     if (Pr.on) Pr.begin(1, s, launch_bytes(w, 1, sizeof(V)));
-    launch(k_primal_lr<V>, grid, LRF_NT, lrf_smem<V>(per, w.r), s, pa, j);
+    launch_early(k_primal_lr<V>, grid, LRF_NT, lrf_smem<V>(per, w.r), s, pa, j);
     if (Pr.on) Pr.end(s);
   }
 }

@@ -25,6 +25,34 @@ static inline void launch(void (*kern)(KArgs...), dim3 grid, int block, size_t s
   count_launch();
 }
 
+// The same, with programmatic stream serialisation: the grid may start once
+// every block of the kernel before it has called grid_trigger() (or ended), so
+// that its launch and its first loads overlap that kernel's last blocks.  Such
+// a kernel calls grid_wait() before it touches anything an earlier kernel of
+// the iteration loop writes, and before any block of it ends.
+template <typename... KArgs, typename... Args>
+static inline void launch_early(void (*kern)(KArgs...), int grid, int block, size_t smem, cudaStream_t s,
+                                Args... args) {
+  if (grid <= 0) return;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
+  count_launch();
+}
+// the kernels before this one have ended and their writes are visible (returns
+// at once in a normal launch)
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+// this block no longer holds back the next kernel's launch
+__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+
 static inline int cdiv(long long a, long long b) { return (int)((a + b - 1) / b); }
 
 // Deterministic sum over the block (valid in every thread).
@@ -139,8 +167,8 @@ __device__ __forceinline__ void stage_products(const BCsr<V>& M, const X* __rest
 // float64 row sums are fused multiply-adds (r_dot), so their blocks stage the
 // values in prod and the gathered entries in sx.  `mid` runs between the first
 // quads' loads (of the matrix, which no kernel of the loop writes) and the first
-// gather: it fetches the rows' operands;
-// false ends the staging.
+// gather: it waits for the kernels before this one and fetches the rows'
+// operands; false ends the staging.
 template <int NT, typename V, typename Mid>
 __device__ __forceinline__ bool stage_rows(const BCsr<V>& M, const V* __restrict__ vec, int e0, int ne, int r0, int nr,
                                            V* prod, V* sx, int* srp, Mid mid) {
