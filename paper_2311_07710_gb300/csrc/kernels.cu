@@ -285,14 +285,14 @@ __device__ __forceinline__ void kkt_n_row(const KktB& a, double (&f)[15], int r,
 // iterate keeps every field index known at compile time (the fields stay in
 // registers).  Row sums by FMA over the staged values and entries.
 template <int NIT>
-__global__ void __launch_bounds__(BNT) k_kkt_m(KktB a) {
+__device__ __forceinline__ void kkt_m_group(const KktB& a, int g) {
   extern __shared__ __align__(16) double kkt_sm[];
   double* sval = kkt_sm;
   double* sx = kkt_sm + BNNZ;
   int* srp = reinterpret_cast<int*>(kkt_sm + (NIT + 1) * BNNZ);
   double f[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
   const int tid = threadIdx.x;
-  const KktGroup G = kkt_group(a, 0, blockIdx.x);
+  const KktGroup G = kkt_group(a, 0, g);
   if (a.st && a.st[G.inst].status != ST_RUNNING) return;
   for (int bk = G.b0; bk < G.b1; ++bk) {   // the group's row blocks, one after another
     if (bk > G.b0) __syncthreads();          // the staging buffers are read up to here
@@ -333,14 +333,15 @@ __global__ void __launch_bounds__(BNT) k_kkt_m(KktB a) {
   }
   block_reduce_smem<9, BNT, 0x133u>(f, kkt_sm);
   if (tid == 0)
-    for (int k = 0; k < 9; ++k) a.part_m[(size_t)k * a.ngrp_m + blockIdx.x] = f[k];
+    for (int k = 0; k < 9; ++k) a.part_m[(size_t)k * a.ngrp_m + g] = f[k];
+}
+template <int NIT>
+__global__ void __launch_bounds__(BNT) k_kkt_m(KktB a) {
+  kkt_m_group<NIT>(a, blockIdx.x);
 }
 
-// 3 blocks per SM (80 registers): capped at 64 for 4 blocks it spills and is
-// slower (n=1e6 checks 4.67 -> 5.15 ms per solve), left alone it takes 100 and
-// runs 2 (a batch's checks 23.5 -> 29.4 ms)
 template <int NIT, bool LR>
-__global__ void __launch_bounds__(BNT, 3) k_kkt_n(KktB a) {
+__device__ __forceinline__ void kkt_n_group(const KktB& a, int g) {
   extern __shared__ __align__(16) double kkt_sm[];
   double* sval = kkt_sm;
   double* sx = kkt_sm + BNNZ;
@@ -350,7 +351,7 @@ __global__ void __launch_bounds__(BNT, 3) k_kkt_n(KktB a) {
 #pragma unroll
   for (int k = 0; k < 15; ++k) f[k] = 0.0;
   const int tid = threadIdx.x;
-  const KktGroup G = kkt_group(a, 1, blockIdx.x);
+  const KktGroup G = kkt_group(a, 1, g);
   if (a.st && a.st[G.inst].status != ST_RUNNING) return;
   const int n = a.n;
   for (int bk = G.b0; bk < G.b1; ++bk) {   // the group's row blocks, one after another
@@ -399,7 +400,22 @@ __global__ void __launch_bounds__(BNT, 3) k_kkt_n(KktB a) {
   }
   block_reduce_smem<15, BNT, 0x4387u>(f, kkt_sm);
   if (tid == 0)
-    for (int k = 0; k < 15; ++k) a.part_n[(size_t)k * a.ngrp_n + blockIdx.x] = f[k];
+    for (int k = 0; k < 15; ++k) a.part_n[(size_t)k * a.ngrp_n + g] = f[k];
+}
+// 3 blocks per SM (80 registers): capped at 64 for 4 blocks it spills and is
+// slower (n=1e6 checks 4.67 -> 5.15 ms per solve), left alone it takes 100 and
+// runs 2 (a batch's checks 23.5 -> 29.4 ms)
+template <int NIT, bool LR>
+__global__ void __launch_bounds__(BNT, 3) k_kkt_n(KktB a) {
+  kkt_n_group<NIT, LR>(a, blockIdx.x);
+}
+// Both sides in one launch, P's groups (the longer ones) first: where together
+// they do not fill the chip once, the two launches would run one after the
+// other on a few SMs (n = 1000: 33 + 16 us).
+template <int NIT, bool LR>
+__global__ void __launch_bounds__(BNT, 3) k_kkt_both(KktB a) {
+  if ((int)blockIdx.x < a.ngrp_n) kkt_n_group<NIT, LR>(a, blockIdx.x);
+  else kkt_m_group<NIT>(a, blockIdx.x - a.ngrp_n);
 }
 
 // Segment sums of the long rows for the relKKT kernels: one CUDA block per
@@ -460,7 +476,17 @@ static void launch_kkt(const Work& w, const KktB& a0, cudaStream_t s) {
     cudaFuncSetAttribute(k_kkt_m<NIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kkt_smem_bytes<NIT>());
     cudaFuncSetAttribute(k_kkt_n<NIT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kkt_smem_bytes<NIT>());
     cudaFuncSetAttribute(k_kkt_n<NIT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kkt_smem_bytes<NIT>());
+    cudaFuncSetAttribute(k_kkt_both<NIT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)kkt_smem_bytes<NIT>());
+    cudaFuncSetAttribute(k_kkt_both<NIT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)kkt_smem_bytes<NIT>());
   });
+  if (w.m > 0 && w.ngrp_A + w.ngrp_P <= 3 * w.num_sms) {
+    const int grid = w.ngrp_A + w.ngrp_P;
+    if (a.lr) launch(k_kkt_both<NIT, true>, grid, BNT, kkt_smem_bytes<NIT>(), s, a);
+    else launch(k_kkt_both<NIT, false>, grid, BNT, kkt_smem_bytes<NIT>(), s, a);
+    return;
+  }
   if (w.m > 0) launch(k_kkt_m<NIT>, w.ngrp_A, BNT, kkt_smem_bytes<NIT>(), s, a);
   if (a.lr) launch(k_kkt_n<NIT, true>, w.ngrp_P, BNT, kkt_smem_bytes<NIT>(), s, a);
   else launch(k_kkt_n<NIT, false>, w.ngrp_P, BNT, kkt_smem_bytes<NIT>(), s, a);
@@ -619,8 +645,9 @@ static void launch_kkt_il(Work& w, const KktB& a, cudaStream_t s) {
 
 // reduce the field-major partials of k_kkt_m / k_kkt_n (blocks [bm0, bm1) of
 // [nbm] and [bn0, bn1) of [nbn]) into F[0..23] (thread 0)
-__device__ void reduce_kkt_blocks(const double* __restrict__ pm, int nbm, int bm0, int bm1,
-                                  const double* __restrict__ pn, int nbn, int bn0, int bn1, double* F) {
+// (at: the value of field k of block b, by side)
+template <typename AtM, typename AtN>
+__device__ __forceinline__ void reduce_kkt_fields(int bm0, int bm1, AtM at_m, int bn0, int bn1, AtN at_n, double* F) {
   double f[24];
 #pragma unroll
   for (int k = 0; k < 24; ++k) f[k] = 0.0;
@@ -630,18 +657,24 @@ __device__ void reduce_kkt_blocks(const double* __restrict__ pm, int nbm, int bm
   for (int b = bm0 + threadIdx.x; b < bm1; b += blockDim.x)
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-      const double v = pm[(size_t)k * nbm + b];
+      const double v = at_m(k, b);
       f[k] = is_max[k] ? nmax(f[k], v) : f[k] + v;
     }
   for (int b = bn0 + threadIdx.x; b < bn1; b += blockDim.x)
 #pragma unroll
     for (int k = 0; k < 15; ++k) {
-      const double v = pn[(size_t)k * nbn + b];
+      const double v = at_n(k, b);
       f[9 + k] = is_max[9 + k] ? nmax(f[9 + k], v) : f[9 + k] + v;
     }
   block_reduce<24>(f, is_max);
   if (threadIdx.x == 0)
     for (int k = 0; k < 24; ++k) F[k] = f[k];
+}
+__device__ __forceinline__ void reduce_kkt_blocks(const double* __restrict__ pm, int nbm, int bm0, int bm1,
+                                                  const double* __restrict__ pn, int nbn, int bn0, int bn1, double* F) {
+  reduce_kkt_fields(
+      bm0, bm1, [&](int k, int b) { return pm[(size_t)k * nbm + b]; }, bn0, bn1,
+      [&](int k, int b) { return pn[(size_t)k * nbn + b]; }, F);
 }
 
 // --------------------------------------------------------------------------
@@ -1555,6 +1588,24 @@ __device__ void decide_thread0(DevState* __restrict__ st, const double* F, const
 // kernel reads tens of values, not thousands.  gfm, gfn: first group of each
 // instance (A, P).
 constexpr int KKT_GPC = KKT_CHUNK / KKT_GROUP;   // groups per chunk (8: lanes 0..7)
+// one chunk's sums of one side in a warp: first group g0 of the chunk, end of
+// the instance's groups ge; put(k, value) in lane 0
+template <int NF, unsigned MAXMASK, typename Put>
+__device__ __forceinline__ void kkt_chunk_sums(const double* __restrict__ part, int ng, int g0, int ge, Put put) {
+  const int lane = threadIdx.x & 31, g = g0 + lane;
+  const bool on = lane < KKT_GPC && g < ge;
+#pragma unroll
+  for (int k = 0; k < NF; ++k) {
+    const bool mx = (MAXMASK >> k) & 1u;
+    double v = on ? part[(size_t)k * ng + g] : 0.0;
+#pragma unroll
+    for (int o = KKT_GPC / 2; o > 0; o >>= 1) {
+      const double t = __shfl_xor_sync(0xffffffffu, v, o);
+      v = mx ? nmax(v, t) : v + t;
+    }
+    if (lane == 0) put(k, v);
+  }
+}
 __global__ void __launch_bounds__(32) k_kkt_chunks(const Inst* __restrict__ insts, const int* __restrict__ gfm,
                                                    const double* __restrict__ pm, int ngm,
                                                    const int* __restrict__ gfn, const double* __restrict__ pn,
@@ -1562,65 +1613,81 @@ __global__ void __launch_bounds__(32) k_kkt_chunks(const Inst* __restrict__ inst
                                                    double* __restrict__ cn, int ncn) {
   const int i = blockIdx.x;
   const Inst in = insts[i];
-  const int lane = threadIdx.x, c = blockIdx.y;
-  if (in.bP0 + c * KKT_CHUNK < in.bP1) {
-    const bool is_max[15] = {true, true, true, false, false, false, false,
-                             true, true, true, false, false, false, false, true};
-    const int g = gfn[i] + c * KKT_GPC + lane;
-    const bool on = lane < KKT_GPC && g < gfn[i + 1];
-#pragma unroll
-    for (int k = 0; k < 15; ++k) {
-      double v = on ? pn[(size_t)k * ngn + g] : 0.0;
-#pragma unroll
-      for (int o = KKT_GPC / 2; o > 0; o >>= 1) {
-        const double t = __shfl_xor_sync(0xffffffffu, v, o);
-        v = is_max[k] ? nmax(v, t) : v + t;
-      }
-      if (lane == 0) cn[(size_t)k * ncn + in.cP0 + c] = v;
-    }
-  }
-  if (in.m > 0 && in.bA0 + c * KKT_CHUNK < in.bA1) {
-    const bool is_max[9] = {true, true, false, false, true, true, false, false, true};
-    const int g = gfm[i] + c * KKT_GPC + lane;
-    const bool on = lane < KKT_GPC && g < gfm[i + 1];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      double v = on ? pm[(size_t)k * ngm + g] : 0.0;
-#pragma unroll
-      for (int o = KKT_GPC / 2; o > 0; o >>= 1) {
-        const double t = __shfl_xor_sync(0xffffffffu, v, o);
-        v = is_max[k] ? nmax(v, t) : v + t;
-      }
-      if (lane == 0) cm[(size_t)k * ncm + in.cA0 + c] = v;
-    }
-  }
+  const int c = blockIdx.y;
+  if (in.bP0 + c * KKT_CHUNK < in.bP1)
+    kkt_chunk_sums<15, 0x4387u>(pn, ngn, gfn[i] + c * KKT_GPC, gfn[i + 1],
+                                [&](int k, double v) { cn[(size_t)k * ncn + in.cP0 + c] = v; });
+  if (in.m > 0 && in.bA0 + c * KKT_CHUNK < in.bA1)
+    kkt_chunk_sums<9, 0x133u>(pm, ngm, gfm[i] + c * KKT_GPC, gfm[i + 1],
+                              [&](int k, double v) { cm[(size_t)k * ncm + in.cA0 + c] = v; });
 }
 
 
 // mode 0: evaluate z^{0,0} (anchor, maybe already optimal); mode 1: a check
 // after `chunk_len` more iterations (Section 6 restart rule, termination
 // eq. (terminate), iteration limit).
-// one CUDA block of 64 threads per instance (one step-table entry per thread)
-__global__ void __launch_bounds__(64) k_decide(DevState* __restrict__ sts, const Inst* __restrict__ insts,
-                                                const double* __restrict__ pm, int nbm,
-                                                const double* __restrict__ pn, int nbn,
-                                                StepEntry* __restrict__ tabs, int C, SolveParams p, int mode,
-                                                long long chunk_len, const InfState* __restrict__ inf) {
+// one CUDA block of 64 threads per instance (one step-table entry per thread).
+// Where no instance has more than DEC_CHUNKS chunks a side, the block forms its
+// chunk sums itself (gf: the first groups; the launch of k_kkt_chunks falls away),
+// and a single instance's counters for the host are written here as well (bst).
+constexpr int DEC_CHUNKS = 4;
+struct DecideArgs {
+  DevState* sts;
+  const Inst* insts;
+  const double *pm, *pn;       // chunk sums, or the group partials (gf_m set)
+  int nbm, nbn;
+  const int *gf_m, *gf_n;      // null: pm, pn hold chunk sums
+  StepEntry* tabs;
+  int C;
+  const InfState* inf;
+  BatchState* bst;             // one instance: its counters (null: k_count_running)
+  const int *rpA, *rpP;
+};
+__device__ __forceinline__ void write_running(const DevState& st, const Inst& in, const int* __restrict__ rpA,
+                                              const int* __restrict__ rpP, BatchState* bst) {
+  const bool r = st.status == ST_RUNNING;
+  bst->running = r;
+  bst->lz_running = !(st.pi_done[0] && st.pi_done[1]);
+  bst->run_n = r ? in.n : 0.0;
+  bst->run_m = r ? in.m : 0.0;
+  bst->run_nnzA = r && in.m > 0 ? rpA[in.yoff + in.m] - rpA[in.yoff] : 0.0;
+  bst->run_nnzP = r ? rpP[in.xoff + in.n] - rpP[in.xoff] : 0.0;
+}
+__global__ void __launch_bounds__(64) k_decide(DecideArgs a, SolveParams p, int mode, long long chunk_len) {
   const int i = blockIdx.x;
-  DevState* st = sts + i;
-  if (mode == 1 && st->status != ST_RUNNING) return;     // uniform
-  const Inst in = insts[i];
+  DevState* st = a.sts + i;
+  const Inst in = a.insts[i];
+  if (mode == 1 && st->status != ST_RUNNING) {           // uniform
+    if (a.bst && threadIdx.x == 0) write_running(*st, in, a.rpA, a.rpP, a.bst);
+    return;
+  }
   __shared__ double F[24];
-  // pm / pn hold the chunk sums of k_kkt_chunks
-  reduce_kkt_blocks(pm, nbm, in.cA0, in.m > 0 ? in.cA0 + kkt_chunks(in.bA0, in.bA1) : in.cA0, pn, nbn, in.cP0,
-                    in.cP0 + kkt_chunks(in.bP0, in.bP1), F);
-  if (threadIdx.x == 0) decide_thread0(st, F, p, mode, chunk_len, inf ? inf[i].status : 0);
+  const int cm = in.m > 0 ? kkt_chunks(in.bA0, in.bA1) : 0, cn = kkt_chunks(in.bP0, in.bP1);
+  if (a.gf_m) {
+    __shared__ double sc[24][DEC_CHUNKS];
+    if (threadIdx.x < 32) {
+      for (int c = 0; c < cn; ++c)
+        kkt_chunk_sums<15, 0x4387u>(a.pn, a.nbn, a.gf_n[i] + c * KKT_GPC, a.gf_n[i + 1],
+                                    [&](int k, double v) { sc[9 + k][c] = v; });
+    } else {
+      for (int c = 0; c < cm; ++c)
+        kkt_chunk_sums<9, 0x133u>(a.pm, a.nbm, a.gf_m[i] + c * KKT_GPC, a.gf_m[i + 1],
+                                  [&](int k, double v) { sc[k][c] = v; });
+    }
+    __syncthreads();
+    reduce_kkt_fields(
+        0, cm, [&](int k, int b) { return sc[k][b]; }, 0, cn, [&](int k, int b) { return sc[9 + k][b]; }, F);
+  } else {
+    reduce_kkt_blocks(a.pm, a.nbm, in.cA0, in.cA0 + cm, a.pn, a.nbn, in.cP0, in.cP0 + cn, F);
+  }
+  if (threadIdx.x == 0) decide_thread0(st, F, p, mode, chunk_len, a.inf ? a.inf[i].status : 0);
   __syncthreads();
-  if (st->status == ST_RUNNING) fill_steps_block(*st, p, tabs + (size_t)i * C);
+  if (a.bst && threadIdx.x == 0) write_running(*st, in, a.rpA, a.rpP, a.bst);
+  if (st->status == ST_RUNNING) fill_steps_block(*st, p, a.tabs + (size_t)i * a.C);
 }
 
 // number of instances still iterating / still estimating norms
-__global__ void k_count_running(const DevState* __restrict__ sts, const Inst* __restrict__ inst,
+__global__ void __launch_bounds__(1024) k_count_running(const DevState* __restrict__ sts, const Inst* __restrict__ inst,
                                 const int* __restrict__ rpA, const int* __restrict__ rpP, int count,
                                 BatchState* bst) {
   int run = 0, lz = 0;
@@ -1804,18 +1871,20 @@ __global__ void k_pair_iterates(int n, int m, const double* __restrict__ x, cons
   }
 }
 
-__global__ void k_materialize(MixedArgs a) {
+// all: every instance's iterates (the start point); else those of the instances
+// still running (the others' are those of the check that ended them)
+__global__ void k_materialize(MixedArgs a, int all) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < max(a.n, a.m); i += gridDim.x * blockDim.x) {
-    if (i < a.n) {
+    if (i < a.n && (all || a.sts[a.inst_n[i]].status == ST_RUNNING)) {
       const double h = a.xhi[i], lo = a.ls[i], hi = a.us[i];
-      const double v0 = fmin(fmax(h + (double)a.fx[i], lo), hi), v1 = fmin(fmax(h + (double)a.fxbar[i], lo), hi);
+      const double v0 = fmin(fmax(h + f2d(a.fx[i]), lo), hi), v1 = fmin(fmax(h + f2d(a.fxbar[i]), lo), hi);
       a.x64[0][i] = v0;
       a.x64[1][i] = v1;
       if (a.xx) a.xx[i] = make_double2(v0, v1);
     }
-    if (i < a.m) {
+    if (i < a.m && (all || a.sts[a.inst_m[i]].status == ST_RUNNING)) {
       const double h = a.yhi[i];
-      double v0 = h + (double)a.fy[i], v1 = h + (double)a.fybar[i];
+      double v0 = h + f2d(a.fy[i]), v1 = h + f2d(a.fybar[i]);
       if (a.ineq[i]) { v0 = fmax(v0, 0.0); v1 = fmax(v1, 0.0); }
       a.y64[0][i] = v0;
       a.y64[1][i] = v1;
@@ -2037,8 +2106,8 @@ void lanczos_compact(Work& w, cudaStream_t s) {
 }
 
 void count_running(Work& w, cudaStream_t s) {
-  launch(k_count_running, 1, 256, 0, s, (const DevState*)w.st, (const Inst*)w.inst, (const int*)w.A.rp,
-         (const int*)w.P.rp, w.count, w.bst);
+  launch(k_count_running, 1, w.count > 256 ? 1024 : 256, 0, s, (const DevState*)w.st, (const Inst*)w.inst,
+         (const int*)w.A.rp, (const int*)w.P.rp, w.count, w.bst);
 }
 
 void norms_finish(Work& w, double normA_opt, double normQ_opt, cudaStream_t s) {
@@ -2312,7 +2381,7 @@ void check(Work& w, const SolveParams& p, int mode, long long chunk_len, bool mi
   if (mixed) {
     MixedArgs ma = mixed_args(w);
     if (pairs) { ma.xx = w.kkt_xx; ma.yy = w.kkt_yy; }
-    launch(k_materialize, grid_v, 256, 0, s, ma);
+    launch(k_materialize, grid_v, 256, 0, s, ma, mode == 0 || w.count == 1 ? 1 : 0);
   } else if (pairs) {
     launch(k_pair_iterates, grid_v, 256, 0, s, w.n, w.m, (const double*)w.x, (const double*)w.xbar,
            (const double*)w.y, (const double*)w.ybar, w.kkt_xx, w.kkt_yy);
@@ -2342,7 +2411,8 @@ void check(Work& w, const SolveParams& p, int mode, long long chunk_len, bool mi
   } else {
     launch_kkt<2>(w, a, s);
   }
-  {
+  const bool own_chunks = std::max(w.maxchunk_n, w.maxchunk_m) <= DEC_CHUNKS;   // k_decide forms them
+  if (!own_chunks) {
     const dim3 grid(w.count, std::max(w.maxchunk_n, w.maxchunk_m));
     launch(k_kkt_chunks, grid, 32, 0, s, (const Inst*)w.inst, (const int*)w.grp_first_A, (const double*)w.part_m,
            w.ngrp_A, (const int*)w.grp_first_P, (const double*)w.part_n, w.ngrp_P, w.cpart_m,
@@ -2350,17 +2420,20 @@ void check(Work& w, const SolveParams& p, int mode, long long chunk_len, bool mi
   }
   const bool certify = w.detect && w.inf && mode == 1;
   if (certify) infeas_check(w, a, s);
-  launch(k_decide, w.count, 64, 0, s, w.st, (const Inst*)w.inst, (const double*)w.cpart_m,
-         std::max(w.nchunk_m, 1), (const double*)w.cpart_n, std::max(w.nchunk_n, 1), w.tab, w.tab_stride, p, mode,
-         chunk_len, certify ? (const InfState*)w.inf : (const InfState*)nullptr);
+  DecideArgs da{w.st, w.inst, w.cpart_m, w.cpart_n, std::max(w.nchunk_m, 1), std::max(w.nchunk_n, 1), nullptr, nullptr,
+                w.tab, w.tab_stride, certify ? w.inf : nullptr, w.count == 1 ? w.bst : nullptr, w.A.rp, w.P.rp};
+  if (own_chunks) {
+    da.pm = w.part_m; da.nbm = w.ngrp_A; da.gf_m = w.grp_first_A;
+    da.pn = w.part_n; da.nbn = w.ngrp_P; da.gf_n = w.grp_first_P;
+  }
+  launch(k_decide, w.count, 64, 0, s, da, p, mode, chunk_len);
   if (mixed) {
     launch(k_mixed_rebase, grid_v, 256, 0, s, mixed_args(w), mode == 0 ? 1 : 0);
   } else if (mode == 1) {
     launch(k_restart_apply, grid_v, 256, 0, s, (const DevState*)w.st, (const int*)w.row_inst_n,
            (const int*)w.row_inst_m, w.n, w.m, w.x, w.xbar, w.Z[0], w.xt, w.ax, w.y, w.ybar, w.ay);
   }
-  launch(k_count_running, 1, 256, 0, s, (const DevState*)w.st, (const Inst*)w.inst, (const int*)w.A.rp,
-         (const int*)w.P.rp, w.count, w.bst);
+  if (w.count > 1) count_running(w, s);   // (one instance: k_decide)
   if (w.count > 1) {   // the running instances' row blocks, for compacted launches
     cudaMemsetAsync(&w.bst->act_A, 0, 2 * sizeof(int), s);
     // -1 past the count: the padding blocks of a replayed compacted grid skip
