@@ -337,6 +337,8 @@ __device__ __forceinline__ void kkt_m_group(const KktB& a, int g) {
 }
 template <int NIT>
 __global__ void __launch_bounds__(BNT) k_kkt_m(KktB a) {
+  grid_trigger();
+  grid_wait();
   kkt_m_group<NIT>(a, blockIdx.x);
 }
 
@@ -407,6 +409,8 @@ __device__ __forceinline__ void kkt_n_group(const KktB& a, int g) {
 // runs 2 (a batch's checks 23.5 -> 29.4 ms)
 template <int NIT, bool LR>
 __global__ void __launch_bounds__(BNT, 3) k_kkt_n(KktB a) {
+  grid_trigger();
+  grid_wait();
   kkt_n_group<NIT, LR>(a, blockIdx.x);
 }
 // Both sides in one launch, P's groups (the longer ones) first: where together
@@ -414,6 +418,8 @@ __global__ void __launch_bounds__(BNT, 3) k_kkt_n(KktB a) {
 // other on a few SMs (n = 1000: 33 + 16 us).
 template <int NIT, bool LR>
 __global__ void __launch_bounds__(BNT, 3) k_kkt_both(KktB a) {
+  grid_trigger();
+  grid_wait();
   if ((int)blockIdx.x < a.ngrp_n) kkt_n_group<NIT, LR>(a, blockIdx.x);
   else kkt_m_group<NIT>(a, blockIdx.x - a.ngrp_n);
 }
@@ -483,13 +489,13 @@ static void launch_kkt(const Work& w, const KktB& a0, cudaStream_t s) {
   });
   if (w.m > 0 && w.ngrp_A + w.ngrp_P <= 3 * w.num_sms) {
     const int grid = w.ngrp_A + w.ngrp_P;
-    if (a.lr) launch(k_kkt_both<NIT, true>, grid, BNT, kkt_smem_bytes<NIT>(), s, a);
-    else launch(k_kkt_both<NIT, false>, grid, BNT, kkt_smem_bytes<NIT>(), s, a);
+    if (a.lr) launch_early(k_kkt_both<NIT, true>, grid, BNT, kkt_smem_bytes<NIT>(), s, a);
+    else launch_early(k_kkt_both<NIT, false>, grid, BNT, kkt_smem_bytes<NIT>(), s, a);
     return;
   }
-  if (w.m > 0) launch(k_kkt_m<NIT>, w.ngrp_A, BNT, kkt_smem_bytes<NIT>(), s, a);
-  if (a.lr) launch(k_kkt_n<NIT, true>, w.ngrp_P, BNT, kkt_smem_bytes<NIT>(), s, a);
-  else launch(k_kkt_n<NIT, false>, w.ngrp_P, BNT, kkt_smem_bytes<NIT>(), s, a);
+  if (w.m > 0) launch_early(k_kkt_m<NIT>, w.ngrp_A, BNT, kkt_smem_bytes<NIT>(), s, a);
+  if (a.lr) launch_early(k_kkt_n<NIT, true>, w.ngrp_P, BNT, kkt_smem_bytes<NIT>(), s, a);
+  else launch_early(k_kkt_n<NIT, false>, w.ngrp_P, BNT, kkt_smem_bytes<NIT>(), s, a);
 }
 
 // --------------------------------------------------------------------------
@@ -876,6 +882,8 @@ __device__ __forceinline__ double* lz_be(const LzArgs& a, int i, int o) { return
 template <typename V, int NT>
 __global__ void __launch_bounds__(NT, MinBlocks<V, NT>::value) k_lz_m(BCsr<V> A, LzArgs la, const V* __restrict__ vA,
                                                                    V* __restrict__ wm) {
+  grid_trigger();
+  grid_wait();
   const int bk = la.actA ? la.actA[blockIdx.x] : (int)blockIdx.x;
   const DevState& st = la.st[la.blk_inst_A[bk]];
   if (st.pi_done[0]) return;
@@ -910,6 +918,8 @@ __global__ void __launch_bounds__(NT, MinBlocks<V, NT, LR>::value) k_lz_n(BCsr<V
                                                                    V* __restrict__ wQ, double* __restrict__ part,
                                                                    const V* __restrict__ F,
                                                                    const V* __restrict__ wlr, int rk) {
+  grid_trigger();
+  grid_wait();
   __shared__ __align__(16) V prod[BNNZ];
   __shared__ int srp[BROWS + 1];
   __shared__ int ssp[BROWS];
@@ -991,6 +1001,8 @@ __device__ __forceinline__ void lz_block_sums(const double* __restrict__ part, i
 // one CUDA block per instance: alpha_k = sum of its chunk sums
 template <int NT>
 __global__ void __launch_bounds__(NT) k_lz_alpha(LzArgs a) {
+  grid_trigger();
+  grid_wait();
   const int i = blockIdx.x;
   DevState& st = a.st[i];
   if (st.pi_done[0] && st.pi_done[1]) return;
@@ -1008,7 +1020,9 @@ __global__ void __launch_bounds__(NT) k_lz_alpha(LzArgs a) {
 
 // r = w - alpha v - beta_prev v_prev over v_prev, one warp per P row block (8
 // per CTA: the per-block prologue of the instance's scalars runs in parallel);
-// partial |r|^2 per row block.  With lazy normalisation v is the stored vector
+// partial |r|^2 per row block.  own_alpha: no instance has more than
+// LZ_OWN_CHUNKS chunks, and each warp sums its instance's alphas itself instead
+// of a launch of k_lz_alpha between the products and this kernel.  With lazy normalisation v is the stored vector
 // times 1/beta of the last step, written back here as the normalised vector
 // that the next step's three-term update reads as v_prev.  The update runs in
 // the vectors' precision (two FMAs), only |r|^2 in float64.
@@ -1016,7 +1030,10 @@ template <typename V>
 __global__ void __launch_bounds__(256) k_lz_orth(LzArgs a, BCsr<V> P, const V* __restrict__ wA,
                                                  const V* __restrict__ wQ, V* __restrict__ vA,
                                                  V* __restrict__ vA_prev, V* __restrict__ vQ,
-                                                 V* __restrict__ vQ_prev, double* __restrict__ part) {
+                                                 V* __restrict__ vQ_prev, double* __restrict__ part,
+                                                 int own_alpha) {
+  grid_trigger();
+  grid_wait();
   const int q = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (q >= (a.actP ? a.nactP : a.nblkP)) return;   // warp-uniform
   const int b = a.actP ? a.actP[q] : q;
@@ -1025,7 +1042,26 @@ __global__ void __launch_bounds__(256) k_lz_orth(LzArgs a, BCsr<V> P, const V* _
   const bool doA = !st.pi_done[0], doQ = !st.pi_done[1];
   if (!doA && !doQ) return;
   const int k = st.pi_iters;
-  const V alA = (V)(doA ? lz_al(a, i, 0)[k] : 0.0), alQ = (V)(doQ ? lz_al(a, i, 1)[k] : 0.0);
+  double al[2];
+  if (own_alpha) {   // the few chunk sums, in k_lz_alpha's order; the instance's first row block keeps them
+    const Inst in = a.inst[i];
+    const int nc = kkt_chunks(in.bP0, in.bP1);
+#pragma unroll
+    for (int o = 0; o < 2; ++o) {
+      double v = lane < nc ? a.cpart[(size_t)o * a.nchunk + in.cP0 + lane] : 0.0;
+      v += __shfl_xor_sync(0xffffffffu, v, 2);
+      v += __shfl_xor_sync(0xffffffffu, v, 1);
+      al[o] = __shfl_sync(0xffffffffu, v, 0);
+    }
+    if (b == in.bP0 && lane == 0) {
+      if (doA) lz_al(a, i, 0)[k] = al[0];
+      if (doQ) lz_al(a, i, 1)[k] = al[1];
+    }
+  } else {
+    al[0] = doA ? lz_al(a, i, 0)[k] : 0.0;
+    al[1] = doQ ? lz_al(a, i, 1)[k] : 0.0;
+  }
+  const V alA = (V)(doA ? al[0] : 0.0), alQ = (V)(doQ ? al[1] : 0.0);
   const V bpA = (V)((doA && k > 0) ? lz_be(a, i, 0)[k - 1] : 0.0);
   const V bpQ = (V)((doQ && k > 0) ? lz_be(a, i, 1)[k - 1] : 0.0);
   const V gA = lz_scale<V>(a, st, 0), gQ = lz_scale<V>(a, st, 1);
@@ -1266,6 +1302,8 @@ __device__ void confirm_bracket_warp(const double* __restrict__ al, const double
 // 2 floats) bytes).
 template <int NT>
 __global__ void __launch_bounds__(NT) k_lz_beta(LzArgs a, double tol, int max_steps, int kcap) {
+  grid_trigger();
+  grid_wait();
   const int i = blockIdx.x;
   DevState& st = a.st[i];
   if (st.pi_done[0] && st.pi_done[1]) return;     // uniform: nothing left to do
@@ -1419,6 +1457,8 @@ __global__ void __launch_bounds__(NT) k_lz_beta(LzArgs a, double tol, int max_st
 // v_next = r / beta (in the buffer that held v_prev)
 template <typename V>
 __global__ void k_lz_norm(LzArgs a, V* __restrict__ vA_next, V* __restrict__ vQ_next) {
+  grid_trigger();
+  grid_wait();
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < a.n; r += gridDim.x * blockDim.x) {
     const DevState& st = a.st[a.row_inst_n[r]];
     // pi_inv_norm changes only when the operator continues; the product in the
@@ -1654,6 +1694,8 @@ __device__ __forceinline__ void write_running(const DevState& st, const Inst& in
   bst->run_nnzP = r ? rpP[in.xoff + in.n] - rpP[in.xoff] : 0.0;
 }
 __global__ void __launch_bounds__(64) k_decide(DecideArgs a, SolveParams p, int mode, long long chunk_len) {
+  grid_trigger();
+  grid_wait();
   const int i = blockIdx.x;
   DevState* st = a.sts + i;
   const Inst in = a.insts[i];
@@ -1788,6 +1830,8 @@ __global__ void k_compact_blocks(const int* __restrict__ blk_inst, int nblk, con
 __global__ void k_restart_apply(const DevState* __restrict__ sts, const int* __restrict__ inst_n,
                                 const int* __restrict__ inst_m, int n, int m, double* x, double* xbar,
                                 double* xmd0, double* xt, double* ax, double* y, double* ybar, double* ay) {
+  grid_trigger();
+  grid_wait();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < max(n, m); i += gridDim.x * blockDim.x) {
     if (i < n) {
       const DevState& s = sts[inst_n[i]];
@@ -1865,6 +1909,8 @@ __global__ void k_init_mixed(MixedArgs a, const double* __restrict__ x0, const d
 __global__ void k_pair_iterates(int n, int m, const double* __restrict__ x, const double* __restrict__ xbar,
                                 const double* __restrict__ y, const double* __restrict__ ybar,
                                 double2* __restrict__ xx, double2* __restrict__ yy) {
+  grid_trigger();
+  grid_wait();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < max(n, m); i += gridDim.x * blockDim.x) {
     if (i < n) xx[i] = make_double2(x[i], xbar[i]);
     if (i < m) yy[i] = make_double2(y[i], ybar[i]);
@@ -1874,6 +1920,8 @@ __global__ void k_pair_iterates(int n, int m, const double* __restrict__ x, cons
 // all: every instance's iterates (the start point); else those of the instances
 // still running (the others' are those of the check that ended them)
 __global__ void k_materialize(MixedArgs a, int all) {
+  grid_trigger();
+  grid_wait();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < max(a.n, a.m); i += gridDim.x * blockDim.x) {
     if (i < a.n && (all || a.sts[a.inst_n[i]].status == ST_RUNNING)) {
       const double h = a.xhi[i], lo = a.ls[i], hi = a.us[i];
@@ -1896,6 +1944,8 @@ __global__ void k_materialize(MixedArgs a, int all) {
 // Move the base to the candidate (or, with force, re-derive the shifted data
 // at the current base) and zero the float32 deltas.
 __global__ void k_mixed_rebase(MixedArgs a, int force) {
+  grid_trigger();
+  grid_wait();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < max(a.n, a.m); i += gridDim.x * blockDim.x) {
     if (i < a.n) {
       const DevState& s = a.sts[a.inst_n[i]];
@@ -2051,29 +2101,31 @@ static void lanczos_step_t(Work& w, int t, const SolveParams& p, BCsr<V> A, BCsr
   const LzArgs la = lz_args(w);
   // all row blocks, or late in a batch's estimates those of the instances still running
   const int gA = w.lz_compact ? w.bst_host->act_A : w.A.nblk, gP = w.lz_compact ? w.bst_host->act_P : w.P.nblk;
-  if (w.m > 0) launch(k_lz_m<V, NT>, gA, NT, 0, s, A, la, (const V*)pu[cur], pz[cur] + w.n);
+  if (w.m > 0) launch_early(k_lz_m<V, NT>, gA, NT, 0, s, A, la, (const V*)pu[cur], pz[cur] + w.n);
   const V* F = nullptr;
   if (w.r > 0) {
     F = lr_factor<V>(w);
     lowrank_ft<V, V>(w, F, (const V*)pz[cur], (const V*)nullptr, s);
   }
   if (F)
-    launch(k_lz_n<V, NT, true>, gP, NT, 0, s, P, la, (const V*)pz[cur], (const V*)pu[cur], lw[0], lw[1],
+    launch_early(k_lz_n<V, NT, true>, gP, NT, 0, s, P, la, (const V*)pz[cur], (const V*)pu[cur], lw[0], lw[1],
            w.part_n, F, lr_weights<V>(w), w.r);
   else
-    launch(k_lz_n<V, NT, false>, gP, NT, 0, s, P, la, (const V*)pz[cur], (const V*)pu[cur], lw[0], lw[1],
+    launch_early(k_lz_n<V, NT, false>, gP, NT, 0, s, P, la, (const V*)pz[cur], (const V*)pu[cur], lw[0], lw[1],
            w.part_n, F, lr_weights<V>(w), w.r);
   // the per-instance reductions read the chunk sums (a few hundred for the
   // largest instance), so 128 threads each suffice
-  launch(k_lz_alpha<128>, w.count, 128, 0, s, la);
-  launch(k_lz_orth<V>, cdiv(gP, 8), 256, 0, s, la, P, (const V*)lw[0], (const V*)lw[1], pu[cur], pu[prv],
-         pz[cur], pz[prv], w.part_n);
+  constexpr int LZ_OWN_CHUNKS = 4;
+  const int own_alpha = w.maxchunk_n <= LZ_OWN_CHUNKS;
+  if (!own_alpha) launch_early(k_lz_alpha<128>, w.count, 128, 0, s, la);
+  launch_early(k_lz_orth<V>, cdiv(gP, 8), 256, 0, s, la, P, (const V*)lw[0], (const V*)lw[1], pu[cur], pu[prv],
+               pz[cur], pz[prv], w.part_n, own_alpha);
   // the tridiagonals have t + 1 rows at step t: shared memory for that many
   // (the blocks per SM grow as the arrays shrink)
   const int kcap = (t + 1 + 3) & ~3;
-  launch(k_lz_beta<128>, w.count, 128, (size_t)kcap * 2 * (3 * sizeof(double) + 2 * sizeof(float)), s, la,
+  launch_early(k_lz_beta<128>, w.count, 128, (size_t)kcap * 2 * (3 * sizeof(double) + 2 * sizeof(float)), s, la,
          p.norm_tol, p.norm_iters < LZ_MAX ? p.norm_iters : LZ_MAX, kcap);
-  if (!la.lazy) launch(k_lz_norm<V>, std::min(cdiv(w.n, 256), 4 * w.num_sms), 256, 0, s, la, pu[prv], pz[prv]);
+  if (!la.lazy) launch_early(k_lz_norm<V>, std::min(cdiv(w.n, 256), 4 * w.num_sms), 256, 0, s, la, pu[prv], pz[prv]);
 }
 
 // The norm estimates run at one width whatever the iteration kernels' variant
@@ -2426,11 +2478,11 @@ void check(Work& w, const SolveParams& p, int mode, long long chunk_len, bool mi
     da.pm = w.part_m; da.nbm = w.ngrp_A; da.gf_m = w.grp_first_A;
     da.pn = w.part_n; da.nbn = w.ngrp_P; da.gf_n = w.grp_first_P;
   }
-  launch(k_decide, w.count, 64, 0, s, da, p, mode, chunk_len);
+  launch_early(k_decide, w.count, 64, 0, s, da, p, mode, chunk_len);
   if (mixed) {
-    launch(k_mixed_rebase, grid_v, 256, 0, s, mixed_args(w), mode == 0 ? 1 : 0);
+    launch_early(k_mixed_rebase, grid_v, 256, 0, s, mixed_args(w), mode == 0 ? 1 : 0);
   } else if (mode == 1) {
-    launch(k_restart_apply, grid_v, 256, 0, s, (const DevState*)w.st, (const int*)w.row_inst_n,
+    launch_early(k_restart_apply, grid_v, 256, 0, s, (const DevState*)w.st, (const int*)w.row_inst_n,
            (const int*)w.row_inst_m, w.n, w.m, w.x, w.xbar, w.Z[0], w.xt, w.ax, w.y, w.ybar, w.ay);
   }
   if (w.count > 1) count_running(w, s);   // (one instance: k_decide)
