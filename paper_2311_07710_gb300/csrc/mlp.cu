@@ -888,79 +888,110 @@ __global__ void k_gather_rows(const bf16* __restrict__ src, int ld, long long a,
   }
 }
 
-// Gradient tiles (32 rows x 32 features per block of 32 x 8 threads).
+// Gradient tiles (32 rows x 64 features per block of 256 threads: a warp per
+// row, two features per lane).
 // MODE 0 (output layer): g = (o - t) * scale with t the target row of sample
 // visit(row0 + r); also the squared-error partial of the block.
 // MODE 1 (hidden layer): g = in.
 // Writes g as bf16 row-major [rows x ldg] and transposed [F x ldgt], and the
-// float32 column sums of the tile to colpart[blockIdx.y][f].
+// float32 column sums of the tile (rows in order) to colpart[blockIdx.y][f].
+// Every leading dimension is even.
+constexpr int GT_F = 64;
 template <int MODE>
 __global__ void __launch_bounds__(256) k_grad_tiles(const float* __restrict__ in, int ldi, const float* __restrict__ T,
                                                     int ldt, long long a, long long sft, long long count,
                                                     long long row0, int rows, int F, float scale, bf16* __restrict__ gb,
                                                     int ldg, bf16* __restrict__ gt, int ldgt,
                                                     float* __restrict__ colpart, int ldc, double* __restrict__ lossp) {
-  __shared__ float tile[32][33];
+  __shared__ float tile[32][GT_F + 1];
   __shared__ double red[8];
   __shared__ long long smp_of[32];
-  const int f0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const int f = f0 + tx;
+  const int f0 = blockIdx.x * GT_F, r0 = blockIdx.y * 32;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int f = f0 + 2 * lane;
+  const bool on0 = f < F, on1 = f + 1 < F;
   // the squared error in float32 pairs (product and sum with their exact
-  // rounding errors, about 2^-48 relative): a thread's four terms would take
-  // eight float64-pipe operations (conversions included), one conversion pair
-  // here; terms whose square or its error leaves float32's range go to ld
+  // rounding errors, about 2^-48 relative): in float64 each term would take
+  // two operations of that pipe, conversion included; terms whose square or
+  // its error leaves float32's range go to ld
   float lh = 0.f, ll = 0.f;
   double ld = 0.0;
   if (MODE == 0) {   // the rows' samples, one 64-bit remainder each
-    if (ty == 0 && r0 + tx < rows) smp_of[tx] = visit(a, sft, count, row0 + r0 + tx);
+    if (w == 0 && r0 + lane < rows) smp_of[lane] = visit(a, sft, count, row0 + r0 + lane);
     __syncthreads();
   }
+  float2 o[4], t[4];
 #pragma unroll
-  for (int i = ty; i < 32; i += 8) {
-    const int r = r0 + i;
-    float g = 0.f;
-    if (r < rows && f < F) {
-      const float o = in[(size_t)r * ldi + f];
-      if (MODE == 0) {
-        const float d = __fsub_rn(o, T[(size_t)smp_of[i] * ldt + f]);
-        if (fabsf(d) > 1e-10f && fabsf(d) < 1e15f) {
-          const float ph = __fmul_rn(d, d);
-          pair_add(lh, ll, ph, __fmaf_rn(d, d, -ph));
-        } else {
-          ld += (double)d * (double)d;
-        }
-        g = __fmul_rn(d, scale);
+  for (int k = 0; k < 4; ++k) {
+    const int i = w + 8 * k, r = r0 + i;
+    o[k] = t[k] = make_float2(0.f, 0.f);
+    if (r < rows && on0) {
+      const float* po = in + (size_t)r * ldi + f;
+      const float* pt = MODE == 0 ? T + (size_t)smp_of[i] * ldt + f : nullptr;
+      if (on1) {
+        o[k] = *reinterpret_cast<const float2*>(po);
+        if (MODE == 0) t[k] = *reinterpret_cast<const float2*>(pt);
       } else {
-        g = o;
+        o[k].x = *po;
+        if (MODE == 0) t[k].x = *pt;
       }
-      gb[(size_t)r * ldg + f] = __float2bfloat16_rn(g);
     }
-    tile[i][tx] = g;
+  }
+  auto square = [&](float d) {
+    if (fabsf(d) > 1e-10f && fabsf(d) < 1e15f) {
+      const float ph = __fmul_rn(d, d);
+      pair_add(lh, ll, ph, __fmaf_rn(d, d, -ph));
+    } else if (d != 0.f) {
+      ld += (double)d * (double)d;
+    }
+  };
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int i = w + 8 * k, r = r0 + i;
+    float2 g = o[k];
+    if (MODE == 0) {
+      const float2 d = make_float2(__fsub_rn(o[k].x, t[k].x), __fsub_rn(o[k].y, t[k].y));   // 0 outside the tile
+      square(d.x);
+      square(d.y);
+      g = make_float2(__fmul_rn(d.x, scale), __fmul_rn(d.y, scale));
+    }
+    if (r < rows && on0) {
+      bf16* p = gb + (size_t)r * ldg + f;
+      if (on1) *reinterpret_cast<__nv_bfloat162*>(p) = __floats2bfloat162_rn(g.x, g.y);
+      else *p = __float2bfloat16_rn(g.x);
+    }
+    tile[i][2 * lane] = g.x;
+    tile[i][2 * lane + 1] = g.y;
   }
   __syncthreads();
-  if (ty == 0 && f < F) {
+  if (threadIdx.x < GT_F && f0 + threadIdx.x < F) {
     float s = 0.f;
-    for (int i = 0; i < 32; ++i) s += tile[i][tx];
-    colpart[(size_t)blockIdx.y * ldc + f] = s;
+#pragma unroll
+    for (int i = 0; i < 32; ++i) s += tile[i][threadIdx.x];
+    colpart[(size_t)blockIdx.y * ldc + f0 + threadIdx.x] = s;
   }
-  for (int i = ty; i < 32; i += 8) {
-    const int ff = f0 + i, rr = r0 + tx;
-    if (ff < F && rr < rows) gt[(size_t)ff * ldgt + rr] = __float2bfloat16_rn(tile[tx][i]);
+  const int rp = 2 * (lane & 15), rr = r0 + rp;    // ldgt is even: pairs of rows in 4 bytes
+#pragma unroll
+  for (int k = 0; k < GT_F / 16; ++k) {
+    const int fl = 2 * (w + 8 * k) + (lane >> 4);
+    if (f0 + fl >= F || rr >= rows) continue;
+    bf16* p = gt + (size_t)(f0 + fl) * ldgt + rr;
+    if (rr + 1 < rows) *reinterpret_cast<__nv_bfloat162*>(p) = __floats2bfloat162_rn(tile[rp][fl], tile[rp + 1][fl]);
+    else *p = __float2bfloat16_rn(tile[rp][fl]);
   }
   if (MODE == 0) {
-    for (int o = 16; o > 0; o >>= 1) {
-      const float xh = __shfl_down_sync(0xffffffffu, lh, o), xl = __shfl_down_sync(0xffffffffu, ll, o);
+    for (int s = 16; s > 0; s >>= 1) {
+      const float xh = __shfl_down_sync(0xffffffffu, lh, s), xl = __shfl_down_sync(0xffffffffu, ll, s);
       pair_add(lh, ll, xh, xl);
     }
     if (__any_sync(0xffffffffu, ld != 0.0))       // warp-uniform (a NaN too)
-      for (int o = 16; o > 0; o >>= 1) ld += __shfl_down_sync(0xffffffffu, ld, o);
-    if (tx == 0) red[ty] = (double)lh + (double)ll + ld;
+      for (int s = 16; s > 0; s >>= 1) ld += __shfl_down_sync(0xffffffffu, ld, s);
+    if (lane == 0) red[w] = (double)lh + (double)ll + ld;
     __syncthreads();
-    if (tx == 0 && ty == 0) {
-      double t = 0.0;
-      for (int i = 0; i < 8; ++i) t += red[i];
-      lossp[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = t;
+    if (threadIdx.x == 0) {
+      double s = 0.0;
+      for (int i = 0; i < 8; ++i) s += red[i];
+      lossp[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = s;
     }
   }
 }
@@ -1453,9 +1484,9 @@ void backward(pdqp_ws_s* w, int rows, const float* T, long long a, long long sft
   const int F = w->F, Fp = w->Fp, mb = w->maxb;
   const int rt = (rows + 31) / 32;
   {
-    dim3 grid((F + 31) / 32, rt), blk(32, 8);
+    dim3 grid((F + GT_F - 1) / GT_F, rt);
     const float scale = (float)(2.0 / ((double)rows * F));
-    k_grad_tiles<0><<<grid, blk, 0, s>>>(w->O, Fp, T, Fp, a, sft, count, row0, rows, F, scale, w->dOb, Fp, w->dOt,
+    k_grad_tiles<0><<<grid, 256, 0, s>>>(w->O, Fp, T, Fp, a, sft, count, row0, rows, F, scale, w->dOb, Fp, w->dOt,
                                          mb, w->colpart, w->ldc, w->lossp);
     k_loss_acc<<<1, 1024, 0, s>>>(w->lossp, (int)(grid.x * grid.y), 1.0 / ((double)rows * F), w->lossacc);
   }
@@ -1473,8 +1504,8 @@ void backward(pdqp_ws_s* w, int rows, const float* T, long long a, long long sft
   for (int j = w->depth - 1; j >= 0; --j) {
     WsLayer& l = w->L[j];
     {
-      dim3 grid((l.out + 31) / 32, rt), blk(32, 8);
-      k_grad_tiles<1><<<grid, blk, 0, s>>>(w->G, l.out, nullptr, 0, 1, 0, 1LL << 62, 0, rows, l.out, 1.f, w->dZb,
+      dim3 grid((l.out + GT_F - 1) / GT_F, rt);
+      k_grad_tiles<1><<<grid, 256, 0, s>>>(w->G, l.out, nullptr, 0, 1, 0, 1LL << 62, 0, rows, l.out, 1.f, w->dZb,
                                            l.out, w->dZt, mb, w->colpart, w->ldc, nullptr);
     }
     k_colsum<<<(l.out + 255) / 256, 256, 0, s>>>(w->colpart, rt, l.out, w->ldc, l.gb);
