@@ -21,20 +21,20 @@ namespace pdqp {
 template <typename V>
 struct DualB {
   BCsr<V> A;
-  const V* __restrict__ xt;      // extrapolated primal point x_tilde
-  const V* __restrict__ yold;    // y^k
-  V* __restrict__ ynew;          // y^{k+1}
-  V* __restrict__ ybar;
-  const V* __restrict__ b;
-  const V* __restrict__ ylo;     // lower bound of inequality duals (mixed-mode shift) or null (0)
-  const StepEntry* __restrict__ tab;    // [instance][C]
+  const V* xt;      // extrapolated primal point x_tilde
+  const V* yold;    // y^k
+  V* ynew;          // y^{k+1}
+  V* ybar;
+  const V* b;
+  const V* ylo;     // lower bound of inequality duals (mixed-mode shift) or null (0)
+  const StepEntry* tab;    // [instance][C]
   const int* __restrict__ blk_inst;     // instance of each row block
-  const DevState* __restrict__ st;      // per instance
+  const DevState* st;      // per instance
   const unsigned char* __restrict__ ineq;   // per row: inequality
   int C;
   const int2* __restrict__ blk_seg;     // long rows: {first segment, segments} per block (null: none)
-  const V* __restrict__ lpart;          // segment sums of the long rows
-  const int* __restrict__ act;          // row block of each CUDA block (null: the block index)
+  const V* lpart;          // segment sums of the long rows
+  const int* act;          // row block of each CUDA block (null: the block index)
   int early;                            // launched by launch_early: no state read before grid_wait()
 };
 
@@ -105,7 +105,7 @@ __device__ __forceinline__ void dual_block(const DualB<V>& a, int bk, int j, V* 
   } else {   // a single row longer than a block
     V s = V(0);
     for (int e = e0 + tid; e < e0 + ne; e += NT)
-      s += a.A.val[e] * __ldg(a.xt + a.A.col[e]);
+      s += a.A.val[e] * a.xt[a.A.col[e]];
     s = block_sum(s);
     if (tid == 0) dual_row(a, a.tab[inst * a.C + j], r0, s, yo, bi, yb, lo);
   }
@@ -128,24 +128,24 @@ __global__ void __launch_bounds__(NT, MinBlocks<V, NT>::value) k_dual(DualB<V> a
 template <typename V>
 struct PrimalB {
   BCsr<V> P;
-  const V* __restrict__ zin;     // [x_md ; y^{k+1}] of this iteration
-  V* __restrict__ zout;          // x_md of the next iteration -> zout[0:n]
-  V* __restrict__ x;
-  V* __restrict__ xbar;
-  V* __restrict__ xt;            // x_tilde of the next iteration
-  const V* __restrict__ c;
-  const V* __restrict__ l;
-  const V* __restrict__ u;
-  const StepEntry* __restrict__ tab;    // [instance][C]
+  const V* zin;     // [x_md ; y^{k+1}] of this iteration
+  V* zout;          // x_md of the next iteration -> zout[0:n]
+  V* x;
+  V* xbar;
+  V* xt;            // x_tilde of the next iteration
+  const V* c;
+  const V* l;
+  const V* u;
+  const StepEntry* tab;    // [instance][C]
   const int* __restrict__ blk_inst;
-  const DevState* __restrict__ st;
+  const DevState* st;
   int C;
-  const V* __restrict__ F;              // low-rank factor F~ (null: none)
-  const V* __restrict__ wlr;            // F~' x_md of this iteration
+  const V* F;              // low-rank factor F~ (null: none)
+  const V* wlr;            // F~' x_md of this iteration
   int r;
   const int2* __restrict__ blk_seg;     // long rows: {first segment, segments} per block (null: none)
-  const V* __restrict__ lpart;          // segment sums of the long rows
-  const int* __restrict__ act;          // row block of each CUDA block (null: the block index)
+  const V* lpart;          // segment sums of the long rows
+  const int* act;          // row block of each CUDA block (null: the block index)
   int early;                            // launched by launch_early: no state read before grid_wait()
 };
 
@@ -203,7 +203,7 @@ __device__ __forceinline__ void primal_block(const PrimalB<V>& a, int bk, int j,
   } else {
     V s = V(0);
     for (int e = e0 + tid; e < e0 + ne; e += NT)
-      s += a.P.val[e] * __ldg(a.zin + a.P.col[e]);
+      s += a.P.val[e] * a.zin[a.P.col[e]];
     s = block_sum(s);
     if (tid == 0) primal_row<V, LR>(a, a.tab[inst * a.C + j], r0, s, xo, xb, cr, lr, ur);
   }
@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(NT) k_dual_pipe(DualB<V> a, const int4* __rest
 #pragma unroll
       for (int k = 0; k < BNNZ / NT; ++k) {
         const int e = tid + k * NT;
-        if (e < ne) sm.prod[e] = pipe_entry(sm.val[s][e + off], __ldg(a.xt + sm.col[s][e + off]));
+        if (e < ne) sm.prod[e] = pipe_entry(sm.val[s][e + off], a.xt[sm.col[s][e + off]]);
       }
       __syncthreads();
       for (int t = tid; t < nr; t += NT) {
@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(NT) k_dual_pipe(DualB<V> a, const int4* __rest
       }
     } else {
       V acc = V(0);
-      for (int e = e0 + tid; e < e0 + ne; e += NT) acc += a.A.val[e] * __ldg(a.xt + a.A.col[e]);
+      for (int e = e0 + tid; e < e0 + ne; e += NT) acc += a.A.val[e] * a.xt[a.A.col[e]];
       acc = block_sum(acc);
       if (tid == 0) dual_row(a, es, r0, acc, yo, bi, yb, lo);
     }
@@ -380,7 +380,7 @@ __global__ void __launch_bounds__(NT) k_primal_pipe(PrimalB<V> a, const int4* __
 #pragma unroll
       for (int k = 0; k < BNNZ / NT; ++k) {
         const int e = tid + k * NT;
-        if (e < ne) sm.prod[e] = pipe_entry(sm.val[s][e + off], __ldg(a.zin + sm.col[s][e + off]));
+        if (e < ne) sm.prod[e] = pipe_entry(sm.val[s][e + off], a.zin[sm.col[s][e + off]]);
       }
       __syncthreads();
       for (int t = tid; t < nr; t += NT) {
@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(NT) k_primal_pipe(PrimalB<V> a, const int4* __
       }
     } else {
       V acc = V(0);
-      for (int e = e0 + tid; e < e0 + ne; e += NT) acc += a.P.val[e] * __ldg(a.zin + a.P.col[e]);
+      for (int e = e0 + tid; e < e0 + ne; e += NT) acc += a.P.val[e] * a.zin[a.P.col[e]];
       acc = block_sum(acc);
       if (tid == 0) {
         if (a.F) primal_row<V, true>(a, es, r0, acc, xo, xb, cr, lr, ur);
@@ -573,18 +573,18 @@ struct FamIL {
   const int* __restrict__ col;
   const V* __restrict__ val;           // scaled values (the same for every member)
   int rows, ld;
-  const V* __restrict__ steps;         // [j - j0][IL_STEPS][ld] step scalars of the chunk (k_il_steps)
-  const int* __restrict__ run;         // [ld] the member iterates
-  const V* __restrict__ zin;           // gathered vector (x_tilde, or [x_md ; y+])
+  const V* steps;         // [j - j0][IL_STEPS][ld] step scalars of the chunk (k_il_steps)
+  const int* run;         // [ld] the member iterates
+  const V* zin;           // gathered vector (x_tilde, or [x_md ; y+])
   // dual: yold, ynew, ybar, b, ylo (may be null), ineq;  primal: x, xbar, zout, xt, c, l, u
-  const V* __restrict__ v0;
-  V* __restrict__ w0;
-  V* __restrict__ w1;
-  V* __restrict__ w2;
-  V* __restrict__ w3;
-  const V* __restrict__ r0;
-  const V* __restrict__ r1;
-  const V* __restrict__ r2;
+  const V* v0;
+  V* w0;
+  V* w1;
+  V* w2;
+  V* w3;
+  const V* r0;
+  const V* r1;
+  const V* r2;
   const unsigned char* __restrict__ ineq;
 };
 
@@ -596,7 +596,7 @@ constexpr int IL_LD_ALIGN = 128;       // members per warp in float32 (the leadi
 
 template <typename V>
 __device__ __forceinline__ void il_load(const V* p, V (&v)[IlVec<V>::W]) {
-  const typename IlVec<V>::T q = __ldg(reinterpret_cast<const typename IlVec<V>::T*>(p));
+  const typename IlVec<V>::T q = *reinterpret_cast<const typename IlVec<V>::T*>(p);
   if constexpr (IlVec<V>::W == 4) { v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w; }
   else { v[0] = q.x; v[1] = q.y; }
 }
@@ -621,10 +621,9 @@ __device__ __forceinline__ void il_store(V* p, const V (&v)[IlVec<V>::W]) {
 // this kernel) moves only the gathered members' values.  Every lane of the
 // warp runs it (the shuffles need the whole warp).
 template <typename V>
-__device__ __forceinline__ void il_row_sum(const FamIL<V>& a, int r, int m0, V (&s)[IlVec<V>::W]) {
+__device__ __forceinline__ void il_row_sum(const FamIL<V>& a, int e0, int e1, int m0, V (&s)[IlVec<V>::W]) {
   constexpr int W = IlVec<V>::W;
   const int lane = threadIdx.x & 31;
-  const int e0 = a.rp[r], e1 = a.rp[r + 1];
 #pragma unroll
   for (int q = 0; q < W; ++q) s[q] = V(0);
   for (int base = e0; base < e1; base += 32) {
@@ -690,7 +689,7 @@ __device__ __forceinline__ bool il_running(const FamIL<V>& a, int m0, int (&run)
   int any = 0;
 #pragma unroll
   for (int q = 0; q < IlVec<V>::W; ++q) {
-    run[q] = __ldg(a.run + m0 + q);
+    run[q] = a.run[m0 + q];
     any |= run[q];
   }
   return __any_sync(0xffffffffu, any != 0);
@@ -700,10 +699,13 @@ __device__ __forceinline__ bool il_running(const FamIL<V>& a, int m0, int (&run)
 template <typename V>
 __global__ void __launch_bounds__(IL_NT, 4) k_dual_il(FamIL<V> a, int k) {
   constexpr int W = IlVec<V>::W;
+  grid_trigger();
   const int lane = threadIdx.x & 31;
   const int r = blockIdx.x * IL_RPB + (threadIdx.x >> 5);
   if (r >= a.rows) return;
   const int m0 = blockIdx.y * 32 * W + lane * W;
+  const int e0 = __ldg(a.rp + r), e1 = __ldg(a.rp + r + 1);
+  grid_wait();
   int run[W];
   if (!il_running(a, m0, run)) return;
   const size_t idx = (size_t)r * a.ld + m0;
@@ -715,7 +717,7 @@ __global__ void __launch_bounds__(IL_NT, 4) k_dual_il(FamIL<V> a, int k) {
   else
 #pragma unroll
     for (int q = 0; q < W; ++q) lo[q] = V(0);
-  il_row_sum(a, r, m0, s);
+  il_row_sum(a, e0, e1, m0, s);
   const bool ineq = a.ineq[r] != 0;
   il_steps(a, k, IL_SIGMA, m0, sg);
   il_steps(a, k, IL_IB, m0, ib);
@@ -731,10 +733,13 @@ __global__ void __launch_bounds__(IL_NT, 4) k_dual_il(FamIL<V> a, int k) {
 template <typename V>
 __global__ void __launch_bounds__(IL_NT, 4) k_primal_il(FamIL<V> a, int k) {
   constexpr int W = IlVec<V>::W;
+  grid_trigger();
   const int lane = threadIdx.x & 31;
   const int r = blockIdx.x * IL_RPB + (threadIdx.x >> 5);
   if (r >= a.rows) return;
   const int m0 = blockIdx.y * 32 * W + lane * W;
+  const int e0 = __ldg(a.rp + r), e1 = __ldg(a.rp + r + 1);
+  grid_wait();
   int run[W];
   if (!il_running(a, m0, run)) return;
   const size_t idx = (size_t)r * a.ld + m0;
@@ -744,7 +749,7 @@ __global__ void __launch_bounds__(IL_NT, 4) k_primal_il(FamIL<V> a, int k) {
   il_load(a.r0 + idx, cr);
   il_load(a.r1 + idx, lr);
   il_load(a.r2 + idx, ur);
-  il_row_sum(a, r, m0, s);
+  il_row_sum(a, e0, e1, m0, s);
   il_steps(a, k, IL_TAU, m0, tau);
   il_steps(a, k, IL_IB, m0, ib);
   il_steps(a, k, IL_IBN, m0, ibn);
@@ -814,13 +819,13 @@ static void run_chunk_il(Work& w, int j0, int len, const V* Aval, const V* Pval,
       da.v0 = I[IL_Z0 + ((j + 1) & 1)] + (size_t)n * ld;   // y^k
       da.w0 = I[IL_Z0 + (j & 1)] + (size_t)n * ld;         // y^{k+1}
       if (Pr.on) Pr.begin(0, s, il_launch_bytes(w, 0, sizeof(V)));
-      launch(k_dual_il<V>, dim3(cdiv(m, IL_RPB), groups), IL_NT, 0, s, da, j - j0);
+      launch_early(k_dual_il<V>, dim3(cdiv(m, IL_RPB), groups), IL_NT, 0, s, da, j - j0);
       if (Pr.on) Pr.end(s);
     }
     pa.zin = I[IL_Z0 + (j & 1)];
     pa.w2 = I[IL_Z0 + ((j + 1) & 1)];
     if (Pr.on) Pr.begin(1, s, il_launch_bytes(w, 1, sizeof(V)));
-    launch(k_primal_il<V>, dim3(cdiv(n, IL_RPB), groups), IL_NT, 0, s, pa, j - j0);
+    launch_early(k_primal_il<V>, dim3(cdiv(n, IL_RPB), groups), IL_NT, 0, s, pa, j - j0);
     if (Pr.on) Pr.end(s);
   }
   // interleaved -> member-major: everything the iterations wrote

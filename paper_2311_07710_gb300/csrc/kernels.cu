@@ -302,9 +302,9 @@ __device__ __forceinline__ void kkt_m_group(const KktB& a, int g) {
     const int ne = a.A.rp[r1] - e0;
     if (ne <= BNNZ) {
       if (NIT == 2 && a.xx)
-        kkt_stage_pairs(a.A, e0, ne, r0, nr, sval, sx, srp, [&](int c) { return __ldg(a.xx + c); });
+        kkt_stage_pairs(a.A, e0, ne, r0, nr, sval, sx, srp, [&](int c) { return a.xx[c]; });
       else
-        kkt_stage<NIT>(a.A, e0, ne, r0, nr, sval, sx, srp, [&](int it, int c) { return __ldg(a.x[it] + c); });
+        kkt_stage<NIT>(a.A, e0, ne, r0, nr, sval, sx, srp, [&](int it, int c) { return a.x[it][c]; });
       __syncthreads();
       for (int q = tid; q < nr * NIT; q += BNT) {
         const int it = q >= nr ? 1 : 0, t = q - it * nr;
@@ -365,10 +365,10 @@ __device__ __forceinline__ void kkt_n_group(const KktB& a, int g) {
     if (ne <= BNNZ) {
       if (NIT == 2 && a.xx)
         kkt_stage_pairs(a.P, e0, ne, r0, nr, sval, sx, srp,
-                        [&](int c) { return c < n ? __ldg(a.xx + c) : __ldg(a.yy + (c - n)); });
+                        [&](int c) { return c < n ? a.xx[c] : a.yy[c - n]; });
       else
         kkt_stage<NIT>(a.P, e0, ne, r0, nr, sval, sx, srp, [&](int it, int c) {
-          return c < n ? __ldg(a.x[it] + c) : __ldg(a.y[it] + (c - n));
+          return c < n ? a.x[it][c] : a.y[it][c - n];
         });
       for (int t = tid; t < nr; t += BNT) ssp[t] = a.P.split[r0 + t] - e0;
       __syncthreads();
@@ -447,8 +447,8 @@ __global__ void __launch_bounds__(256) k_kkt_long(KktB a, const int4* __restrict
     const int c = M.col[e];
 #pragma unroll
     for (int it = 0; it < NIT; ++it) {
-      if (e < sp) s[it] = fma(v, __ldg(a.x[it] + c), s[it]);
-      else t[it] = fma(v, __ldg(a.y[it] + (c - a.n)), t[it]);
+      if (e < sp) s[it] = fma(v, a.x[it][c], s[it]);
+      else t[it] = fma(v, a.y[it][c - a.n], t[it]);
     }
   }
 #pragma unroll
@@ -676,8 +676,8 @@ __device__ __forceinline__ void reduce_kkt_fields(int bm0, int bm1, AtM at_m, in
   if (threadIdx.x == 0)
     for (int k = 0; k < 24; ++k) F[k] = f[k];
 }
-__device__ __forceinline__ void reduce_kkt_blocks(const double* __restrict__ pm, int nbm, int bm0, int bm1,
-                                                  const double* __restrict__ pn, int nbn, int bn0, int bn1, double* F) {
+__device__ __forceinline__ void reduce_kkt_blocks(const double* pm, int nbm, int bm0, int bm1,
+                                                  const double* pn, int nbn, int bn0, int bn1, double* F) {
   reduce_kkt_fields(
       bm0, bm1, [&](int k, int b) { return pm[(size_t)k * nbm + b]; }, bn0, bn1,
       [&](int k, int b) { return pn[(size_t)k * nbn + b]; }, F);
@@ -880,8 +880,8 @@ __device__ __forceinline__ double* lz_al(const LzArgs& a, int i, int o) { return
 __device__ __forceinline__ double* lz_be(const LzArgs& a, int i, int o) { return a.be + ((size_t)i * 2 + o) * LZ_MAX; }
 
 template <typename V, int NT>
-__global__ void __launch_bounds__(NT, MinBlocks<V, NT>::value) k_lz_m(BCsr<V> A, LzArgs la, const V* __restrict__ vA,
-                                                                   V* __restrict__ wm) {
+__global__ void __launch_bounds__(NT, MinBlocks<V, NT>::value) k_lz_m(BCsr<V> A, LzArgs la, const V* vA,
+                                                                   V* wm) {
   grid_trigger();
   grid_wait();
   const int bk = la.actA ? la.actA[blockIdx.x] : (int)blockIdx.x;
@@ -905,7 +905,7 @@ __global__ void __launch_bounds__(NT, MinBlocks<V, NT>::value) k_lz_m(BCsr<V> A,
     }
   } else {
     V s = V(0);
-    for (int e = e0 + tid; e < e0 + ne; e += NT) s += A.val[e] * r_mul(__ldg(vA + A.col[e]), gA);
+    for (int e = e0 + tid; e < e0 + ne; e += NT) s += A.val[e] * r_mul(vA[A.col[e]], gA);
     s = block_sum(s);
     if (tid == 0) wm[r0] = s;
   }
@@ -913,11 +913,11 @@ __global__ void __launch_bounds__(NT, MinBlocks<V, NT>::value) k_lz_m(BCsr<V> A,
 
 // rows of P with input [v_Q ; w_m]: wA = A~'w_m, wQ = Q~ v_Q; partial v'w per row block
 template <typename V, int NT, bool LR = false>
-__global__ void __launch_bounds__(NT, MinBlocks<V, NT, LR>::value) k_lz_n(BCsr<V> P, LzArgs la, const V* __restrict__ zin,
-                                                                   const V* __restrict__ vA, V* __restrict__ wA,
-                                                                   V* __restrict__ wQ, double* __restrict__ part,
-                                                                   const V* __restrict__ F,
-                                                                   const V* __restrict__ wlr, int rk) {
+__global__ void __launch_bounds__(NT, MinBlocks<V, NT, LR>::value) k_lz_n(BCsr<V> P, LzArgs la, const V* zin,
+                                                                   const V* vA, V* wA,
+                                                                   V* wQ, double* part,
+                                                                   const V* F,
+                                                                   const V* wlr, int rk) {
   grid_trigger();
   grid_wait();
   __shared__ __align__(16) V prod[BNNZ];
@@ -959,7 +959,7 @@ __global__ void __launch_bounds__(NT, MinBlocks<V, NT, LR>::value) k_lz_n(BCsr<V
     const int sp = P.split[r0];
     V q = V(0), w = V(0);
     for (int e = e0 + tid; e < e0 + ne; e += NT) {
-      const V x = __ldg(zin + P.col[e]);
+      const V x = zin[P.col[e]];
       const V v = P.val[e] * (e < sp ? r_mul(x, gQ) : x);
       if (e < sp) q += v; else w += v;
     }
@@ -978,7 +978,7 @@ __global__ void __launch_bounds__(NT, MinBlocks<V, NT, LR>::value) k_lz_n(BCsr<V
 
 // Per-thread sums of the two fields (part[b], part[stride + b]) over [b0, b1)
 // (stride blockDim): four independent accumulators, combined in a fixed order.
-__device__ __forceinline__ void lz_block_sums(const double* __restrict__ part, int nblkP, int b0, int b1,
+__device__ __forceinline__ void lz_block_sums(const double* part, int nblkP, int b0, int b1,
                                               double (&f)[2]) {
   double acc[2][4] = {{0.0, 0.0, 0.0, 0.0}, {0.0, 0.0, 0.0, 0.0}};
   const int st = blockDim.x;
@@ -1027,10 +1027,10 @@ __global__ void __launch_bounds__(NT) k_lz_alpha(LzArgs a) {
 // that the next step's three-term update reads as v_prev.  The update runs in
 // the vectors' precision (two FMAs), only |r|^2 in float64.
 template <typename V>
-__global__ void __launch_bounds__(256) k_lz_orth(LzArgs a, BCsr<V> P, const V* __restrict__ wA,
-                                                 const V* __restrict__ wQ, V* __restrict__ vA,
-                                                 V* __restrict__ vA_prev, V* __restrict__ vQ,
-                                                 V* __restrict__ vQ_prev, double* __restrict__ part,
+__global__ void __launch_bounds__(256) k_lz_orth(LzArgs a, BCsr<V> P, const V* wA,
+                                                 const V* wQ, V* vA,
+                                                 V* vA_prev, V* vQ,
+                                                 V* vQ_prev, double* part,
                                                  int own_alpha) {
   grid_trigger();
   grid_wait();
@@ -1076,8 +1076,8 @@ __global__ void __launch_bounds__(256) k_lz_orth(LzArgs a, BCsr<V> P, const V* _
     for (int u = 0; u < U; ++u) {
       const int rr = r + 32 * u;
       if (rr < r1) {
-        if (doA) { w[0][u] = __ldg(wA + rr); v[0][u] = vA[rr]; vp[0][u] = vA_prev[rr]; }
-        if (doQ) { w[1][u] = __ldg(wQ + rr); v[1][u] = vQ[rr]; vp[1][u] = vQ_prev[rr]; }
+        if (doA) { w[0][u] = wA[rr]; v[0][u] = vA[rr]; vp[0][u] = vA_prev[rr]; }
+        if (doQ) { w[1][u] = wQ[rr]; v[1][u] = vQ[rr]; vp[1][u] = vQ_prev[rr]; }
       }
     }
 #pragma unroll
@@ -1456,7 +1456,7 @@ __global__ void __launch_bounds__(NT) k_lz_beta(LzArgs a, double tol, int max_st
 
 // v_next = r / beta (in the buffer that held v_prev)
 template <typename V>
-__global__ void k_lz_norm(LzArgs a, V* __restrict__ vA_next, V* __restrict__ vQ_next) {
+__global__ void k_lz_norm(LzArgs a, V* vA_next, V* vQ_next) {
   grid_trigger();
   grid_wait();
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < a.n; r += gridDim.x * blockDim.x) {
@@ -1618,7 +1618,7 @@ __device__ void fill_steps_block(const DevState& S, const SolveParams& p, StepEn
   for (int j = threadIdx.x; j < p.check_period; j += blockDim.x) tab[j] = make_step(S.k_epoch + j, S, p);
 }
 
-__device__ void decide_thread0(DevState* __restrict__ st, const double* F, const SolveParams& p, int mode,
+__device__ void decide_thread0(DevState* st, const double* F, const SolveParams& p, int mode,
                                long long chunk_len, int inf_status);
 
 // Chunk sums of the relKKT group partials: CUDA block (i, c) reduces chunk c
@@ -1631,7 +1631,7 @@ constexpr int KKT_GPC = KKT_CHUNK / KKT_GROUP;   // groups per chunk (8: lanes 0
 // one chunk's sums of one side in a warp: first group g0 of the chunk, end of
 // the instance's groups ge; put(k, value) in lane 0
 template <int NF, unsigned MAXMASK, typename Put>
-__device__ __forceinline__ void kkt_chunk_sums(const double* __restrict__ part, int ng, int g0, int ge, Put put) {
+__device__ __forceinline__ void kkt_chunk_sums(const double* part, int ng, int g0, int ge, Put put) {
   const int lane = threadIdx.x & 31, g = g0 + lane;
   const bool on = lane < KKT_GPC && g < ge;
 #pragma unroll
@@ -1756,7 +1756,7 @@ __global__ void __launch_bounds__(1024) k_count_running(const DevState* __restri
   }
 }
 
-__device__ void decide_thread0(DevState* __restrict__ st, const double* F, const SolveParams& p, int mode,
+__device__ void decide_thread0(DevState* st, const double* F, const SolveParams& p, int mode,
                                long long chunk_len, int inf_status) {
   DevState& S = *st;
   double P[2][6];
@@ -1827,8 +1827,8 @@ __global__ void k_compact_blocks(const int* __restrict__ blk_inst, int nblk, con
     if (st[blk_inst[b]].status == ST_RUNNING) act[atomicAdd(n, 1)] = b;
 }
 
-__global__ void k_restart_apply(const DevState* __restrict__ sts, const int* __restrict__ inst_n,
-                                const int* __restrict__ inst_m, int n, int m, double* x, double* xbar,
+__global__ void k_restart_apply(const DevState* sts, const int* inst_n,
+                                const int* inst_m, int n, int m, double* x, double* xbar,
                                 double* xmd0, double* xt, double* ax, double* y, double* ybar, double* ay) {
   grid_trigger();
   grid_wait();

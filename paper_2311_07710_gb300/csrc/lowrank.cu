@@ -38,19 +38,19 @@ struct LrPrimal {
   const int* __restrict__ rp;
   const int* __restrict__ col;
   const V* __restrict__ val;
-  const V* __restrict__ zin;
-  V* __restrict__ zout;
-  V* __restrict__ x;
-  V* __restrict__ xbar;
-  V* __restrict__ xt;
-  const V* __restrict__ c;
-  const V* __restrict__ l;
-  const V* __restrict__ u;
-  const StepEntry* __restrict__ tab;
-  const DevState* __restrict__ st;
+  const V* zin;
+  V* zout;
+  V* x;
+  V* xbar;
+  V* xt;
+  const V* c;
+  const V* l;
+  const V* u;
+  const StepEntry* tab;
+  const DevState* st;
   const V* __restrict__ F;
-  const V* __restrict__ w;          // F' x_md of this iteration
-  double* __restrict__ part;        // [tiles][r] partials of the next iteration's
+  const V* w;          // F' x_md of this iteration
+  double* part;        // [tiles][r] partials of the next iteration's
   int n, r, per;
 };
 
@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(LRF_NT) k_primal_lr(LrPrimal<V> a, int j) {
     V s = V(0), xo = V(0), xb0 = V(0), cr = V(0), lr = V(0), ur = V(0);
     if (t < rows) {
       xo = a.x[row]; xb0 = a.xbar[row]; cr = a.c[row]; lr = a.l[row]; ur = a.u[row];
-      for (int k = a.rp[row]; k < a.rp[row + 1]; ++k) s = r_dot(a.val[k], __ldg(a.zin + a.col[k]), s);
+      for (int k = a.rp[row]; k < a.rp[row + 1]; ++k) s = r_dot(a.val[k], a.zin[a.col[k]], s);
     }
     if (base == 0) {
       asm volatile("cp.async.wait_all;\n" ::);
@@ -135,9 +135,9 @@ __global__ void __launch_bounds__(LRF_NT) k_primal_lr(LrPrimal<V> a, int j) {
 // segment sums of A's long rows (independent of each other, one launch).
 template <typename V>
 __global__ void __launch_bounds__(256)
-    k_lr_reduce_long(const double* __restrict__ part, int nparts, int r, double* __restrict__ w, float* __restrict__ wf,
-                     BCsr<V> A, const V* __restrict__ vec, const int4* __restrict__ lseg,
-                     const DevState* __restrict__ st, V* __restrict__ lpart) {
+    k_lr_reduce_long(const double* part, int nparts, int r, double* w, float* wf,
+                     BCsr<V> A, const V* vec, const int4* lseg,
+                     const DevState* st, V* lpart) {
   grid_trigger();
   grid_wait();
   if (st->status != ST_RUNNING) return;

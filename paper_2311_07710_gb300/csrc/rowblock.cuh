@@ -31,14 +31,14 @@ static inline void launch(void (*kern)(KArgs...), dim3 grid, int block, size_t s
 // a kernel calls grid_wait() before it touches anything an earlier kernel of
 // the iteration loop writes, and before any block of it ends.
 template <typename... KArgs, typename... Args>
-static inline void launch_early(void (*kern)(KArgs...), int grid, int block, size_t smem, cudaStream_t s,
+static inline void launch_early(void (*kern)(KArgs...), dim3 grid, int block, size_t smem, cudaStream_t s,
                                 Args... args) {
-  if (grid <= 0) return;
+  if (grid.x == 0 || grid.y == 0) return;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
@@ -48,7 +48,9 @@ static inline void launch_early(void (*kern)(KArgs...), int grid, int block, siz
   count_launch();
 }
 // the kernels before this one have ended and their writes are visible (returns
-// at once in a normal launch)
+// at once in a normal launch).  What they write is read by plain loads through
+// pointers without __restrict__: the compiler may move a non-coherent load
+// (__ldg) or one that it takes to alias nothing above the wait.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 // this block no longer holds back the next kernel's launch
 __device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
@@ -102,7 +104,7 @@ __device__ __forceinline__ void load4(const double* __restrict__ p, double (&v)[
 // SC: the gathered entries of the columns below csplit are multiplied by sc
 // first (a vector kept unnormalised, normalised where it is read).
 template <int NT, typename V, typename X, bool SC = false>
-__device__ __forceinline__ void stage_products(const BCsr<V>& M, const X* __restrict__ vec, int e0, int ne,
+__device__ __forceinline__ void stage_products(const BCsr<V>& M, const X* vec, int e0, int ne,
                                                int r0, int nr, V* prod, int* srp, int cmin = 0, V sc = V(1),
                                                int csplit = 0) {
   // float data: one quad (four gathers) per phase, so that 256 threads fit 32
@@ -149,13 +151,13 @@ __device__ __forceinline__ void stage_products(const BCsr<V>& M, const X* __rest
               const int c = ci[k][i];
               V p = V(0);
               if (c >= cmin) {
-                const V x = (V)__ldg(vec + c);
+                const V x = (V)vec[c];
                 p = vv[k][i] * (c < csplit ? r_mul(x, sc) : x);
               }
               prod[e] = p;
             }
           } else {
-            if (e >= 0 && e < ne) prod[e] = ci[k][i] >= cmin ? vv[k][i] * (V)__ldg(vec + ci[k][i]) : V(0);
+            if (e >= 0 && e < ne) prod[e] = ci[k][i] >= cmin ? vv[k][i] * (V)vec[ci[k][i]] : V(0);
           }
         }
       }
@@ -170,7 +172,7 @@ __device__ __forceinline__ void stage_products(const BCsr<V>& M, const X* __rest
 // gather: it waits for the kernels before this one and fetches the rows'
 // operands; false ends the staging.
 template <int NT, typename V, typename Mid>
-__device__ __forceinline__ bool stage_rows(const BCsr<V>& M, const V* __restrict__ vec, int e0, int ne, int r0, int nr,
+__device__ __forceinline__ bool stage_rows(const BCsr<V>& M, const V* vec, int e0, int ne, int r0, int nr,
                                            V* prod, V* sx, int* srp, Mid mid) {
   constexpr int QPT = BNNZ / NT / 4 + 1;           // quads per thread, one more for the misalignment
   constexpr int QPP = sizeof(V) == 4 ? 1 : 2;   // quads per phase (both phases' quads of one float64 pass in flight)
@@ -206,10 +208,10 @@ __device__ __forceinline__ bool stage_rows(const BCsr<V>& M, const V* __restrict
           const int e = 4 * q + i - o;
           if (e >= 0 && e < ne) {
             if constexpr (sizeof(V) == 4) {
-              prod[e] = vv[k][i] * __ldg(vec + ci[k][i]);
+              prod[e] = vv[k][i] * vec[ci[k][i]];
             } else {
               prod[e] = vv[k][i];
-              sx[e] = __ldg(vec + ci[k][i]);
+              sx[e] = vec[ci[k][i]];
             }
           }
         }
@@ -260,7 +262,7 @@ template <bool LR> struct MinBlocks<double, 512, LR> { static constexpr int valu
 
 // the row term F~_j . w (16-byte loads of the row when r allows)
 template <typename FV, typename V, typename W>
-__device__ __forceinline__ V lr_row(const FV* __restrict__ F, const W* __restrict__ w, int r, int j) {
+__device__ __forceinline__ V lr_row(const FV* F, const W* w, int r, int j) {
   V s = V(0);
   const FV* f = F + (size_t)j * r;
   constexpr int VW = 16 / sizeof(FV);
@@ -283,8 +285,8 @@ __device__ __forceinline__ V lr_row(const FV* __restrict__ F, const W* __restric
 // Column blk of F' v from the block partials of k_lr_ft (vec, k = blk / r, blk %
 // r): a fixed-order tree over 256 threads; a float32 copy for the float32
 // iteration.
-__device__ __forceinline__ void lr_reduce_column(const double* __restrict__ part, int nparts, int r, int nv, int blk,
-                                                 double* __restrict__ w, float* __restrict__ wf) {
+__device__ __forceinline__ void lr_reduce_column(const double* part, int nparts, int r, int nv, int blk,
+                                                 double* w, float* wf) {
   const int q = blk / r, kk = blk % r;
   __shared__ double sh[256];
   double s = 0.0;
@@ -303,10 +305,10 @@ __device__ __forceinline__ void lr_reduce_column(const double* __restrict__ part
 
 // the sum of one segment g = {row, first nonzero, end, row block} of a long row
 template <typename V>
-__device__ __forceinline__ void long_segment_sum(const BCsr<V>& M, const V* __restrict__ vec, int4 g,
-                                                 V* __restrict__ out) {
+__device__ __forceinline__ void long_segment_sum(const BCsr<V>& M, const V* vec, int4 g,
+                                                 V* out) {
   V s = V(0);
-  for (int e = g.y + threadIdx.x; e < g.z; e += 256) s += M.val[e] * __ldg(vec + M.col[e]);
+  for (int e = g.y + threadIdx.x; e < g.z; e += 256) s += M.val[e] * vec[M.col[e]];
   s = block_sum(s);
   if (threadIdx.x == 0) *out = s;
 }
