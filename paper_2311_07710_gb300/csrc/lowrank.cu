@@ -20,6 +20,7 @@
 namespace pdqp {
 
 constexpr int LRF_NT = 256;
+constexpr int LRF_PRE = 4;     // entries of a thread's first row fetched ahead
 
 // shared memory of a tile of `per` rows: F with rows padded so that 16-byte
 // accesses of consecutive rows meet different banks, x_md of the rows, w
@@ -83,7 +84,21 @@ __global__ void __launch_bounds__(LRF_NT) k_primal_lr(LrPrimal<V> a, int j) {
   V* zs = fs + (size_t)a.per * ld;
   V* ws = zs + ((a.per + 3) & ~3);
   lrf_stage<V>(fs, a.F + (size_t)j0 * r, rows, r);
-  grid_wait();                                     // (F is the solve's own: on its way before the wait)
+  // what no kernel of the chunk writes (F, P, c, l, u; the chunk's first kernel
+  // is launched normally) is on its way before the wait
+  V cr0 = V(0), lr0 = V(0), ur0 = V(0), pv[LRF_PRE];
+  int e0 = 0, e1 = 0, pc[LRF_PRE];
+  if (tid < rows) {
+    const int row = j0 + tid;
+    e0 = a.rp[row]; e1 = a.rp[row + 1];
+    cr0 = a.c[row]; lr0 = a.l[row]; ur0 = a.u[row];
+  }
+#pragma unroll
+  for (int k = 0; k < LRF_PRE; ++k) {
+    pc[k] = e0 + k < e1 ? a.col[e0 + k] : 0;
+    pv[k] = e0 + k < e1 ? a.val[e0 + k] : V(0);
+  }
+  grid_wait();
   if (a.st->status != ST_RUNNING) {
     asm volatile("cp.async.wait_all;\n" ::);
     return;
@@ -95,8 +110,21 @@ __global__ void __launch_bounds__(LRF_NT) k_primal_lr(LrPrimal<V> a, int j) {
     const int t = base + tid, row = j0 + t;
     V s = V(0), xo = V(0), xb0 = V(0), cr = V(0), lr = V(0), ur = V(0);
     if (t < rows) {
-      xo = a.x[row]; xb0 = a.xbar[row]; cr = a.c[row]; lr = a.l[row]; ur = a.u[row];
-      for (int k = a.rp[row]; k < a.rp[row + 1]; ++k) s = r_dot(a.val[k], a.zin[a.col[k]], s);
+      xo = a.x[row]; xb0 = a.xbar[row];
+      if (base == 0) {
+        V z[LRF_PRE];
+#pragma unroll
+        for (int k = 0; k < LRF_PRE; ++k) z[k] = e0 + k < e1 ? a.zin[pc[k]] : V(0);
+        cr = cr0; lr = lr0; ur = ur0;
+#pragma unroll
+        for (int k = 0; k < LRF_PRE; ++k)
+          if (e0 + k < e1) s = r_dot(pv[k], z[k], s);
+        for (int k = e0 + LRF_PRE; k < e1; ++k) s = r_dot(a.val[k], a.zin[a.col[k]], s);
+      } else {
+        cr = a.c[row]; lr = a.l[row]; ur = a.u[row];
+        const int q1 = a.rp[row + 1];
+        for (int k = a.rp[row]; k < q1; ++k) s = r_dot(a.val[k], a.zin[a.col[k]], s);
+      }
     }
     if (base == 0) {
       asm volatile("cp.async.wait_all;\n" ::);
@@ -139,10 +167,33 @@ __global__ void __launch_bounds__(256)
                      BCsr<V> A, const V* vec, const int4* lseg,
                      const DevState* st, V* lpart) {
   grid_trigger();
+  if ((int)blockIdx.x < r) {
+    grid_wait();
+    if (st->status != ST_RUNNING) return;
+    lr_reduce_column(part, nparts, r, 1, blockIdx.x, w, wf);
+    return;
+  }
+  // long_segment_sum with the segment's entries fetched before the wait
+  constexpr int PER = (LSEG + 255) / 256;
+  const int4 g = lseg[blockIdx.x - r];
+  V v[PER];
+  int c[PER];
+#pragma unroll
+  for (int k = 0; k < PER; ++k) {
+    const int e = g.y + threadIdx.x + 256 * k;
+    v[k] = e < g.z ? A.val[e] : V(0);
+    c[k] = e < g.z ? A.col[e] : 0;
+  }
   grid_wait();
   if (st->status != ST_RUNNING) return;
-  if ((int)blockIdx.x < r) lr_reduce_column(part, nparts, r, 1, blockIdx.x, w, wf);
-  else long_segment_sum(A, vec, lseg[blockIdx.x - r], lpart + (blockIdx.x - r));
+  V z[PER], s = V(0);
+#pragma unroll
+  for (int k = 0; k < PER; ++k) z[k] = g.y + threadIdx.x + 256 * k < g.z ? vec[c[k]] : V(0);
+#pragma unroll
+  for (int k = 0; k < PER; ++k)
+    if (g.y + (int)threadIdx.x + 256 * k < g.z) s += v[k] * z[k];
+  s = block_sum(s);
+  if (threadIdx.x == 0) lpart[blockIdx.x - r] = s;
 }
 
 // Low-rank row terms (F w0)_j and (F w1)_j of a float64 check: 64 rows of F
