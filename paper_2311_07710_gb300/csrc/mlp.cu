@@ -64,7 +64,37 @@ struct Epi {
   int ldo, ldm;
   int relu;
   int vec;                       // the outputs and the mask start on 16 (8) bytes: 4 columns per access
+  // The network's last product writes its prediction [px | py] = pmean + pstd * value
+  // in float64 (row lengths pn, N - pn; either array may be null) and nothing else.
+  const float *pmean = nullptr, *pstd = nullptr;
+  double *px = nullptr, *py = nullptr;
+  int pn = 0, pm = 0;
+  int pvec = 0;                  // pn and pm even, both arrays on 16 bytes: 2 columns per access
 };
+
+// A kernel of the network starts with early_start() and is launched by early():
+// its blocks are set up while the last blocks of the kernel before it still run
+// (every block of that kernel has started by then), and wait for its end before
+// they touch memory (plain loads through pointers without __restrict__, which
+// the compiler cannot move above the wait).  A training step is about 40 launches of a few microseconds:
+// the gaps between them were 0.8 of 5.0 ms for 2048 samples.
+__device__ __forceinline__ void early_start() {
+  asm volatile("griddepcontrol.launch_dependents;\ngriddepcontrol.wait;\n" ::: "memory");
+}
+template <typename... KArgs, typename... Args>
+static void early(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
+}
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -146,6 +176,55 @@ __device__ __forceinline__ float epi_value(float r, int row, int col, const Epi&
   return r;
 }
 
+constexpr int EPI_LD = 20;                     // floats per row of an epilogue warp's stage
+constexpr int EPI_WARPS = 8;
+constexpr int GEMM_NT = 64 + 32 * EPI_WARPS;   // TMA, MMA and epilogue warps
+
+// float -> double by integer instructions (the conversion instruction issues on
+// the float64 pipe): the same value for every float (NaN payloads aside)
+__device__ __forceinline__ double widen(float x) {
+  const unsigned u = __float_as_uint(x), e = (u >> 23) & 0xFFu;
+  if (e - 1u >= 254u) return (double)x;           // zero, subnormal, infinite, NaN
+  return __hiloint2double((int)((u & 0x80000000u) | (((u >> 3) & 0x0FFFFFFFu) + 0x38000000u)), (int)(u << 29));
+}
+
+// Where the prediction of (row, col) goes, or null.  Its value is
+// pmean + pstd * v: the product of two floats is exact in float64, so one fused
+// multiply-add rounds like the separate addition.
+__device__ __forceinline__ double* pred_at(const Epi& e, int row, int col) {
+  double* d = col < e.pn ? e.px : e.py;
+  return d ? d + (size_t)row * (col < e.pn ? e.pn : e.pm) + (col < e.pn ? col : col - e.pn) : nullptr;
+}
+__device__ __forceinline__ void put_value(const Epi& e, int row, int col, float x) {
+  if (e.pstd) {
+    if (double* d = pred_at(e, row, col)) *d = __fma_rn((double)e.pstd[col], (double)x, (double)e.pmean[col]);
+    return;
+  }
+  const size_t o = (size_t)row * e.ldo + col;
+  if (e.out_f) e.out_f[o] = x;
+  if (e.out_b) e.out_b[o] = __float2bfloat16_rn(x);
+}
+
+// The predictions of 32 rows x 16 columns staged as in store_chunk: eight lanes
+// store a row's 128 contiguous bytes, two columns each.  Two columns per lane
+// widen their statistics once for their eight rows; the value itself is widened
+// by integer instructions, which leaves the float64 pipe one operation a value.
+__device__ __forceinline__ void store_pred(const float* stg, int row0, int cb, const Epi& e) {
+  const int lane = threadIdx.x & 31, col = cb + (lane & 7) * 2, row = row0 + (lane >> 3);
+  double* d = pred_at(e, row, col);
+  if (!d) return;
+  const size_t ld = 4 * (size_t)(col < e.pn ? e.pn : e.pm);
+  const double s0 = widen(e.pstd[col]), s1 = widen(e.pstd[col + 1]);
+  const double m0 = widen(e.pmean[col]), m1 = widen(e.pmean[col + 1]);
+  const float b0 = e.bias ? e.bias[col] : 0.f, b1 = e.bias ? e.bias[col + 1] : 0.f;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    float2 v = *reinterpret_cast<const float2*>(stg + (4 * i + (lane >> 3)) * EPI_LD + (lane & 7) * 2);
+    if (e.bias) { v.x += b0; v.y += b1; }
+    *reinterpret_cast<double2*>(d + i * ld) = make_double2(__fma_rn(s0, widen(v.x), m0), __fma_rn(s1, widen(v.y), m1));
+  }
+}
+
 // Epilogue of a warp's 32 x 16 accumulator values (rows row0.., columns cb..
 // below nend), staged in `stg` (32 rows of EPI_LD floats): the raw float32 split-K
 // partial of split z (ld = N), or the fused epilogue into the outputs.  A lane
@@ -156,15 +235,16 @@ __device__ __forceinline__ float epi_value(float r, int row, int col, const Epi&
 // 64: 31 us with four epilogue warps, float32 or bf16 alike), so the common
 // case reads all its values first and takes its branches outside the loops,
 // and eight warps drain an accumulator, two per 32 TMEM lanes.
-constexpr int EPI_LD = 20;
-constexpr int EPI_WARPS = 8;
-constexpr int GEMM_NT = 64 + 32 * EPI_WARPS;   // TMA, MMA and epilogue warps
 __device__ __forceinline__ void store_chunk(const float* stg, int row0, int cb, int z, int M, int N, int nend,
-                                            const Epi& epi, float* __restrict__ partial) {
+                                            const Epi& epi, float* partial) {
   const int lane = threadIdx.x & 31;
   const bool vec = cb + 16 <= nend && row0 + 32 <= M && epi.vec &&
                    (partial ? (N & 3) == 0 : (epi.ldo & 3) == 0 && (!epi.mask || (epi.ldm & 3) == 0));
-  if (vec) {
+  if (epi.pvec && !partial && cb + 16 <= nend && row0 + 32 <= M) {
+    store_pred(stg, row0, cb, epi);
+    return;
+  }
+  if (vec && (partial || !epi.pstd)) {
     const int col = cb + (lane & 3) * 4, row = row0 + (lane >> 2);
     float4 v[4];
 #pragma unroll
@@ -177,8 +257,7 @@ __device__ __forceinline__ void store_chunk(const float* stg, int row0, int cb, 
       return;
     }
     if (epi.bias) {
-      const float4 b = make_float4(__ldg(epi.bias + col), __ldg(epi.bias + col + 1), __ldg(epi.bias + col + 2),
-                                   __ldg(epi.bias + col + 3));
+      const float4 b = make_float4(epi.bias[col], epi.bias[col + 1], epi.bias[col + 2], epi.bias[col + 3]);
 #pragma unroll
       for (int i = 0; i < 4; ++i) { v[i].x += b.x; v[i].y += b.y; v[i].z += b.z; v[i].w += b.w; }
     }
@@ -232,10 +311,7 @@ __device__ __forceinline__ void store_chunk(const float* stg, int row0, int cb, 
       partial[((size_t)z * M + row) * N + col] = v;
       continue;
     }
-    const float x = epi_value(v, row, col, epi);
-    const size_t o = (size_t)row * epi.ldo + col;
-    if (epi.out_f) epi.out_f[o] = x;
-    if (epi.out_b) epi.out_b[o] = __float2bfloat16_rn(x);
+    put_value(epi, row, col, epi_value(v, row, col, epi));
   }
 }
 
@@ -252,7 +328,7 @@ __device__ __forceinline__ void tmem_ld16(uint32_t (&v)[16], uint32_t taddr) {
 // One warp's share of an accumulator (TMEM base address of its lanes, columns
 // 16 half, 16 half + 32, ... of width) through its stage into the outputs.
 __device__ __forceinline__ void drain(float* stg, uint32_t tmem, int half, int width, int row0, int n0, int z, int M,
-                                      int N, const Epi& epi, float* __restrict__ partial) {
+                                      int N, const Epi& epi, float* partial) {
   const int lane = threadIdx.x & 31, nend = min(n0 + width, N);
   for (int c0 = 16 * half; c0 < width && n0 + c0 < N; c0 += 32) {
     uint32_t v[16];
@@ -282,7 +358,7 @@ __device__ __forceinline__ void drain(float* stg, uint32_t tmem, int half, int w
 template <int BN>
 __global__ void __launch_bounds__(GEMM_NT, 1)
     k_gemm_tn_p(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int M, int N,
-                int K, int ktps, int splits, Epi epi, float* __restrict__ partial, int* err) {
+                int K, int ktps, int splits, Epi epi, float* partial, int* err) {
   constexpr int STAGE_BYTES = Tile<BN>::STAGE_BYTES;
   extern __shared__ __align__(1024) unsigned char smraw[];
   unsigned char* sm = (unsigned char*)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
@@ -323,6 +399,7 @@ __global__ void __launch_bounds__(GEMM_NT, 1)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;\n");
   const uint32_t tmem = *tmem_slot;
+  early_start();
 
   // tiles in bands of GROUP tile rows, column-major inside a band: the CTAs
   // running together cover about GROUP rows of A and gridDim / GROUP columns of
@@ -476,7 +553,7 @@ __device__ __forceinline__ void commit_pair(uint64_t* bar) {   // arrives on thi
 
 __global__ void __launch_bounds__(GEMM_NT, 1) __cluster_dims__(2, 1, 1)
     k_gemm_tn_pair(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int M, int N,
-                   int K, int bn, int ktps, int splits, Epi epi, float* __restrict__ partial, int* err) {
+                   int K, int bn, int ktps, int splits, Epi epi, float* partial, int* err) {
   extern __shared__ __align__(1024) unsigned char smraw[];
   unsigned char* sm = (unsigned char*)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
   uint64_t* full = (uint64_t*)(sm + P_STAGES * P_STAGE_BYTES);
@@ -521,6 +598,7 @@ __global__ void __launch_bounds__(GEMM_NT, 1) __cluster_dims__(2, 1, 1)
   cluster_sync();                            // the peer's barriers are initialised
   asm volatile("tcgen05.fence::after_thread_sync;\n");
   const uint32_t tmem = *tmem_slot;
+  early_start();
 
   // tiles in bands of tile rows, as k_gemm_tn_p (4 x 256 rows)
   constexpr int GROUP = 4;
@@ -650,7 +728,8 @@ __global__ void k_wait_probe(int* err) {
 // Sum of the split-K partials in a fixed order, then the epilogue: W columns
 // per thread (4 where N and the leading dimensions allow), a row per grid y.
 template <int W>
-__global__ void __launch_bounds__(128) k_splitk_epi(const float* __restrict__ part, int splits, int M, int N, Epi epi) {
+__global__ void __launch_bounds__(128) k_splitk_epi(const float* part, int splits, int M, int N, Epi epi) {
+  early_start();
   const size_t MN = (size_t)M * N;
   const int col = (blockIdx.x * 128 + threadIdx.x) * W;
   if (col >= N) return;
@@ -667,13 +746,8 @@ __global__ void __launch_bounds__(128) k_splitk_epi(const float* __restrict__ pa
         r[0] += p[z * MN];
       }
     }
-    const size_t o = (size_t)row * epi.ldo + col;
 #pragma unroll
-    for (int i = 0; i < W; ++i) {
-      const float v = epi_value(r[i], row, col + i, epi);
-      if (epi.out_f) epi.out_f[o + i] = v;
-      if (epi.out_b) epi.out_b[o + i] = __float2bfloat16_rn(v);
-    }
+    for (int i = 0; i < W; ++i) put_value(epi, row, col + i, epi_value(r[i], row, col + i, epi));
   }
 }
 
@@ -694,7 +768,7 @@ constexpr int ROWS_PER = 16;
 constexpr int BATCH = 8;            // rows loaded before the first is used
 
 template <int W>
-__device__ __forceinline__ void load_cols(const double* __restrict__ p, double (&v)[W]) {
+__device__ __forceinline__ void load_cols(const double* p, double (&v)[W]) {
   if constexpr (W == 2) {
     const double2 q = __ldcs(reinterpret_cast<const double2*>(p));
     v[0] = q.x;
@@ -707,8 +781,9 @@ __device__ __forceinline__ void load_cols(const double* __restrict__ p, double (
 // u = bf16((fl32(v) - mean) * scale) for rows [row0, row0+rows) of v = [C | B]
 template <int W>
 __global__ void __launch_bounds__(256)
-    k_prep_input(const double* __restrict__ C, const double* __restrict__ B, int n, int m, long long row0, int rows,
-                 const float* __restrict__ mean, const float* __restrict__ scale, bf16* __restrict__ U, int ldu) {
+    k_prep_input(const double* C, const double* B, int n, int m, long long row0, int rows,
+                 const float* mean, const float* scale, bf16* U, int ldu) {
+  early_start();
   const int f = (blockIdx.x * 256 + threadIdx.x) * W;
   if (f >= n + m) return;
   const double* src = f < n ? C + (size_t)row0 * n + f : B + (size_t)row0 * m + (f - n);
@@ -738,8 +813,9 @@ __global__ void __launch_bounds__(256)
 // t = (fl32(v) - omean) * oinv, float32, for rows [0, count) of [X | Y]
 template <int W>
 __global__ void __launch_bounds__(256)
-    k_prep_target(const double* __restrict__ X, const double* __restrict__ Y, int n, int m, long long count,
-                  const float* __restrict__ omean, const float* __restrict__ oinv, float* __restrict__ T, int ldt) {
+    k_prep_target(const double* X, const double* Y, int n, int m, long long count,
+                  const float* omean, const float* oinv, float* T, int ldt) {
+  early_start();
   const int f = (blockIdx.x * 256 + threadIdx.x) * W;
   if (f >= n + m) return;
   const double* src = f < n ? X + f : Y + (f - n);
@@ -877,8 +953,9 @@ __global__ void __launch_bounds__(128) k_fit_merge(FitPair a, long long count, i
   if (o.stdv[z]) o.stdv[z][f] = (float)sd;
 }
 
-__global__ void k_gather_rows(const bf16* __restrict__ src, int ld, long long a, long long s, long long count,
-                              long long row0, int rows, int d, bf16* __restrict__ dst, int ldd) {
+__global__ void k_gather_rows(const bf16* src, int ld, long long a, long long s, long long count,
+                              long long row0, int rows, int d, bf16* dst, int ldd) {
+  early_start();
   const int vec = d / 8;   // d is a multiple of 8
   const long long total = (long long)rows * vec;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
@@ -898,11 +975,12 @@ __global__ void k_gather_rows(const bf16* __restrict__ src, int ld, long long a,
 // Every leading dimension is even.
 constexpr int GT_F = 64;
 template <int MODE>
-__global__ void __launch_bounds__(256) k_grad_tiles(const float* __restrict__ in, int ldi, const float* __restrict__ T,
+__global__ void __launch_bounds__(256) k_grad_tiles(const float* in, int ldi, const float* T,
                                                     int ldt, long long a, long long sft, long long count,
-                                                    long long row0, int rows, int F, float scale, bf16* __restrict__ gb,
-                                                    int ldg, bf16* __restrict__ gt, int ldgt,
-                                                    float* __restrict__ colpart, int ldc, double* __restrict__ lossp) {
+                                                    long long row0, int rows, int F, float scale, bf16* gb,
+                                                    int ldg, bf16* gt, int ldgt,
+                                                    float* colpart, int ldc, double* lossp) {
+  early_start();
   __shared__ float tile[32][GT_F + 1];
   __shared__ double red[8];
   __shared__ long long smp_of[32];
@@ -996,7 +1074,8 @@ __global__ void __launch_bounds__(256) k_grad_tiles(const float* __restrict__ in
   }
 }
 
-__global__ void k_colsum(const float* __restrict__ part, int ntiles, int F, int ld, float* __restrict__ out) {
+__global__ void k_colsum(const float* part, int ntiles, int F, int ld, float* out) {
+  early_start();
   const int f = blockIdx.x * blockDim.x + threadIdx.x;
   if (f >= F) return;
   float s = 0.f;
@@ -1005,8 +1084,9 @@ __global__ void k_colsum(const float* __restrict__ part, int ntiles, int F, int 
 }
 
 // acc += inv * sum(parts) (one block of 1024 threads, fixed order)
-__global__ void __launch_bounds__(1024) k_loss_acc(const double* __restrict__ parts, int n, double inv,
-                                                   double* __restrict__ acc) {
+__global__ void __launch_bounds__(1024) k_loss_acc(const double* parts, int n, double inv,
+                                                   double* acc) {
+  early_start();
   __shared__ double red[32];
   double s = 0.0;
 #pragma unroll 4
@@ -1021,8 +1101,9 @@ __global__ void __launch_bounds__(1024) k_loss_acc(const double* __restrict__ pa
   }
 }
 
-__global__ void k_transpose_bf16(const bf16* __restrict__ in, int ldi, int rows, int cols, bf16* __restrict__ out,
+__global__ void k_transpose_bf16(const bf16* in, int ldi, int rows, int cols, bf16* out,
                                  int ldo) {
+  early_start();
   __shared__ bf16 t[32][34];
   const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
   for (int i = threadIdx.y; i < 32; i += blockDim.y) {
@@ -1053,10 +1134,11 @@ __device__ __forceinline__ float adam_one(float w, float g, float& m, float& v, 
 // for the copies): 64 x 64 tiles, four columns per thread in 16-byte accesses,
 // the transposed copy in 128-byte runs.
 constexpr int ADAM_T = 64;
-__global__ void __launch_bounds__(256) k_adam_mat(float* __restrict__ W, float* __restrict__ mW,
-                                                  float* __restrict__ vW, const float* __restrict__ g, int rows,
-                                                  int cols, AdamArgs a, bf16* __restrict__ Wb, int ldb,
-                                                  bf16* __restrict__ Wt, int ldt) {
+__global__ void __launch_bounds__(256) k_adam_mat(float* W, float* mW,
+                                                  float* vW, const float* g, int rows,
+                                                  int cols, AdamArgs a, bf16* Wb, int ldb,
+                                                  bf16* Wt, int ldt) {
+  early_start();
   __shared__ bf16 t[ADAM_T][ADAM_T + 2];          // [column][row]
   const int c0 = blockIdx.x * ADAM_T, r0 = blockIdx.y * ADAM_T;
   const int cl = (threadIdx.x & 15) * 4, c = c0 + cl;
@@ -1100,8 +1182,9 @@ __global__ void __launch_bounds__(256) k_adam_mat(float* __restrict__ W, float* 
   }
 }
 
-__global__ void k_adam_vec(float* __restrict__ b, float* __restrict__ mb, float* __restrict__ vb,
-                           const float* __restrict__ g, int n, AdamArgs a) {
+__global__ void k_adam_vec(float* b, float* mb, float* vb,
+                           const float* g, int n, AdamArgs a) {
+  early_start();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n || !a.update) return;
   float m = mb[i], v = vb[i];
@@ -1115,58 +1198,6 @@ __global__ void k_f32_to_bf16_2d(const float* __restrict__ in, int rows, int col
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
     const int r = (int)(i / cols), c = (int)(i % cols);
     out[(size_t)r * ldo + c] = __float2bfloat16_rn(in[i]);
-  }
-}
-
-// float -> double by integer instructions (the conversion instruction issues on
-// the float64 pipe): the same value for every float (NaN payloads aside)
-__device__ __forceinline__ double widen(float x) {
-  const unsigned u = __float_as_uint(x), e = (u >> 23) & 0xFFu;
-  if (e - 1u >= 254u) return (double)x;           // zero, subnormal, infinite, NaN
-  return __hiloint2double((int)((u & 0x80000000u) | (((u >> 3) & 0x0FFFFFFFu) + 0x38000000u)), (int)(u << 29));
-}
-
-// [x0 | y0] = omean + ostd * o in float64, rows [row0, row0+rows).  The product
-// of two floats is exact in float64, so one fused multiply-add rounds like the
-// separate addition: one float64-pipe operation per value instead of five.
-template <int W>
-__global__ void __launch_bounds__(256)
-    k_write_pred(const float* __restrict__ O, int ldo, int rows, int n, int m, const float* __restrict__ omean,
-                 const float* __restrict__ ostd, long long row0, double* __restrict__ X0, double* __restrict__ Y0) {
-  const int f = (blockIdx.x * 256 + threadIdx.x) * W;
-  if (f >= n + m) return;
-  double* dst = f < n ? X0 : Y0;
-  if (!dst) return;
-  const size_t ld = f < n ? n : m;
-  dst += (size_t)row0 * ld + (f < n ? f : f - n);
-  double mu[W], sd[W];
-#pragma unroll
-  for (int i = 0; i < W; ++i) { mu[i] = (double)omean[f + i]; sd[i] = (double)ostd[f + i]; }
-  const int r1 = min(rows, (int)(blockIdx.y + 1) * ROWS_PER);
-  for (int r = blockIdx.y * ROWS_PER; r < r1; r += BATCH) {
-    float o[BATCH][W];
-#pragma unroll
-    for (int k = 0; k < BATCH; ++k) {
-      if (r + k >= r1) break;
-      const float* p = O + (size_t)(r + k) * ldo + f;
-      if constexpr (W == 2) {
-        const float2 q = __ldcs(reinterpret_cast<const float2*>(p));
-        o[k][0] = q.x;
-        o[k][1] = q.y;
-      } else {
-        o[k][0] = __ldcs(p);
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < BATCH; ++k) {
-      if (r + k >= r1) break;
-      double* d = dst + (r + k) * ld;
-      if constexpr (W == 2)
-        *reinterpret_cast<double2*>(d) =
-            make_double2(__fma_rn(sd[0], widen(o[k][0]), mu[0]), __fma_rn(sd[1], widen(o[k][1]), mu[1]));
-      else
-        *d = __fma_rn(sd[0], widen(o[k][0]), mu[0]);
-    }
   }
 }
 
@@ -1295,20 +1326,20 @@ cudaError_t gemm_tn(const bf16* A, int lda, const bf16* B, int ldb, int M, int N
   const int bm = plan.pair ? 2 * BM : BM;
   const long long units = (long long)((N + BN - 1) / BN) * ((M + bm - 1) / bm) * sp;
   if (plan.pair)
-    k_gemm_tn_pair<<<2 * (int)std::min<long long>(units, num_sms() / 2), GEMM_NT, P_SMEM_BYTES, s>>>(
-        ma, mb, M, N, K, BN, ktps, sp, ep, work, err);
+    early(k_gemm_tn_pair, 2 * (int)std::min<long long>(units, num_sms() / 2), GEMM_NT, P_SMEM_BYTES, s, ma, mb, M, N,
+          K, BN, ktps, sp, ep, work, err);
   else if (BN == 256)
-    k_gemm_tn_p<256><<<(int)std::min<long long>(units, num_sms()), GEMM_NT, Tile<256>::SMEM_BYTES, s>>>(
-        ma, mb, M, N, K, ktps, sp, ep, work, err);
+    early(k_gemm_tn_p<256>, (int)std::min<long long>(units, num_sms()), GEMM_NT, Tile<256>::SMEM_BYTES, s, ma, mb, M,
+          N, K, ktps, sp, ep, work, err);
   else
-    k_gemm_tn_p<128><<<(int)std::min<long long>(units, num_sms()), GEMM_NT, Tile<128>::SMEM_BYTES, s>>>(
-        ma, mb, M, N, K, ktps, sp, ep, work, err);
+    early(k_gemm_tn_p<128>, (int)std::min<long long>(units, num_sms()), GEMM_NT, Tile<128>::SMEM_BYTES, s, ma, mb, M,
+          N, K, ktps, sp, ep, work, err);
   if (sp > 1) {
     const int rows = std::min(M, 32768);
     if ((N & 3) == 0 && ((uintptr_t)work & 15) == 0)
-      k_splitk_epi<4><<<dim3((N / 4 + 127) / 128, rows), 128, 0, s>>>(work, sp, M, N, epi);
+      early(k_splitk_epi<4>, dim3((N / 4 + 127) / 128, rows), 128, 0, s, work, sp, M, N, epi);
     else
-      k_splitk_epi<1><<<dim3((N + 127) / 128, rows), 128, 0, s>>>(work, sp, M, N, epi);
+      early(k_splitk_epi<1>, dim3((N + 127) / 128, rows), 128, 0, s, work, sp, M, N, epi);
   }
   return cudaGetLastError();
 }
@@ -1467,13 +1498,21 @@ Epi epi_of(float* of, bf16* ob, int ldo, const float* bias, int relu, const bf16
 }
 
 // forward from H[0] (rows x d) to O; hidden activations in H[1..depth]
-void forward(pdqp_ws_s* w, int rows, cudaStream_t s) {
+// (with x0 or y0: to the prediction of rows from those pointers on)
+void forward(pdqp_ws_s* w, int rows, cudaStream_t s, double* x0 = nullptr, double* y0 = nullptr) {
   for (int j = 0; j < w->depth; ++j) {
     const WsLayer& l = w->L[j];
     gemm(w, w->H[j], l.in, l.Wb, l.in, rows, l.out, l.in, epi_of(nullptr, w->H[j + 1], l.out, l.b, 1), s);
   }
   const WsLayer& o = w->L[w->depth];
-  gemm(w, w->H[w->depth], o.in, o.Wb, o.in, rows, w->F, o.in, epi_of(w->O, nullptr, w->Fp, o.b, 0), s);
+  Epi e = epi_of(w->O, nullptr, w->Fp, o.b, 0);
+  if (x0 || y0) {
+    e.out_f = nullptr;
+    e.pmean = w->out_mean; e.pstd = w->out_std;
+    e.px = x0; e.py = y0; e.pn = w->n; e.pm = w->m;
+    e.pvec = two_columns(w->n, w->m, x0, y0);
+  }
+  gemm(w, w->H[w->depth], o.in, o.Wb, o.in, rows, w->F, o.in, e, s);
 }
 
 // Backward of the mean squared error against targets T (the target of row r
@@ -1486,16 +1525,16 @@ void backward(pdqp_ws_s* w, int rows, const float* T, long long a, long long sft
   {
     dim3 grid((F + GT_F - 1) / GT_F, rt);
     const float scale = (float)(2.0 / ((double)rows * F));
-    k_grad_tiles<0><<<grid, 256, 0, s>>>(w->O, Fp, T, Fp, a, sft, count, row0, rows, F, scale, w->dOb, Fp, w->dOt,
-                                         mb, w->colpart, w->ldc, w->lossp);
-    k_loss_acc<<<1, 1024, 0, s>>>(w->lossp, (int)(grid.x * grid.y), 1.0 / ((double)rows * F), w->lossacc);
+    early(k_grad_tiles<0>, grid, 256, 0, s, w->O, Fp, T, Fp, a, sft, count, row0, rows, F, scale, w->dOb, Fp, w->dOt,
+          mb, w->colpart, w->ldc, w->lossp);
+    early(k_loss_acc, 1, 1024, 0, s, w->lossp, (int)(grid.x * grid.y), 1.0 / ((double)rows * F), w->lossacc);
   }
   WsLayer& o = w->L[w->depth];
-  k_colsum<<<(F + 255) / 256, 256, 0, s>>>(w->colpart, rt, F, w->ldc, o.gb);
+  early(k_colsum, (F + 255) / 256, 256, 0, s, w->colpart, rt, F, w->ldc, o.gb);
   {
     const int c = o.in;
     dim3 grid((c + 31) / 32, rt), blk(32, 8);
-    k_transpose_bf16<<<grid, blk, 0, s>>>(w->H[w->depth], c, rows, c, w->Ht[w->depth], mb);
+    early(k_transpose_bf16, grid, blk, 0, s, w->H[w->depth], c, rows, c, w->Ht[w->depth], mb);
   }
   // gW_out = dO' H_depth  (F x width), K = rows
   gemm(w, w->dOt, mb, w->Ht[w->depth], mb, F, o.in, rows, epi_of(o.gW, nullptr, o.in, nullptr, 0), s);
@@ -1505,13 +1544,13 @@ void backward(pdqp_ws_s* w, int rows, const float* T, long long a, long long sft
     WsLayer& l = w->L[j];
     {
       dim3 grid((l.out + GT_F - 1) / GT_F, rt);
-      k_grad_tiles<1><<<grid, 256, 0, s>>>(w->G, l.out, nullptr, 0, 1, 0, 1LL << 62, 0, rows, l.out, 1.f, w->dZb,
-                                           l.out, w->dZt, mb, w->colpart, w->ldc, nullptr);
+      early(k_grad_tiles<1>, grid, 256, 0, s, w->G, l.out, nullptr, 0, 1, 0, 1LL << 62, 0, rows, l.out, 1.f, w->dZb,
+            l.out, w->dZt, mb, w->colpart, w->ldc, nullptr);
     }
-    k_colsum<<<(l.out + 255) / 256, 256, 0, s>>>(w->colpart, rt, l.out, w->ldc, l.gb);
+    early(k_colsum, (l.out + 255) / 256, 256, 0, s, w->colpart, rt, l.out, w->ldc, l.gb);
     {
       dim3 grid((l.in + 31) / 32, rt), blk(32, 8);
-      k_transpose_bf16<<<grid, blk, 0, s>>>(w->H[j], l.in, rows, l.in, w->Ht[j], mb);
+      early(k_transpose_bf16, grid, blk, 0, s, w->H[j], l.in, rows, l.in, w->Ht[j], mb);
     }
     gemm(w, w->dZt, mb, w->Ht[j], mb, l.out, l.in, rows, epi_of(l.gW, nullptr, l.in, nullptr, 0), s);
     if (j > 0)
@@ -1532,8 +1571,8 @@ void adam(pdqp_ws_s* w, float lr, float b1, float b2, float eps, cudaStream_t s)
   a.update = 1;
   for (WsLayer& l : w->L) {
     dim3 grid((l.in + ADAM_T - 1) / ADAM_T, (l.out + ADAM_T - 1) / ADAM_T);
-    k_adam_mat<<<grid, 256, 0, s>>>(l.W, l.mW, l.vW, l.gW, l.out, l.in, a, l.Wb, l.in, l.Wt, l.ldt);
-    k_adam_vec<<<(l.out + 255) / 256, 256, 0, s>>>(l.b, l.mb, l.vb, l.gb, l.out, a);
+    early(k_adam_mat, grid, 256, 0, s, l.W, l.mW, l.vW, l.gW, l.out, l.in, a, l.Wb, l.in, l.Wt, l.ldt);
+    early(k_adam_vec, (l.out + 255) / 256, 256, 0, s, l.b, l.mb, l.vb, l.gb, l.out, a);
   }
 }
 
@@ -1541,7 +1580,7 @@ void refresh_copies(WsLayer& l, cudaStream_t s) {
   AdamArgs a{};
   a.update = 0;
   dim3 grid((l.in + ADAM_T - 1) / ADAM_T, (l.out + ADAM_T - 1) / ADAM_T);
-  k_adam_mat<<<grid, 256, 0, s>>>(l.W, l.mW, l.vW, l.gW, l.out, l.in, a, l.Wb, l.in, l.Wt, l.ldt);
+  early(k_adam_mat, grid, 256, 0, s, l.W, l.mW, l.vW, l.gW, l.out, l.in, a, l.Wb, l.in, l.Wt, l.ldt);
 }
 
 // the elementwise kernels' grid over `rows` rows of arrays p, q
@@ -1553,8 +1592,7 @@ dim3 row_grid(const pdqp_ws_s* w, const void* p, const void* q, long long rows) 
 // normalised inputs of rows [row0, row0+rows) -> U -> H0 = U P'
 void project(pdqp_ws_s* w, const double* C, const double* B, long long row0, int rows, bf16* H0, cudaStream_t s) {
   auto prep = two_columns(w->n, w->m, C, B) ? k_prep_input<2> : k_prep_input<1>;
-  prep<<<row_grid(w, C, B, rows), 256, 0, s>>>(C, B, w->n, w->m, row0, rows, w->in_mean,
-                                                                w->in_scale, w->U, w->Fp);
+  early(prep, row_grid(w, C, B, rows), 256, 0, s, C, B, w->n, w->m, row0, rows, w->in_mean, w->in_scale, w->U, w->Fp);
   gemm(w, w->U, w->Fp, w->P, w->Fp, rows, w->d, w->F, epi_of(nullptr, H0, w->d, nullptr, 0), s);
 }
 
@@ -1861,8 +1899,8 @@ pdqp_status pdqp_ws_grad(pdqp_ws_handle w, const double* C, const double* B, con
         x(X, (size_t)count * n, mem, s), y(Y, (size_t)count * m, mem, s);
     float* T = walloc<float>(w, (size_t)count * w->Fp);
     try {
-      (two_columns(n, m, x.p, y.p) ? k_prep_target<2> : k_prep_target<1>)<<<row_grid(w, x.p, y.p, count), 256, 0, s>>>(
-          x.p, y.p, n, m, count, w->out_mean, w->out_inv, T, w->Fp);
+      early((two_columns(n, m, x.p, y.p) ? k_prep_target<2> : k_prep_target<1>), row_grid(w, x.p, y.p, count), 256,
+            0, s, x.p, y.p, n, m, count, w->out_mean, w->out_inv, T, w->Fp);
       project(w, c.p, b.p, 0, (int)count, w->H[0], s);
       forward(w, (int)count, s);
       WCK(cudaMemsetAsync(w->lossacc, 0, sizeof(double), s));
@@ -1916,8 +1954,8 @@ pdqp_status pdqp_ws_train(pdqp_ws_handle w, const pdqp_ws_train_options* opt, co
     }
     {
       DevView<double> x(X, (size_t)count * n, mem, s), y(Y, (size_t)count * m, mem, s);
-      (two_columns(n, m, x.p, y.p) ? k_prep_target<2> : k_prep_target<1>)<<<row_grid(w, x.p, y.p, count), 256, 0, s>>>(
-          x.p, y.p, n, m, count, w->out_mean, w->out_inv, w->Tall, Fp);
+      early((two_columns(n, m, x.p, y.p) ? k_prep_target<2> : k_prep_target<1>), row_grid(w, x.p, y.p, count), 256,
+            0, s, x.p, y.p, n, m, count, w->out_mean, w->out_inv, w->Tall, Fp);
       finish(w, s);
     }
     const long long steps = count / batch;
@@ -1927,8 +1965,8 @@ pdqp_status pdqp_ws_train(pdqp_ws_handle w, const pdqp_ws_train_options* opt, co
       WCK(cudaMemsetAsync(w->lossacc, 0, sizeof(double), s));
       for (long long st = 0; st < steps; ++st) {
         const long long row0 = st * batch;
-        k_gather_rows<<<grid_for((long long)batch * d / 8), 256, 0, s>>>(w->H0all, d, a, sft, count, row0, batch, d,
-                                                                         w->H[0], d);
+        early(k_gather_rows, grid_for((long long)batch * d / 8), 256, 0, s, w->H0all, d, a, sft, count, row0, batch,
+              d, w->H[0], d);
         forward(w, batch, s);
         backward(w, batch, w->Tall, a, sft, count, row0, s);
         adam(w, opt->lr, opt->beta1, opt->beta2, opt->eps, s);
@@ -1964,9 +2002,7 @@ pdqp_status pdqp_ws_infer(pdqp_ws_handle w, const double* C, const double* B, in
       for (long long r0 = 0; r0 < count; r0 += w->maxb) {
         const int rows = (int)std::min<long long>(w->maxb, count - r0);
         project(w, c.p, b.p, r0, rows, w->H[0], s);
-        forward(w, rows, s);
-        (two_columns(n, m, x0, y0) ? k_write_pred<2> : k_write_pred<1>)<<<row_grid(w, x0, y0, rows), 256, 0, s>>>(w->O, w->Fp, rows, n, m, w->out_mean,
-                                                                      w->out_std, r0, x0, y0);
+        forward(w, rows, s, x0 ? x0 + (size_t)r0 * n : nullptr, y0 ? y0 + (size_t)r0 * m : nullptr);
       }
       finish(w, s);
       if (tx) WCK(cudaMemcpy(X0, tx, (size_t)count * n * sizeof(double), cudaMemcpyDeviceToHost));
