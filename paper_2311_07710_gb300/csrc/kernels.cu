@@ -2604,7 +2604,7 @@ Profiler::~Profiler() {
 // (pick_lanes), so at most MAX_ROWS / 8 blocks ever touch the scratch
 static_assert(PDQP_NOALLOC_MAX_BLOCKS * (256 / 32) >= PDQP_NOALLOC_MAX_ROWS, "noalloc scratch too small");
 
-// 8192 blocks x 32 partial sums x 8 bytes = 2 MiB per device.
+// 2 x 8192 blocks (of A, of Q and A') x 16 partial sums x 8 bytes = 2 MiB per device.
 static __device__ __align__(256) double g_noalloc_scratch[PDQP_NOALLOC_MAX_BLOCKS * 32];
 // blocks of the call in flight that have written their partial sums
 static __device__ unsigned g_noalloc_ticket;
@@ -2628,95 +2628,188 @@ struct NoallocArgs {
   Csr<double> A, Q, At;
   const double *x, *y, *b, *c, *l, *u;
   int n, m, m_eq, LA, LN, gm, gn;
-  double* part;         // [max(gm, gn)][32]
-  unsigned* ticket;     // 0 at launch
+  double* part;         // [gm + gn][NOALLOC_LD] (k_kkt_noalloc)
+  unsigned* ticket;     // 0 at launch (k_kkt_noalloc)
   double* out;
 };
 
-// Relative KKT error (Section 5 "Progress metric", equality/bound form) in
-// float64 of one point on the original problem, on separate Q, A, A' arrays.
-// Blocks [0, gm) take rows of A, blocks [gm, gm + gn) rows of Q and A', L lanes
-// per row; the last block to finish folds the partial sums.  A control-loop
-// problem (n = 172) is all latency: one launch behind the ticket's reset took
-// the place of a 2 KB reset and three launches.
-__global__ void __launch_bounds__(256) k_kkt_noalloc(NoallocArgs a) {
-  if ((int)blockIdx.x < a.gm) {
-    // fields: 0 max|viol|, 1 max|Ax|, 2 b'y, 8 max|b| (3..7 stay 0)
-    double f[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-    const int L = a.LA, row = blockIdx.x * (256 / L) + threadIdx.x / L, lane = threadIdx.x & (L - 1);
+// The fields of a relKKT evaluation on separate Q, A, A' arrays: maxima (of
+// values >= 0) first, then sums.  A block of rows of A fills NA_VIOL, NA_AX,
+// NA_B and NA_BY, a block of rows of Q and A' the others.
+enum { NA_VIOL = 0, NA_AX, NA_B, NA_RES, NA_QX, NA_ATY, NA_C, NA_MAXIMA, NA_BY = NA_MAXIMA, NA_XQX, NA_CX, NA_BTERM,
+       NA_FIELDS };
+
+// The fields of this thread's row (L lanes a row; lane 0 of them holds the row's).
+__device__ __forceinline__ void noalloc_row(const NoallocArgs& a, int blk, int nt, double (&f)[NA_FIELDS]) {
+#pragma unroll
+  for (int k = 0; k < NA_FIELDS; ++k) f[k] = 0.0;
+  if (blk < a.gm) {
+    const int L = a.LA, row = blk * (nt / L) + threadIdx.x / L, lane = threadIdx.x & (L - 1);
     const bool valid = row < a.m;
-    double s = 0.0;
-    if (valid)
-      for (int k = a.A.rp[row] + lane; k < a.A.rp[row + 1]; k += L) s = fma(a.A.val[k], a.x[a.A.col[k]], s);
+    double s = 0.0, bi = 0.0, yi = 0.0;
+    if (valid) {
+      const int e1 = a.A.rp[row + 1];
+      if (lane == 0) { bi = a.b[row]; yi = a.y[row]; }
+      for (int k = a.A.rp[row] + lane; k < e1; k += L) s = fma(a.A.val[k], a.x[a.A.col[k]], s);
+    }
     s = lanes_sum(s, L);
     if (valid && lane == 0) {
-      const double bi = a.b[row];
-      f[0] = row < a.m_eq ? fabs(s - bi) : fmax(bi - s, 0.0);
-      f[1] = fabs(s);
-      f[2] = bi * a.y[row];
-      f[8] = fabs(bi);
+      f[NA_VIOL] = row < a.m_eq ? fabs(s - bi) : fmax(bi - s, 0.0);
+      f[NA_AX] = fabs(s);
+      f[NA_B] = fabs(bi);
+      f[NA_BY] = bi * yi;
     }
-    const bool is_max[9] = {true, true, false, false, true, true, false, false, true};
-    block_reduce<9>(f, is_max);
-    if (threadIdx.x == 0)
-      for (int k = 0; k < 9; ++k) a.part[(size_t)blockIdx.x * 32 + k] = f[k];
-  } else {
-    // fields: 0 max|res|, 1 max|Qx|, 2 max|A'y|, 3 x'Qx, 4 c'x, 5 sum(l lam+ - u lam-), 14 max|c|
-    double f[15];
-#pragma unroll
-    for (int k = 0; k < 15; ++k) f[k] = 0.0;
-    const int blk = (int)blockIdx.x - a.gm;
-    const int L = a.LN, row = blk * (256 / L) + threadIdx.x / L, lane = threadIdx.x & (L - 1);
+  } else if (blk < a.gm + a.gn) {
+    const int L = a.LN, row = (blk - a.gm) * (nt / L) + threadIdx.x / L, lane = threadIdx.x & (L - 1);
     const bool valid = row < a.n;
-    double sq = 0.0, sa = 0.0;
+    double sq = 0.0, sa = 0.0, cj = 0.0, lj = 0.0, uj = 0.0, xj = 0.0;
     if (valid) {
-      for (int k = a.Q.rp[row] + lane; k < a.Q.rp[row + 1]; k += L) sq = fma(a.Q.val[k], a.x[a.Q.col[k]], sq);
-      if (a.m > 0)
-        for (int k = a.At.rp[row] + lane; k < a.At.rp[row + 1]; k += L) sa = fma(a.At.val[k], a.y[a.At.col[k]], sa);
+      const int q1 = a.Q.rp[row + 1], t0 = a.m > 0 ? a.At.rp[row] : 0, t1 = a.m > 0 ? a.At.rp[row + 1] : 0;
+      if (lane == 0) { cj = a.c[row]; lj = a.l[row]; uj = a.u[row]; xj = a.x[row]; }
+      for (int k = a.Q.rp[row] + lane; k < q1; k += L) sq = fma(a.Q.val[k], a.x[a.Q.col[k]], sq);
+      for (int k = t0 + lane; k < t1; k += L) sa = fma(a.At.val[k], a.y[a.At.col[k]], sa);
     }
     sq = lanes_sum(sq, L);
     sa = lanes_sum(sa, L);
     if (valid && lane == 0) {
-      const double cj = a.c[row], lj = a.l[row], uj = a.u[row], xj = a.x[row];
       const bool lf = isfinite(lj), uf = isfinite(uj);
       const double g = sq + cj - sa;
       const double lam = (lf && uf) ? g : (lf ? fmax(g, 0.0) : (uf ? fmin(g, 0.0) : 0.0));
-      f[0] = fabs(g - lam);
-      f[1] = fabs(sq);
-      f[2] = fabs(sa);
-      f[3] = xj * sq;
-      f[4] = cj * xj;
-      f[5] = (lam > 0.0 ? lj * lam : 0.0) - (lam < 0.0 ? uj * (-lam) : 0.0);
-      f[14] = fabs(cj);
+      f[NA_RES] = fabs(g - lam);
+      f[NA_QX] = fabs(sq);
+      f[NA_ATY] = fabs(sa);
+      f[NA_C] = fabs(cj);
+      f[NA_XQX] = xj * sq;
+      f[NA_CX] = cj * xj;
+      f[NA_BTERM] = (lam > 0.0 ? lj * lam : 0.0) - (lam < 0.0 ? uj * (-lam) : 0.0);
     }
-    const bool is_max[15] = {true, true, true, false, false, false, false,
-                             true, true, true, false, false, false, false, true};
-    block_reduce<15>(f, is_max);
-    if (threadIdx.x == 0)
-      for (int k = 0; k < 15; ++k) a.part[(size_t)blk * 32 + 9 + k] = f[k];
+  }
+}
+
+// The fields over a warp, of which every L-th lane holds values: maxima by
+// integers (nmax), a sum's tree stops at the lanes that hold none.
+__device__ __forceinline__ void noalloc_warp(double (&f)[NA_FIELDS], int L, bool rows_of_A) {
+  for (int o = 16; o >= L; o >>= 1) {
+#pragma unroll
+    for (int k = 0; k < NA_FIELDS; ++k) {
+      const bool of_A = k <= NA_B || k == NA_BY;
+      if (of_A != rows_of_A) continue;             // uniform over the block
+      const double t = __shfl_xor_sync(0xffffffffu, f[k], o);
+      f[k] = k < NA_MAXIMA ? nmax(f[k], t) : f[k] + t;
+    }
+  }
+}
+
+// one field over the lanes of a warp
+__device__ __forceinline__ double noalloc_fold(double v, bool is_max) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double t = __shfl_xor_sync(0xffffffffu, v, o);
+    v = is_max ? nmax(v, t) : v + t;
+  }
+  return v;
+}
+
+__device__ __forceinline__ void noalloc_out(const double* F, double* out) {
+  double G[24];
+#pragma unroll
+  for (int k = 0; k < 24; ++k) G[k] = 0.0;
+  G[0] = F[NA_VIOL]; G[1] = F[NA_AX]; G[2] = F[NA_BY]; G[8] = F[NA_B];
+  G[9] = F[NA_RES]; G[10] = F[NA_QX]; G[11] = F[NA_ATY]; G[12] = F[NA_XQX]; G[13] = F[NA_CX]; G[14] = F[NA_BTERM];
+  G[23] = F[NA_C];
+  kkt_from_fields(G, 0, out);
+}
+
+// Relative KKT error (Section 5 "Progress metric", equality/bound form) in
+// float64 of one point on the original problem, on separate Q, A, A' arrays.
+// Blocks [0, gm) take rows of A, blocks [gm, gm + gn) rows of Q and A', L lanes
+// per row; the last block to finish folds the partial sums (one warp per field).
+constexpr int NOALLOC_NT = 256;
+constexpr int NOALLOC_LD = 16;                     // doubles per block in the scratch
+static_assert(NOALLOC_LD >= NA_FIELDS && sizeof(g_noalloc_scratch) / sizeof(double) >= 2 * PDQP_NOALLOC_MAX_BLOCKS * NOALLOC_LD,
+              "noalloc scratch too small");
+__global__ void __launch_bounds__(NOALLOC_NT) k_kkt_noalloc(NoallocArgs a) {
+  __shared__ double sh[NOALLOC_NT / 32][NA_FIELDS];
+  __shared__ double F[NA_FIELDS];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const bool rows_of_A = (int)blockIdx.x < a.gm;
+  double f[NA_FIELDS];
+  noalloc_row(a, blockIdx.x, NOALLOC_NT, f);
+  noalloc_warp(f, rows_of_A ? a.LA : a.LN, rows_of_A);
+  if (lane == 0)
+#pragma unroll
+    for (int k = 0; k < NA_FIELDS; ++k) sh[w][k] = f[k];
+  __syncthreads();
+  if (threadIdx.x < NA_FIELDS) {
+    const int k = threadIdx.x;
+    double t = sh[0][k];
+    for (int q = 1; q < NOALLOC_NT / 32; ++q) t = k < NA_MAXIMA ? nmax(t, sh[q][k]) : t + sh[q][k];
+    a.part[(size_t)blockIdx.x * NOALLOC_LD + k] = t;
+    __threadfence();
   }
   __shared__ bool last;
+  __syncthreads();
   if (threadIdx.x == 0) {
-    __threadfence();
     last = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
     __threadfence();
   }
   __syncthreads();
   if (!last) return;
-  double f[24];
-#pragma unroll
-  for (int k = 0; k < 24; ++k) f[k] = 0.0;
-  const bool is_max[24] = {true, true, false, false, true, true, false, false, true,
-                           true, true, true, false, false, false, false,
-                           true, true, true, false, false, false, false, true};
-  for (int b = threadIdx.x; b < max(a.gm, a.gn); b += 256)
-#pragma unroll
-    for (int k = 0; k < 24; ++k) {
-      const double v = b < (k < 9 ? a.gm : a.gn) ? __ldcg(a.part + (size_t)b * 32 + k) : 0.0;
-      f[k] = is_max[k] ? nmax(f[k], v) : f[k] + v;
+  for (int k = w; k < NA_FIELDS; k += NOALLOC_NT / 32) {
+    const bool of_A = k <= NA_B || k == NA_BY;
+    const int b0 = of_A ? 0 : a.gm, b1 = of_A ? a.gm : a.gm + a.gn;
+    double v = 0.0;
+    for (int b = b0 + lane; b < b1; b += 32) {
+      const double t = __ldcg(a.part + (size_t)b * NOALLOC_LD + k);
+      v = k < NA_MAXIMA ? nmax(v, t) : v + t;
     }
-  block_reduce<24>(f, is_max);
-  if (threadIdx.x == 0) kkt_from_fields(f, 0, a.out);
+    v = noalloc_fold(v, k < NA_MAXIMA);
+    if (lane == 0) F[k] = v;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) noalloc_out(F, a.out);
+}
+
+// The same for a problem whose rows fill at most eight blocks of 512 threads: one
+// cluster, whose first block reads the others' fields from their shared memory.
+// A control-loop problem (n = 172) is all latency: no counter to reset before
+// the launch, and no trip of the partial sums through L2.
+constexpr int NOALLOC_CNT = 512;
+constexpr int NOALLOC_CMAX = 8;
+__global__ void __launch_bounds__(NOALLOC_CNT) k_kkt_noalloc_cluster(NoallocArgs a) {
+  constexpr int NW = NOALLOC_CNT / 32;
+  __shared__ double sh[NW][NA_FIELDS];
+  __shared__ double F[NA_FIELDS];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, ctas = gridDim.x;
+  const bool rows_of_A = (int)blockIdx.x < a.gm;
+  double f[NA_FIELDS];
+  noalloc_row(a, blockIdx.x, NOALLOC_CNT, f);
+  noalloc_warp(f, rows_of_A ? a.LA : a.LN, rows_of_A);
+  if (lane == 0)
+#pragma unroll
+    for (int k = 0; k < NA_FIELDS; ++k) sh[w][k] = f[k];
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+  if (blockIdx.x == 0) {
+    if (w < NA_FIELDS) {                            // one warp per field: NW values of every CTA
+      const unsigned base = (unsigned)__cvta_generic_to_shared(&sh[0][w]);
+      double v = 0.0;
+      for (int q = lane; q < ctas * NW; q += 32) {
+        unsigned at;
+        double t;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n"
+                     : "=r"(at)
+                     : "r"(base + (unsigned)((q % NW) * NA_FIELDS * sizeof(double))), "r"(q / NW));
+        asm volatile("ld.shared::cluster.f64 %0, [%1];\n" : "=d"(t) : "r"(at) : "memory");
+        v = w < NA_MAXIMA ? nmax(v, t) : v + t;
+      }
+      v = noalloc_fold(v, w < NA_MAXIMA);
+      if (lane == 0) F[w] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) noalloc_out(F, a.out);
+  }
+  // no CTA leaves while its fields are read
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
 
 }  // namespace pdqp
@@ -2775,9 +2868,7 @@ extern "C" pdqp_status pdqp_kkt_noalloc(int64_t n, int64_t m, int64_t m_eq, cons
   const int LN = pdqp::pick_lanes(nnz_Q + nnz_A, n);
   const int gm = m > 0 ? pdqp::cdiv(m, 256 / LA) : 0;
   const int gn = pdqp::cdiv(n, 256 / LN);
-  const int nblk = gm > gn ? gm : gn;
-  if (nblk > PDQP_NOALLOC_MAX_BLOCKS) return PDQP_ERR_INVALID;   // unreachable by the sizes above
-  if (cudaMemsetAsync(mem.ticket, 0, sizeof(unsigned), s) != cudaSuccess) return PDQP_ERR_CUDA;
+  if (gm + gn > 2 * PDQP_NOALLOC_MAX_BLOCKS) return PDQP_ERR_INVALID;   // unreachable by the sizes above
   pdqp::NoallocArgs a{};
   a.A = Csr<double>{A_rowptr, A_col, A_val};
   a.Q = Csr<double>{Q_rowptr, Q_col, Q_val};
@@ -2786,6 +2877,27 @@ extern "C" pdqp_status pdqp_kkt_noalloc(int64_t n, int64_t m, int64_t m_eq, cons
   a.n = (int)n; a.m = (int)m; a.m_eq = (int)m_eq;
   a.LA = LA; a.LN = LN; a.gm = gm; a.gn = gn;
   a.part = mem.scratch; a.ticket = mem.ticket; a.out = parts;
-  pdqp::launch(pdqp::k_kkt_noalloc, gm + gn, 256, 0, s, a);
+  const int cm = m > 0 ? pdqp::cdiv(m, pdqp::NOALLOC_CNT / LA) : 0, cn = pdqp::cdiv(n, pdqp::NOALLOC_CNT / LN);
+  if (cm + cn <= pdqp::NOALLOC_CMAX) {
+    int ctas = 1;                                   // 1, 2, 4 or 8: a CTA beyond the rows adds zeros
+    while (ctas < cm + cn) ctas *= 2;
+    a.gm = cm; a.gn = cn;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = ctas;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(pdqp::NOALLOC_CNT);
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, pdqp::k_kkt_noalloc_cluster, a);
+    pdqp::count_launch();
+  } else {
+    if (cudaMemsetAsync(mem.ticket, 0, sizeof(unsigned), s) != cudaSuccess) return PDQP_ERR_CUDA;
+    pdqp::launch(pdqp::k_kkt_noalloc, gm + gn, pdqp::NOALLOC_NT, 0, s, a);
+  }
   return cudaGetLastError() == cudaSuccess ? PDQP_OK : PDQP_ERR_CUDA;
 }
