@@ -360,7 +360,7 @@ void alloc_il(pdqp_problem* h, bool mixed, int period) {
     if (mixed && !w.ilf[k]) w.ilf[k] = dalloc<float>(h, len[k] * ld);
     if (!mixed && !w.ild[k]) w.ild[k] = dalloc<double>(h, len[k] * ld);
   }
-  if (!w.il_run) w.il_run = dalloc<int>(h, ld);
+  if (!w.il_slot) w.il_slot = dalloc<int>(h, ld);
   int& have = w.il_steps_len[mixed ? 1 : 0];
   if (have < period) {   // a longer check period replaces the buffer the graphs point into
     if (mixed) w.il_steps_f = dalloc<float>(h, 5 * (size_t)period * ld);

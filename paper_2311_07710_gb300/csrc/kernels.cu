@@ -517,23 +517,17 @@ struct KktIL {
   double* sA[2];                                 // interleaved row sums: A x [m x ld]
   double* sQ[2];                                 // Q x [n x ld]
   double* sT[2];                                 // A'y [n x ld] (P's -A' part summed)
-  int n, m, ld, count;
-  const DevState* st;
+  int n, m, ld;
+  const int* slot;                               // [ld] member, or -1
 };
 
 constexpr int KIL_MEM = 64;   // members per warp (two float64 per lane)
 
 __global__ void __launch_bounds__(256, 4) k_kkt_sums_il(KktIL a, int side) {
-  __shared__ int run_any;
   const int lane = threadIdx.x & 31, r = blockIdx.x * 8 + (threadIdx.x >> 5);
   const int m0 = blockIdx.y * KIL_MEM + 2 * lane;
-  const bool run0 = m0 < a.count && a.st[m0].status == ST_RUNNING;
-  const bool run1 = m0 + 1 < a.count && a.st[m0 + 1].status == ST_RUNNING;
-  if (threadIdx.x == 0) run_any = 0;
-  __syncthreads();
-  if (run0 || run1) run_any = 1;
-  __syncthreads();
-  if (!run_any) return;
+  const bool on = a.slot[m0] >= 0;          // slots are filled from the first on
+  if (!__any_sync(0xffffffffu, on)) return;
   const int rows = side == 0 ? a.m : a.n;
   if (r >= rows) return;    // uniform over the warp: every lane stays for the shuffles
   const size_t ld = (size_t)a.ld;
@@ -551,6 +545,7 @@ __global__ void __launch_bounds__(256, 4) k_kkt_sums_il(KktIL a, int side) {
       for (int k = 0; k < cnt; ++k) {
         const double v = __shfl_sync(0xffffffffu, vl, k);
         const size_t c = (size_t)(__shfl_sync(0xffffffffu, cl, k) - coff) * ld + m0;
+        if (!on) continue;
         const double2 z0 = __ldg(reinterpret_cast<const double2*>(z[0] + c));
         const double2 z1 = __ldg(reinterpret_cast<const double2*>(z[1] + c));
         s[part][0][0] = r_fma(v, z0.x, s[part][0][0]);
@@ -563,12 +558,14 @@ __global__ void __launch_bounds__(256, 4) k_kkt_sums_il(KktIL a, int side) {
   const size_t idx = (size_t)r * ld + m0;
   if (side == 0) {
     accum(a.colA, a.valA, a.rpA[r], a.rpA[r + 1], 0, a.x, 0);
+    if (!on) return;
     for (int it = 0; it < 2; ++it)
       *reinterpret_cast<double2*>(a.sA[it] + idx) = make_double2(s[0][it][0], s[0][it][1]);
   } else {
     const int sp = a.splitP[r];
     accum(a.colP, a.valP, a.rpP[r], sp, 0, a.x, 0);
     accum(a.colP, a.valP, sp, a.rpP[r + 1], 1, a.y, a.n);
+    if (!on) return;
     for (int it = 0; it < 2; ++it) {
       *reinterpret_cast<double2*>(a.sQ[it] + idx) = make_double2(s[0][it][0], s[0][it][1]);
       *reinterpret_cast<double2*>(a.sT[it] + idx) = make_double2(s[1][it][0], s[1][it][1]);
@@ -620,30 +617,59 @@ __global__ void __launch_bounds__(BNT) k_kkt_n_sums(KktB a, const double* __rest
     for (int k = 0; k < 15; ++k) a.part_n[(size_t)k * a.ngrp_n + blockIdx.x] = f[k];
 }
 
+// The slots of a family's interleaved vectors: the running members in order,
+// then -1.  One CUDA block; rank by ballots and a scan over the warps.
+__global__ void __launch_bounds__(1024) k_il_slots(const DevState* __restrict__ st, int count, int ld,
+                                                   int* __restrict__ slot) {
+  __shared__ int sums[32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int total = 0;
+  for (int base = 0; base < count; base += 1024) {
+    const int mem = base + threadIdx.x;
+    const bool on = mem < count && st[mem].status == ST_RUNNING;
+    const unsigned ball = __ballot_sync(0xffffffffu, on);
+    if (lane == 0) sums[w] = __popc(ball);
+    __syncthreads();
+    int before = 0, all = 0;
+    for (int q = 0; q < 32; ++q) {
+      if (q < w) before += sums[q];
+      all += sums[q];
+    }
+    if (on) slot[total + before + __popc(ball & ((1u << lane) - 1u))] = mem;
+    total += all;
+    __syncthreads();
+  }
+  for (int k = total + threadIdx.x; k < ld; k += 1024) slot[k] = -1;
+}
+void il_slots(Work& w, cudaStream_t s) {
+  launch(k_il_slots, 1, 1024, 0, s, (const DevState*)w.st, w.fam_count, w.fam_ld, w.il_slot);
+}
+
 // the check's relKKT partials of a family handle through the interleaved sums
 static void launch_kkt_il(Work& w, const KktB& a, cudaStream_t s) {
   const int n = w.fam_n, m = w.fam_m, cnt = w.fam_count, ld = w.fam_ld;
   double* const* I = w.ilk;
-  to_il<double>(a.x[0], n, n, cnt, I[ILK_X0], ld, s);
-  to_il<double>(a.x[1], n, n, cnt, I[ILK_X1], ld, s);
-  to_il<double>(a.y[0], m, m, cnt, I[ILK_Y0], ld, s);
-  to_il<double>(a.y[1], m, m, cnt, I[ILK_Y1], ld, s);
+  il_slots(w, s);
+  to_il<double>(a.x[0], n, n, w.il_slot, cnt, I[ILK_X0], ld, s);
+  to_il<double>(a.x[1], n, n, w.il_slot, cnt, I[ILK_X1], ld, s);
+  to_il<double>(a.y[0], m, m, w.il_slot, cnt, I[ILK_Y0], ld, s);
+  to_il<double>(a.y[1], m, m, w.il_slot, cnt, I[ILK_Y1], ld, s);
   KktIL k{};
   k.rpA = w.A.rp; k.colA = w.A.col; k.valA = w.A.sval;
   k.rpP = w.P.rp; k.colP = w.famP_col; k.valP = w.P.sval; k.splitP = w.P.split;
   k.x[0] = I[ILK_X0]; k.x[1] = I[ILK_X1]; k.y[0] = I[ILK_Y0]; k.y[1] = I[ILK_Y1];
   k.sA[0] = I[ILK_SA0]; k.sA[1] = I[ILK_SA1];
   k.sQ[0] = I[ILK_SQ0]; k.sQ[1] = I[ILK_SQ1]; k.sT[0] = I[ILK_ST0]; k.sT[1] = I[ILK_ST1];
-  k.n = n; k.m = m; k.ld = ld; k.count = cnt; k.st = w.st;
+  k.n = n; k.m = m; k.ld = ld; k.slot = w.il_slot;
   if (m > 0) launch(k_kkt_sums_il, dim3(cdiv(m, 8), ld / KIL_MEM), 256, 0, s, k, 0);
   launch(k_kkt_sums_il, dim3(cdiv(n, 8), ld / KIL_MEM), 256, 0, s, k, 1);
   double* const* S = w.kks;
-  from_il<double>(I[ILK_SA0], ld, m, cnt, S[0], m, s);
-  from_il<double>(I[ILK_SA1], ld, m, cnt, S[1], m, s);
-  from_il<double>(I[ILK_SQ0], ld, n, cnt, S[2], n, s);
-  from_il<double>(I[ILK_SQ1], ld, n, cnt, S[3], n, s);
-  from_il<double>(I[ILK_ST0], ld, n, cnt, S[4], n, s);
-  from_il<double>(I[ILK_ST1], ld, n, cnt, S[5], n, s);
+  from_il<double>(I[ILK_SA0], ld, m, w.il_slot, cnt, S[0], m, s);
+  from_il<double>(I[ILK_SA1], ld, m, w.il_slot, cnt, S[1], m, s);
+  from_il<double>(I[ILK_SQ0], ld, n, w.il_slot, cnt, S[2], n, s);
+  from_il<double>(I[ILK_SQ1], ld, n, w.il_slot, cnt, S[3], n, s);
+  from_il<double>(I[ILK_ST0], ld, n, w.il_slot, cnt, S[4], n, s);
+  from_il<double>(I[ILK_ST1], ld, n, w.il_slot, cnt, S[5], n, s);
   if (w.m > 0) launch(k_kkt_m_sums, w.ngrp_A, BNT, 0, s, a, (const double*)S[0], (const double*)S[1]);
   launch(k_kkt_n_sums, w.ngrp_P, BNT, 0, s, a, (const double*)S[2], (const double*)S[3], (const double*)S[4],
          (const double*)S[5]);

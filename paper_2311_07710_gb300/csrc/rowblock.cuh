@@ -313,50 +313,52 @@ __device__ __forceinline__ void long_segment_sum(const BCsr<V>& M, const V* vec,
   if (threadIdx.x == 0) *out = s;
 }
 
-// member-major [count][L] (member stride `stride`) <-> interleaved [L][ld],
-// through 32 x 32 shared-memory tiles
+// member-major [count][L] (member stride `stride`) <-> interleaved [L][ld] of the
+// members in slot[0..ld) (-1: none), through 32 x 32 shared-memory tiles
 template <typename V>
-__global__ void __launch_bounds__(256) k_to_il(const V* __restrict__ src, long long stride, int L, int count,
-                                               V* __restrict__ dst, int ld) {
+__global__ void __launch_bounds__(256) k_to_il(const V* __restrict__ src, long long stride, int L,
+                                               const int* __restrict__ slot, V* __restrict__ dst, int ld) {
   __shared__ V t[32][33];
   const int j0 = blockIdx.x * 32, m0 = blockIdx.y * 32;
   for (int k = threadIdx.y; k < 32; k += 8) {
-    const int mem = m0 + k, jj = j0 + threadIdx.x;
-    if (mem < count && jj < L) t[k][threadIdx.x] = src[(size_t)mem * stride + jj];
+    const int mem = slot[m0 + k], jj = j0 + threadIdx.x;
+    if (mem >= 0 && jj < L) t[k][threadIdx.x] = src[(size_t)mem * stride + jj];
   }
   __syncthreads();
   for (int k = threadIdx.y; k < 32; k += 8) {
-    const int jj = j0 + k, mem = m0 + threadIdx.x;
-    if (jj < L && mem < count) dst[(size_t)jj * ld + mem] = t[threadIdx.x][k];
+    const int jj = j0 + k, m = m0 + threadIdx.x;
+    if (jj < L && slot[m] >= 0) dst[(size_t)jj * ld + m] = t[threadIdx.x][k];
   }
 }
 template <typename V>
-__global__ void __launch_bounds__(256) k_from_il(const V* __restrict__ src, int ld, int L, int count,
-                                                 V* __restrict__ dst, long long stride) {
+__global__ void __launch_bounds__(256) k_from_il(const V* __restrict__ src, int ld, int L,
+                                                 const int* __restrict__ slot, V* __restrict__ dst,
+                                                 long long stride) {
   __shared__ V t[32][33];
   const int j0 = blockIdx.x * 32, m0 = blockIdx.y * 32;
   for (int k = threadIdx.y; k < 32; k += 8) {
-    const int jj = j0 + k, mem = m0 + threadIdx.x;
-    if (jj < L && mem < count) t[k][threadIdx.x] = src[(size_t)jj * ld + mem];
+    const int jj = j0 + k, m = m0 + threadIdx.x;
+    if (jj < L && slot[m] >= 0) t[k][threadIdx.x] = src[(size_t)jj * ld + m];
   }
   __syncthreads();
   for (int k = threadIdx.y; k < 32; k += 8) {
-    const int mem = m0 + k, jj = j0 + threadIdx.x;
-    if (mem < count && jj < L) dst[(size_t)mem * stride + jj] = t[threadIdx.x][k];
+    const int mem = slot[m0 + k], jj = j0 + threadIdx.x;
+    if (mem >= 0 && jj < L) dst[(size_t)mem * stride + jj] = t[threadIdx.x][k];
   }
 }
 
 // the transposes take a 2-D block of 32 x 8 threads
 template <typename V>
-static void to_il(const V* src, long long stride, int L, int count, V* dst, int ld, cudaStream_t s) {
+static void to_il(const V* src, long long stride, int L, const int* slot, int count, V* dst, int ld, cudaStream_t s) {
   if (L <= 0 || !src) return;
-  k_to_il<V><<<dim3(cdiv(L, 32), cdiv(count, 32)), dim3(32, 8), 0, s>>>(src, stride, L, count, dst, ld);
+  k_to_il<V><<<dim3(cdiv(L, 32), cdiv(count, 32)), dim3(32, 8), 0, s>>>(src, stride, L, slot, dst, ld);
   count_launch();
 }
 template <typename V>
-static void from_il(const V* src, int ld, int L, int count, V* dst, long long stride, cudaStream_t s) {
+static void from_il(const V* src, int ld, int L, const int* slot, int count, V* dst, long long stride,
+                    cudaStream_t s) {
   if (L <= 0) return;
-  k_from_il<V><<<dim3(cdiv(L, 32), cdiv(count, 32)), dim3(32, 8), 0, s>>>(src, ld, L, count, dst, stride);
+  k_from_il<V><<<dim3(cdiv(L, 32), cdiv(count, 32)), dim3(32, 8), 0, s>>>(src, ld, L, slot, dst, stride);
   count_launch();
 }
 

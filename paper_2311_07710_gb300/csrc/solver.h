@@ -211,7 +211,7 @@ struct Work {
   double eps_inf = 1e-8;
   // Family handles (members that share the matrix): one member's sizes and
   // its P columns in local numbering (the A' part at fam_n + k), and the
-  // member-interleaved copies of the iteration vectors, v[j * fam_ld + member],
+  // member-interleaved copies of the iteration vectors, v[j * fam_ld + slot],
   // that the family iteration kernels run on within a chunk (slots IL_*).
   int fam_count = 0, fam_n = 0, fam_m = 0, fam_ld = 0;
   long long fam_nnzP = 0, fam_nnzA = 0;
@@ -219,10 +219,10 @@ struct Work {
   bool fam_il = false;                       // eligible: no long rows, no low-rank term
   double* ild[11] = {};                      // float64 (allocated on first use)
   float* ilf[11] = {};                       // float32
-  float* il_steps_f = nullptr;               // [check period][5][fam_ld] step scalars of a chunk, member order
+  float* il_steps_f = nullptr;               // [check period][5][fam_ld] step scalars of a chunk, slot order
   double* il_steps_d = nullptr;
   int il_steps_len[2] = {0, 0};              // iterations they hold (float64, mixed)
-  int* il_run = nullptr;                     // [fam_ld] the member iterates
+  int* il_slot = nullptr;                    // [fam_ld] member of each slot of the interleaved vectors, or -1
   double* ilk[10] = {};                      // the check's interleaved iterates and row sums (ILK_*)
   double* kks[6] = {};                       // the check's row sums, member-major: A x (2) [m], Q x (2), A'y (2) [n]
   bool il_active = false;                    // this solve runs the interleaved kernels
@@ -312,6 +312,7 @@ void chunk_fill_values(Work& w, bool mixed, cudaStream_t s);
 void chunk_run(Work& w, int len, bool mixed, cudaStream_t s, int j0);
 // a low-rank term over short rows of P: the fused half-step (lowrank.cu)
 bool lowrank_fused_ok(const Work& w, bool mixed);
+void il_slots(Work& w, cudaStream_t s);   // the running members of a family, densely
 void lowrank_run(Work& w, int len, bool mixed, cudaStream_t s, int j0);
 template <typename V>
 void run_dual(Work& w, int j, BCsr<V> A, V* xt, V* const* Z, V* ybar, const V* b, const V* ylo, cudaStream_t s);
