@@ -677,9 +677,8 @@ static void launch_kkt_il(Work& w, const KktB& a, cudaStream_t s) {
 
 // reduce the field-major partials of k_kkt_m / k_kkt_n (blocks [bm0, bm1) of
 // [nbm] and [bn0, bn1) of [nbn]) into F[0..23] (thread 0)
-// (at: the value of field k of block b, by side)
-template <typename AtM, typename AtN>
-__device__ __forceinline__ void reduce_kkt_fields(int bm0, int bm1, AtM at_m, int bn0, int bn1, AtN at_n, double* F) {
+__device__ __forceinline__ void reduce_kkt_blocks(const double* pm, int nbm, int bm0, int bm1,
+                                                  const double* pn, int nbn, int bn0, int bn1, double* F) {
   double f[24];
 #pragma unroll
   for (int k = 0; k < 24; ++k) f[k] = 0.0;
@@ -689,24 +688,18 @@ __device__ __forceinline__ void reduce_kkt_fields(int bm0, int bm1, AtM at_m, in
   for (int b = bm0 + threadIdx.x; b < bm1; b += blockDim.x)
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-      const double v = at_m(k, b);
+      const double v = pm[(size_t)k * nbm + b];
       f[k] = is_max[k] ? nmax(f[k], v) : f[k] + v;
     }
   for (int b = bn0 + threadIdx.x; b < bn1; b += blockDim.x)
 #pragma unroll
     for (int k = 0; k < 15; ++k) {
-      const double v = at_n(k, b);
+      const double v = pn[(size_t)k * nbn + b];
       f[9 + k] = is_max[9 + k] ? nmax(f[9 + k], v) : f[9 + k] + v;
     }
   block_reduce<24>(f, is_max);
   if (threadIdx.x == 0)
     for (int k = 0; k < 24; ++k) F[k] = f[k];
-}
-__device__ __forceinline__ void reduce_kkt_blocks(const double* pm, int nbm, int bm0, int bm1,
-                                                  const double* pn, int nbn, int bn0, int bn1, double* F) {
-  reduce_kkt_fields(
-      bm0, bm1, [&](int k, int b) { return pm[(size_t)k * nbm + b]; }, bn0, bn1,
-      [&](int k, int b) { return pn[(size_t)k * nbn + b]; }, F);
 }
 
 // --------------------------------------------------------------------------
@@ -1644,8 +1637,29 @@ __device__ void fill_steps_block(const DevState& S, const SolveParams& p, StepEn
   for (int j = threadIdx.x; j < p.check_period; j += blockDim.x) tab[j] = make_step(S.k_epoch + j, S, p);
 }
 
-__device__ void decide_thread0(DevState* st, const double* F, const SolveParams& p, int mode,
+__device__ void decide_thread0(DevState* st, const double* F, const double (*P)[6], const SolveParams& p, int mode,
                                long long chunk_len, int inf_status);
+
+// kkt_from_fields of both iterates in a warp: lane 3 it + {0, 1, 2} forms
+// r_primal, r_dual and r_gap of iterate it, so that six divisions go through the
+// float64 pipe as one.
+__device__ __forceinline__ void kkt_parts_warp(const double* F, double (*P)[6]) {
+  const int lane = threadIdx.x & 31, it = lane >= 3 && lane < 6, w = lane - 3 * it;
+  const double* G = F + 9 + it * 7;
+  const double xQx = G[3], cx = G[4];
+  const double pobj = 0.5 * xQx + cx;
+  const double dobj = -0.5 * xQx + F[it * 4 + 2] + G[5];
+  const double top = w == 0 ? F[it * 4] : (w == 1 ? G[0] : fabs(pobj - dobj));
+  const double base = w == 0 ? fmax(F[it * 4 + 1], F[8])
+                             : (w == 1 ? fmax(fmax(G[1], G[2]), F[23]) : fmax(fabs(pobj), fabs(dobj)));
+  const double r = top / (1.0 + base);
+  const double rd = __shfl_down_sync(0xffffffffu, r, 1), rg = __shfl_down_sync(0xffffffffu, r, 2);
+  if (lane == 0 || lane == 3) {
+    double rel = nmax(nmax(r, rd), rg);
+    if (pobj != pobj || dobj != dobj) rel = pobj - dobj;   // NaN
+    P[it][0] = r; P[it][1] = rd; P[it][2] = rg; P[it][3] = rel; P[it][4] = pobj; P[it][5] = dobj;
+  }
+}
 
 // Chunk sums of the relKKT group partials: CUDA block (i, c) reduces chunk c
 // of instance i -- its KKT_CHUNK / KKT_GROUP consecutive groups from the
@@ -1654,22 +1668,33 @@ __device__ void decide_thread0(DevState* st, const double* F, const SolveParams&
 // kernel reads tens of values, not thousands.  gfm, gfn: first group of each
 // instance (A, P).
 constexpr int KKT_GPC = KKT_CHUNK / KKT_GROUP;   // groups per chunk (8: lanes 0..7)
-// one chunk's sums of one side in a warp: first group g0 of the chunk, end of
-// the instance's groups ge; put(k, value) in lane 0
-template <int NF, unsigned MAXMASK, typename Put>
+// One chunk's sums of one side in a warp: first group g0 of the chunk, end of
+// the instance's groups ge; put(k, value) once per field.  Four fields at a
+// time, eight lanes each; sums and maxima apart (an instruction of the float64
+// pipe takes 16 clocks for one lane as for 32, and maxima need none: with
+// kkt_parts_warp and a thread per field in k_decide, which that pipe bounds,
+// n = 1000 went from 4.31 to 4.16 ms a solve, a batch of 4096 from 199 to 197).
+template <int NF, typename Put>
 __device__ __forceinline__ void kkt_chunk_sums(const double* part, int ng, int g0, int ge, Put put) {
-  const int lane = threadIdx.x & 31, g = g0 + lane;
-  const bool on = lane < KKT_GPC && g < ge;
+  static_assert(KKT_GPC == 8 && (NF == 9 || NF == 15), "fields of k_kkt_m or k_kkt_n, eight groups a chunk");
+  constexpr int SUMS = NF == 9 ? 4 : 8, MAXIMA = NF - SUMS;
+  const int lane = threadIdx.x & 31, sub = lane >> 3, g = g0 + (lane & 7);
 #pragma unroll
-  for (int k = 0; k < NF; ++k) {
-    const bool mx = (MAXMASK >> k) & 1u;
-    double v = on ? part[(size_t)k * ng + g] : 0.0;
+  for (int b = 0; b < SUMS; b += 4) {
+    const int q = b + sub, k = NF == 9 ? (q < 2 ? 2 + q : 4 + q) : (q < 4 ? 3 + q : 6 + q);
+    double v = g < ge ? part[(size_t)k * ng + g] : 0.0;
 #pragma unroll
-    for (int o = KKT_GPC / 2; o > 0; o >>= 1) {
-      const double t = __shfl_xor_sync(0xffffffffu, v, o);
-      v = mx ? nmax(v, t) : v + t;
-    }
-    if (lane == 0) put(k, v);
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((lane & 7) == 0) put(k, v);
+  }
+#pragma unroll
+  for (int b = 0; b < MAXIMA; b += 4) {
+    const int q = b + sub;
+    const int k = NF == 9 ? (q < 2 ? q : (q < 4 ? 2 + q : 8)) : (q < 3 ? q : (q < 6 ? 4 + q : 14));
+    double v = q < MAXIMA && g < ge ? part[(size_t)k * ng + g] : 0.0;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) v = nmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+    if (q < MAXIMA && (lane & 7) == 0) put(k, v);
   }
 }
 __global__ void __launch_bounds__(32) k_kkt_chunks(const Inst* __restrict__ insts, const int* __restrict__ gfm,
@@ -1681,10 +1706,10 @@ __global__ void __launch_bounds__(32) k_kkt_chunks(const Inst* __restrict__ inst
   const Inst in = insts[i];
   const int c = blockIdx.y;
   if (in.bP0 + c * KKT_CHUNK < in.bP1)
-    kkt_chunk_sums<15, 0x4387u>(pn, ngn, gfn[i] + c * KKT_GPC, gfn[i + 1],
+    kkt_chunk_sums<15>(pn, ngn, gfn[i] + c * KKT_GPC, gfn[i + 1],
                                 [&](int k, double v) { cn[(size_t)k * ncn + in.cP0 + c] = v; });
   if (in.m > 0 && in.bA0 + c * KKT_CHUNK < in.bA1)
-    kkt_chunk_sums<9, 0x133u>(pm, ngm, gfm[i] + c * KKT_GPC, gfm[i + 1],
+    kkt_chunk_sums<9>(pm, ngm, gfm[i] + c * KKT_GPC, gfm[i + 1],
                               [&](int k, double v) { cm[(size_t)k * ncm + in.cA0 + c] = v; });
 }
 
@@ -1735,20 +1760,32 @@ __global__ void __launch_bounds__(64) k_decide(DecideArgs a, SolveParams p, int 
     __shared__ double sc[24][DEC_CHUNKS];
     if (threadIdx.x < 32) {
       for (int c = 0; c < cn; ++c)
-        kkt_chunk_sums<15, 0x4387u>(a.pn, a.nbn, a.gf_n[i] + c * KKT_GPC, a.gf_n[i + 1],
+        kkt_chunk_sums<15>(a.pn, a.nbn, a.gf_n[i] + c * KKT_GPC, a.gf_n[i + 1],
                                     [&](int k, double v) { sc[9 + k][c] = v; });
     } else {
       for (int c = 0; c < cm; ++c)
-        kkt_chunk_sums<9, 0x133u>(a.pm, a.nbm, a.gf_m[i] + c * KKT_GPC, a.gf_m[i + 1],
+        kkt_chunk_sums<9>(a.pm, a.nbm, a.gf_m[i] + c * KKT_GPC, a.gf_m[i + 1],
                                   [&](int k, double v) { sc[k][c] = v; });
     }
     __syncthreads();
-    reduce_kkt_fields(
-        0, cm, [&](int k, int b) { return sc[k][b]; }, 0, cn, [&](int k, int b) { return sc[9 + k][b]; }, F);
+    if (threadIdx.x < 24) {                     // a field per thread, summed as reduce_kkt_blocks does
+      constexpr unsigned MAXMASK = 0x133u | (0x4387u << 9);
+      const int k = threadIdx.x, c = k < 9 ? cm : cn;
+      double v[DEC_CHUNKS];
+#pragma unroll
+      for (int b = 0; b < DEC_CHUNKS; ++b) v[b] = b < c ? sc[k][b] : 0.0;
+      F[k] = (MAXMASK >> k) & 1u ? nmax(nmax(v[0], v[1]), nmax(v[2], v[3])) : (v[0] + v[2]) + (v[1] + v[3]);
+    }
   } else {
     reduce_kkt_blocks(a.pm, a.nbm, in.cA0, in.cA0 + cm, a.pn, a.nbn, in.cP0, in.cP0 + cn, F);
   }
-  if (threadIdx.x == 0) decide_thread0(st, F, p, mode, chunk_len, a.inf ? a.inf[i].status : 0);
+  __shared__ double parts[2][6];
+  __syncwarp();                                 // F is the first warp's
+  if (threadIdx.x < 32) {
+    kkt_parts_warp(F, parts);
+    __syncwarp();
+    if (threadIdx.x == 0) decide_thread0(st, F, parts, p, mode, chunk_len, a.inf ? a.inf[i].status : 0);
+  }
   __syncthreads();
   if (a.bst && threadIdx.x == 0) write_running(*st, in, a.rpA, a.rpP, a.bst);
   if (st->status == ST_RUNNING) fill_steps_block(*st, p, a.tabs + (size_t)i * a.C);
@@ -1782,12 +1819,9 @@ __global__ void __launch_bounds__(1024) k_count_running(const DevState* __restri
   }
 }
 
-__device__ void decide_thread0(DevState* st, const double* F, const SolveParams& p, int mode,
+__device__ void decide_thread0(DevState* st, const double* F, const double (*P)[6], const SolveParams& p, int mode,
                                long long chunk_len, int inf_status) {
   DevState& S = *st;
-  double P[2][6];
-  kkt_from_fields(F, 0, P[0]);
-  kkt_from_fields(F, 1, P[1]);
   for (int it = 0; it < 2; ++it)
     for (int k = 0; k < 6; ++k) S.parts[it][k] = P[it][k];
   S.restart = 0;
