@@ -2326,6 +2326,8 @@ pdqp_status pdqp_set_lowrank_Q(pdqp_handle h, int32_t r, const float* F, int32_t
     w.wlr_f = dalloc<float>(h, 2 * (size_t)r);
     w.lr_part = dalloc<double>(h, (size_t)((w.n + LR_ROWS - 1) / LR_ROWS) * 2 * r);
     w.lr_rows = dalloc<double>(h, 2 * (size_t)w.n);
+    w.lr_ticket = dalloc<unsigned>(h, std::max(w.A.nlseg, 1));
+    CK(cudaMemsetAsync(w.lr_ticket, 0, std::max(w.A.nlseg, 1) * sizeof(unsigned), s));
     to_device(w.F, hf.data(), N, s);
     to_device(w.Fo, hd.data(), N, s);
     CK(cudaStreamSynchronize(s));

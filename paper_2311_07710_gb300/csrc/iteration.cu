@@ -482,21 +482,97 @@ static void run_chunk_pipe(Work& w, int j0, int len, BCsr<V> A, BCsr<V> P, V* xt
   }
 }
 
-// The dual half-step of iteration j alone (its long rows' segments summed by
-// the kernel before it, which may still be running: launch_early).
+// The dual half-step beside the reduction of F' x_md from its tiles' partials (the
+// low-rank half-step, lowrank.cu): blocks [0, r) sum a column each, the next take
+// a segment of a long row of A each, the others a row block of short rows.  The
+// last segment of a row to finish (ticket, back at zero for the next launch) adds
+// them in order and updates the row, as dual_block does.  A portfolio has two
+// long rows and nothing else: with the segments and the two rows in launches of
+// their own a solve (n = 1e5, r = 64) took 48.2 ms, so 40.6.
 template <typename V>
-void run_dual(Work& w, int j, BCsr<V> A, V* xt, V* const* Z, V* ybar, const V* b, const V* ylo, cudaStream_t s) {
+struct LrColumns {
+  const double* part;            // [nparts][r]
+  int nparts, r;
+  double* w;
+  float* wf;
+  const int4* __restrict__ lseg;
+  int nlseg;
+  V* lpart;
+  unsigned* ticket;              // [nlseg], at a row's first segment
+};
+template <typename V>
+__global__ void __launch_bounds__(256, MinBlocks<V, 256>::value == 8 ? 4 : MinBlocks<V, 256>::value)
+    k_dual_lr(DualB<V> a, LrColumns<V> q, int j) {
+  __shared__ V prod[BNNZ];
+  __shared__ V sx[sizeof(V) == 8 ? BNNZ : 1];
+  __shared__ int srp[BROWS + 1];
+  grid_trigger();
+  int b = blockIdx.x;
+  if (b < q.r) {
+    grid_wait();
+    if (a.st->status == ST_RUNNING) lr_reduce_column(q.part, q.nparts, q.r, 1, b, q.w, q.wf);
+    return;
+  }
+  b -= q.r;
+  if (b >= q.nlseg) {
+    b -= q.nlseg;
+    if (a.blk_seg && a.blk_seg[b].y > 0) grid_wait();          // a long row
+    else dual_block<V, 256>(a, b, j, prod, sx, srp);
+    return;
+  }
+  // long_segment_sum with the segment's entries fetched before the wait
+  constexpr int PER = (LSEG + 255) / 256;
+  const int4 g = q.lseg[b];                                     // {row, first nonzero, end, row block}
+  const int2 sg = a.blk_seg[g.w];
+  V v[PER];
+  int c[PER];
+#pragma unroll
+  for (int k = 0; k < PER; ++k) {
+    const int e = g.y + threadIdx.x + 256 * k;
+    v[k] = e < g.z ? a.A.val[e] : V(0);
+    c[k] = e < g.z ? a.A.col[e] : 0;
+  }
+  grid_wait();
+  if (a.st->status != ST_RUNNING) return;
+  V z[PER], s = V(0);
+#pragma unroll
+  for (int k = 0; k < PER; ++k) z[k] = g.y + (int)threadIdx.x + 256 * k < g.z ? a.xt[c[k]] : V(0);
+  V yo = V(0), bi = V(0), yb = V(0), lo = V(0);
+  if (threadIdx.x == 0) {
+    yo = a.yold[g.x]; bi = a.b[g.x]; yb = a.ybar[g.x];
+    if (a.ylo) lo = a.ylo[g.x];
+  }
+#pragma unroll
+  for (int k = 0; k < PER; ++k)
+    if (g.y + (int)threadIdx.x + 256 * k < g.z) s += v[k] * z[k];
+  s = block_sum(s);
+  if (threadIdx.x != 0) return;
+  q.lpart[b] = s;
+  __threadfence();
+  if (atomicAdd(q.ticket + sg.x, 1u) != (unsigned)sg.y - 1u) return;
+  __threadfence();
+  q.ticket[sg.x] = 0u;
+  s = V(0);
+  for (int k = 0; k < sg.y; ++k) s += __ldcg(q.lpart + sg.x + k);
+  dual_row(a, a.tab[j], g.x, s, yo, bi, yb, lo);
+}
+
+template <typename V>
+void run_dual_lr(Work& w, int j, int nparts, BCsr<V> A, V* xt, V* const* Z, V* ybar, const V* b, const V* ylo,
+                 cudaStream_t s) {
   DualB<V> da{A, xt, nullptr, nullptr, ybar, b, ylo, w.tab, w.blk_inst_A, w.st, w.row_ineq, w.tab_stride};
   da.yold = Z[(j + 1) & 1] + w.n;
   da.ynew = Z[j & 1] + w.n;
-  if (w.A.nlseg) { da.blk_seg = w.A.blk_seg; da.lpart = sizeof(V) == 4 ? (V*)w.A.lpart_f : (V*)w.A.lpart_d; }
+  V* lp = sizeof(V) == 4 ? (V*)w.A.lpart_f : (V*)w.A.lpart_d;
+  if (w.A.nlseg) { da.blk_seg = w.A.blk_seg; da.lpart = lp; }
   da.early = 1;
-  launch_early(k_dual<V, 256>, w.A.nblk, 256, 0, s, da, j);
+  const LrColumns<V> q{w.lr_part, nparts, w.r, w.wlr, w.wlr_f, w.A.lseg, w.A.nlseg, lp, w.lr_ticket};
+  launch_early(k_dual_lr<V>, w.r + w.A.nlseg + (w.m > 0 ? w.A.nblk : 0), 256, 0, s, da, q, j);
 }
-template void run_dual<float>(Work&, int, BCsr<float>, float*, float* const*, float*, const float*, const float*,
-                              cudaStream_t);
-template void run_dual<double>(Work&, int, BCsr<double>, double*, double* const*, double*, const double*,
-                               const double*, cudaStream_t);
+template void run_dual_lr<float>(Work&, int, int, BCsr<float>, float*, float* const*, float*, const float*,
+                                 const float*, cudaStream_t);
+template void run_dual_lr<double>(Work&, int, int, BCsr<double>, double*, double* const*, double*, const double*,
+                                  const double*, cudaStream_t);
 
 template <typename V, int NT>
 static void run_chunk(Work& w, int j0, int len, BCsr<V> A, BCsr<V> P, V* xt, V* const* Z, V* ybar, const V* b,

@@ -7,9 +7,9 @@
 // row tile of one k_lr_ft block, brings its rows of F to shared memory in
 // contiguous 16-byte copies, finishes its rows and, with x_md of the next
 // iteration in hand, forms the tile's partial of F' x_md from the same copy:
-// F is read once and two launches go.  The three kernels of an iteration start
-// early (launch_early): the tiles' copies of F run while the reduction and the dual
-// half-step, a few blocks each, finish.  Every sum keeps k_lr_ft's, k_lr_reduce's
+// F is read once.  The reduction of the partials runs beside the dual half-step
+// (k_dual_lr), and both kernels of an iteration start early (launch_early): the
+// tiles' copies of F run while that kernel, a few blocks, finishes.  Every sum keeps k_lr_ft's, k_lr_reduce's
 // and lr_row's order and rounding, so the iterates are bitwise the general
 // path's.
 #include <algorithm>
@@ -159,43 +159,6 @@ __global__ void __launch_bounds__(LRF_NT) k_primal_lr(LrPrimal<V> a, int j) {
   }
 }
 
-// Blocks [0, r): column k of F' x_md from the tiles' partials; the others: the
-// segment sums of A's long rows (independent of each other, one launch).
-template <typename V>
-__global__ void __launch_bounds__(256)
-    k_lr_reduce_long(const double* part, int nparts, int r, double* w, float* wf,
-                     BCsr<V> A, const V* vec, const int4* lseg,
-                     const DevState* st, V* lpart) {
-  grid_trigger();
-  if ((int)blockIdx.x < r) {
-    grid_wait();
-    if (st->status != ST_RUNNING) return;
-    lr_reduce_column(part, nparts, r, 1, blockIdx.x, w, wf);
-    return;
-  }
-  // long_segment_sum with the segment's entries fetched before the wait
-  constexpr int PER = (LSEG + 255) / 256;
-  const int4 g = lseg[blockIdx.x - r];
-  V v[PER];
-  int c[PER];
-#pragma unroll
-  for (int k = 0; k < PER; ++k) {
-    const int e = g.y + threadIdx.x + 256 * k;
-    v[k] = e < g.z ? A.val[e] : V(0);
-    c[k] = e < g.z ? A.col[e] : 0;
-  }
-  grid_wait();
-  if (st->status != ST_RUNNING) return;
-  V z[PER], s = V(0);
-#pragma unroll
-  for (int k = 0; k < PER; ++k) z[k] = g.y + threadIdx.x + 256 * k < g.z ? vec[c[k]] : V(0);
-#pragma unroll
-  for (int k = 0; k < PER; ++k)
-    if (g.y + (int)threadIdx.x + 256 * k < g.z) s += v[k] * z[k];
-  s = block_sum(s);
-  if (threadIdx.x == 0) lpart[blockIdx.x - r] = s;
-}
-
 // Low-rank row terms (F w0)_j and (F w1)_j of a float64 check: 64 rows of F
 // through shared memory, one thread per (row, iterate).
 __global__ void __launch_bounds__(128) k_lr_rows(const double* __restrict__ F, int n, int r,
@@ -242,13 +205,10 @@ static void run_chunk_lr(Work& w, int j0, int len, BCsr<V> A, BCsr<V> P, V* xt, 
   const int grid = lr_ft_grid(w), per = cdiv(w.n, grid);
   LrPrimal<V> pa{P.rp, P.col, P.val, nullptr, nullptr, x, xbar, xt, c, l, u, w.tab, w.st, lr_factor<V>(w),
                  lr_weights<V>(w), w.lr_part, w.n, w.r, per};
-  V* lpA = sizeof(V) == 4 ? (V*)w.A.lpart_f : (V*)w.A.lpart_d;
   for (int j = j0; j < j0 + len; ++j) {
     if (Pr.on) Pr.begin(0, s, launch_bytes(w, 0, sizeof(V)));
     if (j == j0) lowrank_ft_part(w, pa.F, (const V*)Z[j & 1], s);   // later ones come from k_primal_lr
-    launch_early(k_lr_reduce_long<V>, w.r + w.A.nlseg, 256, 0, s, (const double*)w.lr_part, grid, w.r, w.wlr, w.wlr_f, A,
-           (const V*)xt, (const int4*)w.A.lseg, (const DevState*)w.st, lpA);
-    if (w.m > 0) run_dual(w, j, A, xt, Z, ybar, b, ylo, s);
+    run_dual_lr(w, j, grid, A, xt, Z, ybar, b, ylo, s);
     if (Pr.on) Pr.end(s);
     pa.zin = Z[j & 1];
     pa.zout = Z[(j + 1) & 1];

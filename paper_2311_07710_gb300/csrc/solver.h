@@ -177,6 +177,7 @@ struct Work {
   float* wlr_f = nullptr;    // [2][r] the same in float32 (float32 iteration)
   double* lr_part = nullptr; // [tiles][2][r] partial sums
   double* lr_rows = nullptr; // [2][n] the check's row terms F~ (F~' v)
+  unsigned* lr_ticket = nullptr; // [A's segments] segments of a long row done (0 between launches)
   // Lanczos vectors: pu[p] (n) for A~'A~, pz[p] = [v_Q ; A~v_A] (n+m) the P input
   double *pu[2] = {nullptr, nullptr}, *pz[2] = {nullptr, nullptr};
   float *fpu[2] = {nullptr, nullptr}, *fpz[2] = {nullptr, nullptr};
@@ -315,7 +316,8 @@ bool lowrank_fused_ok(const Work& w, bool mixed);
 void il_slots(Work& w, cudaStream_t s);   // the running members of a family, densely
 void lowrank_run(Work& w, int len, bool mixed, cudaStream_t s, int j0);
 template <typename V>
-void run_dual(Work& w, int j, BCsr<V> A, V* xt, V* const* Z, V* ybar, const V* b, const V* ylo, cudaStream_t s);
+void run_dual_lr(Work& w, int j, int nparts, BCsr<V> A, V* xt, V* const* Z, V* ybar, const V* b, const V* ylo,
+                 cudaStream_t s);
 void check(Work& w, const SolveParams& p, int mode, long long chunk_len, bool mixed, cudaStream_t s);
 
 // infeasibility certificates: fill the recession-cone bounds once the
