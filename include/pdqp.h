@@ -131,7 +131,11 @@ typedef struct {
                                 per iteration (pdqp_info reports them as 4, which
                                 cannot be asked for); else the first full chunk of a
                                 handle's first solve in each precision times two
-                                rounds of 4 iterations of each of 256, 512 and 1 and
+                                rounds of 4 iterations of each of 256, 512, 1 and, for
+                                a large single problem without long rows, a row per
+                                thread on a second copy of the matrices (reported as
+                                5, which cannot be asked for; at most half of the free
+                                device memory, else left out), and
                                 keeps the fastest for that precision; the choice is
                                 also kept for the process per problem shape, so later
                                 handles of the same sizes, nonzeros and row blocks

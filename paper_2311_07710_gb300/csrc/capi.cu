@@ -42,7 +42,7 @@ struct pdqp_problem {
   std::vector<pdqp_info> infos;                       // per instance, from the last solve
   std::vector<void*> allocs;
   int tuned_nt[2] = {0, 0};                           // autotuned variant per precision (0: not yet)
-  cudaEvent_t tune_ev[4] = {nullptr, nullptr, nullptr, nullptr};
+  cudaEvent_t tune_ev[5] = {};
   // Where the last solve stopped (what pdqp_get_state exports): its parameters,
   // the step-table position (iterations run since the table was last filled;
   // 0 at a check) and the iterations of the solve loop.
@@ -636,6 +636,7 @@ void tuned_store(const Work& w, bool mixed, int nt) {
 }
 
 void alloc_chunk(pdqp_problem* h, bool mixed, cudaStream_t s);   // with the device scans, below
+bool alloc_slices(pdqp_problem* h, bool mixed, cudaStream_t s);
 
 // options.spmv_threads = 2: at most 64 row blocks of A and of P, no row longer
 // than a row block, no low-rank term, and 3n + 2m values (with a row block's
@@ -701,6 +702,10 @@ pdqp_status solve_impl(pdqp_problem* h, const pdqp_options& o, const double* x0,
   const bool autotune = o.spmv_threads == 0 && !use_il && !mp && !use_chunk && !use_lr;
   int& tuned = h->tuned_nt[mixed ? 1 : 0];
   if (autotune && !tuned) tuned = tuned_lookup(w, mixed);
+  constexpr int TUNE_PERIOD = 48;   // the shortest check period that is tuned
+  const bool use_slices =
+      autotune && (tuned == 5 || (tuned == 0 && o.check_period >= TUNE_PERIOD)) && alloc_slices(h, mixed, s);
+  if (tuned == 5 && !use_slices) tuned = 0;
   w.mp = mp ? 1 : 0;
   w.mp_accelerate = p.accelerate;
   if (mp) {
@@ -771,6 +776,7 @@ pdqp_status solve_impl(pdqp_problem* h, const pdqp_options& o, const double* x0,
   }
   pdqp::scale_apply(w, mixed, s, rep_vals ? &sw : nullptr);
   if (use_chunk) pdqp::chunk_fill_values(w, mixed, s);
+  if (use_slices) pdqp::slices_fill_values(w, mixed, s);
 
   // spectral norms of the scaled matrices (a resumed solve keeps its own)
   const bool run_lanczos = !resuming && !(o.norm_A > 0.0 && o.norm_Q > 0.0);
@@ -834,25 +840,27 @@ pdqp_status solve_impl(pdqp_problem* h, const pdqp_options& o, const double* x0,
   // graph and replayed, as the solve loop runs them (direct launches would
   // charge the per-iteration variants launch gaps that graphs do not have);
   // with the event profiler on, they are launched directly.
-  static const int kCand[3] = {256, 512, 1};
-  constexpr int ncand = 3;
+  static const int kCand[4] = {256, 512, 1, 5};
+  constexpr int MAX_CAND = 4;
+  const int ncand = use_slices ? 4 : 3;
   constexpr int TUNE = 4, ROUNDS = 2;
+  static_assert(MAX_CAND * ROUNDS * TUNE <= TUNE_PERIOD, "the tuned chunk holds every candidate's rounds");
   if (autotune && tuned) p.spmv_threads = tuned;
   while (w.bst_host->running > 0) {
     const long long len = std::min<long long>(o.check_period, o.max_iter - k_total);
-    const bool tune_now = autotune && !tuned && len == o.check_period && len >= 2 * ncand * ROUNDS * TUNE;
+    const bool tune_now = autotune && !tuned && len == o.check_period && len >= TUNE_PERIOD;
     // per-kernel event timing needs direct launches (events recorded by graph
     // nodes cannot be timed), so profiling bypasses the graph
     if (tune_now) {
       for (auto& e : h->tune_ev)
         if (!e) CK(cudaEventCreate(&e));
-      float best_ms[ncand] = {0.f, 0.f, 0.f};
+      float best_ms[MAX_CAND] = {};
       int j = 0;
       const bool replay = !w.prof.on && !o.no_graphs;
       if (replay) pdqp::iterate(w, 0, mixed, 1, s, 0);   // one-time setup of the pipelined variant
       for (int r = 0; r < ROUNDS; ++r) {
-        cudaGraphExec_t ex[ncand] = {nullptr, nullptr, nullptr};
-        long long kern[ncand] = {0, 0, 0};
+        cudaGraphExec_t ex[MAX_CAND] = {};
+        long long kern[MAX_CAND] = {};
         if (replay)
           for (int c = 0; c < ncand; ++c) ex[c] = capture_iterations(h, TUNE, mixed, kCand[c], j + c * TUNE, &kern[c]);
         CK(cudaEventRecord(h->tune_ev[0], s));
@@ -1837,6 +1845,57 @@ void alloc_chunk(pdqp_problem* h, bool mixed, cudaStream_t s) {
   if (mixed && !ck.valf) ck.valf = dalloc<float2>(h, (size_t)ck.ngroups * 32);
   if (!mixed && !ck.vald) ck.vald = dalloc<double2>(h, (size_t)ck.ngroups * 32);
   if (ck.cls[mixed ? 1 : 0].empty()) pdqp::chunk_plan_classes(w, mixed);
+}
+
+// The slice layout of a large instance (iteration.cu), as alloc_chunk; false where
+// it is not taken: rows too uneven (more than half as many pads as entries), or
+// not within half of the free memory.
+bool alloc_slices(pdqp_problem* h, bool mixed, cudaStream_t s) {
+  Work& w = h->w;
+  SlicePlan& q = w.slices;
+  if (q.state < 0 || !pdqp::slices_ok(w, mixed)) return false;
+  const size_t mark = h->allocs.size();
+  try {
+    size_t free_b = 0, total_b = 0;
+    auto fits = [&](size_t bytes) { return cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && bytes <= free_b / 2; };
+    if (q.state == 0) {
+      q.nsA = (w.m + 31) / 32;
+      q.nsP = (w.n + 31) / 32;
+      const int ns = q.nsA + q.nsP;
+      TmpFree tmp;
+      tmp.s = s;
+      int* wid = (int*)pool_alloc((size_t)ns * sizeof(int), s);
+      tmp.v.push_back(wid);
+      q.sp = dalloc<int>(h, (size_t)ns + 1);
+      pdqp::slices_width(w, wid, s);
+      device_scan(wid, ns, q.sp, tmp.v, s);
+      int groups = 0;
+      CK(cudaMemcpyAsync(&groups, q.sp + ns, sizeof(int), cudaMemcpyDeviceToHost, s));
+      CK(cudaStreamSynchronize(s));
+      q.groups = groups;
+      const bool take = groups >= 0 && 2 * 64LL * groups <= 3 * (w.A.nnz + w.P.nnz) && fits((size_t)groups * 32 * 16);
+      if (take) {
+        q.idx = dalloc<int2>(h, (size_t)groups * 32);
+        pdqp::slices_fill_index(w, s);
+      }
+      q.state = take ? 1 : -1;
+    }
+    if (q.state == 1 && mixed && !q.valf) {
+      if (!fits((size_t)q.groups * 32 * sizeof(float2))) return false;
+      q.valf = dalloc<float2>(h, (size_t)q.groups * 32);
+    }
+    if (q.state == 1 && !mixed && !q.vald) {
+      if (!fits((size_t)q.groups * 32 * sizeof(double2))) return false;
+      q.vald = dalloc<double2>(h, (size_t)q.groups * 32);
+    }
+  } catch (const Fail& f) {
+    if (f.st != PDQP_ERR_OOM) throw;
+    for (size_t k = mark; k < h->allocs.size(); ++k) cudaFreeAsync(h->allocs[k], s);
+    h->allocs.resize(mark);
+    q = SlicePlan{};
+    q.state = -1;
+  }
+  return q.state == 1;
 }
 
 // A batch handed over as one block-diagonal problem: instance i owns the

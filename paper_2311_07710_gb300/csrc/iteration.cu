@@ -239,6 +239,217 @@ __global__ void __launch_bounds__(256) k_long_partials(BCsr<V> M, const V* __res
 
 
 // ==========================================================================
+// One row per thread on a slice layout (one instance without long rows): 32 rows a
+// slice, entry pairs of a slice's rows side by side, so that a warp's index and
+// value loads are contiguous and nothing is staged in shared memory.
+// The staged row blocks fill 2.4 (P) and 1.2 (A) waves of an n = 300007 problem
+// and wait at a barrier each; here all warps of an SM have gathers in flight and
+// L2's sectors (one of 32 bytes for a value) are the bound.
+// ==========================================================================
+constexpr int SL_U = 2;                  // pairs of a row in flight
+// Warps per SM against pairs in flight, n = 1e6 in float32 / 300007 in float64:
+// 64 / 32 warps and two pairs 115 / 52 us an iteration, 48 / 40 and two 118 / 58,
+// 48 / 32 and three 115 / 54, 40 / 24 and four 120 / 64.
+template <typename V> struct Sl;
+template <> struct Sl<float> { static constexpr int NT = 128, MINB = 16; };
+template <> struct Sl<double> { static constexpr int NT = 64, MINB = 16; };
+
+template <typename V> struct V2;
+template <> struct V2<float> { using T = float2; };
+template <> struct V2<double> { using T = double2; };
+
+// the matrix passes through once: not kept in L1, which the gathered vector needs
+__device__ __forceinline__ int2 ld_once(const int2* p) {
+  int2 v;
+  asm("ld.global.nc.L1::no_allocate.v2.s32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float2 ld_once(const float2* p) {
+  float2 v;
+  asm("ld.global.nc.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double2 ld_once(const double2* p) {
+  double2 v;
+  asm("ld.global.nc.L1::no_allocate.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+  return v;
+}
+
+template <typename V>
+struct SliceM {
+  const int* __restrict__ rp;            // the CSR row pointers
+  const int* __restrict__ sp;            // slice starts, in groups of 32 pairs
+  const int2* __restrict__ idx;
+  const typename V2<V>::T* __restrict__ val;
+};
+// a thread's row: its length and its first pairs
+template <typename V>
+struct SliceRow {
+  int len;
+  const int2* c;
+  const typename V2<V>::T* v;
+  int2 hc[SL_U];
+  typename V2<V>::T hv[SL_U];
+};
+template <typename V>
+__device__ __forceinline__ void slice_head(const SliceM<V>& M, int r, bool on, SliceRow<V>& h) {
+  h.len = on ? M.rp[r + 1] - M.rp[r] : 0;
+  const size_t at = on ? (size_t)M.sp[r >> 5] * 32 + (r & 31) : 0;
+  h.c = M.idx + at;
+  h.v = M.val + at;
+#pragma unroll
+  for (int k = 0; k < SL_U; ++k)
+    if (2 * k < h.len) { h.hc[k] = ld_once(h.c + 32 * k); h.hv[k] = ld_once(h.v + 32 * k); }
+}
+// the row's sum, its entries in CSR order by r_dot as in every variant
+template <typename V>
+__device__ __forceinline__ V slice_sum(SliceRow<V>& h, const V* vec) {
+  V s = V(0);
+  for (int e = 0; e < h.len; e += 2 * SL_U) {
+    V x[2 * SL_U];
+    typename V2<V>::T v[SL_U];
+#pragma unroll
+    for (int k = 0; k < SL_U; ++k) {
+      x[2 * k] = e + 2 * k < h.len ? vec[h.hc[k].x] : V(0);
+      x[2 * k + 1] = e + 2 * k + 1 < h.len ? vec[h.hc[k].y] : V(0);
+      v[k] = h.hv[k];
+    }
+#pragma unroll
+    for (int k = 0; k < SL_U; ++k) {
+      const int p = (e >> 1) + SL_U + k;
+      if (2 * p < h.len) { h.hc[k] = ld_once(h.c + 32 * p); h.hv[k] = ld_once(h.v + 32 * p); }
+    }
+#pragma unroll
+    for (int k = 0; k < SL_U; ++k) {
+      if (e + 2 * k < h.len) s = r_dot(v[k].x, x[2 * k], s);
+      if (e + 2 * k + 1 < h.len) s = r_dot(v[k].y, x[2 * k + 1], s);
+    }
+  }
+  return s;
+}
+
+template <typename V>
+__global__ void __launch_bounds__(Sl<V>::NT, Sl<V>::MINB) k_dual_sl(DualB<V> a, SliceM<V> M, int m, int j) {
+  grid_trigger();
+  const int r = blockIdx.x * Sl<V>::NT + threadIdx.x;
+  const bool on = r < m;
+  SliceRow<V> h;
+  slice_head(M, r, on, h);
+  grid_wait();
+  if (!on || a.st->status != ST_RUNNING) return;
+  const V s = slice_sum(h, a.xt);
+  dual_row(a, a.tab[j], r, s, a.yold[r], a.b[r], a.ybar[r], a.ylo ? a.ylo[r] : V(0));
+}
+template <typename V>
+__global__ void __launch_bounds__(Sl<V>::NT, Sl<V>::MINB) k_primal_sl(PrimalB<V> a, SliceM<V> M, int n, int j) {
+  grid_trigger();
+  const int r = blockIdx.x * Sl<V>::NT + threadIdx.x;
+  const bool on = r < n;
+  SliceRow<V> h;
+  slice_head(M, r, on, h);
+  grid_wait();
+  if (!on || a.st->status != ST_RUNNING) return;
+  const V s = slice_sum(h, a.zin);
+  primal_row<V, false>(a, a.tab[j], r, s, a.x[r], a.xbar[r], a.c[r], a.l[r], a.u[r]);
+}
+
+template <typename V>
+static void run_chunk_sl(Work& w, int j0, int len, V* xt, V* const* Z, V* ybar, const V* b, const V* ylo, V* x, V* xbar,
+                         const V* c, const V* l, const V* u, cudaStream_t s) {
+  using T = typename V2<V>::T;
+  Profiler& Pr = w.prof;
+  const SlicePlan& q = w.slices;
+  const T* val = sizeof(V) == 4 ? (const T*)q.valf : (const T*)q.vald;
+  DualB<V> da{};
+  da.xt = xt; da.ybar = ybar; da.b = b; da.ylo = ylo; da.tab = w.tab; da.st = w.st; da.ineq = w.row_ineq;
+  PrimalB<V> pa{};
+  pa.x = x; pa.xbar = xbar; pa.xt = xt; pa.c = c; pa.l = l; pa.u = u; pa.tab = w.tab; pa.st = w.st;
+  const SliceM<V> A{w.A.rp, q.sp, q.idx, val}, P{w.P.rp, q.sp + q.nsA, q.idx, val};
+  for (int j = j0; j < j0 + len; ++j) {
+    if (w.m > 0) {
+      da.yold = Z[(j + 1) & 1] + w.n;
+      da.ynew = Z[j & 1] + w.n;
+      if (Pr.on) Pr.begin(0, s, launch_bytes(w, 0, sizeof(V)));
+      launch_early(k_dual_sl<V>, cdiv(w.m, Sl<V>::NT), Sl<V>::NT, 0, s, da, A, w.m, j);
+      if (Pr.on) Pr.end(s);
+    }
+    pa.zin = Z[j & 1];
+    pa.zout = Z[(j + 1) & 1];
+    if (Pr.on) Pr.begin(1, s, launch_bytes(w, 1, sizeof(V)));
+    launch_early(k_primal_sl<V>, cdiv(w.n, Sl<V>::NT), Sl<V>::NT, 0, s, pa, P, w.n, j);
+    if (Pr.on) Pr.end(s);
+  }
+}
+
+// The slice layout from the CSR arrays: A's slices, then P's.
+// width of a slice in pairs: its longest row, rounded up
+__global__ void __launch_bounds__(256) k_slice_width(const int* __restrict__ arp, int m, int nsA,
+                                                     const int* __restrict__ prp, int n, int ns,
+                                                     int* __restrict__ wid) {
+  const int s = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (s >= ns) return;
+  const bool isA = s < nsA;
+  const int r = 32 * (isA ? s : s - nsA) + lane;
+  const int* rp = isA ? arp : prp;
+  const int len = __reduce_max_sync(0xffffffffu, r < (isA ? m : n) ? rp[r + 1] - rp[r] : 0);
+  if (lane == 0) wid[s] = (len + 1) >> 1;
+}
+// columns (val null) or values; the second half of a row's last pair may be a pad
+template <typename V, bool VALUES>
+__global__ void __launch_bounds__(256) k_slice_fill(BCsr<V> A, int m, int nsA, BCsr<V> P, int n, int ns,
+                                                    const int* __restrict__ sp, int2* __restrict__ idx,
+                                                    typename V2<V>::T* __restrict__ val) {
+  const int s = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (s >= ns) return;
+  const bool isA = s < nsA;
+  const int r = 32 * (isA ? s : s - nsA) + lane;
+  if (r >= (isA ? m : n)) return;
+  const int* rp = isA ? A.rp : P.rp;
+  const int e1 = rp[r + 1];
+  size_t at = (size_t)sp[s] * 32 + lane;
+  for (int e = rp[r]; e < e1; e += 2, at += 32) {
+    if constexpr (VALUES) {
+      const V* v = isA ? A.val : P.val;
+      typename V2<V>::T q;
+      q.x = v[e];
+      q.y = e + 1 < e1 ? v[e + 1] : V(0);
+      val[at] = q;
+    } else {
+      const int* c = isA ? A.col : P.col;
+      idx[at] = make_int2(c[e], e + 1 < e1 ? c[e + 1] : 0);
+    }
+  }
+}
+// One row per thread has a longer chain than a staged row block: below some 24 MB
+// of matrix the row blocks are faster (n = 60000 in float64: 22.5 against 30.2 us
+// an iteration, n = 300007 in float32: 41.1 against 49.6), above it the solve's
+// tuning decides (n = 300007 in float64: 85.1 against 51.9, n = 1e6 in float32:
+// 123.9 against 115.0).
+bool slices_ok(const Work& w, bool mixed) {
+  return w.count == 1 && w.r == 0 && w.A.nlseg == 0 && w.P.nlseg == 0 && w.P.nblk > 0 &&
+         (w.A.nnz + w.P.nnz) * (mixed ? 8 : 12) >= 24LL << 20;
+}
+void slices_width(Work& w, int* wid, cudaStream_t s) {
+  const SlicePlan& q = w.slices;
+  launch(k_slice_width, cdiv(q.nsA + q.nsP, 8), 256, 0, s, (const int*)w.A.rp, w.m, q.nsA, (const int*)w.P.rp, w.n,
+         q.nsA + q.nsP, wid);
+}
+void slices_fill_index(Work& w, cudaStream_t s) {
+  const SlicePlan& q = w.slices;
+  launch(k_slice_fill<float, false>, cdiv(q.nsA + q.nsP, 8), 256, 0, s, w.A.bscaled_f(), w.m, q.nsA, w.P.bscaled_f(),
+         w.n, q.nsA + q.nsP, (const int*)q.sp, q.idx, (float2*)nullptr);
+}
+void slices_fill_values(Work& w, bool mixed, cudaStream_t s) {
+  const SlicePlan& q = w.slices;
+  if (mixed)
+    launch(k_slice_fill<float, true>, cdiv(q.nsA + q.nsP, 8), 256, 0, s, w.A.bscaled_f(), w.m, q.nsA, w.P.bscaled_f(),
+           w.n, q.nsA + q.nsP, (const int*)q.sp, (int2*)nullptr, q.valf);
+  else
+    launch(k_slice_fill<double, true>, cdiv(q.nsA + q.nsP, 8), 256, 0, s, w.A.bscaled(), w.m, q.nsA, w.P.bscaled(),
+           w.n, q.nsA + q.nsP, (const int*)q.sp, (int2*)nullptr, q.vald);
+}
+
+// ==========================================================================
 // Pipelined persistent variants of the two half-steps.  Each CUDA block loops
 // over row blocks b = blockIdx.x, blockIdx.x + gridDim.x, ...; while it
 // gathers and finishes block b, the index, value and row-pointer ranges of its
@@ -947,6 +1158,16 @@ void iterate_chunk(Work& w, int len, bool mixed, int nt, cudaStream_t s, int j0,
   }
   if (nt == 4) {   // a low-rank term over short rows
     lowrank_run(w, len, mixed, s, j0);
+    return;
+  }
+  if (nt == 5) {   // a row per thread on the slice layout
+    if (mixed) {
+      run_chunk_sl<float>(w, j0, len, w.fxt, w.fZ, w.fybar, w.fb, w.fylo, w.fx, w.fxbar, w.fc, w.fl, w.fu, s);
+      w.fy = w.fZ[(j0 + len - 1) & 1] + w.n;
+    } else {
+      run_chunk_sl<double>(w, j0, len, w.xt, w.Z, w.ybar, w.bs, nullptr, w.x, w.xbar, w.cs, w.ls, w.us, s);
+      w.y = w.Z[(j0 + len - 1) & 1] + w.n;
+    }
     return;
   }
   if (nt == 1) {   // pipelined persistent kernels, 256 threads

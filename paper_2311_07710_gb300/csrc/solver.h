@@ -133,6 +133,17 @@ struct ChunkPlan {
   cudaEvent_t fork = nullptr, join[2] = {nullptr, nullptr};
 };
 
+// The slice layout of a large instance (iteration.cu): slices of 32 rows, A's then P's.
+struct SlicePlan {
+  int state = 0;                          // 0 not looked at, 1 built, -1 not taken
+  int nsA = 0, nsP = 0;
+  long long groups = 0;                   // of 32 pairs of entries
+  int* sp = nullptr;                      // [nsA + nsP + 1] starts, in groups
+  int2* idx = nullptr;                    // [groups][32] columns
+  float2* valf = nullptr;                 // [groups][32] scaled values
+  double2* vald = nullptr;
+};
+
 struct Work {
   int n = 0, m = 0, m_eq = 0;   // totals over the batch (m_eq: single-instance value)
   int count = 1;                // instances stacked block-diagonally
@@ -242,6 +253,7 @@ struct Work {
   double *mp_ax = nullptr, *mp_axb = nullptr, *mp_qxb = nullptr, *mp_aty = nullptr, *mp_atyb = nullptr;
   double *mp_sA[2] = {nullptr, nullptr}, *mp_sQ[2] = {nullptr, nullptr};
   ChunkPlan chunk;
+  SlicePlan slices;
   Profiler prof;
 };
 
@@ -283,7 +295,8 @@ void init_iterates(Work& w, const double* x0, const double* y0, const SolveParam
 // compact: launch only the row blocks of the running instances (batches; the
 // counts of the last check must be in bst_host).
 // nt: 256 or 512 threads per row block, 1 the pipelined persistent kernels, 2
-// the whole chunk in one launch (only where chunk_ok, plan and values built), 4
+// the whole chunk in one launch (only where chunk_ok, plan and values built), 5 the
+// slice layout (built), 4
 // the low-rank kernels (only where lowrank_fused_ok), 3 the
 // member-interleaved family kernels (only where w.fam_il, buffers allocated).
 void iterate_chunk(Work& w, int len, bool mixed, int nt, cudaStream_t s, int j0 = 0, bool compact = false);
@@ -311,6 +324,11 @@ void chunk_plan_classes(Work& w, bool mixed);             // w.chunk.ctas, cls o
 void chunk_fill_index(Work& w, cudaStream_t s);
 void chunk_fill_values(Work& w, bool mixed, cudaStream_t s);
 void chunk_run(Work& w, int len, bool mixed, cudaStream_t s, int j0);
+// the slice layout: whether it can be taken, and its parts
+bool slices_ok(const Work& w, bool mixed);
+void slices_width(Work& w, int* wid, cudaStream_t s);
+void slices_fill_index(Work& w, cudaStream_t s);
+void slices_fill_values(Work& w, bool mixed, cudaStream_t s);
 // a low-rank term over short rows of P: the fused half-step (lowrank.cu)
 bool lowrank_fused_ok(const Work& w, bool mixed);
 void il_slots(Work& w, cudaStream_t s);   // the running members of a family, densely
