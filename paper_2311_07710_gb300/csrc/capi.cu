@@ -1837,8 +1837,9 @@ void alloc_chunk(pdqp_problem* h, bool mixed, cudaStream_t s) {
     pdqp::chunk_fill_index(w, s);
     for (auto& t : ck.side)
       if (!t) CK(cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking));
-    for (cudaEvent_t* e : {&ck.fork, &ck.join[0], &ck.join[1]})
-      if (!*e) CK(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+    if (!ck.fork) CK(cudaEventCreateWithFlags(&ck.fork, cudaEventDisableTiming));
+    for (auto& e : ck.join)
+      if (!e) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     CK(cudaGetLastError());
     ck.built = true;
   }
@@ -2634,7 +2635,8 @@ void pdqp_destroy(pdqp_handle h) {
   if (h->cap) cudaStreamDestroy(h->cap);
   for (auto& t : h->w.chunk.side)
     if (t) cudaStreamDestroy(t);
-  for (cudaEvent_t e : {h->w.chunk.fork, h->w.chunk.join[0], h->w.chunk.join[1]})
+  if (h->w.chunk.fork) cudaEventDestroy(h->w.chunk.fork);
+  for (auto& e : h->w.chunk.join)
     if (e) cudaEventDestroy(e);
   if (h->tmpl) pdqp_destroy(h->tmpl);
   delete h;

@@ -23,6 +23,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <functional>
 #include <mutex>
 
 #include "rowblock.cuh"
@@ -449,23 +450,88 @@ static void prepare_chunk() {   // once per process
   std::call_once(once, [] { g_chunk_max_ctas = std::min(chunk_resident_ctas<float>(), chunk_resident_ctas<double>()); });
 }
 
-// CTAs per instance: with at least as many instances as SMs one each; fewer
-// instances share the SMs out (a power of two, at most one slice of P per CTA).
-// In float64 up to two CTAs an SM: the float64 pipes bind there, and a second
-// round of small instances costs less than half the pipes idle.
-static int chunk_ctas(const Work& w, bool mixed) {
-  int big = 1;
-  for (const Inst& I : w.inst_host) big = std::max(big, cdiv(I.n, 32));
-  int k = 1;
-  while (2 * k <= g_chunk_max_ctas && 2 * k * w.count <= (mixed ? 1 : 2) * w.num_sms && 2 * k <= big) k *= 2;
-  return k;
+// CTAs of every instance: one each with at least as many instances as SMs.
+// Fewer instances share out the SMs by their rows, so that no CTA has much more to
+// do than another and all run at once: the least bound on a CTA's rows under which
+// the clusters fit the SMs (a cluster lies within one GPC, taken as 19 SMs of which
+// pairs give 18 to clusters; without that, 30 control QPs in float64 took 9.0 us an
+// iteration, with it 5.9).  A power of two of CTAs for all, as before, leaves the
+// launch waiting for the largest: 77 control QPs of horizons 10 to 100 took 12.7 us
+// in float64 and 5.4 in mixed precision against 9.8 and 4.1.
+// In float64, more than half as many instances as SMs keep two CTAs each where that
+// finishes earlier (pairs dealt out largest first to the SMs as they fall free): the
+// float64 pipes bind there, and a second round of small instances costs less than
+// idle pipes (151 of them 17.7 us against 23.2, 120 of them 14.1 against 17.2).
+static std::vector<int> chunk_ctas(const Work& w, bool mixed) {
+  std::vector<int> out(w.count, 1);
+  if (w.count >= w.num_sms) return out;
+  static const int kSizes[] = {1, 2, 3, 4, 6, 8, 12, 16};
+  const int gpcs = std::max(1, w.num_sms / 19);
+  // larger clusters pay with their barriers: 1500 rows (n = 1000) take 3.26 us an
+  // iteration on 8 CTAs, 3.45 on 16; 2824 (a control QP of horizon 100) 3.15, 3.30 on
+  // 12 and 3.46; 1000 rows 2.69 on 4 and 2.96 on 16; 6000 rows 4.69 on 12 and 4.90, in
+  // float64 10.0 on 16 and 11.6 on 12
+  auto cap = [&](const Inst& I) {
+    int k = 1;
+    for (int q : kSizes) {
+      const int rows = q <= 4 ? 100 : q <= 8 ? 187 : q <= 12 || !mixed ? 250 : 500;   // at least, a CTA
+      if (q <= g_chunk_max_ctas && 32 * (q - 1) < I.n && (long long)q * rows <= I.n + I.m) k = q;
+    }
+    return k;
+  };
+  auto split = [&](long long rows) {              // at most `rows` rows per CTA: whether all CTAs fit
+    int all = 0, of_size[17] = {};
+    for (int i = 0; i < w.count; ++i) {
+      const Inst& I = w.inst_host[i];
+      int k = 1;
+      for (int q : kSizes)
+        if (q <= cap(I) && (long long)k * rows < I.n + I.m) k = q;
+      all += out[i] = k;
+      ++of_size[k];
+    }
+    std::vector<int> room(gpcs, 18);
+    for (int k = 16; k > 1; --k)
+      for (int c = 0; c < of_size[k]; ++c) {
+        auto g = std::find_if(room.begin(), room.end(), [&](int r) { return r >= k; });
+        if (g == room.end()) return false;
+        *g -= k;
+      }
+    return all <= w.num_sms;
+  };
+  long long lo = 1, hi = 1;
+  for (const Inst& I : w.inst_host) hi = std::max<long long>(hi, I.n + I.m);
+  while (lo < hi) {
+    const long long mid = (lo + hi) / 2;
+    if (split(mid)) hi = mid;
+    else lo = mid + 1;
+  }
+  split(hi);
+  if (mixed || 2 * w.count <= w.num_sms) return out;
+  double most = 0.0;                               // rows of the fullest CTA
+  std::vector<int> rows(w.count);
+  for (int i = 0; i < w.count; ++i) {
+    rows[i] = w.inst_host[i].n + w.inst_host[i].m;
+    most = std::max(most, (double)rows[i] / out[i]);
+  }
+  constexpr int k = 2;
+  std::sort(rows.begin(), rows.end(), std::greater<int>());
+  std::vector<double> busy(w.num_sms, 0.0);
+  for (int r : rows) {
+    std::partial_sort(busy.begin(), busy.begin() + k, busy.end());
+    std::fill(busy.begin(), busy.begin() + k, busy[k - 1] + (double)r / k);
+  }
+  if (*std::max_element(busy.begin(), busy.end()) < 0.9 * most)
+    for (int i = 0; i < w.count; ++i) out[i] = std::min(k, cap(w.inst_host[i]));
+  return out;
 }
 
 template <typename V>
-static bool chunk_fits(const Work& w, int ctas) {
-  for (const Inst& I : w.inst_host) {
+static bool chunk_fits(const Work& w, const std::vector<int>& ctas) {
+  for (int i = 0; i < w.count; ++i) {
+    const Inst& I = w.inst_host[i];
     if (I.n + I.m > 65535) return false;          // 16-bit columns, the pads' slot included
-    if (chunk_fixed_bytes<V>(I.n, I.m, cdiv(cdiv(I.m, 32), ctas), cdiv(cdiv(I.n, 32), ctas)) > (size_t)CHUNK_SMEM_MAX)
+    if (chunk_fixed_bytes<V>(I.n, I.m, cdiv(cdiv(I.m, 32), ctas[i]), cdiv(cdiv(I.n, 32), ctas[i])) >
+        (size_t)CHUNK_SMEM_MAX)
       return false;
   }
   return true;
@@ -474,7 +540,7 @@ static bool chunk_fits(const Work& w, int ctas) {
 bool chunk_ok(const Work& w, bool mixed) {
   if (w.r != 0 || w.A.nlseg != 0 || w.P.nlseg != 0 || w.n < 1) return false;
   prepare_chunk();
-  const int k = chunk_ctas(w, mixed);
+  const std::vector<int> k = chunk_ctas(w, mixed);
   return mixed ? chunk_fits<float>(w, k) : chunk_fits<double>(w, k);
 }
 
@@ -486,9 +552,10 @@ bool chunk_ok(const Work& w, bool mixed) {
 // 2.7 us (n = 1000, 4e3 nonzeros per CTA) against 7.5, 8.1 (n = 1e4, 19e3) against
 // 8.0; in float64 10.5 (n = 4000, 8e3) against 13.
 bool chunk_pays(const Work& w, bool mixed) {
-  const int k = chunk_ctas(w, mixed);
   if (w.count >= 20) return true;
-  return (w.A.nnz + w.P.nnz) / ((long long)w.count * k) <= (mixed ? 18000 : 8000);
+  long long k = 0;
+  for (int c : chunk_ctas(w, mixed)) k += c;
+  return (w.A.nnz + w.P.nnz) / k <= (mixed ? 18000 : 8000);
 }
 
 // The launches of one precision: the instances, in launch order (largest
@@ -502,23 +569,24 @@ bool chunk_pays(const Work& w, bool mixed) {
 template <typename V>
 static void chunk_classes(Work& w, std::vector<ChunkClass>& out) {
   ChunkPlan& ck = w.chunk;
-  const int ctas = ck.ctas[sizeof(V) == 4 ? 1 : 0];
   out.clear();
   const size_t gb = chunk_group_bytes<V>();
   int cls_of_prev = -1;
   for (int i = 0; i < w.count; ++i) {
     const ChunkInst& I = ck.order[i];
+    const int ctas = ck.ctas[I.id];
     const int oA = cdiv(I.nsA, ctas), oP = cdiv(I.nsP, ctas);
     const size_t fixed = chunk_fixed_bytes<V>(I.n, I.m, oA, oP);
     // a CTA's share of the groups, rounded up by a slice's worth
     const size_t own = ((size_t)ck.groups[i].x + ck.groups[i].y) / ctas;
     const size_t need = fixed + (ctas > 1 ? own + own / 8 + 64 : own) * gb;
     int c = 0;
-    if (ctas == 1)
+    if (ctas > 1) c = 2 + ctas;
+    else if (w.count >= w.num_sms)
       c = need <= 64 * 1024 && fixed <= 48 * 1024 ? 2
           : (need <= 130 * 1024 || w.count >= 2 * w.num_sms) && fixed <= 108 * 1024 ? 1 : 0;
     if (c != cls_of_prev) {
-      out.push_back(ChunkClass{i, 0, 0, 0});
+      out.push_back(ChunkClass{i, 0, 0, ctas, 0});
       cls_of_prev = c;
     }
     ChunkClass& k = out.back();
@@ -547,12 +615,15 @@ void chunk_plan_order(Work& w, const std::vector<int2>& groups) {   // groups: b
   ChunkPlan& ck = w.chunk;
   auto total = [&](const ChunkInst& p) { return (long long)groups[p.id].x + groups[p.id].y; };
   std::stable_sort(ck.order.begin(), ck.order.end(),
-                   [&](const ChunkInst& p, const ChunkInst& q) { return total(p) > total(q); });
+                   [&](const ChunkInst& p, const ChunkInst& q) {
+                     const int rp = p.n + p.m, rq = q.n + q.m;   // with few instances the rows set the CTAs
+                     return w.count < w.num_sms && rp != rq ? rp > rq : total(p) > total(q);
+                   });
   ck.groups.resize(w.count);
   for (int i = 0; i < w.count; ++i) ck.groups[i] = groups[ck.order[i].id];
 }
 void chunk_plan_classes(Work& w, bool mixed) {
-  w.chunk.ctas[mixed ? 1 : 0] = chunk_ctas(w, mixed);
+  w.chunk.ctas = chunk_ctas(w, mixed);
   if (mixed) chunk_classes<float>(w, w.chunk.cls[1]);
   else chunk_classes<double>(w, w.chunk.cls[0]);
 }
@@ -567,10 +638,9 @@ static void run_chunk(Work& w, int j0, int len, const typename Pair<V>::T* val, 
   // kind 3: one launch holds both half-steps of `len` iterations
   if (Pr.on) Pr.begin(3, s, len * (launch_bytes(w, 0, sizeof(V)) + launch_bytes(w, 1, sizeof(V))));
   const std::vector<ChunkClass>& cls = ck.cls[sizeof(V) == 4 ? 1 : 0];
-  const int ctas = ck.ctas[sizeof(V) == 4 ? 1 : 0];
   // the classes run side by side (forked onto the plan's own streams), so that
   // their CTAs share the SMs and no class's last wave leaves the chip idle
-  const size_t sides = std::min<size_t>(cls.size() - 1, 2);
+  const size_t sides = std::min<size_t>(cls.size() - 1, ChunkPlan::SIDES);
   if (sides) cudaEventRecord(ck.fork, s);
   for (size_t k = 0; k < sides; ++k) cudaStreamWaitEvent(ck.side[k], ck.fork, 0);
   for (size_t k = 0; k < cls.size(); ++k) {
@@ -578,8 +648,8 @@ static void run_chunk(Work& w, int j0, int len, const typename Pair<V>::T* val, 
     a.smem = (int)q.smem;
     cudaLaunchAttribute at[1];
     const cudaLaunchConfig_t cfg =
-        chunk_cfg<V>(ctas, q.count, q.threads, q.smem, k == 0 ? s : ck.side[(k - 1) % 2], at);
-    if (ctas > 1) cudaLaunchKernelEx(&cfg, k_chunk<V, true>, a, q.first, j0, len);
+        chunk_cfg<V>(q.ctas, q.count, q.threads, q.smem, k == 0 ? s : ck.side[(k - 1) % ChunkPlan::SIDES], at);
+    if (q.ctas > 1) cudaLaunchKernelEx(&cfg, k_chunk<V, true>, a, q.first, j0, len);
     else cudaLaunchKernelEx(&cfg, k_chunk<V, false>, a, q.first, j0, len);
     count_launch();
   }

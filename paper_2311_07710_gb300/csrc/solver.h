@@ -113,12 +113,12 @@ struct ChunkInst {
 };
 // Instances [first, first + count) of the launch order in one launch.
 struct ChunkClass {
-  int first, count, threads;
+  int first, count, threads, ctas;
   size_t smem;
 };
 struct ChunkPlan {
   bool built = false;
-  int ctas[2] = {1, 1};                   // CTAs per instance (a cluster when > 1): float64, mixed
+  std::vector<int> ctas;                  // CTAs per instance (a cluster when > 1), of the classes planned last
   int slices = 0;
   long long ngroups = 0;
   std::vector<ChunkInst> order;           // launch order, largest first
@@ -129,8 +129,9 @@ struct ChunkPlan {
   double2* vald = nullptr;
   std::vector<int2> groups;               // {of A, of P} per instance, in launch order
   std::vector<ChunkClass> cls[2];         // launches: float64, mixed
-  cudaStream_t side[2] = {nullptr, nullptr};   // the second and later launches' streams
-  cudaEvent_t fork = nullptr, join[2] = {nullptr, nullptr};
+  static constexpr int SIDES = 7;
+  cudaStream_t side[SIDES] = {};          // the second and later launches' streams
+  cudaEvent_t fork = nullptr, join[SIDES] = {};
 };
 
 // The slice layout of a large instance (iteration.cu): slices of 32 rows, A's then P's.
@@ -320,7 +321,7 @@ void chunk_plan_instances(Work& w);                       // w.chunk.order, slic
 void chunk_widths(Work& w, int* wid, cudaStream_t s);     // pairs per slice
 void chunk_groups(Work& w, int2* out, cudaStream_t s);    // groups of A and of P per instance
 void chunk_plan_order(Work& w, const std::vector<int2>& groups);   // largest instances first
-void chunk_plan_classes(Work& w, bool mixed);             // w.chunk.ctas, cls of one precision
+void chunk_plan_classes(Work& w, bool mixed);             // cls of one precision
 void chunk_fill_index(Work& w, cudaStream_t s);
 void chunk_fill_values(Work& w, bool mixed, cudaStream_t s);
 void chunk_run(Work& w, int len, bool mixed, cudaStream_t s, int j0);
