@@ -431,7 +431,7 @@ def run_ours(args, world, rank, local):
                      "speedup_of_value": value / (world * k64 * per_step / (t64 / 1e3)),
                      "setup_ms": 1e3 * info64.setup_seconds, "iterate_ms": 1e3 * info64.iterate_seconds,
                      "kernel_ms": {k: v["ms"] for k, v in prof64.items()},
-                     "roofline": roofline_fp64(prof64, nnz_A, nnz_P, N, M)}
+                     "roofline": roofline_fp64(prof64, nnz_A, nnz_P, N, M, period=args.check_period or 64)}
         # the same float64 solves with maintained products: the iteration
         # carries A x, A x_bar, Q x_bar, A'y, A'y_bar, and a check gathers x
         # once for A x and once for Q x
@@ -488,15 +488,18 @@ def run_ours(args, world, rank, local):
 
     # ---- roofline of the dominant kernel ----
     hbm_peak, hbm_src = peak_of("hbm_gbs")
-    # "other": the one-launch cluster chunk (both half-steps of a chunk per launch)
+    # "other": the one-launch chunk (both half-steps of a chunk per launch)
     kinds = {k: v for k, v in prof.items() if k in ("dual", "primal", "other") and v["launches"]}
     dom = max(kinds, key=lambda k: kinds[k]["ms"])
     d = prof[dom]
     avg_s = d["ms"] / d["launches"] / 1e3
+    d = launch_once(d, dom, args.check_period or 64)
     achieved_gbs = d["bytes"] / avg_s / 1e9
-    kname = {"dual": "k_dual", "primal": "k_primal", "other": "k_chunk_cluster"}[dom]
+    kname = {"dual": "k_dual", "primal": "k_primal", "other": "k_chunk"}[dom]
     if args.maintained_products:
         kname += "_mp"
+    elif infos[-1].spmv_threads == 5:
+        kname += "_sl"
     nnz_rows = (nnz_A, M, 8) if dom == "dual" else (nnz_P, N, 15)
     flops = 2.0 * nnz_rows[0] + nnz_rows[2] * nnz_rows[1]
     if args.precision == "fp64" and dom != "other":
@@ -617,21 +620,32 @@ def _timed(stream, fn):
     return e0.elapsed_time(e1) / 1e3, out
 
 
-def roofline_fp64(prof, nnz_A, nnz_P, N, M, names=("k_dual", "k_primal")):
+def launch_once(d, kind, period):
+    """A kind's profile with the bytes that one launch cannot do without: the
+    one-launch chunk ("other") is counted both half-steps of each of its `period`
+    iterations, and reads and writes each matrix and vector once for all of them."""
+    return dict(d, bytes=d["bytes"] / period) if kind == "other" else d
+
+
+def roofline_fp64(prof, nnz_A, nnz_P, N, M, names=("k_dual", "k_primal"), period=64):
     """Roofline of the dominant iteration kernel of a float64 solve: against
     HBM by its algorithmic bytes and against the nominal float64 rate by its
     flops (2 per nonzero and ~15 per row of the update); the larger fraction
     names the bound."""
     hbm_peak, hbm_src = peak_of("hbm_gbs")
-    kinds = {k: v for k, v in prof.items() if k in ("dual", "primal") and v["launches"]}
+    kinds = {k: v for k, v in prof.items() if k in ("dual", "primal", "other") and v["launches"]}
     dom = max(kinds, key=lambda k: kinds[k]["ms"])
     d = prof[dom]
     avg_s = d["ms"] / d["launches"] / 1e3
     nnz, rows, per_row = (nnz_A, M, 8) if dom == "dual" else (nnz_P, N, 15)
     flops = 2.0 * nnz + per_row * rows
+    if dom == "other":     # the one-launch chunk: `period` iterations of the instances that run (by their bytes)
+        d = launch_once(d, dom, period)
+        whole = 12.0 * (nnz_A + nnz_P) + 4.0 * (M + N + 2) + 8.0 * (11.0 * N + 6.0 * M)
+        flops = period * (2.0 * (nnz_A + nnz_P) + 8.0 * M + 15.0 * N) * d["bytes"] / whole
     frac_hbm = d["bytes"] / avg_s / 1e9 / hbm_peak
     frac_alu = flops / avg_s / (FP64_NOMINAL_TFLOPS * 1e12)
-    roof = {"kernel": {"dual": names[0], "primal": names[1]}[dom], "avg_launch_us": avg_s * 1e6,
+    roof = {"kernel": {"dual": names[0], "primal": names[1], "other": "k_chunk"}[dom], "avg_launch_us": avg_s * 1e6,
             "launches": d["launches"], "algorithmic_bytes_per_launch": d["bytes"],
             "hbm": {"achieved_gbs": d["bytes"] / avg_s / 1e9, "peak": hbm_peak, "frac": frac_hbm,
                     "peak_source": hbm_src},
@@ -723,13 +737,13 @@ def plain_fp64_cold(pdqp, insts, stream, dev):
 
 
 def _roofline_of(prof, hbm_peak, hbm_src, note):
-    kinds = {k: v for k, v in prof.items() if k in ("dual", "primal") and v["launches"]}
+    kinds = {k: v for k, v in prof.items() if k in ("dual", "primal", "other") and v["launches"]}
     dom = max(kinds, key=lambda k: kinds[k]["ms"])
-    d = prof[dom]
+    d = launch_once(prof[dom], dom, 64)
     avg_s = d["ms"] / d["launches"] / 1e3
     return {"bound": "hbm", "achieved": d["bytes"] / avg_s / 1e9, "peak": hbm_peak, "unit": "GB/s",
             "frac": d["bytes"] / avg_s / 1e9 / hbm_peak, "peak_source": hbm_src,
-            "kernel": {"dual": "k_dual", "primal": "k_primal"}[dom], "avg_launch_us": avg_s * 1e6,
+            "kernel": {"dual": "k_dual", "primal": "k_primal", "other": "k_chunk"}[dom], "avg_launch_us": avg_s * 1e6,
             "launches": d["launches"], "algorithmic_bytes_per_launch": d["bytes"],
             "bytes_counted": note, "traffic": None, "timing": PROFILED_PASS}
 
@@ -1048,7 +1062,7 @@ def run_gemm(args, world, rank, local):
                        "l2": "operands 128 MiB each at 8192, larger than L2 with the output"},
             "roofline": {"bound": "tensor", "achieved": top["tflops"], "peak": peak, "unit": "TFLOP/s",
                          "frac": top["frac"], "peak_source": peak_src,
-                         "kernel": "k_gemm_tn_p", "traffic": None},
+                         "kernel": "k_gemm_tn_pair", "traffic": None},
             "shapes": results, "gpu_launches": args.steps * sum(1 + (r["splits"] > 1) for r in results)}
     if rank == 0:
         print(json.dumps(line), flush=True)

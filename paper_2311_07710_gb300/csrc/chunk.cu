@@ -470,12 +470,15 @@ static std::vector<int> chunk_ctas(const Work& w, bool mixed) {
   // larger clusters pay with their barriers: 1500 rows (n = 1000) take 3.26 us an
   // iteration on 8 CTAs, 3.45 on 16; 2824 (a control QP of horizon 100) 3.15, 3.30 on
   // 12 and 3.46; 1000 rows 2.69 on 4 and 2.96 on 16; 6000 rows 4.69 on 12 and 4.90, in
-  // float64 10.0 on 16 and 11.6 on 12
+  // float64 10.0 on 16 and 11.6 on 12.  Rows much longer than these (15 to 43 thousand
+  // nonzeros in all) pay for more: 5000 nonzeros a CTA, counted by the rows.
+  const double per_row = (double)(w.A.nnz + w.P.nnz) / std::max<long long>(1, (long long)w.n + w.m);
   auto cap = [&](const Inst& I) {
     int k = 1;
     for (int q : kSizes) {
       const int rows = q <= 4 ? 100 : q <= 8 ? 187 : q <= 12 || !mixed ? 250 : 500;   // at least, a CTA
-      if (q <= g_chunk_max_ctas && 32 * (q - 1) < I.n && (long long)q * rows <= I.n + I.m) k = q;
+      const bool enough = (long long)q * rows <= I.n + I.m || q * 5000.0 <= per_row * (I.n + I.m);
+      if (q <= g_chunk_max_ctas && 32 * (q - 1) < I.n && enough) k = q;
     }
     return k;
   };
@@ -544,9 +547,9 @@ bool chunk_ok(const Work& w, bool mixed) {
   return mixed ? chunk_fits<float>(w, k) : chunk_fits<double>(w, k);
 }
 
-// Whether the chunk beats the per-iteration kernels.  From 20 instances on
-// (at most 4 CTAs each; 8 in float64) it always did: 1200 control QPs 17 us per
-// iteration against 88, 160 of them 3.8 against 12, 77 in float64 11 against 16.
+// Whether the chunk beats the per-iteration kernels.  From 20 instances on it
+// always did: 1200 control QPs 17 us per iteration against 88, 160 of them 3.8
+// against 12, 77 in float64 9.8 against 16.
 // A few instances on many CTAs pay for the cluster barriers and, on random
 // patterns, for bank conflicts: random sparse QPs, per iteration in float32,
 // 2.7 us (n = 1000, 4e3 nonzeros per CTA) against 7.5, 8.1 (n = 1e4, 19e3) against

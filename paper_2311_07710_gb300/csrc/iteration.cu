@@ -5,9 +5,10 @@
 //   k_primal : rows of P = [Q | -A'] gathering [x_md ; y+] -- g = Q x_md + c - A'y+,
 //              x+ = proj_[l,u](x - tau g), x_bar+ = (1 - 1/beta) x_bar + x+/beta,
 //              and the next iteration's x_md and x_tilde
-// with their pipelined persistent variants, the member-interleaved family
-// kernels, the segment sums of long rows, and the host loop that launches a
-// chunk of iterations (a whole chunk in one launch: chunk.cu).
+// with their pipelined persistent variants, the kernels of a row per thread on
+// the slice layout, the member-interleaved family kernels, the segment sums of
+// long rows, and the host loop that launches a chunk of iterations (a whole chunk
+// in one launch: chunk.cu).
 #include <algorithm>
 
 #include "rowblock.cuh"
