@@ -124,9 +124,10 @@ typedef struct {
                                 by member, v[j * members + i], one warp per row for 32
                                 members, so one matrix entry meets 128 members in one
                                 coalesced load,
-                                0 = chosen: 3 for an eligible family handle; 2 where
-                                every instance's vectors fit a CTA's shared memory and
-                                the instances are many or small; for a low-rank term
+                                0 = chosen: 2 where every instance's vectors fit a
+                                CTA's shared memory and the instances are many or
+                                small (a family: up to 300 thousand rows in all); 3
+                                for the other eligible family handles; for a low-rank term
                                 over short rows of P, kernels that read the factor once
                                 per iteration (pdqp_info reports them as 4, which
                                 cannot be asked for); else the first full chunk of a

@@ -676,7 +676,14 @@ pdqp_status solve_impl(pdqp_problem* h, const pdqp_options& o, const double* x0,
     throw Fail{PDQP_ERR_INVALID, "options.maintained_products: a row of A or P holds more nonzeros than a row block"};
   if (mp && h->resume)
     throw Fail{PDQP_ERR_INVALID, "options.maintained_products: a solve resumed from pdqp_set_state is not supported"};
-  const bool use_il = il_ok && !mp && (o.spmv_threads == 0 || o.spmv_threads == 3);
+  // A family of up to 300 thousand rows in all takes the one-launch chunk like any
+  // batch: two launches an iteration and a few busy lanes cost the interleaved
+  // kernels as much as a large family (members of 420 + 210 rows: 12 of them 8.9 ms
+  // a solve against 2.3, 300 of them 9.6 against 4.9; of 1000 + 500: 200 of them 15.0
+  // against 12.3; of 2500 + 1250: 60 of them 14.4 against 10.1, 160 of them 17.9
+  // against 23.1, and there the shared matrix read once wins).
+  const bool fam_chunk = il_ok && chunk_ok && (long long)w.n + w.m <= 300000 && pdqp::chunk_pays(w, mixed);
+  const bool use_il = il_ok && !mp && ((o.spmv_threads == 0 && !fam_chunk) || o.spmv_threads == 3);
   if (mixed) alloc_mixed(h);
   if (use_il) alloc_il(h, mixed, o.check_period);
   w.il_active = use_il;
