@@ -852,7 +852,11 @@ struct LzArgs {
   // (its readers multiply by pi_inv_norm, k_lz_orth writes v = r / beta back);
   // 0: k_lz_norm normalises it in place (a low-rank term reads it as well)
   int lazy;
-  double* cpart;                   // [2][nchunk] chunk sums of the row-block partials
+  // [2][nchunk] chunk sums of the row-block partials: of v'w (k_lz_n; the alphas)
+  // and of |r|^2 (k_lz_orth).  Apart, since a warp of k_lz_orth may read its
+  // instance's v'w after another chunk of the instance has closed its |r|^2.
+  double* cpart;
+  double* rpart;
   unsigned* ticket;                // [nchunk] zero between launches
   int nchunk;
   // batches late in the estimates: the row blocks of the instances still
@@ -864,13 +868,13 @@ struct LzArgs {
 // After row block b of instance i wrote its two partials (part[b],
 // part[nblkP + b]; one thread): the last of its chunk's blocks to finish -- a
 // ticket taken after a fence -- sums the chunk's partials in block order into
-// the chunk sums and resets the ticket.  Chunks are KKT_CHUNK consecutive row
+// the chunk sums `out` and resets the ticket.  Chunks are KKT_CHUNK consecutive row
 // blocks from the instance's first, so a batch, a family member and a
 // standalone solve sum alike, and the per-instance reductions (one CUDA block
 // each) read tens of chunk sums instead of thousands of partials.  No waits:
 // every block of a chunk runs the kernel to this point or none does (the
 // early exits test the instance's state only).
-__device__ __forceinline__ void lz_chunk_close(const LzArgs& a, const double* part, int b, int i) {
+__device__ __forceinline__ void lz_chunk_close(const LzArgs& a, const double* part, int b, int i, double* out) {
   const Inst in = a.inst[i];
   const int c = (b - in.bP0) / KKT_CHUNK;
   const int c0 = in.bP0 + c * KKT_CHUNK, c1 = min(c0 + KKT_CHUNK, in.bP1);
@@ -883,8 +887,8 @@ __device__ __forceinline__ void lz_chunk_close(const LzArgs& a, const double* pa
     s0 += __ldcg(part + k);
     s1 += __ldcg(part + (size_t)a.nblkP + k);
   }
-  a.cpart[g] = s0;
-  a.cpart[(size_t)a.nchunk + g] = s1;
+  out[g] = s0;
+  out[(size_t)a.nchunk + g] = s1;
   a.ticket[g] = 0u;
 }
 
@@ -991,7 +995,7 @@ __global__ void __launch_bounds__(NT, MinBlocks<V, NT, LR>::value) k_lz_n(BCsr<V
   if (tid == 0) {
     part[bk] = f[0];
     part[(size_t)la.nblkP + bk] = f[1];
-    lz_chunk_close(la, part, bk, la.blk_inst_P[bk]);
+    lz_chunk_close(la, part, bk, la.blk_inst_P[bk], la.cpart);
   }
 }
 
@@ -1128,7 +1132,7 @@ __global__ void __launch_bounds__(256) k_lz_orth(LzArgs a, BCsr<V> P, const V* w
   if (lane == 0) {
     part[b] = f[0];
     part[(size_t)a.nblkP + b] = f[1];
-    lz_chunk_close(a, part, b, i);
+    lz_chunk_close(a, part, b, i, a.rpart);
   }
 }
 
@@ -1328,7 +1332,7 @@ __global__ void __launch_bounds__(NT) k_lz_beta(LzArgs a, double tol, int max_st
   if (st.pi_done[0] && st.pi_done[1]) return;     // uniform: nothing left to do
   const Inst in = a.inst[i];
   double f[2] = {0.0, 0.0};
-  lz_block_sums(a.cpart, a.nchunk, in.cP0, in.cP0 + kkt_chunks(in.bP0, in.bP1), f);
+  lz_block_sums(a.rpart, a.nchunk, in.cP0, in.cP0 + kkt_chunks(in.bP0, in.bP1), f);
   const bool is_max[2] = {false, false};
   block_reduce<2>(f, is_max);
   __shared__ double beta[2], s_lo[2], s_hi[2], s_theta[2][2];
@@ -2138,7 +2142,9 @@ static LzArgs lz_args(Work& w) {
   la.blk_inst_P = w.blk_inst_P; la.blk_inst_A = w.blk_inst_A; la.row_inst_n = w.row_inst_n;
   la.nblkP = w.P.nblk;
   la.lazy = w.r == 0 ? 1 : 0;
-  la.cpart = w.cpart_n; la.ticket = w.lz_ticket; la.nchunk = w.nchunk_n;
+  la.cpart = w.cpart_n;                        // (15 chunk sums a chunk, of which these take four)
+  la.rpart = w.cpart_n + 2 * (size_t)w.nchunk_n;
+  la.ticket = w.lz_ticket; la.nchunk = w.nchunk_n;
   if (w.lz_compact) { la.actA = w.act_A; la.actP = w.act_P; la.nactP = w.bst_host->act_P; }
   return la;
 }
