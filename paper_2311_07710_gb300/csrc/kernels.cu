@@ -1880,8 +1880,6 @@ __device__ void decide_thread0(DevState* st, const double* F, const double (*P)[
   }
 }
 
-// Restart of the outer loop from the candidate: x = x_bar = x_md = x_tilde = x_c,
-// y = y_bar = y_c, anchors = z_c (Algorithm 1 "restart the outer loop").
 // Row blocks of the instances still running (batches): indices in act, their
 // number in *n (in any order: a block's rows do not depend on its place in
 // the grid).
@@ -1891,9 +1889,16 @@ __global__ void k_compact_blocks(const int* __restrict__ blk_inst, int nblk, con
     if (st[blk_inst[b]].status == ST_RUNNING) act[atomicAdd(n, 1)] = b;
 }
 
+// Restart of the outer loop from the candidate: x = x_bar = x_md = x_tilde = x_c,
+// y = y_bar = y_c, anchors = z_c (Algorithm 1 "restart the outer loop").
+// y_other (batches): the half of Z whose y part y is not.  A member that has
+// stopped keeps its y in both halves: later chunks leave its rows alone, and
+// one of odd length (an iteration limit inside a period) moves the handle's y
+// to the other half.
 __global__ void k_restart_apply(const DevState* sts, const int* inst_n,
                                 const int* inst_m, int n, int m, double* x, double* xbar,
-                                double* xmd0, double* xt, double* ax, double* y, double* ybar, double* ay) {
+                                double* xmd0, double* xt, double* ax, double* y, double* ybar, double* ay,
+                                double* y_other) {
   grid_trigger();
   grid_wait();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < max(n, m); i += gridDim.x * blockDim.x) {
@@ -1909,6 +1914,8 @@ __global__ void k_restart_apply(const DevState* sts, const int* inst_n,
       if (s.status == ST_RUNNING && s.restart) {
         const double v = s.cand_avg ? ybar[i] : y[i];
         y[i] = v; ybar[i] = v; ay[i] = v;
+      } else if (y_other && s.status != ST_RUNNING) {
+        y_other[i] = y[i];
       }
     }
   }
@@ -2547,9 +2554,10 @@ void check(Work& w, const SolveParams& p, int mode, long long chunk_len, bool mi
   launch_early(k_decide, w.count, 64, 0, s, da, p, mode, chunk_len);
   if (mixed) {
     launch_early(k_mixed_rebase, grid_v, 256, 0, s, mixed_args(w), mode == 0 ? 1 : 0);
-  } else if (mode == 1) {
+  } else if (mode == 1 || w.count > 1) {   // (at the start point nothing restarts; members may stop)
+    double* const y_other = w.count > 1 ? (w.y == w.Z[1] + w.n ? w.Z[0] : w.Z[1]) + w.n : nullptr;
     launch_early(k_restart_apply, grid_v, 256, 0, s, (const DevState*)w.st, (const int*)w.row_inst_n,
-           (const int*)w.row_inst_m, w.n, w.m, w.x, w.xbar, w.Z[0], w.xt, w.ax, w.y, w.ybar, w.ay);
+           (const int*)w.row_inst_m, w.n, w.m, w.x, w.xbar, w.Z[0], w.xt, w.ax, w.y, w.ybar, w.ay, y_other);
   }
   if (w.count > 1) count_running(w, s);   // (one instance: k_decide)
   if (w.count > 1) {   // the running instances' row blocks, for compacted launches
