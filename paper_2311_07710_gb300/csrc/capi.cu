@@ -635,7 +635,8 @@ void tuned_store(const Work& w, bool mixed, int nt) {
   g_tuned[tune_key(w, mixed)] = nt;
 }
 
-void alloc_chunk(pdqp_problem* h, bool mixed, cudaStream_t s);   // with the device scans, below
+void plan_chunk(pdqp_problem* h, cudaStream_t s);                // with the device scans, below
+void alloc_chunk(pdqp_problem* h, bool mixed, cudaStream_t s);
 bool alloc_slices(pdqp_problem* h, bool mixed, cudaStream_t s);
 
 // options.spmv_threads = 2: at most 64 row blocks of A and of P, no row longer
@@ -682,8 +683,16 @@ pdqp_status solve_impl(pdqp_problem* h, const pdqp_options& o, const double* x0,
   // a solve against 2.3, 300 of them 9.6 against 4.9; of 1000 + 500: 200 of them 15.0
   // against 12.3; of 2500 + 1250: 60 of them 14.4 against 10.1, 160 of them 17.9
   // against 23.1, and there the shared matrix read once wins).
-  const bool fam_chunk = il_ok && chunk_ok && (long long)w.n + w.m <= 300000 && pdqp::chunk_pays(w, mixed);
-  const bool use_il = il_ok && !mp && ((o.spmv_threads == 0 && !fam_chunk) || o.spmv_threads == 3);
+  const bool il_small = il_ok && (long long)w.n + w.m <= 300000;
+  // the one-launch chunk: asked for, or chosen where every instance fits it
+  bool use_chunk = !mp && chunk_ok &&
+                   (o.spmv_threads == 2 ||
+                    (o.spmv_threads == 0 && (!il_ok || il_small) && pdqp::chunk_pays(w, mixed)));
+  if (use_chunk) {
+    plan_chunk(h, s);
+    if (o.spmv_threads == 0) use_chunk = pdqp::chunk_even(w, mixed);
+  }
+  const bool use_il = il_ok && !mp && ((o.spmv_threads == 0 && !use_chunk) || o.spmv_threads == 3);
   if (mixed) alloc_mixed(h);
   if (use_il) alloc_il(h, mixed, o.check_period);
   w.il_active = use_il;
@@ -696,8 +705,6 @@ pdqp_status solve_impl(pdqp_problem* h, const pdqp_options& o, const double* x0,
   if (w.detect) alloc_infeas(h, s);
   SolveParams p = make_params(o);
   if (use_il) p.spmv_threads = 3;
-  // the one-launch chunk: asked for, or chosen where every instance fits it
-  const bool use_chunk = !use_il && !mp && chunk_ok && (o.spmv_threads == 2 || (o.spmv_threads == 0 && pdqp::chunk_pays(w, mixed)));
   if (use_chunk) {
     alloc_chunk(h, mixed, s);
     p.spmv_threads = 2;
@@ -1813,34 +1820,45 @@ void device_scan(const int* in, int len, int* out, std::vector<void*>& tmp, cuda
   CK(cudaGetLastError());
 }
 
-// The one-launch chunk's slice layout (chunk.cu), built on the first solve that
-// runs it: structure once per handle, the scaled values by every solve.
+// The one-launch chunk's slices (chunk.cu): their starts and the instances' shapes,
+// once per handle on the first solve that may run it.  (The widths' sum fits 32
+// bits: a slice is as wide as one of its rows is long.)
+void plan_chunk(pdqp_problem* h, cudaStream_t s) {
+  Work& w = h->w;
+  ChunkPlan& ck = w.chunk;
+  if (ck.state >= 1) return;
+  pdqp::chunk_plan_instances(w);
+  if (!ck.inst) ck.inst = dalloc<ChunkInst>(h, w.count);
+  to_device(ck.inst, ck.order.data(), ck.order.size(), s);
+  if (!ck.sp) ck.sp = dalloc<int>(h, (size_t)ck.slices + 1);
+  TmpFree tmp;
+  tmp.s = s;
+  int* wid = (int*)pool_alloc((size_t)std::max(ck.slices, 1) * sizeof(int), s);
+  tmp.v.push_back(wid);
+  int2* even = (int2*)pool_alloc((size_t)std::max(ck.slices, 1) * sizeof(int2), s);
+  tmp.v.push_back(even);
+  pdqp::chunk_widths(w, wid, even, s);
+  device_scan(wid, ck.slices, ck.sp, tmp.v, s);
+  int4* ds = (int4*)pool_alloc((size_t)w.count * sizeof(int4), s);
+  tmp.v.push_back(ds);
+  pdqp::chunk_shapes(w, even, ds, s);
+  ck.shape.resize((size_t)w.count);
+  CK(cudaMemcpyAsync(ck.shape.data(), ds, ck.shape.size() * sizeof(int4), cudaMemcpyDeviceToHost, s));
+  CK(cudaStreamSynchronize(s));
+  ck.ngroups = 0;
+  for (const int4& g : ck.shape) ck.ngroups += (long long)g.x + g.y;
+  pdqp::chunk_plan_order(w);
+  to_device(ck.inst, ck.order.data(), ck.order.size(), s);
+  ck.state = 1;
+}
+
+// ... and the layout itself: the columns once per handle, the scaled values by
+// every solve.
 void alloc_chunk(pdqp_problem* h, bool mixed, cudaStream_t s) {
   Work& w = h->w;
   ChunkPlan& ck = w.chunk;
-  if (!ck.built) {
-    pdqp::chunk_plan_instances(w);
-    ck.inst = dalloc<ChunkInst>(h, w.count);
-    to_device(ck.inst, ck.order.data(), ck.order.size(), s);
-    ck.sp = dalloc<int>(h, (size_t)ck.slices + 1);
-    TmpFree tmp;
-    tmp.s = s;
-    int* wid = (int*)pool_alloc((size_t)std::max(ck.slices, 1) * sizeof(int), s);
-    tmp.v.push_back(wid);
-    pdqp::chunk_widths(w, wid, s);
-    device_scan(wid, ck.slices, ck.sp, tmp.v, s);
-    int2* dg = (int2*)pool_alloc((size_t)w.count * sizeof(int2), s);
-    tmp.v.push_back(dg);
-    pdqp::chunk_groups(w, dg, s);
-    std::vector<int2> groups((size_t)w.count);
-    CK(cudaMemcpyAsync(groups.data(), dg, groups.size() * sizeof(int2), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-    long long total = 0;
-    for (const int2& g : groups) total += (long long)g.x + g.y;
-    ck.ngroups = total;
-    pdqp::chunk_plan_order(w, groups);
-    to_device(ck.inst, ck.order.data(), ck.order.size(), s);
-    ck.idx = dalloc<unsigned>(h, (size_t)total * 32);
+  if (ck.state < 2) {
+    ck.idx = dalloc<unsigned>(h, (size_t)ck.ngroups * 32);
     pdqp::chunk_fill_index(w, s);
     for (auto& t : ck.side)
       if (!t) CK(cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking));
@@ -1848,7 +1866,7 @@ void alloc_chunk(pdqp_problem* h, bool mixed, cudaStream_t s) {
     for (auto& e : ck.join)
       if (!e) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     CK(cudaGetLastError());
-    ck.built = true;
+    ck.state = 2;
   }
   if (mixed && !ck.valf) ck.valf = dalloc<float2>(h, (size_t)ck.ngroups * 32);
   if (!mixed && !ck.vald) ck.vald = dalloc<double2>(h, (size_t)ck.ngroups * 32);

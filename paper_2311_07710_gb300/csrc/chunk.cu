@@ -307,31 +307,50 @@ __global__ void __launch_bounds__(1024, 1) k_chunk(ChunkArgs<V> a, int first, in
 // The slice layout, built from the handle's CSR arrays (blockIdx.x = the
 // instance's place in launch order; the slices of an instance over blockIdx.y)
 // --------------------------------------------------------------------------
-// width of every slice in pairs (its longest row, rounded up to a pair)
+// width of every slice in pairs (its longest row, rounded up to a pair) and {the
+// width were its rows all of their mean length, the entries of its longest row past that}
 __global__ void __launch_bounds__(256) k_chunk_width(const ChunkInst* __restrict__ inst, const int* __restrict__ arp,
-                                                     const int* __restrict__ prp, int* __restrict__ wid) {
+                                                     const int* __restrict__ prp, int* __restrict__ wid,
+                                                     int2* __restrict__ even) {
   const ChunkInst in = inst[blockIdx.x];
   const int lane = threadIdx.x & 31, step = gridDim.y * 8;
   for (int s = blockIdx.y * 8 + (threadIdx.x >> 5); s < in.nsA + in.nsP; s += step) {
     const bool isA = s < in.nsA;
-    const int r = 32 * (isA ? s : s - in.nsA) + lane;
+    const int r0 = 32 * (isA ? s : s - in.nsA), r = r0 + lane;
+    const int rows = min(32, (isA ? in.m : in.n) - r0);
     int len = 0;
-    if (r < (isA ? in.m : in.n)) {
+    if (lane < rows) {
       const int* rp = isA ? arp + in.yoff : prp + in.xoff;
       len = rp[r + 1] - rp[r];
     }
-    len = __reduce_max_sync(0xffffffffu, len);
-    if (lane == 0) wid[(isA ? in.sA + s : in.sP + s - in.nsA)] = (len + 1) >> 1;
+    const int width = (__reduce_max_sync(0xffffffffu, len) + 1) >> 1;
+    const int mean = (__reduce_add_sync(0xffffffffu, len) + 2 * rows - 1) / (2 * rows);
+    if (lane == 0) {
+      const int gs = isA ? in.sA + s : in.sP + s - in.nsA;
+      wid[gs] = width;
+      even[gs] = make_int2(mean, 2 * (width - mean));
+    }
   }
 }
 
-// {groups of A, groups of P} of every instance, in launch order
-__global__ void k_chunk_groups(const ChunkInst* __restrict__ inst, int count, const int* __restrict__ sp,
-                               int2* __restrict__ out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+// {groups of A, groups of P, groups were the rows of every slice of its mean
+// length, the most entries of a row past that} of every instance, in the order of
+// inst; a warp each
+__global__ void __launch_bounds__(256) k_chunk_shape(const ChunkInst* __restrict__ inst, int count,
+                                                     const int* __restrict__ sp, const int2* __restrict__ even,
+                                                     int4* __restrict__ out) {
+  const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (i >= count) return;
   const ChunkInst in = inst[i];
-  out[i] = make_int2(sp[in.sA + in.nsA] - sp[in.sA], sp[in.sP + in.nsP] - sp[in.sP]);
+  int sum = 0, most = 0;
+  for (int s = lane; s < in.nsA + in.nsP; s += 32) {
+    const int2 e = even[s < in.nsA ? in.sA + s : in.sP + s - in.nsA];
+    sum += e.x;
+    most = max(most, e.y);
+  }
+  sum = __reduce_add_sync(0xffffffffu, sum);
+  most = __reduce_max_sync(0xffffffffu, most);
+  if (lane == 0) out[i] = make_int4(sp[in.sA + in.nsA] - sp[in.sA], sp[in.sP + in.nsP] - sp[in.sP], sum, most);
 }
 
 // Columns (val null) or values of every slice; pads: the zero slot, value 0.
@@ -387,13 +406,13 @@ static dim3 chunk_grid(const Work& w) {
   return dim3(w.count, std::max(1, std::min(cdiv(big, 8), cdiv(8 * w.num_sms, w.count))));
 }
 
-void chunk_widths(Work& w, int* wid, cudaStream_t s) {
+void chunk_widths(Work& w, int* wid, int2* even, cudaStream_t s) {
   launch(k_chunk_width, chunk_grid(w), 256, 0, s, (const ChunkInst*)w.chunk.inst, (const int*)w.A.rp,
-         (const int*)w.P.rp, wid);
+         (const int*)w.P.rp, wid, even);
 }
-void chunk_groups(Work& w, int2* out, cudaStream_t s) {
-  launch(k_chunk_groups, cdiv(w.count, 256), 256, 0, s, (const ChunkInst*)w.chunk.inst, w.count,
-         (const int*)w.chunk.sp, out);
+void chunk_shapes(Work& w, const int2* even, int4* out, cudaStream_t s) {
+  launch(k_chunk_shape, cdiv(w.count, 8), 256, 0, s, (const ChunkInst*)w.chunk.inst, w.count,
+         (const int*)w.chunk.sp, even, out);
 }
 void chunk_fill_index(Work& w, cudaStream_t s) {
   launch(k_chunk_fill<float, false>, chunk_grid(w), 256, 0, s, (const ChunkInst*)w.chunk.inst, (const int*)w.chunk.sp,
@@ -547,9 +566,12 @@ bool chunk_ok(const Work& w, bool mixed) {
   return mixed ? chunk_fits<float>(w, k) : chunk_fits<double>(w, k);
 }
 
-// Whether the chunk beats the per-iteration kernels.  From 20 instances on it
-// always did: 1200 control QPs 17 us per iteration against 88, 160 of them 3.8
-// against 12, 77 in float64 9.8 against 16.
+// Whether the chunk beats the per-iteration kernels where the rows are even
+// (chunk_even).  From 20 instances on it always did: 1200 control QPs 17 us per
+// iteration against 88, 160 of them 3.8 against 12, 77 in float64 9.8 against 16;
+// random patterns, 20 of n = 1e4 (3e5 nonzeros each) 13.1 against 28.7, 80 of
+// n = 5000 22.7 against 46.4, 304 of n = 2500 28.5 against 77.3, in float64 20 of
+// n = 5000 16.1 against 37.1 and 304 of n = 2500 92.9 against 185.
 // A few instances on many CTAs pay for the cluster barriers and, on random
 // patterns, for bank conflicts: random sparse QPs, per iteration in float32,
 // 2.7 us (n = 1000, 4e3 nonzeros per CTA) against 7.5, 8.1 (n = 1e4, 19e3) against
@@ -559,6 +581,44 @@ bool chunk_pays(const Work& w, bool mixed) {
   long long k = 0;
   for (int c : chunk_ctas(w, mixed)) k += c;
   return (w.A.nnz + w.P.nnz) / k <= (mixed ? 18000 : 8000);
+}
+
+// Whether the rows are even enough for the slices (the plan's shapes known).  A
+// slice is as wide as its longest row: one long row is walked by one warp, mostly on
+// pads and past some length from L2, and many of them make the streams mostly pads.
+// Measured, us an iteration, chunk against the faster row-block kernel:
+// - one long row among rows of 10.  Float32, n = 1000 alone: 5.5 / 6.7 at 256 entries,
+//   6.5 / 7.0 at 320, 8.7 / 7.0 at 384, 23.0 / 9.3 at 1000; n = 4000 at 2000 45.7 / 13.8;
+//   a batch hides more of it: 160 of n = 1000 13.0 / 16.4 at 256, 29.0 / 19.5 at 1000.
+//   Float64, n = 1000 alone: 23.3 / 24.5 at 384, 30.4 / 29.3 at 512; 24 of them
+//   13.6 / 14.7 at 64, 19.2 / 17.5 at 128, 30.4 / 22.0 at 256; 160 of n = 300 19.2 / 22.2
+//   at 128, 24.7 / 24.2 at 192; 160 of n = 2000 71.8 / 70.2 at 256.
+// - a long row in every slice of A (groups over even groups).  Float32, where the
+//   matrices stay in shared memory: n = 1000 alone 5.9 / 7.2 (6.5), 160 of n = 300 6.9 /
+//   10.5 (4.7); where they do not: 160 of n = 2000 21.5 / 27.0 (2.7), 41.5 / 32.2 (4.3),
+//   1200 of n = 300 28.9 / 30.5 (4.7), 47.7 / 38.6 (6.3).  Float64, which has time for
+//   the streams: 160 of n = 1000 60.6 / 60.8 (4.4), 100 / 91 (6.5), 1200 of n = 300 74 /
+//   125 (4.7).
+bool chunk_even(const Work& w, bool mixed) {
+  const ChunkPlan& ck = w.chunk;
+  const std::vector<int> ctas = chunk_ctas(w, mixed);
+  const size_t cap = w.count >= 2 * w.num_sms ? 112 * 1024 : CHUNK_SMEM_MAX;
+  long long groups = 0, even = 0;
+  int most = 0;
+  bool resident = true;
+  for (int i = 0; i < w.count; ++i) {
+    const Inst& I = w.inst_host[i];
+    const int4 g = ck.shape[i];
+    const int k = ctas[i], oA = cdiv(cdiv(I.m, 32), k), oP = cdiv(cdiv(I.n, 32), k);
+    const size_t fixed = mixed ? chunk_fixed_bytes<float>(I.n, I.m, oA, oP) : chunk_fixed_bytes<double>(I.n, I.m, oA, oP);
+    resident = resident && fixed + ((size_t)g.x + g.y) / k * (mixed ? chunk_group_bytes<float>() : chunk_group_bytes<double>()) <= cap;
+    groups += (long long)g.x + g.y;
+    even += g.z;
+    most = std::max(most, g.w);
+  }
+  const double millions = 1e-6 * (double)(w.A.nnz + w.P.nnz);
+  const double row = mixed ? 320 + 50 * millions : (w.count < 20 ? 384 : 128) + 30 * millions;
+  return most <= row && groups <= (mixed ? (resident ? 8 : 4) : 6) * even;
 }
 
 // The launches of one precision: the instances, in launch order (largest
@@ -581,7 +641,7 @@ static void chunk_classes(Work& w, std::vector<ChunkClass>& out) {
     const int oA = cdiv(I.nsA, ctas), oP = cdiv(I.nsP, ctas);
     const size_t fixed = chunk_fixed_bytes<V>(I.n, I.m, oA, oP);
     // a CTA's share of the groups, rounded up by a slice's worth
-    const size_t own = ((size_t)ck.groups[i].x + ck.groups[i].y) / ctas;
+    const size_t own = ((size_t)ck.shape[I.id].x + ck.shape[I.id].y) / ctas;
     const size_t need = fixed + (ctas > 1 ? own + own / 8 + 64 : own) * gb;
     int c = 0;
     if (ctas > 1) c = 2 + ctas;
@@ -614,16 +674,14 @@ void chunk_plan_instances(Work& w) {
   }
   ck.slices = sP;
 }
-void chunk_plan_order(Work& w, const std::vector<int2>& groups) {   // groups: by instance
+void chunk_plan_order(Work& w) {
   ChunkPlan& ck = w.chunk;
-  auto total = [&](const ChunkInst& p) { return (long long)groups[p.id].x + groups[p.id].y; };
+  auto total = [&](const ChunkInst& p) { return (long long)ck.shape[p.id].x + ck.shape[p.id].y; };
   std::stable_sort(ck.order.begin(), ck.order.end(),
                    [&](const ChunkInst& p, const ChunkInst& q) {
                      const int rp = p.n + p.m, rq = q.n + q.m;   // with few instances the rows set the CTAs
                      return w.count < w.num_sms && rp != rq ? rp > rq : total(p) > total(q);
                    });
-  ck.groups.resize(w.count);
-  for (int i = 0; i < w.count; ++i) ck.groups[i] = groups[ck.order[i].id];
 }
 void chunk_plan_classes(Work& w, bool mixed) {
   w.chunk.ctas = chunk_ctas(w, mixed);

@@ -117,7 +117,7 @@ struct ChunkClass {
   size_t smem;
 };
 struct ChunkPlan {
-  bool built = false;
+  int state = 0;                          // 0 not looked at, 1 slices and shapes known, 2 columns laid out
   std::vector<int> ctas;                  // CTAs per instance (a cluster when > 1), of the classes planned last
   int slices = 0;
   long long ngroups = 0;
@@ -127,7 +127,7 @@ struct ChunkPlan {
   unsigned* idx = nullptr;                // [groups][32] two 16-bit columns
   float2* valf = nullptr;                 // [groups][32] scaled values
   double2* vald = nullptr;
-  std::vector<int2> groups;               // {of A, of P} per instance, in launch order
+  std::vector<int4> shape;                // per instance {groups of A, of P, even groups, excess of the longest row}
   std::vector<ChunkClass> cls[2];         // launches: float64, mixed
   static constexpr int SIDES = 7;
   cudaStream_t side[SIDES] = {};          // the second and later launches' streams
@@ -318,9 +318,10 @@ double launch_bytes(const Work& w, int kind, double sv);
 bool chunk_ok(const Work& w, bool mixed);
 bool chunk_pays(const Work& w, bool mixed);               // chosen over the per-iteration kernels
 void chunk_plan_instances(Work& w);                       // w.chunk.order, slices (instance order)
-void chunk_widths(Work& w, int* wid, cudaStream_t s);     // pairs per slice
-void chunk_groups(Work& w, int2* out, cudaStream_t s);    // groups of A and of P per instance
-void chunk_plan_order(Work& w, const std::vector<int2>& groups);   // largest instances first
+void chunk_widths(Work& w, int* wid, int2* even, cudaStream_t s);   // pairs per slice, of even rows
+void chunk_shapes(Work& w, const int2* even, int4* out, cudaStream_t s);   // w.chunk.shape
+void chunk_plan_order(Work& w);                           // largest instances first
+bool chunk_even(const Work& w, bool mixed);               // rows even enough (shapes known)
 void chunk_plan_classes(Work& w, bool mixed);             // cls of one precision
 void chunk_fill_index(Work& w, cudaStream_t s);
 void chunk_fill_values(Work& w, bool mixed, cudaStream_t s);
