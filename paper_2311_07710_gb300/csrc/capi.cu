@@ -636,7 +636,7 @@ void tuned_store(const Work& w, bool mixed, int nt) {
 }
 
 void plan_chunk(pdqp_problem* h, cudaStream_t s);                // with the device scans, below
-void alloc_chunk(pdqp_problem* h, bool mixed, cudaStream_t s);
+bool alloc_chunk(pdqp_problem* h, bool mixed, bool asked, cudaStream_t s);
 bool alloc_slices(pdqp_problem* h, bool mixed, cudaStream_t s);
 
 // options.spmv_threads = 2: at most 64 row blocks of A and of P, no row longer
@@ -688,12 +688,13 @@ pdqp_status solve_impl(pdqp_problem* h, const pdqp_options& o, const double* x0,
   bool use_chunk = !mp && chunk_ok &&
                    (o.spmv_threads == 2 ||
                     (o.spmv_threads == 0 && (!il_ok || il_small) && pdqp::chunk_pays(w, mixed)));
+  if (mixed) alloc_mixed(h);   // (first: what every variant needs)
   if (use_chunk) {
+    const bool asked = o.spmv_threads == 2;
     plan_chunk(h, s);
-    if (o.spmv_threads == 0) use_chunk = pdqp::chunk_even(w, mixed);
+    use_chunk = (asked || pdqp::chunk_even(w, mixed)) && alloc_chunk(h, mixed, asked, s);
   }
   const bool use_il = il_ok && !mp && ((o.spmv_threads == 0 && !use_chunk) || o.spmv_threads == 3);
-  if (mixed) alloc_mixed(h);
   if (use_il) alloc_il(h, mixed, o.check_period);
   w.il_active = use_il;
   if (!use_il && !w.kkt_xx) {   // the row-block checks gather both iterates of a column at once
@@ -705,10 +706,7 @@ pdqp_status solve_impl(pdqp_problem* h, const pdqp_options& o, const double* x0,
   if (w.detect) alloc_infeas(h, s);
   SolveParams p = make_params(o);
   if (use_il) p.spmv_threads = 3;
-  if (use_chunk) {
-    alloc_chunk(h, mixed, s);
-    p.spmv_threads = 2;
-  }
+  if (use_chunk) p.spmv_threads = 2;
   // the iteration-kernel variant, where nothing above fixes it: the one this
   // shape was tuned to, or timed on the first chunk (below)
   const bool use_lr = o.spmv_threads == 0 && !use_il && !mp && pdqp::lowrank_fused_ok(w, mixed);
@@ -1852,13 +1850,46 @@ void plan_chunk(pdqp_problem* h, cudaStream_t s) {
   ck.state = 1;
 }
 
+// Bytes this process can still take: the device's free memory and what the pool
+// holds unused.
+size_t memory_room() {
+  size_t free_b = 0, total_b = 0;
+  uint64_t held = 0, used = 0;
+  CK(cudaMemGetInfo(&free_b, &total_b));
+  CK(cudaMemPoolGetAttribute(lib_pool(), cudaMemPoolAttrReservedMemCurrent, &held));
+  CK(cudaMemPoolGetAttribute(lib_pool(), cudaMemPoolAttrUsedMemCurrent, &used));
+  return free_b + (size_t)(held > used ? held - used : 0);
+}
+
 // ... and the layout itself: the columns once per handle, the scaled values by
-// every solve.
-void alloc_chunk(pdqp_problem* h, bool mixed, cudaStream_t s) {
+// every solve.  It is a second copy of the matrices: unless the chunk is asked for,
+// at most half of the memory left, and without it (false) the solve runs the
+// kernels that need none.
+bool alloc_chunk(pdqp_problem* h, bool mixed, bool asked, cudaStream_t s) {
   Work& w = h->w;
   ChunkPlan& ck = w.chunk;
-  if (ck.state < 2) {
-    ck.idx = dalloc<unsigned>(h, (size_t)ck.ngroups * 32);
+  const size_t pairs = (size_t)ck.ngroups * 32;
+  const bool need_idx = ck.state < 2, need_val = mixed ? !ck.valf : !ck.vald;
+  const size_t bytes = (need_idx ? pairs * sizeof(unsigned) : 0) +
+                       (need_val ? pairs * (mixed ? sizeof(float2) : sizeof(double2)) : 0);
+  if (!asked && bytes > (64ULL << 20) && bytes > memory_room() / 2) return false;
+  const size_t mark = h->allocs.size();
+  try {
+    if (need_idx) ck.idx = dalloc<unsigned>(h, pairs);
+    if (need_val && mixed) ck.valf = dalloc<float2>(h, pairs);
+    if (need_val && !mixed) ck.vald = dalloc<double2>(h, pairs);
+  } catch (const Fail& f) {
+    while (h->allocs.size() > mark) {
+      cudaFreeAsync(h->allocs.back(), s);
+      h->allocs.pop_back();
+    }
+    if (need_idx) ck.idx = nullptr;
+    if (need_val && mixed) ck.valf = nullptr;
+    if (need_val && !mixed) ck.vald = nullptr;
+    if (asked || f.st != PDQP_ERR_OOM) throw;
+    return false;
+  }
+  if (need_idx) {
     pdqp::chunk_fill_index(w, s);
     for (auto& t : ck.side)
       if (!t) CK(cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking));
@@ -1868,9 +1899,8 @@ void alloc_chunk(pdqp_problem* h, bool mixed, cudaStream_t s) {
     CK(cudaGetLastError());
     ck.state = 2;
   }
-  if (mixed && !ck.valf) ck.valf = dalloc<float2>(h, (size_t)ck.ngroups * 32);
-  if (!mixed && !ck.vald) ck.vald = dalloc<double2>(h, (size_t)ck.ngroups * 32);
   if (ck.cls[mixed ? 1 : 0].empty()) pdqp::chunk_plan_classes(w, mixed);
+  return true;
 }
 
 // The slice layout of a large instance (iteration.cu), as alloc_chunk; false where
