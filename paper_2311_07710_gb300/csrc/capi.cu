@@ -661,7 +661,7 @@ pdqp_status solve_impl(pdqp_problem* h, const pdqp_options& o, const double* x0,
   check_space(x_out, mem, "x_out");
   check_space(y_out, mem, "y_out");
   const bool mixed = o.precision == PDQP_PREC_MIXED;
-  const bool chunk_ok = pdqp::chunk_ok(w, mixed);
+  const bool chunk_ok = pdqp::chunk_ok(w, mixed, o.spmv_threads == 2);
   if (o.spmv_threads == 2 && !(chunk_ok && chunk_asked_ok(w, mixed)))
     throw Fail{PDQP_ERR_INVALID, "options.spmv_threads = 2 needs at most 64 row blocks of A and of P, no row "
                                  "longer than a row block, no low-rank term and 3n + 2m values within 200 KB"};

@@ -481,10 +481,10 @@ static void prepare_chunk() {   // once per process
 // finishes earlier (pairs dealt out largest first to the SMs as they fall free): the
 // float64 pipes bind there, and a second round of small instances costs less than
 // idle pipes (151 of them 17.7 us against 23.2, 120 of them 14.1 against 17.2).
+static const int kChunkSizes[] = {1, 2, 3, 4, 6, 8, 12, 16};
 static std::vector<int> chunk_ctas(const Work& w, bool mixed) {
   std::vector<int> out(w.count, 1);
   if (w.count >= w.num_sms) return out;
-  static const int kSizes[] = {1, 2, 3, 4, 6, 8, 12, 16};
   const int gpcs = std::max(1, w.num_sms / 19);
   // larger clusters pay with their barriers: 1500 rows (n = 1000) take 3.26 us an
   // iteration on 8 CTAs, 3.45 on 16; 2824 (a control QP of horizon 100) 3.15, 3.30 on
@@ -494,7 +494,7 @@ static std::vector<int> chunk_ctas(const Work& w, bool mixed) {
   const double per_row = (double)(w.A.nnz + w.P.nnz) / std::max<long long>(1, (long long)w.n + w.m);
   auto cap = [&](const Inst& I) {
     int k = 1;
-    for (int q : kSizes) {
+    for (int q : kChunkSizes) {
       const int rows = q <= 4 ? 100 : q <= 8 ? 187 : q <= 12 || !mixed ? 250 : 500;   // at least, a CTA
       const bool enough = (long long)q * rows <= I.n + I.m || q * 5000.0 <= per_row * (I.n + I.m);
       if (q <= g_chunk_max_ctas && 32 * (q - 1) < I.n && enough) k = q;
@@ -506,7 +506,7 @@ static std::vector<int> chunk_ctas(const Work& w, bool mixed) {
     for (int i = 0; i < w.count; ++i) {
       const Inst& I = w.inst_host[i];
       int k = 1;
-      for (int q : kSizes)
+      for (int q : kChunkSizes)
         if (q <= cap(I) && (long long)k * rows < I.n + I.m) k = q;
       all += out[i] = k;
       ++of_size[k];
@@ -547,23 +547,30 @@ static std::vector<int> chunk_ctas(const Work& w, bool mixed) {
   return out;
 }
 
-template <typename V>
-static bool chunk_fits(const Work& w, const std::vector<int>& ctas) {
-  for (int i = 0; i < w.count; ++i) {
-    const Inst& I = w.inst_host[i];
-    if (I.n + I.m > 65535) return false;          // 16-bit columns, the pads' slot included
-    if (chunk_fixed_bytes<V>(I.n, I.m, cdiv(cdiv(I.m, 32), ctas[i]), cdiv(cdiv(I.n, 32), ctas[i])) >
-        (size_t)CHUNK_SMEM_MAX)
-      return false;
-  }
-  return true;
+// Whether the vectors of an instance on k CTAs fit shared memory.
+static bool chunk_fits(const Inst& I, int k, bool mixed) {
+  const int oA = cdiv(cdiv(I.m, 32), k), oP = cdiv(cdiv(I.n, 32), k);
+  return I.n + I.m <= 65535 &&                     // 16-bit columns, the pads' slot included
+         (mixed ? chunk_fixed_bytes<float>(I.n, I.m, oA, oP) : chunk_fixed_bytes<double>(I.n, I.m, oA, oP)) <=
+             (size_t)CHUNK_SMEM_MAX;
+}
+// Asked for, an instance that chunk_ctas gives too few CTAs for its vectors (rows
+// of few variables: n = 100, m = 10000 in float64) takes the fewest that hold them.
+static std::vector<int> chunk_ctas_asked(const Work& w, bool mixed) {
+  std::vector<int> k = chunk_ctas(w, mixed);
+  for (int i = 0; i < w.count && w.count < w.num_sms; ++i)
+    for (int q : kChunkSizes)
+      if (q > k[i] && q <= g_chunk_max_ctas && !chunk_fits(w.inst_host[i], k[i], mixed)) k[i] = q;
+  return k;
 }
 
-bool chunk_ok(const Work& w, bool mixed) {
+bool chunk_ok(const Work& w, bool mixed, bool asked) {
   if (w.r != 0 || w.A.nlseg != 0 || w.P.nlseg != 0 || w.n < 1) return false;
   prepare_chunk();
-  const std::vector<int> k = chunk_ctas(w, mixed);
-  return mixed ? chunk_fits<float>(w, k) : chunk_fits<double>(w, k);
+  const std::vector<int> k = asked ? chunk_ctas_asked(w, mixed) : chunk_ctas(w, mixed);
+  for (int i = 0; i < w.count; ++i)
+    if (!chunk_fits(w.inst_host[i], k[i], mixed)) return false;
+  return true;
 }
 
 // Whether the chunk beats the per-iteration kernels where the rows are even
@@ -684,7 +691,7 @@ void chunk_plan_order(Work& w) {
                    });
 }
 void chunk_plan_classes(Work& w, bool mixed) {
-  w.chunk.ctas = chunk_ctas(w, mixed);
+  w.chunk.ctas = chunk_ctas_asked(w, mixed);       // (chunk_ctas' where these fit)
   if (mixed) chunk_classes<float>(w, w.chunk.cls[1]);
   else chunk_classes<double>(w, w.chunk.cls[0]);
 }

@@ -315,7 +315,7 @@ double launch_bytes(const Work& w, int kind, double sv);
 
 // The one-launch chunk (chunk.cu): whether every instance's vectors fit a CTA
 // (no long rows, no low-rank term); the plan's parts, in the order they are built.
-bool chunk_ok(const Work& w, bool mixed);
+bool chunk_ok(const Work& w, bool mixed, bool asked);
 bool chunk_pays(const Work& w, bool mixed);               // chosen over the per-iteration kernels
 void chunk_plan_instances(Work& w);                       // w.chunk.order, slices (instance order)
 void chunk_widths(Work& w, int* wid, int2* even, cudaStream_t s);   // pairs per slice, of even rows

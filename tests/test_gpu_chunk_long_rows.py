@@ -84,3 +84,23 @@ def test_family_with_a_long_row_runs_interleaved():
             pd.pdqp_destroy(h)
     assert out[0][1] == 3
     np.testing.assert_array_equal(out[0][0], out[256][0])
+
+
+@pytest.mark.parametrize("precision,n,m", [(0, 100, 10000), (0, 40, 11500), (1, 40, 24000), (0, 7600, 0), (1, 15900, 0)])
+def test_asked_for_within_its_limit(precision, n, m):
+    """Up to 3n + 2m values in 200 KB the chunk runs where it is asked for, whatever the shape."""
+    G.lib()
+    inst = _qp(n, m, 4, seed=5) if n >= 100 and m else None
+    if inst is None and m == 0:
+        inst = qpgen.diagonal_box_qp(qpgen.SEED_BASE + 8100, n=n)
+    if inst is None:
+        rng = np.random.default_rng(6)
+        cols = (rng.integers(0, n, (m, 1)) + np.arange(3)) % n
+        A = sp.csr_matrix((rng.standard_normal(3 * m) / np.sqrt(m), (np.repeat(np.arange(m), 3), cols.ravel())), (m, n))
+        inst = qpgen.QPInstance("tall", n, m, 0, _as32(sp.identity(n)), _as32(A), rng.standard_normal(n),
+                                np.asarray(A @ np.full(n, 0.1)).ravel() - 0.1, np.full(n, -1.0), np.full(n, 1.0))
+    a = G.solve(inst, precision=precision, spmv_threads=256, max_iter=70, eps=0.0)
+    b = G.solve(inst, precision=precision, spmv_threads=2, max_iter=70, eps=0.0)
+    assert b[1].spmv_threads == 2 and a[0] == b[0]
+    np.testing.assert_array_equal(a[2], b[2])
+    np.testing.assert_array_equal(a[3], b[3])
