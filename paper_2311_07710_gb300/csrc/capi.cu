@@ -1899,7 +1899,12 @@ bool alloc_chunk(pdqp_problem* h, bool mixed, bool asked, cudaStream_t s) {
     CK(cudaGetLastError());
     ck.state = 2;
   }
-  if (ck.cls[mixed ? 1 : 0].empty()) pdqp::chunk_plan_classes(w, mixed);
+  const int q = mixed ? 1 : 0;
+  if (ck.cls[q].empty()) {
+    if (!ck.launch[q]) ck.launch[q] = dalloc<ChunkInst>(h, w.count);
+    pdqp::chunk_plan_classes(w, mixed);
+    to_device(ck.launch[q], ck.launch_host[q].data(), ck.launch_host[q].size(), s);
+  }
   return true;
 }
 

@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(1024, 1) k_chunk(ChunkArgs<V> a, int first, in
 
 // --------------------------------------------------------------------------
 // The slice layout, built from the handle's CSR arrays (blockIdx.x = the
-// instance's place in launch order; the slices of an instance over blockIdx.y)
+// instance's place in the plan's order; the slices of an instance over blockIdx.y)
 // --------------------------------------------------------------------------
 // width of every slice in pairs (its longest row, rounded up to a pair) and {the
 // width were its rows all of their mean length, the entries of its longest row past that}
@@ -628,8 +628,8 @@ bool chunk_even(const Work& w, bool mixed) {
   return most <= row && groups <= (mixed ? (resident ? 8 : 4) : 6) * even;
 }
 
-// The launches of one precision: the instances, in launch order (largest
-// first), split by the shared memory their vectors and matrices take, so that
+// The launches of one precision, one a class: the instances by the shared memory
+// their vectors and matrices take, largest first within a class, so that
 // smaller ones share an SM: up to 64 KB four a SM, up to 130 KB two (the part
 // that does not fit streams from L2).  A batch of at least two instances an SM
 // takes two a SM however large they are (two half-resident instances hide each
@@ -637,13 +637,14 @@ bool chunk_even(const Work& w, bool mixed) {
 // 103.7); with fewer, a larger one keeps its SM to itself (160 instances: 3.8
 // against 6.1).
 template <typename V>
-static void chunk_classes(Work& w, std::vector<ChunkClass>& out) {
+static void chunk_classes(Work& w, std::vector<ChunkClass>& out, std::vector<ChunkInst>& launch) {
   ChunkPlan& ck = w.chunk;
-  out.clear();
   const size_t gb = chunk_group_bytes<V>();
-  int cls_of_prev = -1;
-  for (int i = 0; i < w.count; ++i) {
-    const ChunkInst& I = ck.order[i];
+  constexpr int CLASSES = 3 + 16;                  // by what shares an SM (0..2), by the cluster's CTAs
+  std::vector<ChunkInst> of[CLASSES];
+  ChunkClass cls[CLASSES] = {};
+  std::vector<int> seen;                           // in the order of their largest instances
+  for (const ChunkInst& I : ck.order) {
     const int ctas = ck.ctas[I.id];
     const int oA = cdiv(I.nsA, ctas), oP = cdiv(I.nsP, ctas);
     const size_t fixed = chunk_fixed_bytes<V>(I.n, I.m, oA, oP);
@@ -655,16 +656,22 @@ static void chunk_classes(Work& w, std::vector<ChunkClass>& out) {
     else if (w.count >= w.num_sms)
       c = need <= 64 * 1024 && fixed <= 48 * 1024 ? 2
           : (need <= 130 * 1024 || w.count >= 2 * w.num_sms) && fixed <= 108 * 1024 ? 1 : 0;
-    if (c != cls_of_prev) {
-      out.push_back(ChunkClass{i, 0, 0, ctas, 0});
-      cls_of_prev = c;
-    }
-    ChunkClass& k = out.back();
-    ++k.count;
+    if (of[c].empty()) seen.push_back(c);
+    of[c].push_back(I);
+    ChunkClass& k = cls[c];
+    k.ctas = ctas;
     const size_t cap = c == 2 ? 55 * 1024 : c == 1 ? 112 * 1024 : (size_t)CHUNK_SMEM_MAX;
     k.smem = std::max(k.smem, std::min(need, cap));
     const int own_slices = std::max(oA, oP);
     k.threads = std::max(k.threads, std::min(c == 2 ? 256 : c == 1 ? 512 : 1024, 32 * std::max(4, own_slices)));
+  }
+  out.clear();
+  launch.clear();
+  for (int c : seen) {
+    cls[c].first = (int)launch.size();
+    cls[c].count = (int)of[c].size();
+    out.push_back(cls[c]);
+    launch.insert(launch.end(), of[c].begin(), of[c].end());
   }
 }
 
@@ -692,8 +699,8 @@ void chunk_plan_order(Work& w) {
 }
 void chunk_plan_classes(Work& w, bool mixed) {
   w.chunk.ctas = chunk_ctas_asked(w, mixed);       // (chunk_ctas' where these fit)
-  if (mixed) chunk_classes<float>(w, w.chunk.cls[1]);
-  else chunk_classes<double>(w, w.chunk.cls[0]);
+  if (mixed) chunk_classes<float>(w, w.chunk.cls[1], w.chunk.launch_host[1]);
+  else chunk_classes<double>(w, w.chunk.cls[0], w.chunk.launch_host[0]);
 }
 
 template <typename V>
@@ -701,7 +708,7 @@ static void run_chunk(Work& w, int j0, int len, const typename Pair<V>::T* val, 
                       const V* b, const V* ylo, V* x, V* xbar, const V* c, const V* l, const V* u, cudaStream_t s) {
   Profiler& Pr = w.prof;
   ChunkPlan& ck = w.chunk;
-  ChunkArgs<V> a{ck.inst, ck.sp, ck.idx, val, xt, Z[0], Z[1], x, xbar, ybar, b, ylo, c, l, u, w.row_ineq, w.tab, w.st,
+  ChunkArgs<V> a{ck.launch[sizeof(V) == 4 ? 1 : 0], ck.sp, ck.idx, val, xt, Z[0], Z[1], x, xbar, ybar, b, ylo, c, l, u, w.row_ineq, w.tab, w.st,
                  w.tab_stride, w.n, 0};
   // kind 3: one launch holds both half-steps of `len` iterations
   if (Pr.on) Pr.begin(3, s, len * (launch_bytes(w, 0, sizeof(V)) + launch_bytes(w, 1, sizeof(V))));

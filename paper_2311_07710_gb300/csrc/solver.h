@@ -104,8 +104,7 @@ struct InfState {
 constexpr int KKT_GROUP = 4;
 static_assert(KKT_CHUNK % KKT_GROUP == 0, "a relKKT chunk holds whole groups");
 
-// The one-launch chunk (chunk.cu): an instance with its slices of 32 rows, in
-// launch order; its row in sp (A's slices of all instances come first, then P's).
+// The one-launch chunk (chunk.cu): an instance with its slices of 32 rows; its row in sp (A's slices of all instances come first, then P's).
 struct ChunkInst {
   int n, m, xoff, yoff;
   int sA, nsA, sP, nsP;
@@ -121,8 +120,10 @@ struct ChunkPlan {
   std::vector<int> ctas;                  // CTAs per instance (a cluster when > 1), of the classes planned last
   int slices = 0;
   long long ngroups = 0;
-  std::vector<ChunkInst> order;           // launch order, largest first
+  std::vector<ChunkInst> order;           // largest first
   ChunkInst* inst = nullptr;              // [count] on the device
+  std::vector<ChunkInst> launch_host[2];  // launch order of a precision: class by class (float64, mixed)
+  ChunkInst* launch[2] = {};              // ... on the device
   int* sp = nullptr;                      // [slices + 1] starts, in groups of 32 pairs of entries
   unsigned* idx = nullptr;                // [groups][32] two 16-bit columns
   float2* valf = nullptr;                 // [groups][32] scaled values
