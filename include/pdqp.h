@@ -128,7 +128,8 @@ typedef struct {
                                 CTA's shared memory and the instances are many or
                                 small (a family: up to 300 thousand rows in all); 3
                                 for the other eligible family handles; for a low-rank term
-                                over short rows of P, kernels that read the factor once
+                                over short rows of P (eight entries on average, none
+                                of more than 192), kernels that read the factor once
                                 per iteration (pdqp_info reports them as 4, which
                                 cannot be asked for); else the first full chunk of a
                                 handle's first solve in each precision times two

@@ -2450,6 +2450,8 @@ pdqp_status pdqp_set_lowrank_Q(pdqp_handle h, int32_t r, const float* F, int32_t
     CK(cudaMemsetAsync(w.lr_ticket, 0, std::max(w.A.nlseg, 1) * sizeof(unsigned), s));
     to_device(w.F, hf.data(), N, s);
     to_device(w.Fo, hd.data(), N, s);
+    const std::vector<int32_t> rp = fetch<int32_t>(w.P.rp, (size_t)w.n + 1, PDQP_MEM_DEVICE, s);
+    for (int j = 0; j < w.n; ++j) w.longest_P = std::max(w.longest_P, rp[j + 1] - rp[j]);
     CK(cudaStreamSynchronize(s));
     w.r = r;
     drop_graphs(h);

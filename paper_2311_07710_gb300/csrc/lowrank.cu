@@ -189,8 +189,15 @@ void lowrank_rows(Work& w, const double* F, int nit, cudaStream_t s) {
 
 constexpr int LRF_SMEM_MAX = 220 * 1024;
 
+// Rows of P are short, on average and each of them: a thread walks a row, entry
+// after entry, while its block waits.  With one variable in K rows of A, us an iteration
+// against the faster general kernel: n = 2000, r = 16 in float32 15.3 / 21.9 (K = 0),
+// 19.6 / 22.3 (128), 32.8 / 24.1 (512), 82.8 / 28.8 (2000), in float64 103 / 107 (128),
+// 136 / 123 (512); n = 20000, r = 32 in float32 12.8 / 19.8 (128), 27.0 / 22.1 (512);
+// n = 1e5, r = 64 31.3 / 33.5 (512), 82.9 / 33.6 (2000).
+constexpr int LRF_ROW_MAX = 192;
 bool lowrank_fused_ok(const Work& w, bool mixed) {
-  if (w.r < 1 || w.count != 1 || w.P.nlseg != 0 || w.P.nnz > 8LL * w.n) return false;
+  if (w.r < 1 || w.count != 1 || w.P.nnz > 8LL * w.n || w.longest_P > LRF_ROW_MAX) return false;
   const int grid = lr_ft_grid(w), per = cdiv(w.n, grid);
   return (mixed ? lrf_smem<float>(per, w.r) : lrf_smem<double>(per, w.r)) <= (size_t)LRF_SMEM_MAX;
 }

@@ -182,6 +182,7 @@ struct Work {
   double *prodAx = nullptr, *prodQx = nullptr, *prodATy = nullptr;      // [2][m], [2][n], [2][n]
   // low-rank factor (Q_total = Q + F F'), row-major n x r
   int r = 0;
+  int longest_P = 0;         // entries of P's longest row (set with the low-rank term)
   float* F = nullptr;        // original, float32
   double* Fo = nullptr;      // original, float64
   float* Fs = nullptr;       // D2 F, float32
