@@ -884,8 +884,8 @@ __device__ __forceinline__ void pair_add(float& hi, float& lo, float x, float xl
 // (1.27 ms for 4096 x 60000 values at that pipe's rate); it takes the difference
 // there, and the sums run on float32 pairs: the difference's bits split into
 // 24 + 23 (truncated at 2^-46 of it), products and sums with their exact
-// rounding errors.  Values whose square or its error leaves float32's range
-// take the float64 sums.  Two arrays per launch (grid z) and short ranges, so
+// rounding errors.  Values whose square, its error or a range's sum of squares
+// leaves float32's range take the float64 sums.  Two arrays per launch (grid z) and short ranges, so
 // that the blocks fill whole waves (ranges of 256 rows, one array a launch: a
 // little over two waves, 1.48 ms; the two-pass form before, 157 blocks of one
 // column per thread: 4.8 ms).
@@ -915,7 +915,7 @@ __global__ void __launch_bounds__(256) k_fit_part(FitPair a, long long count, in
         const double d = v[k] - K;
         const unsigned hw = (unsigned)__double2hiint(d), lw = (unsigned)__double2loint(d);
         const unsigned e = (hw >> 20) & 0x7FFu, sg = hw & 0x80000000u;
-        if (e - 973u <= 113u) {                    // 2^-50 <= |d| < 2^64
+        if (e - 973u <= 109u) {                    // 2^-50 <= |d| < 2^60: FIT_ROWS squares stay below 2^126
           const float hi = __uint_as_float(sg | ((e - 896u) << 23) | (__funnelshift_l(lw, hw, 3) & 0x7FFFFFu));
           const float lo = __fmul_rn(__fsub_rn(__uint_as_float(0x4B000000u | ((lw >> 6) & 0x7FFFFFu)), 8388608.f),
                                      __uint_as_float(sg | ((e - 942u) << 23)));
