@@ -638,6 +638,7 @@ void tuned_store(const Work& w, bool mixed, int nt) {
 void plan_chunk(pdqp_problem* h, cudaStream_t s);                // with the device scans, below
 bool alloc_chunk(pdqp_problem* h, bool mixed, bool asked, cudaStream_t s);
 bool alloc_slices(pdqp_problem* h, bool mixed, cudaStream_t s);
+void drop_slices(pdqp_problem* h, bool mixed, cudaStream_t s);
 
 // options.spmv_threads = 2: at most 64 row blocks of A and of P, no row longer
 // than a row block, no low-rank term, and 3n + 2m values (with a row block's
@@ -900,6 +901,7 @@ pdqp_status solve_impl(pdqp_problem* h, const pdqp_options& o, const double* x0,
         if (best_ms[c] < best_ms[bc]) bc = c;
       tuned = kCand[bc];
       tuned_store(w, mixed, tuned);
+      if (use_slices && tuned != 5) drop_slices(h, mixed, s);
       p.spmv_threads = tuned;
       pdqp::iterate(w, (int)len - j, mixed, p.spmv_threads, s, j);
       pdqp::check(w, p, 1, len, mixed, s);
@@ -1957,6 +1959,26 @@ bool alloc_slices(pdqp_problem* h, bool mixed, cudaStream_t s) {
     q.state = -1;
   }
   return q.state == 1;
+}
+
+// One precision runs another variant: its copy of the values goes back, and with
+// it the layout where the other precision holds none (it is built anew if that
+// one comes to be tuned).
+void drop_slices(pdqp_problem* h, bool mixed, cudaStream_t s) {
+  SlicePlan& q = h->w.slices;
+  auto give_back = [&](auto*& p) {
+    auto it = std::find(h->allocs.begin(), h->allocs.end(), (void*)p);
+    if (it == h->allocs.end()) return;
+    h->allocs.erase(it);
+    cudaFreeAsync(p, s);
+    p = nullptr;
+  };
+  if (mixed) give_back(q.valf);
+  else give_back(q.vald);
+  if (q.valf || q.vald) return;
+  give_back(q.idx);
+  give_back(q.sp);
+  q = SlicePlan{};
 }
 
 // A batch handed over as one block-diagonal problem: instance i owns the
