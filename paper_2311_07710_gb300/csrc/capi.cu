@@ -362,6 +362,7 @@ void alloc_il(pdqp_problem* h, bool mixed, int period) {
   }
   if (!w.il_slot) w.il_slot = dalloc<int>(h, ld);
   int& have = w.il_steps_len[mixed ? 1 : 0];
+  period = std::min(period, IL_STEP_ITERS);
   if (have < period) {   // a longer check period replaces the buffer the graphs point into
     if (mixed) w.il_steps_f = dalloc<float>(h, 5 * (size_t)period * ld);
     else w.il_steps_d = dalloc<double>(h, 5 * (size_t)period * ld);

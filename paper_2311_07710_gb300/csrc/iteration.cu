@@ -864,7 +864,7 @@ struct FamIL {
   const int* __restrict__ col;
   const V* __restrict__ val;           // scaled values (the same for every member)
   int rows, ld;
-  const V* steps;         // [j - j0][IL_STEPS][ld] step scalars of the chunk (k_il_steps)
+  const V* steps;         // [k][IL_STEPS][ld] step scalars of up to IL_STEP_ITERS iterations (k_il_steps)
   const int* slot;        // [ld] member, or -1
   const V* zin;           // gathered vector (x_tilde, or [x_md ; y+])
   // dual: yold, ynew, ybar, b, ylo (may be null), ineq;  primal: x, xbar, zout, xt, c, l, u
@@ -986,7 +986,7 @@ __device__ __forceinline__ bool il_running(const FamIL<V>& a, int m0, int (&run)
   return any != 0;
 }
 
-// k: the iteration within the chunk
+// k: the iteration among those whose step scalars are laid out
 template <typename V>
 __global__ void __launch_bounds__(IL_NT, 4) k_dual_il(FamIL<V> a, int k) {
   constexpr int W = IlVec<V>::W;
@@ -1102,8 +1102,6 @@ static void run_chunk_il(Work& w, int j0, int len, const V* Aval, const V* Pval,
   tin(ylo, m, m, I[IL_YLO]);
   const int groups = ld / (32 * IlVec<V>::W);
   V* steps = sizeof(V) == 4 ? (V*)w.il_steps_f : (V*)w.il_steps_d;
-  launch(k_il_steps<V>, dim3(cdiv(ld, 128), len), 128, 0, s, (const StepEntry*)w.tab, w.tab_stride,
-         (const int*)w.il_slot, ld, j0, steps);
   FamIL<V> da{};
   da.rp = w.A.rp; da.col = w.A.col; da.val = Aval;
   da.rows = m; da.ld = ld; da.steps = steps; da.slot = w.il_slot;
@@ -1114,17 +1112,21 @@ static void run_chunk_il(Work& w, int j0, int len, const V* Aval, const V* Pval,
   pa.rows = n; pa.ld = ld; pa.steps = steps; pa.slot = w.il_slot;
   pa.w0 = I[IL_X]; pa.w1 = I[IL_XBAR]; pa.w3 = I[IL_XT]; pa.r0 = I[IL_C]; pa.r1 = I[IL_L]; pa.r2 = I[IL_U];
   for (int j = j0; j < j0 + len; ++j) {
+    const int k = (j - j0) % IL_STEP_ITERS;
+    if (k == 0)
+      launch(k_il_steps<V>, dim3(cdiv(ld, 128), std::min(IL_STEP_ITERS, j0 + len - j)), 128, 0, s,
+             (const StepEntry*)w.tab, w.tab_stride, (const int*)w.il_slot, ld, j, steps);
     if (m > 0) {
       da.v0 = I[IL_Z0 + ((j + 1) & 1)] + (size_t)n * ld;   // y^k
       da.w0 = I[IL_Z0 + (j & 1)] + (size_t)n * ld;         // y^{k+1}
       if (Pr.on) Pr.begin(0, s, il_launch_bytes(w, 0, sizeof(V)));
-      launch_early(k_dual_il<V>, dim3(cdiv(m, IL_RPB), groups), IL_NT, 0, s, da, j - j0);
+      launch_early(k_dual_il<V>, dim3(cdiv(m, IL_RPB), groups), IL_NT, 0, s, da, k);
       if (Pr.on) Pr.end(s);
     }
     pa.zin = I[IL_Z0 + (j & 1)];
     pa.w2 = I[IL_Z0 + ((j + 1) & 1)];
     if (Pr.on) Pr.begin(1, s, il_launch_bytes(w, 1, sizeof(V)));
-    launch_early(k_primal_il<V>, dim3(cdiv(n, IL_RPB), groups), IL_NT, 0, s, pa, j - j0);
+    launch_early(k_primal_il<V>, dim3(cdiv(n, IL_RPB), groups), IL_NT, 0, s, pa, k);
     if (Pr.on) Pr.end(s);
   }
   // interleaved -> member-major: everything the iterations wrote

@@ -15,6 +15,10 @@ enum { IL_Z0 = 0, IL_Z1, IL_X, IL_XBAR, IL_XT, IL_YBAR, IL_C, IL_L, IL_U, IL_B, 
 // ... and of the family check (float64): the iterates and the row sums.
 enum { ILK_X0 = 0, ILK_X1, ILK_Y0, ILK_Y1, ILK_SA0, ILK_SA1, ILK_SQ0, ILK_SQ1, ILK_ST0, ILK_ST1, ILK_SLOTS };
 
+// Iterations whose step scalars a family's slots hold at a time (20 to 40 bytes each a
+// member: the whole of a long check period would outgrow the members' vectors).
+constexpr int IL_STEP_ITERS = 256;
+
 // Row blocks: every CUDA block of the SpMV kernels takes whole rows
 // [blk[b], blk[b+1]) holding at most BNNZ nonzeros and BROWS rows; a row longer
 // than BNNZ forms a block of its own.
@@ -234,7 +238,7 @@ struct Work {
   bool fam_il = false;                       // eligible: no long rows, no low-rank term
   double* ild[11] = {};                      // float64 (allocated on first use)
   float* ilf[11] = {};                       // float32
-  float* il_steps_f = nullptr;               // [check period][5][fam_ld] step scalars of a chunk, slot order
+  float* il_steps_f = nullptr;               // [il_steps_len][5][fam_ld] step scalars, slot order
   double* il_steps_d = nullptr;
   int il_steps_len[2] = {0, 0};              // iterations they hold (float64, mixed)
   int* il_slot = nullptr;                    // [fam_ld] member of each slot of the interleaved vectors, or -1
