@@ -125,8 +125,11 @@ typedef struct {
                                 members, so one matrix entry meets 128 members in one
                                 coalesced load,
                                 0 = chosen: 2 where every instance's vectors fit a
-                                CTA's shared memory and the instances are many or
-                                small (a family: up to 300 thousand rows in all); 3
+                                CTA's shared memory, the instances are many or
+                                small (a family: up to 300 thousand rows in all), no
+                                row is much longer than its neighbours and a second
+                                copy of the matrices takes at most half of the memory
+                                left; 3
                                 for the other eligible family handles; for a low-rank term
                                 over short rows of P (eight entries on average, none
                                 of more than 192), kernels that read the factor once
@@ -137,7 +140,8 @@ typedef struct {
                                 a large single problem without long rows, a row per
                                 thread on a second copy of the matrices (reported as
                                 5, which cannot be asked for; at most half of the free
-                                device memory, else left out), and
+                                device memory, else left out; given back where another
+                                variant is faster), and
                                 keeps the fastest for that precision; the choice is
                                 also kept for the process per problem shape, so later
                                 handles of the same sizes, nonzeros and row blocks
